@@ -586,10 +586,11 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
                                                        chunk[g], es));
     }
     const int per_sm = res_term + res_hand <= 200 * 1024 ? resident_blocks_per_sm(o.precision, res_term + res_hand) : 0;
-    if (per_sm < 1 || chunks_of(chunk[0]) > (long)per_sm * n_sms) {
+    const long chunks = chunks_of(chunk[0]);  // reads the handle's games
+    if (per_sm < 1 || chunks > (long)per_sm * n_sms) {
       delete t;
       return fail(CFR_EINVAL, "the resident schedule needs every chunk of hands resident at once (" +
-                                  std::to_string(chunks_of(chunk[0])) + " chunks, " + std::to_string(per_sm * n_sms) +
+                                  std::to_string(chunks) + " chunks, " + std::to_string(per_sm * n_sms) +
                                   " blocks fit)");
     }
   }
