@@ -151,7 +151,7 @@ int launch_terminals(const cfr_tree* t, int player_mask, int use_bar, cudaStream
 
 // Kernels one terminal stage launches.
 int terminal_launches(const cfr_tree* t) {
-  return (t->ctx.n_term_work > 0 ? 1 : 0) + (t->ro_n8 > 0 ? 1 : 0) + (t->ro_n16 > 0 ? 1 : 0);
+  return (t->ctx.n_term_work > 0 ? 1 : 0) + (t->ro_n8 + t->ro_n16 > 0 ? 1 : 0);
 }
 
 // One device block for every subgame's tables and state: the tables are staged on the host
@@ -726,7 +726,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   for (int g = 0; g < n_games; ++g) t->dev[g].br_out = t->d_br_all + 2 * g;
   if (!ro.tables.empty()) {  // the run-out tables, from each showdown board's tie groups
     const HostGame& h = t->host[0];
-    // tops sorted by table, in groups of up to kRunoutGroup that share a table (one block each)
+    // tops sorted by table, in groups of up to kRunoutGroup that share a table
     std::vector<RunoutItem> items;
     std::vector<RunoutGroup> groups[2];
     for (const std::vector<RunoutItem>* list : {&ro.items8, &ro.items16}) {

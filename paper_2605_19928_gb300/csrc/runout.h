@@ -33,7 +33,7 @@ struct RunoutTable {  // E of one run-out board, stored [o][hstride] as unsigned
   int32_t pad;
 };
 
-struct RunoutGroup {  // up to kRunoutGroup top nodes of one table, evaluated by one block
+struct RunoutGroup {  // up to kRunoutGroup top nodes of one table, evaluated together
   int32_t table;
   int32_t item0;      // its first item (items sorted by table)
   int32_t count;
@@ -55,7 +55,7 @@ int launch_runout_build(const RunoutTable* tables, int n_tables, const RunoutBoa
 // Values of the players in player_mask (1, 2 or 3) at every run-out top node of game 0, from
 // the opponent's reach (use_bar: the average-strategy reach, into cfv_br), FP32 values.  The
 // groups8 use uint8 tables, groups16 uint16 ones; items are the top nodes, sorted by table.
-// One launch per non-empty group list.
+// One launch (none without groups).
 int launch_runout_values(const GameDev* games, const RunoutItem* items, const RunoutGroup* groups8, int n8,
                          const RunoutGroup* groups16, int n16, const RunoutTable* tables, const unsigned char* pool,
                          int n_hands, int player_mask, int use_bar, void* stream);
