@@ -130,10 +130,11 @@ typedef struct cfr_game_spec {
  * average-strategy sums S are FP64 in both.
  * schedule: how the update launch (Stages 1, 6 and 7 of one player) is laid out; results
  * are the same bits either way.  CFR_SCHEDULE_LEVEL: one CUDA block per chunk_hands hands
- * walks the tree level by level (lowest latency for one subgame).  CFR_SCHEDULE_STREAM: one
- * warp per 32 hands walks a depth-first program of its tree with no block barriers and no
- * inner-node state in DRAM (highest throughput for batches; needs at most 8 actions per
- * decision node; warp_hands sets 32 or 64 hands per warp).  CFR_SCHEDULE_WIDE: every pass (update, initial strategy, average, best
+ * walks the tree level by level (lowest latency for one subgame).  CFR_SCHEDULE_STREAM: for
+ * batches (highest throughput; needs at most 8 actions per decision node): one block per tile
+ * of 8 to 32 hands keeps its subgame's values, strategy and reach in shared memory and streams R
+ * and S; where a tree is too large for a tile, or warp_hands is 64, or chunk_hands is above 8, one
+ * warp per 32 (or 64) hands walks a depth-first program of its tree instead.  CFR_SCHEDULE_WIDE: every pass (update, initial strategy, average, best
  * response) is one launch per tree level over all of that level's (node, hand) pairs, one
  * thread each (for one tree too large for a block to stage in shared memory: exact turns
  * and flops; one subgame per handle, at most 8 actions per decision node).
@@ -149,13 +150,14 @@ typedef struct cfr_game_spec {
  * CFR_ETIMEOUT and the handle's state is undefined.
  * CFR_SCHEDULE_AUTO (0) picks STREAM when the handle has at least 1216 such warps (8 per
  * SM) and every tree allows it, WIDE for one subgame too large to stage, else LEVEL.
- * term_nodes: fold and showdown nodes per CUDA block of the terminal launch (nodes of one
- * board; 0 = automatic: one while the nodes do not fill the GPU eight times over, up to
- * eight when they do; otherwise 1 to 8).  Results are the same bits for every value.
- * warp_hands: hands per warp of the stream schedule's update launch: 32 (one per lane), 64
- * (two per lane: the walk's control work is shared by two hands; needs every subgame's
- * hand rows padded to a multiple of 64, i.e. the hand count rounded up to 32 is a multiple
- * of 64, CFR_EINVAL otherwise), or 0 = automatic (32; cfr_autotune tries both).  Other
+ * term_nodes: fold and showdown nodes a block of the terminal launch evaluates together (nodes
+ * of one board and kind; 0 = automatic: one while the nodes do not fill the GPU many times over,
+ * four when they do -- two with pair values; otherwise 1 to 8, of which at most those many are
+ * taken).  Results are the same bits for every value.
+ * warp_hands: 64 asks the stream schedule for its one-warp walk with two hands per lane (needs
+ * every subgame's hand rows padded to a multiple of 64, i.e. the hand count rounded up to 32 is a
+ * multiple of 64, CFR_EINVAL otherwise); 0 (automatic) and 32: hand tiles, or the walk with one
+ * hand per lane where they do not apply (cfr_autotune tries 32 and 64).  Other
  * schedules ignore it.  Results are the same bits either way.
  * runout_tables: 1 evaluates every all-in run-out -- a chance node below a decision whose
  * subtree holds only chance and showdown nodes (nobody acts again) -- in one step instead of

@@ -24,6 +24,9 @@ using namespace pcfr;
 
 namespace {
 
+// Terminal nodes from which the launch evaluates them in groups (see create_impl).
+constexpr int kTermGroupMin = 152 * 16;
+
 thread_local std::string g_last_error;
 cfr_alloc_fn g_alloc = nullptr;
 cfr_free_fn g_free = nullptr;
@@ -52,11 +55,13 @@ struct cfr_tree {
   GameDev* d_games = nullptr;
   Work* d_chunk_work = nullptr;
   Work* d_term_work = nullptr;
-  Work* d_term_runs = nullptr;
+  TermGroup* d_term_groups = nullptr;
+  Work* d_term_segments = nullptr;
   Work* d_warp_work = nullptr;
+  Work* d_tile_work = nullptr;
   int32_t* d_wide_inner = nullptr;  // wide schedule: inner node ids, level by level
   int32_t* d_wide_fwd = nullptr;    // wide schedule: nodes whose reach is stored, level by level
-  int32_t* d_term_src = nullptr;    // reach source of each terminal work entry
+  TermSrc* d_term_src = nullptr;    // reach rows of each terminal work entry
   // all-in run-outs evaluated by win-minus-loss tables (runout_tables; none: all zero)
   RunoutItem* d_ro_items = nullptr;   // top nodes, sorted by table
   RunoutGroup* d_ro_groups8 = nullptr;
@@ -94,6 +99,14 @@ struct cfr_tree {
   int device = -1;              // the device current when the handle was created
   std::vector<std::pair<void*, bool>> blocks;  // (pointer, from hook)
   void* stream_arg = nullptr;
+
+  // The node whose reach row of player p the terminal and leaf launches read for node n.  The one-
+  // warp walk of the stream schedule stores no rows at the opponent's decision nodes, so only an
+  // all-in run-out's rows are shared there.
+  int reach_row(int g, int p, int n) const {
+    const HostGame& h = host[(size_t)g];
+    return ctx.schedule == kScheduleStream && ctx.n_tile_work == 0 ? h.reach_src[(size_t)n] : h.reach_row[p][(size_t)n];
+  }
 
   void* alloc(size_t bytes) {
     bytes = (bytes + 255) / 256 * 256;
@@ -319,6 +332,7 @@ int setup_leaves(cfr_tree* t, const cfr_game_spec* specs, int n_games) {
       LeafDev lf{};
       lf.game = g;
       lf.node = n;
+      for (int p = 0; p < 2; ++p) lf.src[p] = t->reach_row(g, p, n);
       lf.row0 = (int)t->leaf_host.size() * kLeafCards;
       const double pot = h.contrib[2 * (size_t)n] + h.contrib[2 * (size_t)n + 1];
       const double behind = cap - h.contrib[2 * (size_t)n];
@@ -456,7 +470,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   };
   int res_W = 8;
   while (resident && !o.chunk_hands && res_W < 32 && chunks_of(res_W) > n_sms) res_W *= 2;
-  size_t smem_hand = 0, smem_term = 0;
+  size_t smem_hand = 0;
   std::vector<int> chunk(n_games);
   std::vector<int> use_smem(n_games);
   bool all_fit = true;
@@ -469,9 +483,6 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const HostGame& h = t->host[g];
     use_smem[g] = all_fit;
     if (all_fit) smem_hand = std::max(smem_hand, hand_smem(h, chunk[g], es));
-    const TermTab tt(h.n_hands, h.hand_size, h.deck);
-    smem_term = std::max(smem_term, (size_t)tt.len * 2 + 2 * (size_t)h.hstride * es +
-                                        (size_t)(h.hand_size * h.n_hands + 1 + h.n_hands + 1) * 8);
   }
 
   // Update schedule: one warp per 32 hands when the handle has enough of them to fill the
@@ -562,6 +573,37 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   } else if (o.schedule == CFR_SCHEDULE_AUTO && schedule == kScheduleLevel && wide_ok && !all_fit) {
     schedule = kScheduleWide;
   }
+  // Hand tiles: the stream schedule's passes as k_tile, when every tree's values and strategy fit a
+  // tile of 8 hands.  Each subgame takes the widest of 32, 16 and 8 hands that fits (32 keeps a warp
+  // on one node; the narrower ones give larger trees the same shared memory): in the eighth of an
+  // SM that a block of 128 threads has, or, where a tree is too large for that or values are
+  // pairs, in the quarter of a block of 256.  warp_hands = 64 asks for the one-warp walk, and
+  // chunk_hands beyond 8 for best-response sums a tile cannot form.
+  bool tiles = schedule == kScheduleStream && o.warp_hands != 64 && chunk[0] <= 8;
+  std::vector<std::vector<uint16_t>> tile_tabs(n_games);
+  std::vector<int> tile_wlog(n_games, 0);
+  size_t smem_tile = 0;
+  int tile_threads = 0;
+  if (tiles) parallel_games(n_games, [&](int g) { tile_tabs[g] = tile_table(t->host[g]); });
+  for (int small = es == 4; tiles && small >= 0 && !tile_threads; --small) {
+    const size_t limit = small ? kTileSmemSmall : kTileSmem;
+    bool fit = true;
+    smem_tile = 0;
+    for (int g = 0; g < n_games && fit; ++g) {
+      const HostGame& h = t->host[g];
+      const int rows_max = std::max(h.row_begin[1] - h.row_begin[0], h.row_begin[2] - h.row_begin[1]);
+      auto bytes = [&](int wl) {
+        return tile_smem_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, 1 << wl, es);
+      };
+      int wl = 5;
+      while (wl > 3 && bytes(wl) > limit) --wl;
+      fit = !tile_tabs[g].empty() && bytes(wl) <= limit;
+      tile_wlog[g] = wl;
+      smem_tile = std::max(smem_tile, bytes(wl));
+    }
+    if (fit) tile_threads = small ? 128 : 256;
+  }
+  tiles = tile_threads > 0;
   RunoutPlan ro;
   if (o.runout_tables) {
     if (schedule != kScheduleWide || t->host[0].hand_size != 2) {
@@ -615,12 +657,21 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     }
   }
 
+  // Terminal nodes a block evaluates together: one while they do not fill the GPU many times over
+  // (a block per node then has the lower latency), else groups of four (two with pair values:
+  // 16-byte entries either way).
+  int n_ends = 0;
+  for (int g = 0; g < n_games; ++g)
+    for (int n : t->host[g].terminals) n_ends += ro.inside.empty() || !ro.inside[(size_t)n];
+  const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= kTermGroupMin ? 4 : 1;
+  const int term_nv = term_nodes == 1 ? 1 : term_nodes < 4 || es == 8 ? 2 : 4;
+
   std::vector<Work> chunk_work, term_work, warp_work;
   // each game's device tables, prepared on the host in parallel, then packed in game order
   struct Prepared {
     std::vector<double> r64;
     std::vector<float> rv, pay32;
-    std::vector<uint16_t> tab;
+    std::vector<uint16_t> tab, rec, tile;
     std::vector<int32_t> rown, decn;
     std::vector<ProgOp> ops;
     int dec_begin[3];
@@ -635,6 +686,8 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       for (int k = 0; k < h.n_hands; ++k) q.r64[p * S + k] = h.range[p][k];
     q.rv = to_value_type(q.r64, o.precision);
     q.tab = pack_term_tables(h);
+    if (term_nv > 1) q.rec = pack_term_records(h);
+    if (tiles) q.tile = std::move(tile_tabs[g]);
     q.rown = row_nodes(h);
     q.decn = decision_nodes(h, q.dec_begin);
     const double kappa = 1.0 / h.Z;
@@ -692,6 +745,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     packer.table(h.payoff, &d.payoff);
     packer.table(pay32, &d.payoff_ff);
     packer.table(tab, &d.term_tab);
+    packer.table(q.rec, &d.term_rec);
+    packer.table(q.tile, &d.tile_tab);
+    d.tile_tab16 = (int)q.tile.size() / 8;
+    d.tile_wlog = tile_wlog[g];
     packer.table(decn, &d.dec_nodes);
     packer.table(ops, &d.prog);
     packer.table(chunk_lists[g], &d.chunks);
@@ -711,12 +768,14 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     packer.zeroed(4, &d.br_done);
     for (int c = 0; c < d.n_chunks; ++c) chunk_work.push_back({g, c});
 
-    // terminals grouped by board table (fold nodes read only the board-free part of table 0)
+    // terminals grouped by board table (fold nodes read only the board-free part of table 0) and
+    // kind
     std::vector<int> term;
     for (int n : h.terminals)
       if (ro.inside.empty() || !ro.inside[(size_t)n]) term.push_back(n);  // run-outs: by their tables
     auto table = [&](int n) { return h.nodes[(size_t)n].type == kShowdown ? h.nodes[(size_t)n].row : 0; };
-    std::stable_sort(term.begin(), term.end(), [&](int a, int b2) { return table(a) < table(b2); });
+    auto key = [&](int n) { return 2 * table(n) + (h.nodes[(size_t)n].type == kShowdown); };
+    std::stable_sort(term.begin(), term.end(), [&](int a, int b2) { return key(a) < key(b2); });
     for (int n : term) term_work.push_back({g, n});
   }
   if ((rc = packer.commit(t))) {
@@ -748,7 +807,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       delete t;
       return rc;
     }
-    t->d_ro_pool = static_cast<unsigned char*>(t->alloc(ro.pool_bytes));
+    t->d_ro_pool = static_cast<unsigned char*>(t->alloc(ro.pool_bytes + (size_t)kRunoutPadRows * h.hstride * 2));
     if (!t->d_ro_pool) {
       delete t;
       return fail(CFR_ENOMEM, "device allocation failed");
@@ -761,43 +820,87 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     t->ro_n8 = (int)groups[0].size();
     t->ro_n16 = (int)groups[1].size();
   }
-  std::vector<int32_t> term_src(term_work.size());
+  t->ctx.schedule = schedule;
+  t->ctx.n_tile_work = tiles;  // its count below
+  std::vector<TermSrc> term_src(term_work.size());
   for (size_t k = 0; k < term_work.size(); ++k)
-    term_src[k] = t->host[term_work[k].game].reach_src[(size_t)term_work[k].unit];
-  // terminal runs: one node per block while the nodes do not fill the GPU many times over,
-  // up to eight per block (same game and board table) when they do
-  std::vector<Work> term_runs;
-  {
-    const int per = o.term_nodes ? o.term_nodes : std::max(1, std::min(8, (int)term_work.size() / (152 * 8)));
-    size_t a = 0;
-    while (a < term_work.size()) {
-      const Work w = term_work[a];
+    for (int p = 0; p < 2; ++p) {
+      const HostGame& h = t->host[term_work[k].game];
+      const int n = term_work[k].unit, row = t->reach_row(term_work[k].game, p, n);
+      term_src[k].row[p] = h.nodes[(size_t)row].board == h.nodes[(size_t)n].board ? row : ~row;
+    }
+  // grouped terminal launch: groups of up to term_nv nodes of one game, board table and kind, and
+  // each block's stretch of them -- two blocks per SM, equal shares of the work (a showdown group
+  // costs about twice a fold group with FP32 values, the same with pairs)
+  std::vector<TermGroup> term_groups;
+  std::vector<Work> term_segments;
+  if (term_nv > 1) {
+    auto key = [&](const Work& w) {
       const NodeDev& nd = t->host[w.game].nodes[(size_t)w.unit];
-      const int tb = nd.type == kShowdown ? nd.row : 0;
-      int cnt = 1;
-      while (cnt < per && a + cnt < term_work.size()) {
-        const Work w2 = term_work[a + cnt];
-        const NodeDev& n2 = t->host[w2.game].nodes[(size_t)w2.unit];
-        if (w2.game != w.game || (n2.type == kShowdown ? n2.row : 0) != tb) break;
-        ++cnt;
+      return nd.type == kShowdown ? nd.row : -1;
+    };
+    for (size_t a = 0; a < term_work.size();) {
+      TermGroup q{};
+      const Work w0 = term_work[a];
+      const HostGame& h = t->host[w0.game];
+      q.game = w0.game;
+      q.kind = h.nodes[(size_t)w0.unit].type;
+      q.table = q.kind == kShowdown ? h.nodes[(size_t)w0.unit].row : 0;
+      for (; q.count < term_nv && a < term_work.size(); ++a, ++q.count) {
+        const Work w = term_work[a];
+        if (w.game != w0.game || key(w) != key(w0)) break;
+        const NodeDev& nd = h.nodes[(size_t)w.unit];
+        q.node[q.count] = w.unit;
+        q.src[q.count] = term_src[a];
+        for (int p = 0; p < 2; ++p) q.below |= (term_src[a].row[p] < 0) << p;
+        q.board[q.count] = nd.board;
+        for (int i = 0; i < 2; ++i) {
+          const float* pay = &prep[w.game].pay32[2 * (size_t)w.unit];
+          const bool neg = nd.type == kFold && nd.player == i;
+          q.pay[i][q.count] = {neg ? -pay[0] : pay[0], neg ? -pay[1] : pay[1]};
+        }
       }
-      term_runs.push_back({(int)a, cnt});
-      a += cnt;
+      for (int v = q.count; v < term_nv; ++v) {  // a short group repeats its last node, unwritten
+        const int last = q.count - 1;
+        q.node[v] = q.node[last];
+        q.src[v] = q.src[last];
+        q.board[v] = q.board[last];
+      }
+      term_groups.push_back(q);
+    }
+    auto cost = [&](const TermGroup& q) { return es == 4 && q.kind == kFold ? 1 : 2; };
+    long total = 0, done = 0, cut = 0;
+    for (const TermGroup& q : term_groups) total += cost(q);
+    const long share = (total + 2 * n_sms - 1) / (2 * n_sms);
+    for (size_t a = 0; a < term_groups.size(); ++a) {
+      if (term_segments.empty() || done >= cut || term_segments.back().unit == kTermSegment) {
+        term_segments.push_back({(int)a, 0});
+        cut = done + share;
+      }
+      term_segments.back().unit += 1;
+      done += cost(term_groups[a]);
     }
   }
+  size_t smem_term = 0;
+  for (const HostGame& h : t->host)
+    smem_term = std::max(smem_term, terminal_smem_size(h.n_hands, h.hand_size, h.deck, h.hstride, es, term_nv));
   // stream schedule: blocks of kStreamWarps warps of one game, largest trees first so that
   // their long walks start at once and the small trees fill in behind them
   std::vector<int> by_size(n_games);
   for (int g = 0; g < n_games; ++g) by_size[g] = g;
   std::stable_sort(by_size.begin(), by_size.end(),
                    [&](int a, int b) { return t->host[a].nodes.size() > t->host[b].nodes.size(); });
+  std::vector<Work> tile_work;
+  for (int g : by_size)
+    for (int u = 0; tiles && u << tile_wlog[g] < t->host[g].n_hands; ++u) tile_work.push_back({g, u});
   const int warp_span = 32 * stream_hp;
   for (int g : by_size)
     for (int u = 0; u < (t->host[g].n_hands + warp_span - 1) / warp_span; u += kStreamWarps) warp_work.push_back({g, u});
   if ((rc = upload(t, t->dev, &t->d_games)) || (rc = upload(t, chunk_work, &t->d_chunk_work)) ||
       (rc = upload(t, term_work, &t->d_term_work)) || (rc = upload(t, warp_work, &t->d_warp_work)) ||
       (rc = upload(t, term_src, &t->d_term_src)) ||
-      (rc = upload(t, term_runs, &t->d_term_runs)) ||
+      (rc = upload(t, term_groups, &t->d_term_groups)) || (rc = upload(t, term_segments, &t->d_term_segments)) ||
+      (rc = upload(t, tile_work, &t->d_tile_work)) ||
       (rc = zeros(t, 1, &t->d_iter)) ||
       (rc = zeros(t, 1, &t->d_done)) || (rc = zeros(t, 1, &t->d_err)) || (rc = zeros(t, 2, &t->d_res_sync)) ||
       (rc = upload(t, discount_table(o, kDiscountCapacity), &t->d_disc))) {
@@ -812,8 +915,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.term_work = t->d_term_work;
   c.term_src = t->d_term_src;
   c.n_term_work = (int)term_work.size();
-  c.term_runs = t->d_term_runs;
-  c.n_term_runs = (int)term_runs.size();
+  c.term_groups = t->d_term_groups;
+  c.term_segments = t->d_term_segments;
+  c.n_term_segments = (int)term_segments.size();
+  c.term_nv = term_nv;
   c.iter = t->d_iter;
   c.done = t->d_done;
   c.err = t->d_err;
@@ -827,6 +932,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.schedule = schedule;
   c.warp_work = t->d_warp_work;
   c.n_warp_work = (int)warp_work.size();
+  c.tile_work = t->d_tile_work;
+  c.n_tile_work = (int)tile_work.size();
+  c.smem_tile = smem_tile;
+  c.tile_threads = tile_threads;
   c.stream_depth = stream_depth;
   c.stream_prog = stream_prog;
   c.stream_half = stream_half;
@@ -1188,8 +1297,8 @@ int cfr_read_values(cfr_tree* t, int game, int what, int player, int node, doubl
     const size_t vf = t->opts.precision == CFR_PRECISION_SINGLE ? 1 : 2;
     std::vector<float> tmp((size_t)H * vf);
     const void* arr = what == CFR_READ_CFV ? d.cfv : what == CFR_READ_BR_CFV ? d.cfv_br : d.reach_bar;
-    // a run-out node's reach is its source's with the hands holding a dealt card zeroed
-    const int at = what == CFR_READ_AVG_REACH ? h.reach_src[(size_t)node] : node;
+    // a node's reach is its source row's with the hands holding a dealt card zeroed
+    const int at = what == CFR_READ_AVG_REACH ? h.reach_row[player][(size_t)node] : node;
     const float* src = static_cast<const float*>(arr) + ((size_t)player * h.nodes.size() + at) * S * vf;
     CK(cudaMemcpyAsync(tmp.data(), src, (size_t)H * 4 * vf, cudaMemcpyDeviceToHost, t->stream));
     CK(cudaStreamSynchronize(t->stream));

@@ -42,9 +42,7 @@ constexpr int kTermThreads = 512;
 // Dekker's exact product.  The _rn intrinsics stop the compiler from contracting or
 // reassociating the error terms.
 
-struct ff {
-  float hi, lo;
-};
+using ff = PairF;  // (hi, lo)
 
 __device__ __forceinline__ ff ff_of(float x) { return {x, 0.f}; }
 __device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
@@ -134,12 +132,11 @@ __device__ __forceinline__ bool ff_gt(ff a, ff b) { return a.hi > b.hi || (a.hi 
 // Exact float -> double by exponent rebias on the integer pipe (IEEE 754 binary32 ->
 // binary64; subnormal floats, below 1.2e-38, become zero).
 __device__ __forceinline__ double f2d(float f) {
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t e = (u >> 23) & 0xffu;
-  const uint64_t sign = (uint64_t)(u & 0x80000000u) << 32;
-  if (e == 0u) return __longlong_as_double((long long)sign);
-  const uint64_t ed = e == 0xffu ? 0x7ffu : (uint64_t)(e + 896u);
-  return __longlong_as_double((long long)(sign | (ed << 52) | ((uint64_t)(u & 0x7fffffu) << 29)));
+  const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+  uint32_t hi = (a >> 3) + 0x38000000u, lo = u << 29;  // exponent + 896, mantissa up by 29 bits
+  if (a >= 0x7f800000u) hi += 0x38000000u;             // infinity and NaN: exponent 0x7ff
+  if (a < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
 }
 __device__ __forceinline__ ff d2ff(double x) {
   const float hi = __double2float_rn(x);
@@ -171,6 +168,7 @@ struct Pairs {  // double-float values
   static __device__ __forceinline__ double to_double(V a) { return ff2d(a); }
   static __device__ __forceinline__ ff to_ff(V a) { return a; }
   static __device__ __forceinline__ V of_ff(ff a) { return a; }
+  static __device__ __forceinline__ V scale(ff u) { return u; }  // a payoff scale as a value
   using Acc = acc2;
   static __device__ __forceinline__ Acc acc0() { return acc_zero(); }
   static __device__ __forceinline__ void acc(Acc& a, V x) { acc_add(a, x); }
@@ -194,6 +192,7 @@ struct Single {  // plain FP32 values
   static __device__ __forceinline__ double to_double(V a) { return f2d(a); }
   static __device__ __forceinline__ ff to_ff(V a) { return ff_of(a); }
   static __device__ __forceinline__ V of_ff(ff a) { return ff_round(a); }
+  static __device__ __forceinline__ V scale(ff u) { return u.hi; }
   using Acc = float;
   static __device__ __forceinline__ Acc acc0() { return 0.f; }
   static __device__ __forceinline__ void acc(Acc& a, V x) { a = __fadd_rn(a, x); }
@@ -551,104 +550,401 @@ __device__ __forceinline__ void terminal_values(const GameDev& G, const NodeDev&
   }
 }
 
-// Terminal values (Stages 2-4).  One block per (player, run): a run is up to eight fold or
-// showdown nodes of one game that read the same board table, which is staged once by a
-// bulk (TMA) copy; the opponent reach rows of the run's nodes arrive by bulk copies into
-// two alternating buffers, each node's row landing while the node before it computes.  A
+// The player of a block of the terminal launch and its item of n (grid: (player, item)).
+__device__ __forceinline__ int terminal_item(int n, int player_mask, int& i) {
+  if (player_mask != 3) {
+    i = player_mask == 1 ? 0 : 1;
+    return blockIdx.x;
+  }
+  i = (int)blockIdx.x >= n;
+  return blockIdx.x - i * n;
+}
+
+// Payoff for player i per unit of (opponent reach) x kappa at node n: the FP64 product as a pair
+// of FP32 rounded once on the host (FP32 values use its high part): no FP64 work per thread.
+__device__ __forceinline__ ff terminal_payoff(const GameDev& G, const NodeDev& nd, int n, int i) {
+  const bool neg = nd.type == kFold && nd.player == i;
+  return {neg ? -G.payoff_ff[2 * n] : G.payoff_ff[2 * n], neg ? -G.payoff_ff[2 * n + 1] : G.payoff_ff[2 * n + 1]};
+}
+
+// Terminal values (Stages 2-4), the one-node form for handles with few terminals (latency: all
+// registers it wants).  One block per (player, node): the board table is staged by a bulk (TMA)
+// copy before the launch waits for its predecessor, the opponent's reach row after it.  A
 // showdown below an all-in run-out reads the run-out's reach row (src) and zeroes the hands
 // holding a dealt card itself (nobody acts below the run-out, so that is its reach).
-// Every wait is bounded: on a timeout the block sets *err, lets its copies drain and leaves.
-// RUNS = false is the one-node form (latency: all registers it wants); RUNS = true fits four
-// blocks per SM for handles whose terminal nodes fill the GPU many times over.
-template <typename P, bool RUNS>
-__global__ void __launch_bounds__(kTermThreads, RUNS ? 4 : 1) k_terminal(const GameDev* __restrict__ games,
+// The wait is bounded: on a timeout the block sets *err, lets its copies drain and leaves.
+template <typename P>
+__global__ void __launch_bounds__(kTermThreads, 1) k_terminal(const GameDev* __restrict__ games,
                                                             const Work* __restrict__ work,
-                                                            const int32_t* __restrict__ src,
-                                                            const Work* __restrict__ runs, int n_runs,
+                                                            const TermSrc* __restrict__ src, int n_work,
                                                             int player_mask, int use_bar, int* err) {
   using V = typename P::V;
-  int item = blockIdx.x;
   int i;
-  if (player_mask == 3) {
-    i = item >= n_runs;
-    item -= i * n_runs;
-  } else {
-    i = player_mask == 1 ? 0 : 1;
-  }
-  const Work run = runs[item];  // (first entry of `work`, count)
-  const int first = run.game, count = RUNS ? run.unit : 1;
+  const int first = terminal_item(n_work, player_mask, i);
   const GameDev& G = games[work[first].game];
+  const int n = work[first].unit;
+  const NodeDev nd = G.nodes[n];
   const int H = G.n_hands, k = G.hand_size;
   const size_t stride = (size_t)G.hstride;
   const TermTab tt(H, k, G.deck);
-  bool show_any = false;
-  int b = 0;
-  for (int j = 0; j < count; ++j) {
-    const NodeDev nd = G.nodes[work[first + j].unit];
-    if (nd.type == kShowdown) show_any = true, b = nd.row;
-  }
-  const unsigned tab_bytes = (unsigned)(show_any ? tt.len : tt.fold_len) * 2u;
+  const bool show = nd.type == kShowdown;
+  const unsigned tab_bytes = (unsigned)(show ? tt.len : tt.fold_len) * 2u;
   const unsigned q_bytes = (unsigned)(stride * sizeof(V));
   const V* qsrc = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + (size_t)(1 - i) * G.n_nodes * stride;
   V* dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
 
   extern __shared__ __align__(128) unsigned char smt[];
-  __shared__ __align__(8) uint64_t bar[2];
-  uint16_t* tab = reinterpret_cast<uint16_t*>(smt);                                // [tt.len]
-  V* qbuf = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);                         // [2][hstride]
-  ff* CP = reinterpret_cast<ff*>(smt + (size_t)tt.len * 2 + 2 * (size_t)q_bytes);   // [k H + 1]
-  ff* Psc = CP + (k * H + 1);                                                       // [H + 1]
+  __shared__ __align__(8) uint64_t bar;
+  uint16_t* tab = reinterpret_cast<uint16_t*>(smt);                            // [tt.len]
+  V* q = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);                        // [hstride]
+  ff* CP = reinterpret_cast<ff*>(smt + (size_t)tt.len * 2 + (size_t)q_bytes);   // [k H + 1]
+  ff* Psc = CP + (k * H + 1);                                                   // [H + 1]
 
   if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {  // the board tables are static: copy them before waiting
+    mbar_arrive_expect_tx(&bar, tab_bytes + q_bytes);
+    bulk_copy_g2s(tab, G.term_tab + (size_t)(show ? nd.row : 0) * tt.len, tab_bytes, &bar);
+  }
+  pdl_wait();  // the reach rows come from the launch just before this one
+  pdl_trigger();
+  const int from = src[first].row[1 - i];
+  if (threadIdx.x == 0) bulk_copy_g2s(q, qsrc + (size_t)term_src_node(from) * stride, q_bytes, &bar);
+  const ff u = terminal_payoff(G, nd, n, i);
+  const bool ok = threadIdx.x >= 32 || mbar_wait_bounded(&bar, 0, g_first_wait_polls);  // one warp polls
+  if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
+    if (threadIdx.x == 0) {
+      atomicExch(err, 1);
+      mbar_wait_bounded(&bar, 0);
+    }
+    __syncthreads();
+    return;
+  }
+  if (from < 0) {  // below an all-in run-out: the run-out's reach, without the hands holding
+    for (int h = threadIdx.x; h < H; h += blockDim.x)  // a card dealt on the way
+      if (holds_board_card(tab + tt.cards, h, k, nd.board)) q[h] = P::zero();
+    __syncthreads();
+  }
+  terminal_values<P>(G, nd, i, u, tt, tab, q, CP, Psc, dst + (size_t)n * stride);
+}
+
+// ---- several nodes at once: the throughput form for handles whose terminals fill the GPU
+//
+// A group is up to NV nodes of one game, one kind (folds or showdowns) and one board table.  The
+// scan arrays of terminal_values become arrays of NV values (16 bytes), so each table entry and
+// each address is read and computed once for NV nodes and a gather is one 16-byte shared-memory
+// access.  Component v runs exactly the one-node form's operations in its order (the same runs
+// of entries per thread, the same combination of threads and warps), so the bits are the same.
+//
+// Blocks are persistent: two per SM, each walking its own contiguous stretch of the groups, so
+// that the board table is reloaded only when it changes, descriptors are staged once, and the
+// reach rows of the next group are in flight (bulk copies, two buffers) while the current one
+// is computed.  A showdown group takes three block barriers: rows landed; each thread has
+// gathered its run of entries into registers and summed it; the prefix sums are written.
+// Bound by random shared-memory gathers (5060 wavefronts a group of four, 45 % of the pipe's rate).
+// Measured against blocks that take their nodes one by one: exact turn 119 -> 88 us per player,
+// 256 rivers 132 -> 129, with one block per group and its descriptors read node by node 147.
+
+// Entries of a thread's run at most, for the 1176 hands a flop leaves: 1176 over 160 threads (8) and
+// 2352 over 352 (7) with FP32 values, 2352 over 256 (10) with pairs.
+template <typename P>
+struct ScanPer {
+  static constexpr int n = std::is_same<P, Single>::value ? 8 : 10;
+};
+
+template <typename P, int NV>
+struct alignas(NV * sizeof(typename P::V)) Vec {
+  typename P::V v[NV];
+};
+template <typename P, int NV>
+struct alignas(16) VecAcc {  // running sums: FP32, or compensated pairs
+  typename P::Acc v[NV];
+};
+__device__ __forceinline__ float acc_up(float a, int o) { return __shfl_up_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ acc2 acc_up(acc2 a, int o) { return acc_shfl_up(a, o); }
+__device__ __forceinline__ float acc_from(float a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ acc2 acc_from(acc2 a, int l) {
+  return {__shfl_sync(0xffffffffu, a.s, l), __shfl_sync(0xffffffffu, a.e, l)};
+}
+__device__ __forceinline__ void acc_join(float& a, float b) { a = __fadd_rn(a, b); }
+__device__ __forceinline__ void acc_join(acc2& a, acc2 b) { acc_merge(a, b); }
+
+// One thread's part of group_exclusive_scan(_f32) over NV arrays: its run's values are in
+// registers (a[0 .. cnt)), x receives the inclusive sum of its warp's runs up to its own, and the
+// warp's total goes to red[warp].
+template <typename P, int NV>
+__device__ __forceinline__ void scan_runs(const Vec<P, NV> (&a)[ScanPer<P>::n], int cnt, VecAcc<P, NV>* red, int gtid,
+                                          VecAcc<P, NV>& x) {
+  const int lane = gtid & 31;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) x.v[v] = P::acc0();
+#pragma unroll
+  for (int e = 0; e < ScanPer<P>::n; ++e)
+    if (e < cnt) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) P::acc(x.v[v], a[e].v[v]);
+    }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const typename P::Acc y = acc_up(x.v[v], o);
+      if (lane >= o) acc_join(x.v[v], y);
+    }
+  if (lane == 31) red[gtid >> 5] = x;
+}
+
+// After the barrier: the exclusive prefix sums of the thread's run into out (out[n] = totals).
+// Every warp scans the GT / 32 warp totals itself, as the one-node form's first warp does.
+template <typename P, int NV, int GT>
+__device__ __forceinline__ void scan_write(const Vec<P, NV> (&a)[ScanPer<P>::n], int begin, int cnt, int n,
+                                           const VecAcc<P, NV>* red, int gtid, const VecAcc<P, NV>& x,
+                                           Vec<P, NV>* out) {
+  const int lane = gtid & 31, warp = gtid >> 5;
+  VecAcc<P, NV> run;
+  Vec<P, NV> total;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    typename P::Acc w = lane < GT / 32 ? red[lane].v[v] : P::acc0();
+#pragma unroll
+    for (int o = 1; o < GT / 32; o <<= 1) {
+      const typename P::Acc y = acc_up(w, o);
+      if (lane >= o) acc_join(w, y);
+    }
+    run.v[v] = acc_up(x.v[v], 1);
+    if (lane == 0) run.v[v] = P::acc0();
+    const typename P::Acc before = acc_from(w, max(warp - 1, 0));
+    if (warp > 0) acc_join(run.v[v], before);
+    total.v[v] = P::value(acc_from(w, GT / 32 - 1));
+  }
+#pragma unroll
+  for (int e = 0; e < ScanPer<P>::n; ++e)
+    if (e < cnt) {
+      Vec<P, NV> o;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        o.v[v] = P::value(run.v[v]);
+        P::acc(run.v[v], a[e].v[v]);
+      }
+      out[begin + e] = o;
+    }
+  if (gtid == 0) out[n] = total;
+}
+
+template <typename P, int NV>
+__global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev* __restrict__ games,
+                                                                const TermGroup* __restrict__ groups,
+                                                                const Work* __restrict__ segments, int n_segments,
+                                                                int player_mask, int use_bar, int* err) {
+  using V = typename P::V;
+  using VV = Vec<P, NV>;
+  constexpr bool single = std::is_same<P, Single>::value;
+  constexpr int kScanPer = ScanPer<P>::n;
+  constexpr int gp = single ? 5 * 32 : kTermThreads / 2;  // threads on the rank order; the rest on the card lists
+  int i;
+  const Work seg = segments[terminal_item(n_segments, player_mask, i)];  // (first group, count <= kTermSegment)
+  const int tid = threadIdx.x, lane = tid & 31;
+
+  extern __shared__ __align__(128) unsigned char smt[];
+  __shared__ __align__(8) uint64_t bar[2];
+  __shared__ VecAcc<P, NV> red[2][kTermThreads / 32];
+  __shared__ float Cs[NV][kMaxDeck], Ts[NV];  // fold groups, FP32 values
+  TermGroup* desc = reinterpret_cast<TermGroup*>(smt);
+  const uint4* gsrc = reinterpret_cast<const uint4*>(groups + seg.game);
+  for (int k = tid; k < seg.unit * (int)(sizeof(TermGroup) / 16); k += kTermThreads)
+    reinterpret_cast<uint4*>(desc)[k] = __ldg(gsrc + k);
+  if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     fence_barrier_init();
   }
   __syncthreads();
-  if (threadIdx.x == 0) {  // the board tables are static: copy them before waiting
-    mbar_arrive_expect_tx(&bar[0], tab_bytes + q_bytes);
-    bulk_copy_g2s(tab, G.term_tab + (size_t)b * tt.len, tab_bytes, &bar[0]);
-  }
+
+  // per (game, table, kind), reloaded when it changes; shared memory by offsets into smt: the table's
+  // fold part (card lists, cards, list offsets) at kTab, then rows [2][NV][hstride], CP [k H + 1],
+  // Ps [H + 1]
+  constexpr int kTab = kTermSegment * (int)sizeof(TermGroup);
+  int game = -1, table = -1, kind = -1, H = 0, k = 0, stride = 0, begin = 0, cnt = 0, rows = 0;
+  V* dst = nullptr;
+  const uint4* rec = nullptr;
+  uint32_t at[kScanPer / 2];  // hands of the thread's run (rank order or card lists), two in a word
+
+  auto copy_rows = [&](int g) {  // one thread: the reach rows of group g into buffer g & 1
+    const TermGroup& d = desc[g];
+    const GameDev& Gg = games[d.game];
+    const size_t S = (size_t)Gg.hstride;
+    const unsigned bytes = (unsigned)(S * sizeof(V));
+    const TermTab tg(Gg.n_hands, Gg.hand_size, Gg.deck);
+    unsigned char* buf = smt + kTab + tg.fold_len * 2 + (g & 1) * NV * bytes;
+    const V* q = static_cast<const V*>(use_bar ? Gg.reach_bar : Gg.reach) + (size_t)(1 - i) * Gg.n_nodes * S;
+    mbar_arrive_expect_tx(&bar[g & 1], NV * bytes);  // a short group repeats its last node
+    for (int v = 0; v < NV; ++v) bulk_copy_g2s(buf + v * bytes, q + (size_t)term_src_node(d.src[v].row[1 - i]) * S, bytes, &bar[g & 1]);
+  };
+
   pdl_wait();  // the reach rows come from the launch just before this one
   pdl_trigger();
-  if (threadIdx.x == 0) {
-    bulk_copy_g2s(qbuf, qsrc + (size_t)src[first] * stride, q_bytes, &bar[0]);
-    if (RUNS && count > 1) {
-      mbar_arrive_expect_tx(&bar[1], q_bytes);
-      bulk_copy_g2s(qbuf + stride, qsrc + (size_t)src[first + 1] * stride, q_bytes, &bar[1]);
+  for (int g = 0; g < seg.unit; ++g) {
+    const TermGroup& d = desc[g];
+    const bool show = d.kind == kShowdown, other = d.game != game;
+    if (other) {
+      // the rows of a game's first group start once the shared memory of the game before is free
+      // (each game lays it out by its own hand count)
+      if (g > 0) __syncthreads();
+      if (tid == 0) copy_rows(g);
     }
-  }
-  for (int j = 0; j < count; ++j) {
-    const int n = work[first + j].unit;
-    const NodeDev nd = G.nodes[n];
-    // payoff for player i per unit of (opponent reach) x kappa: the FP64 product as a pair of
-    // FP32 rounded once on the host (FP32 values use its high part): no FP64 work per thread
-    const bool neg = nd.type == kFold && nd.player == i;
-    const ff u = {neg ? -G.payoff_ff[2 * n] : G.payoff_ff[2 * n], neg ? -G.payoff_ff[2 * n + 1] : G.payoff_ff[2 * n + 1]};
-    const bool ok = threadIdx.x >= 32 ||  // one warp polls
-                    mbar_wait_bounded(&bar[j & 1], (j >> 1) & 1, j == 0 ? g_first_wait_polls : kWaitLimit);
+    if (other || d.table != table || d.kind != kind) {
+      const GameDev& G = games[d.game];
+      H = G.n_hands, k = G.hand_size;
+      const TermTab tt(H, k, G.deck);
+      if (other) {
+        stride = G.hstride;
+        rows = kTab + tt.fold_len * 2;
+        dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
+      }
+      const uint16_t* gt = G.term_tab + (size_t)d.table * tt.len;
+      if (other || d.table != table) {
+        if (!other) __syncthreads();  // the last group's readers of the table are done
+        table = d.table;
+        for (int x = tid; x < tt.fold_len / 8; x += kTermThreads)
+          reinterpret_cast<uint4*>(smt + kTab)[x] = __ldg(reinterpret_cast<const uint4*>(gt) + x);
+        rec = G.term_rec + (size_t)table * H;
+      }
+      game = d.game;
+      kind = d.kind;
+      if (show || !single) {
+        const int n = tid < gp ? H : k * H, gt_n = tid < gp ? gp : kTermThreads - gp, gtid = tid < gp ? tid : tid - gp;
+        const int per = (n + gt_n - 1) / gt_n;
+        begin = min(gtid * per, n);
+        cnt = min(begin + per, n) - begin;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+          const int j = begin + e;
+          const uint32_t h = e >= cnt ? 0 : tid >= gp ? gt[tt.clh + j] : show ? gt[tt.perm + j] : j;
+          at[e / 2] = e & 1 ? at[e / 2] | h << 16 : h;
+        }
+      }
+    }
+    const bool ok = tid >= 32 || mbar_wait_bounded(&bar[g & 1], (g >> 1) & 1, g == 0 ? g_first_wait_polls : kWaitLimit);
     if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
-      if (threadIdx.x == 0) {
+      if (tid == 0) {
         atomicExch(err, 1);
-        mbar_wait_bounded(&bar[j & 1], (j >> 1) & 1);
-        if (j + 1 < count) mbar_wait_bounded(&bar[(j + 1) & 1], ((j + 1) >> 1) & 1);
+        mbar_wait_bounded(&bar[g & 1], (g >> 1) & 1);
       }
       __syncthreads();
       return;
     }
-    if (src[first + j] != n) {  // below an all-in run-out: the run-out's reach, without the
-      V* qb = qbuf + (size_t)(j & 1) * stride;  // hands holding a card dealt on the way
-      for (int h = threadIdx.x; h < H; h += blockDim.x)
-        if (holds_board_card(tab + tt.cards, h, k, nd.board)) qb[h] = P::zero();
+    // the other buffer's last readers are behind the barrier above
+    if (tid == 0 && g + 1 < seg.unit && desc[g + 1].game == game) copy_rows(g + 1);
+    const uint16_t* clh = reinterpret_cast<const uint16_t*>(smt + kTab);
+    const uint16_t* cards = clh + k * H;
+    const uint16_t* cloff = cards + H;
+    V* q = reinterpret_cast<V*>(smt + rows) + (g & 1) * NV * stride;  // node v's row at q + v * stride
+    VV* CP = reinterpret_cast<VV*>(reinterpret_cast<V*>(smt + rows) + 2 * NV * stride);
+    VV* Ps = CP + (k * H + 1);
+    if (d.below >> (1 - i) & 1) {  // nodes below an all-in run-out: its reach, without the hands holding a card dealt since
+      for (int v = 0; v < NV; ++v)
+        if (d.src[v].row[1 - i] < 0)
+          for (int h = tid; h < H; h += kTermThreads)
+            if (holds_board_card(cards, h, k, d.board[v])) q[v * stride + h] = P::zero();
       __syncthreads();
     }
-    terminal_values<P>(G, nd, i, u, tt, tab, qbuf + (size_t)(j & 1) * stride, CP, Psc, dst + (size_t)n * stride);
-    if (!RUNS) break;
-    __syncthreads();  // buffer j & 1 and the scan arrays are free again
-    if (threadIdx.x == 0 && j + 2 < count) {
-      mbar_arrive_expect_tx(&bar[j & 1], q_bytes);
-      bulk_copy_g2s(qbuf + (size_t)(j & 1) * stride, qsrc + (size_t)src[first + j + 2] * stride, q_bytes,
-                    &bar[j & 1]);
+
+    if constexpr (single) {
+      if (!show) {  // terminal_values' FP32 fold sums: T of node v by warp v, C[c] of (v, c) by one thread
+        const int deck = games[game].deck;
+        if (tid < 32 * NV) {
+          const float* qv = q + (tid >> 5) * stride;
+          float t = 0.f;
+#pragma unroll 8
+          for (int h = lane; h < H; h += 32) t = __fadd_rn(t, qv[h]);
+          for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+          if (lane == 0) Ts[tid >> 5] = t;
+        } else if (tid - 32 * NV < NV * deck) {
+          const int x = tid - 32 * NV, v = x / deck, c = x - v * deck;
+          const float* qv = q + v * stride;
+          float s = 0.f;
+#pragma unroll 8
+          for (int j = cloff[c]; j < cloff[c + 1]; ++j) s = __fadd_rn(s, qv[clh[j]]);
+          Cs[v][c] = s;
+        }
+        __syncthreads();
+        for (int h = tid; h < H; h += kTermThreads) {
+          const unsigned cw = cards[h];
+          const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
+          const uint64_t own = (1ull << c1) | (k == 2 ? 1ull << c2 : 0ull);
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+            if (v < d.count) {
+              float m = __fsub_rn(Ts[v], Cs[v][c1]);
+              if (k == 2) m = __fadd_rn(__fsub_rn(m, Cs[v][c2]), q[v * stride + h]);
+              dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? 0.f : __fmul_rn(d.pay[i][v].hi, m);
+            }
+        }
+        continue;
+      }
+    }
+    {  // the reach in rank order (pair values' folds: in hand order) and along the card lists
+      VV a[kScanPer];
+      VecAcc<P, NV> x;
+#pragma unroll
+      for (int e = 0; e < kScanPer; ++e)
+        if (e < cnt) {
+          const V* qe = q + (at[e / 2] >> (e & 1 ? 16 : 0) & 0xffffu);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) a[e].v[v] = qe[v * stride];
+        }
+      const int gtid = tid < gp ? tid : tid - gp;
+      scan_runs<P, NV>(a, cnt, red[tid >= gp], gtid, x);
+      __syncthreads();
+      if (tid < gp)
+        scan_write<P, NV, gp>(a, begin, cnt, H, red[0], gtid, x, Ps);
+      else
+        scan_write<P, NV, kTermThreads - gp>(a, begin, cnt, k * H, red[1], gtid, x, CP);
+    }
+    __syncthreads();
+    for (int h = tid; h < H; h += kTermThreads) {
+      const uint4 hr = __ldg(rec + h);
+      const unsigned c1 = hr.x & 0xffu, c2 = (hr.x >> 8) & 0xffu;
+      uint64_t own = 1ull << c1;
+      VV d0;
+      if (show) {
+        const VV T = Ps[H];
+        VV Wn = Ps[hr.x >> 16], Ln = Ps[hr.y & 0xffffu];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Ln.v[v] = P::sub(T.v[v], Ln.v[v]);
+        auto one = [&](unsigned c, unsigned lo, unsigned hi) {
+          const VV a = CP[lo], a0 = CP[cloff[c]], z0 = CP[cloff[c + 1]], z = CP[hi];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            Wn.v[v] = P::sub(Wn.v[v], P::sub(a.v[v], a0.v[v]));
+            Ln.v[v] = P::sub(Ln.v[v], P::sub(z0.v[v], z.v[v]));
+          }
+        };
+        one(c1, hr.y >> 16, hr.z & 0xffffu);
+        if (k == 2) {
+          one(c2, hr.z >> 16, hr.w & 0xffffu);
+          own |= 1ull << c2;
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) d0.v[v] = P::sub(Wn.v[v], Ln.v[v]);
+      } else {  // pair values' folds
+        const VV T = Ps[H], a = CP[cloff[c1 + 1]], a0 = CP[cloff[c1]];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) d0.v[v] = P::sub(T.v[v], P::sub(a.v[v], a0.v[v]));
+        if (k == 2) {
+          own |= 1ull << c2;
+          const VV b = CP[cloff[c2 + 1]], b0 = CP[cloff[c2]];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) d0.v[v] = P::add(P::sub(d0.v[v], P::sub(b.v[v], b0.v[v])), q[v * stride + h]);
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        if (v < d.count)
+          dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? P::zero() : P::mul(P::scale(d.pay[i][v]), d0.v[v]);
     }
   }
 }
@@ -1082,11 +1378,11 @@ __host__ __device__ inline size_t resident_hand_bytes(int n_nodes, int n_levels,
 // shared memory while the nodes the block evaluates read the same one (tab_game / tab_b name
 // it); the opponent's reach row is read past L1.  Ends with a block barrier.
 template <typename P>
-__device__ __forceinline__ void resident_terminal(const GameDev* __restrict__ games, Work e, int src, int i,
+__device__ __forceinline__ void resident_terminal(const GameDev* __restrict__ games, Work e, TermSrc ts, int i,
                                                   unsigned char* smr, int& tab_game, int& tab_b) {
   using V = typename P::V;
   const GameDev& G = games[e.game];
-  const int n = e.unit;
+  const int n = e.unit, src = ts.row[1 - i];
   const NodeDev nd = G.nodes[n];
   const TermTab tt(G.n_hands, G.hand_size, G.deck);
   const size_t stride = (size_t)G.hstride;
@@ -1105,12 +1401,12 @@ __device__ __forceinline__ void resident_terminal(const GameDev* __restrict__ ga
   }
   {  // the row is a multiple of 128 bytes (hstride is a multiple of 32)
     const uint4* q4 = reinterpret_cast<const uint4*>(static_cast<const V*>(G.reach) +
-                                                     ((size_t)(1 - i) * G.n_nodes + src) * stride);
+                                                     ((size_t)(1 - i) * G.n_nodes + term_src_node(src)) * stride);
     for (int k = threadIdx.x; k < (int)(stride * sizeof(V) / 16); k += blockDim.x)
       reinterpret_cast<uint4*>(qs)[k] = __ldcg(q4 + k);
   }
   __syncthreads();
-  if (src != n) {  // below an all-in run-out: zero the hands holding a card dealt on the way
+  if (src < 0) {  // below an all-in run-out: zero the hands holding a card dealt on the way
     for (int h = threadIdx.x; h < G.n_hands; h += blockDim.x)
       if (holds_board_card(tab + tt.cards, h, G.hand_size, nd.board)) qs[h] = P::zero();
     __syncthreads();
@@ -1129,7 +1425,7 @@ __device__ __forceinline__ void resident_terminal(const GameDev* __restrict__ ga
 template <typename P>
 __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
     const GameDev* __restrict__ games, const Work* __restrict__ chunk_work, int n_chunk_work,
-    const Work* __restrict__ term_work, const int32_t* __restrict__ term_src, int n_term_work, int alternating,
+    const Work* __restrict__ term_work, const TermSrc* __restrict__ term_src, int n_term_work, int alternating,
     int n_iters, int* iter, const Discount* __restrict__ disc_tab, int variant, unsigned* sync, int* err,
     unsigned term_bytes) {
   using V = typename P::V;
@@ -1775,6 +2071,321 @@ __global__ void __launch_bounds__(kStreamWarps * 32) k_stream_update(
   }
 }
 
+// ------------------------------------------------------------------ hand tiles
+//
+// The throughput form of the per-hand passes for handles of many subgames whose trees fit a
+// block's shared memory a few times per SM (batches of rivers).  One block owns W hands (32, 16
+// or 8: the most that fit) of one subgame and one player:
+//   A  the values of the tree's end nodes and the stored strategy come in by cp.async; the inner
+//      nodes' values (Stage 6) are computed level by level in shared memory;
+//   B  the regret and average update (Stage 7) of every row of the player: a flat loop over (row,
+//      hand) items with no order between them, four in flight a thread, so that the FP64 pipe
+//      (64 cycles a warp instruction and scheduler) and the R and S streams stay busy; the
+//      positive parts of the new regrets replace the strategy in shared memory;
+//   C  level by level from the root: regret matching of the player's nodes (Eq. rm) and the
+//      reach of their children (Stage 1), in the array of A.
+// R and S are read and written once, straight from registers; L2 is asked for their lines at the
+// start, before the launch waits for its predecessor.  The arithmetic is k_hand's, in its order.
+// Bound: the FP64 pipe (four operations a row and hand: 88 us on the batch below) and issue slots.
+// Measured, one player's update: 256 rivers, FP32 values 267 -> 180 us against the one-warp walk;
+// 64 rivers, pairs, Predictive CFR+ 321 -> 110 us.  Average pass 780 -> 167, best response 943 ->
+// 150 us (256 rivers, both players; k_hand before).
+
+constexpr int kTileThreads = 256;  // at most; 128 where the tiles are small (see create_impl)
+constexpr int kTileRows = 4;       // (row, hand) items of phase B in flight per thread
+
+__host__ __device__ inline size_t tile_smem_bytes(int tab16, int n_nodes, int rows_max, int W, size_t es) {
+  return (size_t)tab16 * 16 + (size_t)(n_nodes + rows_max) * W * es;
+}
+
+// Copies rows of W values (count of them, row k of the source at row_at(k)) into the tile.
+template <typename V, typename F, typename T>
+__device__ __forceinline__ void tile_copy(V* tile, const V* __restrict__ src, size_t stride, int wlog, int count, F row_at,
+                                          T tile_at) {
+  const int pl = wlog + (sizeof(V) == 8 ? 3 : 2) - 4;  // log2 of a row's 16-byte pieces
+  for (int k = threadIdx.x; k < count << pl; k += blockDim.x) {
+    const int r = k >> pl, part = k & ((1 << pl) - 1);
+    cp_async<16>(reinterpret_cast<unsigned char*>(tile + (tile_at(r) << wlog)) + part * 16,
+                 reinterpret_cast<const unsigned char*>(src + (size_t)row_at(r) * stride) + part * 16);
+  }
+}
+
+// Regret matching (Eq. rm) at a decision node of the player with NA actions from the positive parts
+// s, and the reach of its children from the node's reach x (regret_match_n's operations).
+template <typename P, int NA>
+__device__ __forceinline__ void tile_match(const typename P::V* s, typename P::V* c, int wlog, typename P::V x,
+                                           typename P::V* __restrict__ gs, typename P::V* __restrict__ gc, int stride,
+                                           bool store_reach, bool valid) {
+  using V = typename P::V;
+  V y[NA], tot = P::zero();
+  int npos = 0;
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    y[a] = s[a << wlog];
+    npos += P::positive(y[a]);
+    tot = P::add(tot, y[a]);
+  }
+  const V inv = P::recip(tot);  // unused (and possibly not finite) unless npos > 1
+  const V uni = P::uniform(NA);
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    const V many = P::mul(y[a], inv);
+    y[a] = npos > 1 ? many : npos == 1 ? (P::positive(y[a]) ? P::one() : P::zero()) : uni;
+    const V r = P::mul(x, y[a]);
+    c[a << wlog] = r;
+    if (valid) {
+      gs[(size_t)a * stride] = y[a];
+      if (store_reach) gc[(size_t)a * stride] = r;
+    }
+  }
+}
+
+template <int MODE, typename P, bool DCFR>
+__global__ void __launch_bounds__(kTileThreads, 4) k_tile(const GameDev* __restrict__ games,
+                                                       const Work* __restrict__ work, int n_work, int player_mask,
+                                                       int advance, int* iter, unsigned* done,
+                                                       const Discount* __restrict__ disc_tab, int variant) {
+  using V = typename P::V;
+  extern __shared__ __align__(16) unsigned char smx[];
+  __shared__ Discount disc;
+  int p;
+  const Work wk = work[terminal_item(n_work, player_mask, p)];
+  const GameDev& G = games[wk.game];
+  const int wlog = G.tile_wlog, W = 1 << wlog, tid = threadIdx.x, w = tid & (W - 1), slot = tid >> wlog,
+            nslots = blockDim.x >> wlog;
+  const int h0 = wk.unit << wlog, h = h0 + w;  // < hstride: hstride is a multiple of 32 and W divides 32
+  const bool valid = h < G.n_hands;
+  const int N = G.n_nodes, stride = G.hstride, rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
+  const uint64_t hmask = valid ? G.hand_mask[h] : 0ull;
+  const int tab16 = G.tile_tab16;
+
+  // shared: the tile table, values / reach [N][W], strategy [rows][W]
+  V* tval = reinterpret_cast<V*>(smx + (size_t)tab16 * 16);
+  V* val = tval + w;                 // this lane's column: node n at val[n << wlog]
+  V* sg = val + ((size_t)N << wlog);  // row r at sg[r << wlog]
+  const size_t plane = (size_t)p * N * stride;
+  V* gv = static_cast<V*>(MODE == kModeBR ? G.cfv_br : G.cfv) + plane;
+  V* grch = static_cast<V*>(MODE == kModeAvg ? G.reach_bar : G.reach) + plane;
+  V* gsg = static_cast<V*>(MODE == kModeAvg ? G.sigbar : G.sigma) + (size_t)rb * stride;
+  double* gR = G.R + (size_t)rb * stride;
+  double* gS = G.S + (size_t)rb * stride;
+
+  // ---- what older launches wrote: the table, the strategy, and L2 lines of R and S
+  for (int k = tid; k < tab16; k += blockDim.x)
+    reinterpret_cast<uint4*>(smx)[k] = __ldg(reinterpret_cast<const uint4*>(G.tile_tab) + k);
+  if (MODE == kModeUpdate) {
+    if (tid == 0) disc = disc_tab[*iter];
+    auto same = [](int r) { return r; };
+    tile_copy(tval + ((size_t)N << wlog), gsg + h0, (size_t)stride, wlog, nrows, same, same);
+  }
+  if (MODE != kModeBR) {
+    const int ll = wlog == 5;  // lines of 16 doubles per row: 2, or 1
+    for (int k = tid; k < nrows << ll; k += blockDim.x) {
+      const size_t at = (size_t)(k >> ll) * stride + h0 + (k & ll) * 16;
+      if (MODE != kModeAvg) asm volatile("prefetch.global.L2 [%0];" ::"l"(gR + at));
+      if (MODE != kModeInit) asm volatile("prefetch.global.L2 [%0];" ::"l"(gS + at));
+    }
+  }
+  pdl_wait();  // terminal values come from the launch just before this one
+  pdl_trigger();
+  __syncthreads();
+  const TileHead* head = reinterpret_cast<const TileHead*>(smx);
+  const uint16_t* tab = reinterpret_cast<const uint16_t*>(smx);
+  const TileNode* inner = reinterpret_cast<const TileNode*>(tab + head->inner);
+  const uint16_t* level = tab + head->level;  // inner nodes of level l: [level[l], level[l + 1])
+  const int L = head->levels;
+
+  if (MODE == kModeUpdate || MODE == kModeBR) {
+    // ---- A: end values in, then inner values from the deepest level up
+    const uint16_t* ends = tab + head->ends;
+    auto end = [&](int e) { return (int)ends[e]; };
+    tile_copy(tval, static_cast<const V*>(gv) + h0, (size_t)stride, wlog, head->n_ends, end, end);
+    cp_async_wait_all();
+    __syncthreads();
+    for (int l = L - 1; l >= 0; --l) {
+      const int last = level[l + 1];
+      for (int k = level[l] + slot; k < last; k += nslots) {
+        const TileNode nd = inner[k];
+        const int A = nd.kids & 63, kind = nd.kids >> 6;
+        const V* c = val + (nd.first_kid << wlog);
+        V x;
+        if (MODE == kModeBR && kind == p) {
+          x = c[0];
+          for (int a = 1; a < A; ++a) x = P::vmax(x, c[a << wlog]);
+        } else {
+          typename P::Acc acc = P::acc0();
+          if (kind == 2) {  // children values carry the card probabilities; cards in the hand are out
+            for (int a = 0; a < A; ++a)
+              if (!((hmask >> G.nodes[nd.first_kid + a].deal) & 1ull)) P::acc(acc, c[a << wlog]);
+          } else if (kind != p) {
+#pragma unroll 4
+            for (int a = 0; a < A; ++a) P::acc(acc, c[a << wlog]);
+          } else {
+            const V* s = sg + (nd.row << wlog);
+#pragma unroll 4
+            for (int a = 0; a < A; ++a) P::acc_mul(acc, s[a << wlog], c[a << wlog]);
+          }
+          x = P::value(acc);
+        }
+        val[nd.id << wlog] = x;
+        if (valid && (MODE == kModeBR || l == 0)) gv[(size_t)nd.id * stride + h] = x;
+      }
+      __syncthreads();
+    }
+  }
+  if constexpr (MODE == kModeBR) {
+    // FP64 root sums of the tile's chunks, reduced by the game's last block as in k_hand
+    __shared__ int s_last;
+    __shared__ double red64[kHandThreads];
+    const int C = G.chunk;  // <= W
+    if (tid < W) {
+      double x = valid ? G.range64[(size_t)p * stride + h] * P::to_double(val[0]) : 0.0;
+      const unsigned mask = W == 32 ? 0xffffffffu : (1u << W) - 1u;
+      for (int o = C / 2; o > 0; o >>= 1) x += __shfl_down_sync(mask, x, o, C);
+      if (w % C == 0 && valid) G.br_partial[(size_t)p * G.n_chunks + h / C] = x;
+      __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+      const unsigned chunks = (unsigned)((min(h0 + W, G.n_hands) - h0 + C - 1) / C);
+      s_last = atomicAdd(G.br_done, chunks) + chunks == (unsigned)(2 * G.n_chunks);
+    }
+    __syncthreads();
+    if (s_last) {  // the sums of kHandThreads threads, as k_hand's last block forms them
+      __threadfence();
+      for (int q = 0; q < 2; ++q) {
+        for (int t = tid; t < kHandThreads; t += blockDim.x) {
+          double x = 0.0;
+          for (int c = t; c < G.n_chunks; c += kHandThreads) x += __ldcg(&G.br_partial[(size_t)q * G.n_chunks + c]);
+          red64[t] = x;
+        }
+        __syncthreads();
+        for (int o = kHandThreads / 2; o > 0; o >>= 1) {
+          for (int t = tid; t < o; t += blockDim.x) red64[t] += red64[t + o];
+          __syncthreads();
+        }
+        if (tid == 0) G.br_out[q] = red64[0];
+        __syncthreads();
+      }
+      if (tid == 0) *G.br_done = 0u;
+    }
+    return;
+  }
+
+  // ---- B: every row of the player (sign tests of FP64 values read the sign bit on the integer pipe)
+  {
+    const TileRow* rowmap = reinterpret_cast<const TileRow*>(tab + head->rows[p]);
+    double* gM = G.M ? G.M + (size_t)rb * stride + h : nullptr;
+    const double* src = (MODE == kModeAvg ? gS : gR) + h;
+    for (int r0 = slot; r0 < nrows; r0 += kTileRows * nslots) {
+      double R[kTileRows], S[kTileRows];
+      V pi[kTileRows];
+      TileRow m[kTileRows];
+#pragma unroll
+      for (int e = 0; e < kTileRows; ++e) {
+        const int r = r0 + e * nslots;
+        if (r < nrows) {
+          R[e] = src[(size_t)r * stride];
+          if (MODE == kModeUpdate) {
+            m[e] = rowmap[r];
+            S[e] = gS[(size_t)r * stride + h];
+            pi[e] = grch[(size_t)m[e].src * stride + h];
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < kTileRows; ++e) {
+        const int r = r0 + e * nslots;
+        if (r < nrows) {
+          double x = R[e];
+          if (MODE == kModeUpdate) {
+            const V rr = P::sub(val[m[e].kid << wlog], val[m[e].node << wlog]);  // instantaneous regret
+            const double rd = P::to_double(rr);
+            const double contrib = P::to_double(P::mul(pi[e], sg[r << wlog]));  // pi_i(I) sigma(I, a)
+            x += rd;
+            double sn;
+            if constexpr (DCFR) {
+              x *= __double_as_longlong(x) > 0 ? disc.dpos : disc.dneg;
+              sn = fma(S[e], disc.dS, contrib);
+            } else {
+              if (variant != 0 && __double_as_longlong(x) < 0) x = 0.0;  // CFR+, Predictive CFR+
+              sn = fma(S[e], disc.dS, variant != 0 ? disc.wS * contrib : contrib);
+            }
+            if (valid) {
+              gR[(size_t)r * stride + h] = x;
+              gS[(size_t)r * stride + h] = sn;
+            }
+            if (!DCFR && variant == 3) {
+              if (valid) gM[(size_t)r * stride] = rd;  // the prediction of the next regret
+              x += rd;                                 // Predictive CFR+ matches R + M
+            }
+          } else if (MODE == kModeInit && gM) {
+            x += gM[(size_t)r * stride];
+          }
+          sg[r << wlog] = __double_as_longlong(x) > 0 ? P::of_double(x) : P::zero();
+        }
+      }
+    }
+  }
+  __syncthreads();  // the positive parts are there, and the values have been read: their array takes the reach
+
+  // ---- C: regret matching and reach from the root down, over the nodes that make new rows: the
+  // children of the player's decisions and of chance nodes (every other node shares a row above
+  // it).  An update stores those rows; the other passes every node's
+  if (tid < W) val[0] = valid ? static_cast<const V*>(G.range_v)[(size_t)p * stride + h] : P::zero();
+  __syncthreads();
+  const TileNode* fwd = reinterpret_cast<const TileNode*>(tab + head->fwd[p]);
+  const uint16_t* flevel = tab + head->flevel[p];
+  for (int l = 0; l < head->flevels[p]; ++l) {
+    const int last = flevel[l + 1];
+    for (int k = flevel[l] + slot; k < last; k += nslots) {
+      const TileNode nd = fwd[k];
+      const int A = nd.kids & 63;
+      const V x = val[nd.id << wlog];
+      V* c = val + (nd.first_kid << wlog);
+      V* gc = grch + (size_t)nd.first_kid * stride + h;
+      const V* s = sg + (nd.row << wlog);
+      V* gs = gsg + (size_t)nd.row * stride + h;
+      if (nd.kids >> 6 == 2) {
+        for (int a = 0; a < A; ++a) {
+          const V y = ((hmask >> G.nodes[nd.first_kid + a].deal) & 1ull) ? P::zero() : x;
+          c[a << wlog] = y;
+          if (MODE == kModeUpdate && valid) gc[(size_t)a * stride] = y;
+        }
+        continue;
+      }
+      constexpr bool upd = MODE == kModeUpdate;
+      switch (A) {
+        case 1: tile_match<P, 1>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 2: tile_match<P, 2>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 3: tile_match<P, 3>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 4: tile_match<P, 4>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 5: tile_match<P, 5>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 6: tile_match<P, 6>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        case 7: tile_match<P, 7>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+        default: tile_match<P, 8>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
+      }
+    }
+    __syncthreads();
+  }
+  if (MODE != kModeUpdate && valid) {
+    const uint16_t* all = tab + head->all[p];
+    for (int n = slot; n < N; n += nslots) grch[(size_t)n * stride + h] = val[all[n] << wlog];
+  }
+
+  if (MODE == kModeUpdate && advance) {
+    if (tid == 0) {
+      __threadfence();
+      const unsigned prev = atomicAdd(done, 1u);
+      if (prev == gridDim.x - 1) {  // last block of the launch: every block has read *iter
+        *done = 0u;
+        *iter += 1;
+        __threadfence();
+      }
+    }
+  }
+}
+
 // sigma = RM(R) at every decision node of every game (current strategy, for read-back when
 // the update launches do not store it).
 template <typename P>
@@ -2038,6 +2649,17 @@ size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es)
   return hand_smem_bytes(n_nodes, n_levels, rows_max, W, es);
 }
 
+size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv) {
+  const TermTab tt(n_hands, hand_size, deck);
+  const size_t scan = (size_t)(hand_size * n_hands + 1 + n_hands + 1);
+  if (nv == 1) return (size_t)tt.len * 2 + (size_t)hstride * es + scan * sizeof(ff);
+  return kTermSegment * sizeof(TermGroup) + (size_t)tt.fold_len * 2 + 2 * (size_t)nv * hstride * es + scan * nv * es;
+}
+
+size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es) {
+  return tile_smem_bytes(tab16, n_nodes, rows_max, W, es);
+}
+
 size_t resident_term_size(int n_hands, int hand_size, int deck, int hstride, size_t es) {
   return round16(resident_term_bytes(n_hands, hand_size, deck, hstride, es));
 }
@@ -2077,9 +2699,15 @@ template <typename P>
 static cudaError_t configure_precision() {
   cudaError_t e = configure_hand<P, true>();
   if (e == cudaSuccess) e = configure_hand<P, false>();
-  if (e == cudaSuccess) e = configure_one(k_terminal<P, false>, 200 * 1024);
-  if (e == cudaSuccess) e = configure_one(k_terminal<P, true>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal<P>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal_vec<P, 2>, 200 * 1024);
+  if (e == cudaSuccess && sizeof(typename P::V) == 4) e = configure_one(k_terminal_vec<Single, 4>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_average_rows<P>, 0);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, true>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeAvg, P, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeBR, P, false>, kTileSmem);
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 1>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 2>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_current_rows<P>, 0);
@@ -2238,8 +2866,28 @@ int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advanc
   return back + 1;
 }
 
+template <int MODE>
+static int launch_tile(const LaunchCtx& c, int player_mask, int advance, void* stream, bool pdl) {
+  auto go = [&](auto kernel) {
+    return launch_kernel(kernel, c.n_tile_work * (player_mask == 3 ? 2 : 1), c.tile_threads, c.smem_tile, stream, pdl,
+                         c.games, c.tile_work, c.n_tile_work, player_mask, advance, c.iter, c.done, c.disc, c.variant);
+  };
+  constexpr bool upd = MODE == kModeUpdate;  // the other passes do not depend on the variant
+  cudaError_t e;
+  if (c.precision == kPrecisionSingle)
+    e = upd && c.variant == 2 ? go(k_tile<MODE, Single, upd>) : go(k_tile<MODE, Single, false>);
+  else
+    e = upd && c.variant == 2 ? go(k_tile<MODE, Pairs, upd>) : go(k_tile<MODE, Pairs, false>);
+  if (e != cudaSuccess) {
+    fprintf(stderr, "pcfr: launch of k_tile failed: %s\n", cudaGetErrorString(e));
+    return -1;
+  }
+  return check_launch("k_tile");
+}
+
 int launch_init(const LaunchCtx& c, void* stream) {
   if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeInit, 3, 0, stream);
+  if (c.n_tile_work > 0) return launch_tile<kModeInit>(c, 3, 0, stream, false);
   return launch_hand<kModeInit>(c, 3, 0, stream, false);
 }
 template <typename P, int HP>
@@ -2261,6 +2909,7 @@ static int launch_stream_p(const LaunchCtx& c, int player_mask, int advance, voi
 
 int launch_update(const LaunchCtx& c, int player_mask, int advance, void* stream) {
   if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeUpdate, player_mask, advance, stream);
+  if (c.n_tile_work > 0) return launch_tile<kModeUpdate>(c, player_mask, advance, stream, c.pdl != 0);
   if (c.schedule == kScheduleStream)
     return c.precision == kPrecisionSingle
                ? (c.stream_hp == 2 ? launch_stream_p<Single, 2>(c, player_mask, advance, stream)
@@ -2279,30 +2928,32 @@ int launch_current_rows(const LaunchCtx& c, void* stream) {
 }
 int launch_avg_reach(const LaunchCtx& c, void* stream) {
   if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeAvg, 3, 0, stream);
+  if (c.n_tile_work > 0) return launch_tile<kModeAvg>(c, 3, 0, stream, false);
   return launch_hand<kModeAvg>(c, 3, 0, stream, false);
 }
 int launch_br(const LaunchCtx& c, void* stream) {
   if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeBR, 3, 0, stream);
+  if (c.n_tile_work > 0) return launch_tile<kModeBR>(c, 3, 0, stream, c.pdl != 0);
   return launch_hand<kModeBR>(c, 3, 0, stream, c.pdl != 0);
 }
 
 int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stream) {
-  if (c.n_term_runs == 0) return 0;
+  if (c.n_term_work == 0) return 0;
   const int players = player_mask == 3 ? 2 : 1;
-  const int grid = c.n_term_runs * players;
   const bool pdl = c.pdl != 0;
+  auto one = [&](auto kernel) {
+    return launch_kernel(kernel, c.n_term_work * players, kTermThreads, c.smem_term, stream, pdl, c.games, c.term_work,
+                         c.term_src, c.n_term_work, player_mask, use_bar, c.err);
+  };
+  auto vec = [&](auto kernel) {
+    return launch_kernel(kernel, c.n_term_segments * players, kTermThreads, c.smem_term, stream, pdl, c.games,
+                         c.term_groups, c.term_segments, c.n_term_segments, player_mask, use_bar, c.err);
+  };
   cudaError_t e;
-  const bool runs = c.n_term_runs < c.n_term_work;
   if (c.precision == kPrecisionSingle)
-    e = runs ? launch_kernel(k_terminal<Single, true>, grid, kTermThreads, c.smem_term, stream, pdl, c.games,
-                             c.term_work, c.term_src, c.term_runs, c.n_term_runs, player_mask, use_bar, c.err)
-             : launch_kernel(k_terminal<Single, false>, grid, kTermThreads, c.smem_term, stream, pdl, c.games,
-                             c.term_work, c.term_src, c.term_runs, c.n_term_runs, player_mask, use_bar, c.err);
+    e = c.term_nv == 4 ? vec(k_terminal_vec<Single, 4>) : c.term_nv == 2 ? vec(k_terminal_vec<Single, 2>) : one(k_terminal<Single>);
   else
-    e = runs ? launch_kernel(k_terminal<Pairs, true>, grid, kTermThreads, c.smem_term, stream, pdl, c.games,
-                             c.term_work, c.term_src, c.term_runs, c.n_term_runs, player_mask, use_bar, c.err)
-             : launch_kernel(k_terminal<Pairs, false>, grid, kTermThreads, c.smem_term, stream, pdl, c.games,
-                             c.term_work, c.term_src, c.term_runs, c.n_term_runs, player_mask, use_bar, c.err);
+    e = c.term_nv == 2 ? vec(k_terminal_vec<Pairs, 2>) : one(k_terminal<Pairs>);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_terminal failed: %s\n", cudaGetErrorString(e));
     return -1;
@@ -2325,7 +2976,7 @@ static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stre
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_resident<P>, c.games, c.chunk_work, c.n_chunk_work, c.term_work,
-                            static_cast<const int32_t*>(c.term_src), c.n_term_work, c.alternating, n_iters, c.iter,
+                            c.term_src, c.n_term_work, c.alternating, n_iters, c.iter,
                             c.disc, c.variant, c.resident_sync, c.err, c.resident_term);
 }
 

@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kLeafInThreads) k_leaf_inputs(const GameDev* _
       if (col >= kLeafIn) break;
       const int p = col >= kLeafSlots;
       const bool live = h[u] >= 0 && !(m[u] & nd.board);
-      const float q = live ? vf(reach[((size_t)p * G.n_nodes + lf.node) * stride + h[u]]) : 0.f;
+      const float q = live ? vf(reach[((size_t)p * G.n_nodes + lf.src[p]) * stride + h[u]]) : 0.f;
       qc[col] = q;
       cc[col] = live ? (uint16_t)((__ffsll((long long)m[u]) - 1) | ((63 - __clzll((long long)m[u])) << 8)) : kNoHand;
       if (p == 0) t0 += q, n += live, pos0 += q > 0.f;
@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(kLeafThreads) k_leaf_values(const GameDev* __r
   const NodeDev nd = G.nodes[lf.node];
   const int nh = G.n_hands < kLeafSlots ? G.n_hands : kLeafSlots;
   const size_t stride = (size_t)G.hstride;
-  const V* q = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + ((size_t)(1 - i) * G.n_nodes + lf.node) * stride;
+  const V* q = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + ((size_t)(1 - i) * G.n_nodes + lf.src[1 - i]) * stride;
   V* out = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + ((size_t)i * G.n_nodes + lf.node) * stride;
   const int16_t* slot = L.slot + (size_t)lf.game * L.hstride_max;
   for (int x = threadIdx.x; x < 52 * 52; x += blockDim.x) Q2[x] = 0.f;

@@ -28,6 +28,9 @@
 #ifndef __CUDACC__  // host-only translation units share the small helpers below
 #define __host__
 #define __device__
+struct uint4 {
+  uint32_t x, y, z, w;
+};
 #endif
 
 namespace pcfr {
@@ -72,6 +75,35 @@ struct alignas(16) NodeDev {
   uint64_t board;     // public cards at this node (bit c = card c)
 };
 static_assert(sizeof(NodeDev) == 32, "NodeDev is 32 bytes");
+
+// Hand tiles (k_tile): the table of one subgame, one block of uint16 staged in shared memory.
+// Offsets are in uint16 from its start.
+struct TileHead {
+  int32_t inner;      // TileNode [n_inner]: inner nodes, level by level
+  int32_t level;      // [levels + 1] first inner node of each level
+  int32_t levels;     // levels that hold inner nodes
+  int32_t ends, n_ends;        // node ids of the fold, showdown and leaf nodes
+  int32_t rows[2];             // per player: TileRow of each of its rows
+  // per player: the nodes that make new reach rows (TileNode whose id is the node holding the reach
+  // at it, HostGame::reach_row), level by level; first of each level; levels
+  int32_t fwd[2], flevel[2], flevels[2];
+  int32_t all[2];              // per player: [n_nodes] reach_row
+  int32_t pad;
+};
+static_assert(sizeof(TileHead) % 16 == 0, "the table's TileNodes start 16-byte aligned");
+// One inner node of a tile table, 8 bytes.
+struct alignas(8) TileNode {
+  uint16_t id, first_kid, row;  // row: of the node's first action, from its player's first row
+  uint8_t kids;                 // children | (player, or 2 for a chance node) << 6
+  uint8_t pad;
+};
+static_assert(sizeof(TileNode) == sizeof(uint64_t), "TileNode is 8 bytes");
+struct alignas(8) TileRow {  // a row's child node, its decision node, and the node holding the reach there
+  uint16_t kid, node, src, pad;
+};
+
+constexpr int kTileSmemSmall = 26 * 1024;  // shared memory of a block of 128 threads: eight fit an SM
+constexpr int kTileSmem = 53 * 1024;       // of a block of 256 threads: four fit
 
 // One node of the stream schedule's program (pre-order), 16 bytes.  Offsets are in
 // elements of a per-hand array (multiples of hstride).
@@ -130,8 +162,13 @@ struct GameDev {
   const void* range_v;         // [2][hstride] normalised ranges, value type V
   const double* range64;       // [2][hstride]
   const uint16_t* term_tab;    // [n_boards][TermTab.len]
+  const uint4* term_rec;       // [n_boards][n_hands] (grouped terminal launch): cards, gs, ge, then lo and
+                               // hi per card, as uint16
   const ProgOp* prog;          // [prog_len] inner nodes in depth-first pre-order (stream schedule)
   int prog_len;
+  const uint16_t* tile_tab;    // hand tiles: TileHead and its lists (null: the handle does not use them)
+  int tile_tab16;              // its length in 16-byte units
+  int tile_wlog;               // log2 of the hands per tile
   const int32_t* chunks;       // load chunks of the stream schedule (see stream_tables)
   int chunk_off[4], chunk_count[4];
   const uint32_t* units;       // loads of the stream schedule, in the order the passes use them
@@ -151,6 +188,32 @@ struct GameDev {
   unsigned* br_done;           // blocks of the best-response pass that have finished
 };
 
+struct PairF {  // an FP32 pair: a value hi + lo
+  float hi, lo;
+};
+
+// Per player, the node whose reach row stands for a terminal's (HostGame::reach_row), negated and
+// less one (~node) where the hands holding a card dealt since are to be zeroed.
+struct TermSrc {
+  int32_t row[2];
+};
+__host__ __device__ inline int term_src_node(int32_t row) { return row < 0 ? ~row : row; }
+
+// Up to four terminal nodes of one game, board table and kind, evaluated together.
+struct alignas(16) TermGroup {
+  int32_t game;
+  int32_t table;      // board table (folds read table 0)
+  int16_t kind;       // kFold or kShowdown
+  int16_t count;
+  int32_t below;      // bit p: player p's reach at some node is another's without dealt cards' hands
+  int32_t node[4];
+  TermSrc src[4];
+  uint64_t board[4];
+  PairF pay[2][4];    // per player: payoff * kappa, negative where the player folded
+};
+static_assert(sizeof(TermGroup) == 160, "TermGroup is 160 bytes");
+constexpr int kTermSegment = 16;  // groups a block of the grouped terminal launch walks at most
+
 struct Work {
   int game;
   int unit;  // chunk index (per-hand passes) or node id (terminal pass)
@@ -168,14 +231,14 @@ struct LaunchCtx {
   int n_games;
   const Work* chunk_work;      // device [n_chunk_work]: (game, chunk)
   int n_chunk_work;
-  const Work* term_work;       // device [n_term_work]: (game, terminal node), grouped by game and
-                               // board table
+  const Work* term_work;       // device [n_term_work]: (game, terminal node), grouped by game,
+                               // board table and kind (folds, then showdowns)
   int n_term_work;
-  const Work* term_runs;       // device [n_term_runs]: (first entry of term_work, count), the
-                               // terminal nodes one block evaluates
-  int n_term_runs;
-  const int32_t* term_src;     // device [n_term_work]: node whose reach rows stand for each
-                               // terminal's (HostGame::reach_src)
+  int term_nv;                 // nodes a block evaluates together: 1, or term_groups of up to 2 or 4
+  const TermGroup* term_groups;   // device (term_nv > 1)
+  const Work* term_segments;      // device [n_term_segments]: (first group, count), one block's
+  int n_term_segments;
+  const TermSrc* term_src;     // device [n_term_work]: reach rows of each terminal
   int* iter;                   // device: iterations completed
   unsigned* done;              // device: block arrival counter
   int* err;                    // device: nonzero after a bounded wait gave up
@@ -190,6 +253,10 @@ struct LaunchCtx {
   const Work* warp_work;       // device [n_warp_work]: (game, first group of 32 hands) of each
                                // block of the stream schedule, largest trees first
   int n_warp_work;
+  const Work* tile_work;       // device [n_tile_work]: (game, tile), largest trees first; the stream
+  int n_tile_work;             // schedule's passes run as k_tile when there are any
+  size_t smem_tile;            // dynamic shared memory of k_tile
+  int tile_threads;            // its threads per block
   int stream_depth;            // stack slots per lane of the stream schedule
   int stream_prog;             // nodes of the largest tree, if its program is staged in shared
                                // memory; 0 = read from global memory
@@ -226,12 +293,16 @@ int launch_average_rows(const LaunchCtx& c, void* stream);
 // kModeBR, as the per-hand kernel's modes).
 int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advance);
 int hand_kernel_smem_limit();
+// Shared memory of one block of the terminal launch for one game (nv: LaunchCtx::term_nv).
+size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv);
 // Shared memory the per-hand kernel needs to stage one game (es = bytes per value).
 size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es);
 int configure_kernels();  // once per process, before the first launch
 // Polls of the terminal kernel's first bulk-copy wait on the current device (< 0: the
 // default limit); for tests of the timeout path.  Returns 0 or -1.
 int set_first_wait_polls(long polls);
+// Shared memory of k_tile for one game (tab16: its table in 16-byte units).
+size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es);
 // Resident schedule: shared memory of its two regions for one game, the blocks of k_resident
 // one SM holds with `smem` bytes (0 if none), and the cooperative launch of n_iters iterations.
 size_t resident_term_size(int n_hands, int hand_size, int deck, int hstride, size_t es);
@@ -259,6 +330,7 @@ constexpr int kLeafCards = 48;                          // river cards after 4 b
 
 struct LeafDev {      // one depth-limit leaf
   int game, node;
+  int src[2];         // per player, the node whose reach row stands for the leaf's
   int row0;           // first of its kLeafCards network rows (river cards ascending)
   float feat[2];      // pot / (pot + 2 stack), stack / (pot + 2 stack) at the leaf
 };

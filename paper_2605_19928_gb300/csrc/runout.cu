@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_runout_build(const RunoutTabl
 constexpr int kValueThreads = 64;  // 4 hands a thread: 256 hands a block
 constexpr int kChunk = 64;         // opponent hands staged at a time (one a thread)
 constexpr int kAhead = 8;          // table rows in flight per thread
+static_assert(2 * kAhead <= kRunoutPadRows, "rows loaded past a table's end stay in the pool");
 constexpr int kTops8 = kRunoutGroup, kTops16 = 2, kSubs16 = kRunoutGroup / kTops16;
 static_assert(kChunk == kValueThreads && kChunk % kAhead == 0, "one staged hand per thread");
 
@@ -132,7 +133,8 @@ __device__ __forceinline__ void runout_tops(const GameDev& G, const RunoutItem* 
                                             float* __restrict__ out, ulonglong2* qs) {
   const int H = G.n_hands, tid = threadIdx.x;
   const size_t S = (size_t)G.hstride;
-  const T* E = table + (h0 < H ? h0 : 0);  // a thread past the hands computes hand 0's and drops them
+  const uint32_t ld = (uint32_t)S;
+  uint32_t at = h0 < H ? (uint32_t)h0 : 0u;  // a thread past the hands computes hand 0's and drops them
   const float* src[kTops];
 #pragma unroll
   for (int g = 0; g < kTops; ++g) src[g] = reach + (size_t)items[g < count ? g : 0].node * S;
@@ -149,9 +151,13 @@ __device__ __forceinline__ void runout_tops(const GameDev& G, const RunoutItem* 
 #pragma unroll
     for (int g = 0; g < kTops; g += 2) dst[g / 2] = make_ulonglong2(pack2(q[g], q[g]), pack2(q[g + 1], q[g + 1]));
   };
+  // rows past the last are loaded too (the pool has kRunoutPadRows rows of slack) and not used
   Row4<T> row[kAhead], next[kAhead];
+  auto rows = [&](Row4<T> (&r)[kAhead]) {
 #pragma unroll
-  for (int k = 0; k < kAhead; ++k) row[k] = Row4<T>::load(E + (size_t)min(k, H - 1) * S);
+    for (int k = 0; k < kAhead; ++k, at += ld) r[k] = Row4<T>::load(table + at);
+  };
+  rows(row);
   fetch(tid);
   stage(0);
   __syncthreads();
@@ -159,19 +165,18 @@ __device__ __forceinline__ void runout_tops(const GameDev& G, const RunoutItem* 
     if (c0 + kChunk < H) fetch(c0 + kChunk + tid);
     const ulonglong2* qc = qs + (size_t)buf * kChunk * (kTops / 2);
     const int n = min(kChunk, H - c0);
-    for (int k0 = 0; k0 < n; k0 += kAhead) {
+    for (int k0 = 0; k0 + kAhead <= n; k0 += kAhead) {
+      rows(next);
 #pragma unroll
-      for (int k = 0; k < kAhead; ++k) next[k] = Row4<T>::load(E + (size_t)min(c0 + k0 + kAhead + k, H - 1) * S);
-      if (k0 + kAhead <= n) {
-#pragma unroll
-        for (int k = 0; k < kAhead; ++k) runout_step<T, kTops>(row[k], qc + (size_t)(k0 + k) * (kTops / 2), acc);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kAhead; ++k)
-          if (k0 + k < n) runout_step<T, kTops>(row[k], qc + (size_t)(k0 + k) * (kTops / 2), acc);
-      }
+      for (int k = 0; k < kAhead; ++k) runout_step<T, kTops>(row[k], qc + (k0 + k) * (kTops / 2), acc);
 #pragma unroll
       for (int k = 0; k < kAhead; ++k) row[k] = next[k];
+    }
+    if (n % kAhead) {  // the last chunk's last rows
+      const int k0 = n - n % kAhead;
+#pragma unroll
+      for (int k = 0; k < kAhead - 1; ++k)
+        if (k < n % kAhead) runout_step<T, kTops>(row[k], qc + (k0 + k) * (kTops / 2), acc);
     }
     if (c0 + kChunk < H) stage(buf ^ 1);  // its readers finished before the last barrier
     __syncthreads();

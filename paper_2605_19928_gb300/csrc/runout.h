@@ -40,6 +40,7 @@ struct RunoutGroup {  // up to kRunoutGroup top nodes of one table, evaluated to
   int32_t pad;
 };
 constexpr int kRunoutGroup = 8;
+constexpr int kRunoutPadRows = 16;  // 16-bit rows the pool is allocated beyond its tables (read ahead, not used)
 
 struct RunoutBoard {  // one showdown board of a run-out table
   uint64_t cards;     // the board's public cards

@@ -431,6 +431,16 @@ int build_game(const cfr_game_spec& spec, HostGame& g, std::string& err) {
     const bool passes = nd.type == kChance || nd.type == kShowdown || nd.type == kFold;
     g.reach_src[n] = below_chance && passes ? g.reach_src[nd.parent] : n;
   }
+  for (int p = 0; p < 2; ++p) {
+    std::vector<int32_t>& row = g.reach_row[p];
+    row.resize(N);
+    for (int n = 0; n < N; ++n) {
+      const NodeDev& nd = g.nodes[n];
+      const bool own = nd.parent < 0 || (g.nodes[nd.parent].type == kDecision ? g.nodes[nd.parent].player == p
+                                                                             : g.reach_src[n] == n);
+      row[n] = own ? n : row[nd.parent];
+    }
+  }
 
   // ---- showdown tables, one per board the tree shows down on (table 0 also serves the
   // fold terminals, which only read its card lists)
@@ -536,6 +546,24 @@ std::vector<uint16_t> pack_term_tables(const HostGame& g) {
       }
     }
   }
+  return out;
+}
+
+std::vector<uint16_t> pack_term_records(const HostGame& g) {
+  const size_t H = (size_t)g.n_hands;
+  std::vector<uint16_t> out((size_t)g.n_boards * H * 8, 0);
+  for (size_t b = 0; b < (size_t)g.n_boards; ++b)
+    for (size_t h = 0; h < H; ++h) {
+      uint16_t* r = &out[(b * H + h) * 8];
+      const size_t at = b * H + h;
+      r[0] = (uint16_t)(g.hand_cards[2 * h] | (g.hand_cards[2 * h + 1] << 8));
+      r[1] = (uint16_t)g.sd_gs[at];
+      r[2] = (uint16_t)g.sd_ge[at];
+      for (int s = 0; s < 2; ++s) {
+        r[3 + 2 * s] = (uint16_t)g.cl_lo[2 * at + s];
+        r[4 + 2 * s] = (uint16_t)g.cl_hi[2 * at + s];
+      }
+    }
   return out;
 }
 
@@ -668,6 +696,90 @@ std::vector<uint32_t> node_loads(const HostGame& g, int n, int p, bool backward,
     }
   }
   return mine;
+}
+
+std::vector<uint16_t> tile_table(const HostGame& g) {
+  const int N = (int)g.nodes.size(), L = (int)g.level_start.size() - 1;
+  if (N > 65535 || g.n_rows > 65535) return {};
+  std::vector<TileNode> inner, fwd[2];
+  std::vector<uint16_t> level, ends, flevel[2], all[2];
+  std::vector<TileRow> rows[2];
+  for (int l = 0; l < L; ++l) {
+    const size_t first = inner.size();
+    for (int n = g.level_start[l]; n < g.level_start[l + 1]; ++n) {
+      const NodeDev& nd = g.nodes[(size_t)n];
+      if (is_terminal(nd)) {
+        ends.push_back((uint16_t)n);
+        continue;
+      }
+      if (nd.type == kDecision && nd.n_kids > kStreamMaxActions) return {};
+      TileNode t{};
+      t.id = (uint16_t)n;
+      t.first_kid = (uint16_t)nd.first_kid;
+      t.row = nd.type == kDecision ? (uint16_t)(nd.row - g.row_begin[nd.player]) : 0;
+      t.kids = (uint8_t)(nd.n_kids | (nd.type == kChance ? 2 : nd.player) << 6);
+      inner.push_back(t);
+    }
+    if (inner.size() == first) continue;  // an inner level always lies above: levels stay in order
+    std::stable_sort(inner.begin() + (long)first, inner.end(), [](const TileNode& a, const TileNode& b) {
+      return a.kids < b.kids;  // by kind, then action count
+    });
+    level.push_back((uint16_t)first);
+  }
+  if (inner.empty()) return {};
+  const int levels = (int)level.size();
+  level.push_back((uint16_t)inner.size());
+  for (int p = 0; p < 2; ++p) {
+    rows[p].resize((size_t)(g.row_begin[p + 1] - g.row_begin[p]));
+    for (const TileNode& t : inner)
+      for (int a = 0; t.kids >> 6 == p && a < (t.kids & 63); ++a)
+        rows[p][(size_t)(t.row + a)] = {(uint16_t)(t.first_kid + a), t.id, (uint16_t)g.reach_row[p][t.id], 0};
+  }
+  // the nodes that make new reach rows of a player: its decision nodes, and chance nodes with own
+  // rows below (not run-outs), by how many of them lie above
+  for (int p = 0; p < 2; ++p) {
+    std::vector<int> depth((size_t)N, 0);  // of a node's reach row
+    std::vector<std::vector<TileNode>> by;
+    for (const TileNode& t : inner) {
+      const int kind = t.kids >> 6, src = g.reach_row[p][t.id];
+      if (kind == 1 - p || (kind == 2 && g.reach_row[p][t.first_kid] != t.first_kid)) continue;
+      const size_t d = (size_t)depth[(size_t)src];
+      if (by.size() <= d) by.resize(d + 1);
+      TileNode f = t;
+      f.id = (uint16_t)src;
+      by[d].push_back(f);
+      for (int a = 0; a < (t.kids & 63); ++a) depth[(size_t)t.first_kid + a] = (int)d + 1;
+    }
+    for (const std::vector<TileNode>& l : by) {
+      flevel[p].push_back((uint16_t)fwd[p].size());
+      fwd[p].insert(fwd[p].end(), l.begin(), l.end());
+    }
+    flevel[p].push_back((uint16_t)fwd[p].size());
+    for (int n = 0; n < N; ++n) all[p].push_back((uint16_t)g.reach_row[p][(size_t)n]);
+  }
+  TileHead head{};
+  std::vector<uint16_t> out(sizeof(TileHead) / 2, 0);
+  auto put = [&](const void* data, size_t n16) {
+    const size_t off = (out.size() + 3) / 4 * 4;  // 8-byte aligned
+    out.resize(off + n16);
+    if (n16) memcpy(&out[off], data, n16 * 2);
+    return (int32_t)off;
+  };
+  head.inner = put(inner.data(), inner.size() * sizeof(TileNode) / 2);
+  head.level = put(level.data(), level.size());
+  head.levels = levels;
+  head.ends = put(ends.data(), ends.size());
+  head.n_ends = (int32_t)ends.size();
+  for (int p = 0; p < 2; ++p) {
+    head.rows[p] = put(rows[p].data(), rows[p].size() * sizeof(TileRow) / 2);
+    head.fwd[p] = put(fwd[p].data(), fwd[p].size() * sizeof(TileNode) / 2);
+    head.flevel[p] = put(flevel[p].data(), flevel[p].size());
+    head.flevels[p] = (int32_t)flevel[p].size() - 1;
+    head.all[p] = put(all[p].data(), all[p].size());
+  }
+  memcpy(out.data(), &head, sizeof head);
+  out.resize((out.size() + 7) / 8 * 8, 0);
+  return out;
 }
 
 void plan_runouts(const HostGame& h, RunoutPlan& r) {

@@ -25,6 +25,10 @@ struct HostGame {
   // top chance node of an all-in run-out for the run-out's inner chance nodes and
   // showdowns (nobody acts below it), the node itself otherwise
   std::vector<int32_t> reach_src;
+  // per player: the node whose reach row of that player stands for this node's -- the player's reach
+  // changes only below its own decisions and at dealt cards, so every other node shares its
+  // parent's row (composed with reach_src: below an all-in run-out up to the dealt cards)
+  std::vector<int32_t> reach_row[2];
   // hands
   int n_hands = 0, hstride = 0;
   std::vector<uint8_t> hand_cards;    // [n_hands][2]
@@ -41,6 +45,10 @@ int build_game(const cfr_game_spec& spec, HostGame& out, std::string& err);
 
 // The terminal kernel's per-board uint16 tables (layout: TermTab in pcfr_internal.h).
 std::vector<uint16_t> pack_term_tables(const HostGame& g);
+
+// The grouped terminal launch's per-hand records: per board and hand 8 uint16 -- card ids, gs,
+// ge, lo and hi of the first card, lo and hi of the second, 0 -- one 16-byte load a hand.
+std::vector<uint16_t> pack_term_records(const HostGame& g);
 
 // Decision nodes of player 0 then player 1; begin[p] .. begin[p + 1] are player p's.
 std::vector<int32_t> decision_nodes(const HostGame& g, int begin[3]);
@@ -77,6 +85,12 @@ std::vector<ProgOp> program_ops(const HostGame& g, const std::vector<int32_t>& p
 std::vector<int32_t> stream_tables(const HostGame& g, const std::vector<int32_t>& pre, int half, bool pred,
                                    std::vector<uint32_t>& units, int unit_off[4], int unit_count[4],
                                    int chunk_off[4], int chunk_count[4]);
+
+// The hand-tile table of one subgame (TileHead and its lists, pcfr_internal.h), or empty when its
+// tree does not suit them (node or row ids beyond 16 bits, more actions than a tile's rows hold).
+// Nodes of one level are ordered by kind and action count, so that the slots sharing a warp take the
+// same path; their order changes no result.
+std::vector<uint16_t> tile_table(const HostGame& g);
 
 // All-in run-outs of one game evaluated by win-minus-loss tables (runout.h): a run-out's top
 // is a chance node below a decision whose subtree holds only chance and showdown nodes, all of
