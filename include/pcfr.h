@@ -140,13 +140,13 @@ typedef struct cfr_game_spec {
  * and flops; one subgame per handle, at most 8 actions per decision node).
  * CFR_SCHEDULE_RESIDENT: cfr_iterate runs all its iterations in one cooperative launch;
  * each block keeps one chunk of hands of both players (regrets, strategy sums, strategy,
- * reach) in shared memory for the whole launch, and a grid barrier separates an iteration's
- * phases (the terminal values of a player, then its update), so no phase is a launch of its
- * own (lowest latency for one small subgame).  Every chunk must have a block of its own at
+ * reach) in shared memory for the whole launch, and an iteration's phases (the terminal values
+ * of a player, then its update) wait for each other's values inside it, so no phase is a launch
+ * of its own (lowest latency for one small subgame).  Every chunk must have a block of its own at
  * one block per SM (chunk_hands = 0 takes the smallest of 8, 16 and 32 hands that allows
  * it) and the tree must have no depth-limit leaves: CFR_EINVAL otherwise.  The other passes
- * (initial strategy, average, best response) use the level schedule's kernels.  A grid
- * barrier that waits too long gives up (about a second): cfr_sync then returns
+ * (initial strategy, average, best response) use the level schedule's kernels.  A wait inside
+ * the launch that takes too long gives up (about a second): cfr_sync then returns
  * CFR_ETIMEOUT and the handle's state is undefined.
  * CFR_SCHEDULE_AUTO (0) picks STREAM when the handle has at least 1216 such warps (8 per
  * SM) and every tree allows it, WIDE for one subgame too large to stage, else LEVEL.
@@ -320,9 +320,9 @@ int cfr_sync(cfr_tree* tree);
  * can land.  A block that gives up still waits, with the default limit, for its own copies
  * to land, then sets the handle's device flag and returns without computing its values,
  * so the next synchronising call on the handle reports CFR_ETIMEOUT and the CUDA context
- * stays usable.  The same limit applies to the first grid barrier of each resident-schedule
- * launch (CFR_SCHEDULE_RESIDENT): with 0 every block but the last to arrive gives up, sets
- * the flag, and the others see it at their next barrier and leave.  Call it while none of
+ * stays usable.  The same limit applies to the waits of the first iteration of each resident-
+ * schedule launch (CFR_SCHEDULE_RESIDENT): with 0 every block whose values are not there yet gives
+ * up, sets the flag, and the others see it at their next wait and leave.  Call it while none of
  * the library's kernels are in flight (e.g. after cfr_sync); it applies to every handle on
  * the device until it is called again. */
 int cfr_debug_first_wait_polls(long polls);

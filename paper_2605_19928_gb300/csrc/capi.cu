@@ -85,6 +85,7 @@ struct cfr_tree {
   cfr_solver_opts opts{};
   LaunchCtx ctx{};
   int iters_done = 0;
+  uint32_t resident_stamp = 0;  // resident schedule: the last stamp its launches have used
   int64_t state_gen = 0;        // bumped whenever R or S may change
   int64_t avg_gen = -1;         // state_gen for which sigbar holds k_average_rows' output
   int64_t cur_gen = -1;         // state_gen for which sigma holds RM(R) (stream schedule)
@@ -579,31 +580,49 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // SM that a block of 128 threads has, or, where a tree is too large for that or values are
   // pairs, in the quarter of a block of 256.  warp_hands = 64 asks for the one-warp walk, and
   // chunk_hands beyond 8 for best-response sums a tile cannot form.
-  bool tiles = schedule == kScheduleStream && o.warp_hands != 64 && chunk[0] <= 8;
+  // The level and wide schedules (one subgame, or few) run their passes as the latency form of the
+  // same kernel when every tree fits it with chunk_hands hands a tile (4 or more: 16-byte pieces),
+  // and the resident schedule walks the same tables.
+  const bool stream_tiles = schedule == kScheduleStream && o.warp_hands != 64 && chunk[0] <= 8;
+  const bool staged = schedule != kScheduleStream && chunk[0] >= 4 && !o.runout_tables;
   std::vector<std::vector<uint16_t>> tile_tabs(n_games);
-  std::vector<int> tile_wlog(n_games, 0);
+  std::vector<int> tile_wlog(n_games, 0), tile_group(n_games, 0);
   size_t smem_tile = 0;
   int tile_threads = 0;
-  if (tiles) parallel_games(n_games, [&](int g) { tile_tabs[g] = tile_table(t->host[g]); });
-  for (int small = es == 4; tiles && small >= 0 && !tile_threads; --small) {
+  if (stream_tiles || staged || resident) parallel_games(n_games, [&](int g) { tile_tabs[g] = tile_table(t->host[g]); });
+  auto tile_bytes = [&](int g, int wl, int with_rs) {
+    const HostGame& h = t->host[g];
+    const int rows_max = std::max(h.row_begin[1] - h.row_begin[0], h.row_begin[2] - h.row_begin[1]);
+    return tile_smem_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, 1 << wl, es, with_rs);
+  };
+  for (int small = es == 4; stream_tiles && small >= 0 && !tile_threads; --small) {
     const size_t limit = small ? kTileSmemSmall : kTileSmem;
     bool fit = true;
     smem_tile = 0;
     for (int g = 0; g < n_games && fit; ++g) {
-      const HostGame& h = t->host[g];
-      const int rows_max = std::max(h.row_begin[1] - h.row_begin[0], h.row_begin[2] - h.row_begin[1]);
-      auto bytes = [&](int wl) {
-        return tile_smem_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, 1 << wl, es);
-      };
       int wl = 5;
-      while (wl > 3 && bytes(wl) > limit) --wl;
-      fit = !tile_tabs[g].empty() && bytes(wl) <= limit;
+      while (wl > 3 && tile_bytes(g, wl, 0) > limit) --wl;
+      fit = !tile_tabs[g].empty() && tile_bytes(g, wl, 0) <= limit;
       tile_wlog[g] = wl;
-      smem_tile = std::max(smem_tile, bytes(wl));
+      smem_tile = std::max(smem_tile, tile_bytes(g, wl, 0));
     }
     if (fit) tile_threads = small ? 128 : 256;
   }
-  tiles = tile_threads > 0;
+  if (staged || resident) {
+    bool fit = staged;
+    for (int g = 0; g < n_games; ++g) {
+      while (1 << tile_wlog[g] < chunk[g]) ++tile_wlog[g];
+      if (tile_tabs[g].empty()) {
+        fit = false;
+        continue;
+      }
+      tile_group[g] = tile_walkers(t->host[g], chunk[g]);
+      smem_tile = std::max(smem_tile, tile_bytes(g, tile_wlog[g], 1));
+    }
+    // a wave of blocks takes each phase in one step with 512 threads; more blocks overlap instead
+    if (fit && smem_tile <= (size_t)kTileSmemStaged) tile_threads = chunks_of(chunk[0]) <= n_sms ? 512 : 256;
+  }
+  const bool tiles = tile_threads > 0;
   RunoutPlan ro;
   if (o.runout_tables) {
     if (schedule != kScheduleWide || t->host[0].hand_size != 2) {
@@ -619,15 +638,16 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // Resident schedule: one block per SM holds a chunk's state of both players beside a terminal
   // node's board table, and every chunk has a block.
   size_t res_term = 0, res_hand = 0;
+  bool tabled = true;
   if (resident) {
     for (int g = 0; g < n_games; ++g) {
       const HostGame& h = t->host[g];
       const int rows_max = std::max(h.row_begin[1] - h.row_begin[0], h.row_begin[2] - h.row_begin[1]);
       res_term = std::max(res_term, resident_term_size(h.n_hands, h.hand_size, h.deck, h.hstride, es));
-      res_hand = std::max(res_hand, resident_hand_size((int)h.nodes.size(), (int)h.level_start.size() - 1, rows_max,
-                                                       chunk[g], es));
+      res_hand = std::max(res_hand, resident_hand_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, chunk[g], es));
+      tabled = tabled && !tile_tabs[g].empty();
     }
-    const int per_sm = res_term + res_hand <= 200 * 1024 ? resident_blocks_per_sm(o.precision, res_term + res_hand) : 0;
+    const int per_sm = tabled && res_term + res_hand <= 200 * 1024 ? resident_blocks_per_sm(o.precision, res_term + res_hand) : 0;
     const long chunks = chunks_of(chunk[0]);  // reads the handle's games
     if (per_sm < 1 || chunks > (long)per_sm * n_sms) {
       delete t;
@@ -661,8 +681,13 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // (a block per node then has the lower latency), else groups of four (two with pair values:
   // 16-byte entries either way).
   int n_ends = 0;
+  std::vector<char> shows(n_games, es == 8);  // its records are read: at showdowns, and pairs' folds
   for (int g = 0; g < n_games; ++g)
-    for (int n : t->host[g].terminals) n_ends += ro.inside.empty() || !ro.inside[(size_t)n];
+    for (int n : t->host[g].terminals)
+      if (ro.inside.empty() || !ro.inside[(size_t)n]) {
+        ++n_ends;
+        if (t->host[g].nodes[(size_t)n].type == kShowdown) shows[g] = 1;
+      }
   const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= kTermGroupMin ? 4 : 1;
   const int term_nv = term_nodes == 1 ? 1 : term_nodes < 4 || es == 8 ? 2 : 4;
 
@@ -686,8 +711,8 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       for (int k = 0; k < h.n_hands; ++k) q.r64[p * S + k] = h.range[p][k];
     q.rv = to_value_type(q.r64, o.precision);
     q.tab = pack_term_tables(h);
-    if (term_nv > 1) q.rec = pack_term_records(h);
-    if (tiles) q.tile = std::move(tile_tabs[g]);
+    if (shows[g] && (term_nv > 1 || resident)) q.rec = pack_term_records(h);
+    if (tiles || resident) q.tile = std::move(tile_tabs[g]);
     q.rown = row_nodes(h);
     q.decn = decision_nodes(h, q.dec_begin);
     const double kappa = 1.0 / h.Z;
@@ -749,6 +774,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     packer.table(q.tile, &d.tile_tab);
     d.tile_tab16 = (int)q.tile.size() / 8;
     d.tile_wlog = tile_wlog[g];
+    d.tile_group = tile_group[g];
     packer.table(decn, &d.dec_nodes);
     packer.table(ops, &d.prog);
     packer.table(chunk_lists[g], &d.chunks);
@@ -764,6 +790,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     packer.zeroed(cells * es, &d.cfv);
     packer.zeroed(cells * es, &d.cfv_br);
     if (o.variant == CFR_VARIANT_PCFRPLUS) packer.zeroed(rows * 8, &d.M);
+    if (resident && o.alternating) {
+      packer.zeroed(cells * es * 2, &d.xval);
+      packer.zeroed(cells * es * 2, &d.xreach);
+    }
     packer.zeroed((size_t)2 * d.n_chunks * 8, &d.br_partial);
     packer.zeroed(4, &d.br_done);
     for (int c = 0; c < d.n_chunks; ++c) chunk_work.push_back({g, c});
@@ -936,6 +966,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.n_tile_work = (int)tile_work.size();
   c.smem_tile = smem_tile;
   c.tile_threads = tile_threads;
+  c.tile_staged = tiles && staged;
   c.stream_depth = stream_depth;
   c.stream_prog = stream_prog;
   c.stream_half = stream_half;
@@ -1012,7 +1043,7 @@ int leaf_launches(const cfr_tree* t, int player_mask) {
 
 // Kernels one pass launches: one, or one per level under the wide schedule.
 int pass_launches(const cfr_tree* t, int which, int player_mask, int advance) {
-  if (t->ctx.schedule != kScheduleWide) return 1;
+  if (t->ctx.schedule != kScheduleWide || t->ctx.n_tile_work > 0) return 1;
   return wide_launch_count(t->ctx, which, player_mask, advance);
 }
 
@@ -1106,8 +1137,17 @@ int cfr_iterate(cfr_tree* t, int n_iters) {
   t->state_gen += 1;
   if (t->ctx.resident) {  // one cooperative launch per 2^20 iterations (its barrier count stays in 32 bits)
     for (int done = 0; done < n_iters; done += 1 << 20) {
-      if (launch_resident(t->ctx, std::min(n_iters - done, 1 << 20), t->stream) != 0)
-        return fail(CFR_ECUDA, "resident launch failed");
+      const int n = std::min(n_iters - done, 1 << 20);
+      if (t->resident_stamp > 0xffffffffu - (uint32_t)n) {  // the stamps start again: clear the old ones
+        for (const GameDev& d : t->dev) {
+          const size_t bytes = (size_t)2 * d.n_nodes * d.hstride * (t->opts.precision == CFR_PRECISION_SINGLE ? 8 : 16);
+          if (d.xval) CK(cudaMemsetAsync(d.xval, 0, bytes, t->stream));
+          if (d.xreach) CK(cudaMemsetAsync(d.xreach, 0, bytes, t->stream));
+        }
+        t->resident_stamp = 0;
+      }
+      if (launch_resident(t->ctx, n, t->resident_stamp, t->stream) != 0) return fail(CFR_ECUDA, "resident launch failed");
+      t->resident_stamp += (uint32_t)n;
       t->launches += 1;
     }
     t->iters_done += n_iters;

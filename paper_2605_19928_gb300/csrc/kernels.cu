@@ -206,91 +206,6 @@ __device__ __forceinline__ acc2 acc_shfl_up(acc2 a, int o) {
   return {__shfl_up_sync(0xffffffffu, a.s, o), __shfl_up_sync(0xffffffffu, a.e, o)};
 }
 
-// Exclusive prefix sum of the non-negative values value_at(0 .. n-1) into out[0 .. n]
-// (out[n] = total) by one group of GT consecutive threads (gtid = rank in the group; every
-// thread of the block must call it, so that the block barriers inside line up).  Each
-// thread owns a contiguous run; runs are combined by a warp-shuffle scan and a scan over the
-// group's warp totals in red[GT / 32].  Sums are compensated (acc2).
-template <int GT, typename F>
-__device__ __forceinline__ ff group_exclusive_scan(int n, F value_at, ff* out, acc2* red, int gtid) {
-  const int per = (n + GT - 1) / GT;
-  const int lane = gtid & 31, warp = gtid >> 5;
-  const int begin = min(gtid * per, n), end = min(begin + per, n);
-  acc2 local = acc_zero();
-  for (int j = begin; j < end; ++j) acc_add(local, value_at(j));
-  acc2 x = local;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const acc2 y = acc_shfl_up(x, o);
-    if (lane >= o) acc_merge(x, y);
-  }
-  acc2 run = acc_shfl_up(x, 1);
-  if (lane == 0) run = acc_zero();
-  if (lane == 31) red[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    acc2 wv = lane < GT / 32 ? red[lane] : acc_zero();
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const acc2 y = acc_shfl_up(wv, o);
-      if (lane >= o) acc_merge(wv, y);
-    }
-    if (lane < GT / 32) red[lane] = wv;
-  }
-  __syncthreads();
-  if (warp > 0) acc_merge(run, red[warp - 1]);
-  for (int j = begin; j < end; ++j) {  // value read before out[j] is written: out may be the input
-    const ff v = value_at(j);
-    out[j] = acc_value(run);
-    acc_add(run, v);
-  }
-  const ff total = acc_value(red[GT / 32 - 1]);
-  if (gtid == 0) out[n] = total;
-  __syncthreads();
-  return total;
-}
-
-// The same exclusive prefix sum in plain FP32 (values of the single-precision path; the
-// error of a prefix stays within a few dozen ulps of the total).
-template <int GT, typename F>
-__device__ __forceinline__ float group_exclusive_scan_f32(int n, F value_at, float* out, float* red, int gtid) {
-  const int per = (n + GT - 1) / GT;
-  const int lane = gtid & 31, warp = gtid >> 5;
-  const int begin = min(gtid * per, n), end = min(begin + per, n);
-  float local = 0.f;
-  for (int j = begin; j < end; ++j) local = __fadd_rn(local, value_at(j));
-  float x = local;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x = __fadd_rn(x, y);
-  }
-  float run = __shfl_up_sync(0xffffffffu, x, 1);
-  if (lane == 0) run = 0.f;
-  if (lane == 31) red[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    float wv = lane < GT / 32 ? red[lane] : 0.f;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float y = __shfl_up_sync(0xffffffffu, wv, o);
-      if (lane >= o) wv = __fadd_rn(wv, y);
-    }
-    if (lane < GT / 32) red[lane] = wv;
-  }
-  __syncthreads();
-  if (warp > 0) run = __fadd_rn(run, red[warp - 1]);
-  for (int j = begin; j < end; ++j) {  // value read before out[j] is written: out may be the input
-    const float v = value_at(j);
-    out[j] = run;
-    run = __fadd_rn(run, v);
-  }
-  const float total = red[GT / 32 - 1];
-  if (gtid == 0) out[n] = total;
-  __syncthreads();
-  return total;
-}
-
 // ------------------------------------------------------------------ bulk copies (TMA) into shared memory
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -365,288 +280,17 @@ __device__ __forceinline__ bool holds_board_card(const uint16_t* cards, int h, i
   return (((board >> (cw & 0xffu)) | (k == 2 ? board >> (cw >> 8) : 0ull)) & 1ull) != 0;
 }
 
-// Values of player i at one fold or showdown node n (Stages 2-4), the opponent's reach q
-// at n already in shared memory.  kappa = 1/Z, and the node's payoff already carries the
-// probability of the public cards dealt on its path, so every value is a counterfactual
-// value in the sense of Eq. (cfv).
+// Values of player i at fold and showdown nodes (Stages 2-4) from the opponent's reach q there.
+// kappa = 1/Z, and a node's payoff already carries the probability of the public cards dealt on its
+// path, so every value is a counterfactual value in the sense of Eq. (cfv).
 //   fold (Stage 3):   v_i(h) = u_i kappa (T - C[c1] - C[c2] + q[h]),  T = sum_o q[o],
 //                     C[c] = sum_{o holds c} q[o]  (inclusion-exclusion over the two cards)
 //   showdown (Stage 4): v_i(h) = c kappa (W(h) - L(h)), W / L the opponent reach of weaker /
 //                     stronger hands that share no card with h, from exclusive prefix sums
 //                     over the rank-sorted order minus per-card prefix sums; the tie group
 //                     of h is excluded from both (a split pot pays 0).
-// Sums and differences are double-float with FP32-pair values, plain FP32 with FP32
-// values.  Every thread of the block calls it (it holds block barriers).
-template <typename P>
-__device__ __forceinline__ void terminal_values(const GameDev& G, const NodeDev& nd, int i, ff u,
-                                                const TermTab& tt, const uint16_t* tab,
-                                                const typename P::V* __restrict__ qs, ff* CP, ff* Psc,
-                                                typename P::V* __restrict__ out) {
-  using V = typename P::V;
-  __shared__ acc2 red[2][kTermThreads / 64];
-  const float uf = u.hi;  // FP32 values: the scale rounded once to FP32
-  const int H = G.n_hands, k = G.hand_size;
-  const bool show = nd.type == kShowdown;
-  const uint64_t board = nd.board;
-  const uint16_t* clh = tab + tt.clh;
-  const uint16_t* cards = tab + tt.cards;
-  const uint16_t* cloff = tab + tt.cloff;
-  const uint16_t* perm = tab + tt.perm;
-  if constexpr (std::is_same<P, Single>::value) {
-    if (!show) {
-      // fold (FP32 values): no prefix sums needed.  T: warp 0 keeps 32 lane-strided partial
-      // sums of q and combines them by a fixed xor tree (lane 0's result); C[c]: one thread
-      // per card sums card c's list in list order.  Few warps work and the others wait at
-      // one barrier, which the other blocks on the SM fill.
-      __shared__ float Cs[kMaxDeck];
-      __shared__ float Tsh;
-      const int lane = threadIdx.x & 31;
-      if (threadIdx.x < 32) {
-        float t = 0.f;
-#pragma unroll 8
-        for (int h = lane; h < H; h += 32) t = __fadd_rn(t, qs[h]);
-        for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
-        if (lane == 0) Tsh = t;
-      } else if (threadIdx.x - 32 < G.deck) {
-        const int c = threadIdx.x - 32;
-        float x = 0.f;
-#pragma unroll 4
-        for (int j = cloff[c]; j < cloff[c + 1]; ++j) x = __fadd_rn(x, qs[clh[j]]);
-        Cs[c] = x;
-      }
-      __syncthreads();
-      const float T = Tsh;
-      for (int h = threadIdx.x; h < H; h += kTermThreads) {
-        const unsigned cw = cards[h];
-        const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
-        float m = __fsub_rn(T, Cs[c1]);
-        bool blocked = (board >> c1) & 1ull;
-        if (k == 2) {
-          m = __fadd_rn(__fsub_rn(m, Cs[c2]), qs[h]);
-          blocked = blocked || ((board >> c2) & 1ull);
-        }
-        out[h] = blocked ? 0.f : __fmul_rn(uf, m);
-      }
-      __syncthreads();  // Cs and Tsh are reused by the next node
-      return;
-    }
-    // FP32 values: the same scans and differences in plain FP32 (a value's error stays
-    // within about 1e-6 of the largest value at the node)
-    __shared__ float redf[2][kTermThreads / 32];
-    __shared__ float cps[kMaxDeck], cpe[kMaxDeck];  // prefix at the start / end of each card's list
-    float* CPf = reinterpret_cast<float*>(CP);  // [k H + 1]
-    float* Pf = CPf + (k * H + 1);             // [H + 1]
-    {  // the reach in rank order and along the card lists, gathered once into the scans'
-       // output arrays (lanes on consecutive entries), then scanned in place, each thread
-       // over a contiguous run: the same sums as scanning the gathers directly, with half
-       // the random shared-memory reads.  Two-card hands' card lists hold 2 H entries, so 11
-       // warps scan them and 5 the H rank-ordered entries (about 7 per thread on both sides).
-      for (int j = threadIdx.x; j < H; j += kTermThreads) Pf[j] = qs[show ? perm[j] : j];
-      for (int j = threadIdx.x; j < k * H; j += kTermThreads) CPf[j] = qs[clh[j]];
-      __syncthreads();
-      constexpr int gp = 5 * 32;
-      if (threadIdx.x < gp)
-        group_exclusive_scan_f32<gp>(H, [&](int j) { return Pf[j]; }, Pf, redf[0], threadIdx.x);
-      else
-        group_exclusive_scan_f32<kTermThreads - gp>(k * H, [&](int j) { return CPf[j]; }, CPf, redf[1],
-                                                     threadIdx.x - gp);
-    }
-    for (int c = threadIdx.x; c < G.deck; c += kTermThreads) {
-      cps[c] = CPf[cloff[c]];
-      cpe[c] = CPf[cloff[c + 1]];
-    }
-    __syncthreads();
-    const float T = Pf[H];
-    if (!show) {
-      for (int h = threadIdx.x; h < H; h += kTermThreads) {
-        const unsigned cw = cards[h];
-        const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
-        float m = __fsub_rn(T, __fsub_rn(CPf[cloff[c1 + 1]], CPf[cloff[c1]]));
-        bool blocked = (board >> c1) & 1ull;
-        if (k == 2) {
-          m = __fsub_rn(m, __fsub_rn(CPf[cloff[c2 + 1]], CPf[cloff[c2]]));
-          m = __fadd_rn(m, qs[h]);
-          blocked = blocked || ((board >> c2) & 1ull);
-        }
-        out[h] = blocked ? 0.f : __fmul_rn(uf, m);
-      }
-    } else {
-      const uint16_t* gs = tab + tt.gs;
-      const uint16_t* ge = tab + tt.ge;
-      const uint16_t* lo = tab + tt.lo;
-      const uint16_t* hi = tab + tt.hi;
-      if (k == 2) {  // the same differences, card 1 then card 2, in straight-line code
-        for (int h = threadIdx.x; h < H; h += kTermThreads) {
-          const unsigned cw = cards[h];
-          const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
-          float Wn = Pf[gs[h]];
-          float Ln = __fsub_rn(T, Pf[ge[h]]);
-          Wn = __fsub_rn(Wn, __fsub_rn(CPf[lo[2 * h]], cps[c1]));
-          Ln = __fsub_rn(Ln, __fsub_rn(cpe[c1], CPf[hi[2 * h]]));
-          Wn = __fsub_rn(Wn, __fsub_rn(CPf[lo[2 * h + 1]], cps[c2]));
-          Ln = __fsub_rn(Ln, __fsub_rn(cpe[c2], CPf[hi[2 * h + 1]]));
-          const bool blocked = ((board >> c1) | (board >> c2)) & 1ull;
-          out[h] = blocked ? 0.f : __fmul_rn(uf, __fsub_rn(Wn, Ln));
-        }
-      } else {  // one-card hands (Kuhn, Leduc)
-        for (int h = threadIdx.x; h < H; h += kTermThreads) {
-          const unsigned c = cards[h] & 0xffu;
-          const float Wn = __fsub_rn(Pf[gs[h]], __fsub_rn(CPf[lo[2 * h]], cps[c]));
-          const float Ln = __fsub_rn(__fsub_rn(T, Pf[ge[h]]), __fsub_rn(cpe[c], CPf[hi[2 * h]]));
-          out[h] = ((board >> c) & 1ull) ? 0.f : __fmul_rn(uf, __fsub_rn(Wn, Ln));
-        }
-      }
-    }
-    return;
-  }
-  // Two scans at once, one per half of the block: the first half takes the reach in
-  // rank-sorted order (showdown) or in hand order (fold, for the total T), the second half
-  // the reach along the per-card hand lists.
-  {  // each scan's values gathered once into its output array, then scanned in place
-    for (int j = threadIdx.x; j < H; j += kTermThreads) Psc[j] = P::to_ff(qs[show ? perm[j] : j]);
-    for (int j = threadIdx.x; j < k * H; j += kTermThreads) CP[j] = P::to_ff(qs[clh[j]]);
-    __syncthreads();
-    constexpr int half = kTermThreads / 2;
-    const bool first = threadIdx.x < half;
-    const int gtid = first ? threadIdx.x : threadIdx.x - half;
-    if (first)
-      group_exclusive_scan<half>(H, [&](int j) { return Psc[j]; }, Psc, red[0], gtid);
-    else
-      group_exclusive_scan<half>(k * H, [&](int j) { return CP[j]; }, CP, red[1], gtid);
-  }
-  const ff T = Psc[H];
-
-  if (!show) {
-    for (int h = threadIdx.x; h < H; h += kTermThreads) {
-      const unsigned cw = cards[h];
-      const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
-      ff m = ff_sub(T, ff_sub(CP[cloff[c1 + 1]], CP[cloff[c1]]));
-      bool blocked = (board >> c1) & 1ull;
-      if (k == 2) {
-        m = ff_sub(m, ff_sub(CP[cloff[c2 + 1]], CP[cloff[c2]]));
-        m = ff_add(m, P::to_ff(qs[h]));
-        blocked = blocked || ((board >> c2) & 1ull);
-      }
-      out[h] = blocked ? P::zero() : P::of_ff(ff_mul(u, m));
-    }
-  } else {
-    const uint16_t* gs = tab + tt.gs;
-    const uint16_t* ge = tab + tt.ge;
-    const uint16_t* lo = tab + tt.lo;
-    const uint16_t* hi = tab + tt.hi;
-    for (int h = threadIdx.x; h < H; h += kTermThreads) {
-      const unsigned cw = cards[h];
-      ff Wn = Psc[gs[h]];
-      ff Ln = ff_sub(T, Psc[ge[h]]);
-      bool blocked = false;
-      for (int s = 0; s < k; ++s) {
-        const unsigned c = s == 0 ? (cw & 0xffu) : (cw >> 8);
-        Wn = ff_sub(Wn, ff_sub(CP[lo[2 * h + s]], CP[cloff[c]]));
-        Ln = ff_sub(Ln, ff_sub(CP[cloff[c + 1]], CP[hi[2 * h + s]]));
-        blocked = blocked || ((board >> c) & 1ull);
-      }
-      out[h] = blocked ? P::zero() : P::of_ff(ff_mul(u, ff_sub(Wn, Ln)));
-    }
-  }
-}
-
-// The player of a block of the terminal launch and its item of n (grid: (player, item)).
-__device__ __forceinline__ int terminal_item(int n, int player_mask, int& i) {
-  if (player_mask != 3) {
-    i = player_mask == 1 ? 0 : 1;
-    return blockIdx.x;
-  }
-  i = (int)blockIdx.x >= n;
-  return blockIdx.x - i * n;
-}
-
-// Payoff for player i per unit of (opponent reach) x kappa at node n: the FP64 product as a pair
-// of FP32 rounded once on the host (FP32 values use its high part): no FP64 work per thread.
-__device__ __forceinline__ ff terminal_payoff(const GameDev& G, const NodeDev& nd, int n, int i) {
-  const bool neg = nd.type == kFold && nd.player == i;
-  return {neg ? -G.payoff_ff[2 * n] : G.payoff_ff[2 * n], neg ? -G.payoff_ff[2 * n + 1] : G.payoff_ff[2 * n + 1]};
-}
-
-// Terminal values (Stages 2-4), the one-node form for handles with few terminals (latency: all
-// registers it wants).  One block per (player, node): the board table is staged by a bulk (TMA)
-// copy before the launch waits for its predecessor, the opponent's reach row after it.  A
-// showdown below an all-in run-out reads the run-out's reach row (src) and zeroes the hands
-// holding a dealt card itself (nobody acts below the run-out, so that is its reach).
-// The wait is bounded: on a timeout the block sets *err, lets its copies drain and leaves.
-template <typename P>
-__global__ void __launch_bounds__(kTermThreads, 1) k_terminal(const GameDev* __restrict__ games,
-                                                            const Work* __restrict__ work,
-                                                            const TermSrc* __restrict__ src, int n_work,
-                                                            int player_mask, int use_bar, int* err) {
-  using V = typename P::V;
-  int i;
-  const int first = terminal_item(n_work, player_mask, i);
-  const GameDev& G = games[work[first].game];
-  const int n = work[first].unit;
-  const NodeDev nd = G.nodes[n];
-  const int H = G.n_hands, k = G.hand_size;
-  const size_t stride = (size_t)G.hstride;
-  const TermTab tt(H, k, G.deck);
-  const bool show = nd.type == kShowdown;
-  const unsigned tab_bytes = (unsigned)(show ? tt.len : tt.fold_len) * 2u;
-  const unsigned q_bytes = (unsigned)(stride * sizeof(V));
-  const V* qsrc = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + (size_t)(1 - i) * G.n_nodes * stride;
-  V* dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
-
-  extern __shared__ __align__(128) unsigned char smt[];
-  __shared__ __align__(8) uint64_t bar;
-  uint16_t* tab = reinterpret_cast<uint16_t*>(smt);                            // [tt.len]
-  V* q = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);                        // [hstride]
-  ff* CP = reinterpret_cast<ff*>(smt + (size_t)tt.len * 2 + (size_t)q_bytes);   // [k H + 1]
-  ff* Psc = CP + (k * H + 1);                                                   // [H + 1]
-
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {  // the board tables are static: copy them before waiting
-    mbar_arrive_expect_tx(&bar, tab_bytes + q_bytes);
-    bulk_copy_g2s(tab, G.term_tab + (size_t)(show ? nd.row : 0) * tt.len, tab_bytes, &bar);
-  }
-  pdl_wait();  // the reach rows come from the launch just before this one
-  pdl_trigger();
-  const int from = src[first].row[1 - i];
-  if (threadIdx.x == 0) bulk_copy_g2s(q, qsrc + (size_t)term_src_node(from) * stride, q_bytes, &bar);
-  const ff u = terminal_payoff(G, nd, n, i);
-  const bool ok = threadIdx.x >= 32 || mbar_wait_bounded(&bar, 0, g_first_wait_polls);  // one warp polls
-  if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
-    if (threadIdx.x == 0) {
-      atomicExch(err, 1);
-      mbar_wait_bounded(&bar, 0);
-    }
-    __syncthreads();
-    return;
-  }
-  if (from < 0) {  // below an all-in run-out: the run-out's reach, without the hands holding
-    for (int h = threadIdx.x; h < H; h += blockDim.x)  // a card dealt on the way
-      if (holds_board_card(tab + tt.cards, h, k, nd.board)) q[h] = P::zero();
-    __syncthreads();
-  }
-  terminal_values<P>(G, nd, i, u, tt, tab, q, CP, Psc, dst + (size_t)n * stride);
-}
-
-// ---- several nodes at once: the throughput form for handles whose terminals fill the GPU
-//
-// A group is up to NV nodes of one game, one kind (folds or showdowns) and one board table.  The
-// scan arrays of terminal_values become arrays of NV values (16 bytes), so each table entry and
-// each address is read and computed once for NV nodes and a gather is one 16-byte shared-memory
-// access.  Component v runs exactly the one-node form's operations in its order (the same runs
-// of entries per thread, the same combination of threads and warps), so the bits are the same.
-//
-// Blocks are persistent: two per SM, each walking its own contiguous stretch of the groups, so
-// that the board table is reloaded only when it changes, descriptors are staged once, and the
-// reach rows of the next group are in flight (bulk copies, two buffers) while the current one
-// is computed.  A showdown group takes three block barriers: rows landed; each thread has
-// gathered its run of entries into registers and summed it; the prefix sums are written.
-// Bound by random shared-memory gathers (5060 wavefronts a group of four, 45 % of the pipe's rate).
-// Measured against blocks that take their nodes one by one: exact turn 119 -> 88 us per player,
-// 256 rivers 132 -> 129, with one block per group and its descriptors read node by node 147.
+// Sums and differences are double-float with FP32-pair values (whose folds take T and C[c] from
+// the same prefix sums, in hand order), plain FP32 with FP32 values.
 
 // Entries of a thread's run at most, for the 1176 hands a flop leaves: 1176 over 160 threads (8) and
 // 2352 over 352 (7) with FP32 values, 2352 over 256 (10) with pairs.
@@ -672,9 +316,10 @@ __device__ __forceinline__ acc2 acc_from(acc2 a, int l) {
 __device__ __forceinline__ void acc_join(float& a, float b) { a = __fadd_rn(a, b); }
 __device__ __forceinline__ void acc_join(acc2& a, acc2 b) { acc_merge(a, b); }
 
-// One thread's part of group_exclusive_scan(_f32) over NV arrays: its run's values are in
-// registers (a[0 .. cnt)), x receives the inclusive sum of its warp's runs up to its own, and the
-// warp's total goes to red[warp].
+// Exclusive prefix sums of NV arrays of n values by GT consecutive threads, in two halves with a block
+// barrier between.  Each thread owns a run of ceil(n / GT) entries, whose values are in registers
+// (a[0 .. cnt)): first x receives the inclusive sum of its warp's runs up to its own, and the warp's
+// total goes to red[warp].  Sums are plain FP32 with FP32 values, compensated with pairs.
 template <typename P, int NV>
 __device__ __forceinline__ void scan_runs(const Vec<P, NV> (&a)[ScanPer<P>::n], int cnt, VecAcc<P, NV>* red, int gtid,
                                           VecAcc<P, NV>& x) {
@@ -697,8 +342,8 @@ __device__ __forceinline__ void scan_runs(const Vec<P, NV> (&a)[ScanPer<P>::n], 
   if (lane == 31) red[gtid >> 5] = x;
 }
 
-// After the barrier: the exclusive prefix sums of the thread's run into out (out[n] = totals).
-// Every warp scans the GT / 32 warp totals itself, as the one-node form's first warp does.
+// After the barrier: the exclusive prefix sums of the thread's run into out (out[n] = totals).  Every
+// warp scans the GT / 32 warp totals itself.
 template <typename P, int NV, int GT>
 __device__ __forceinline__ void scan_write(const Vec<P, NV> (&a)[ScanPer<P>::n], int begin, int cnt, int n,
                                            const VecAcc<P, NV>* red, int gtid, const VecAcc<P, NV>& x,
@@ -733,6 +378,264 @@ __device__ __forceinline__ void scan_write(const Vec<P, NV> (&a)[ScanPer<P>::n],
     }
   if (gtid == 0) out[n] = total;
 }
+
+// ---- one node, all of a block of kTermThreads threads: the latency form
+
+constexpr int kTermHands = 3;  // hands per thread: at most 1176 of them
+
+// The threads on the rank order (the others take the card lists), and a thread's run of them.
+template <typename P>
+struct TermRun {
+  static constexpr int gp = std::is_same<P, Single>::value ? 5 * 32 : kTermThreads / 2;
+  int begin, cnt;
+  __device__ __forceinline__ TermRun() : begin(0), cnt(0) {}
+  __device__ __forceinline__ TermRun(int H, int k) {
+    const int tid = threadIdx.x, n = tid < gp ? H : k * H, gn = tid < gp ? gp : kTermThreads - gp,
+              per = (n + gn - 1) / gn;
+    begin = min((tid < gp ? tid : tid - gp) * per, n);
+    cnt = min(begin + per, n) - begin;
+  }
+};
+
+// What a thread reads of a board table for the nodes of one kind: the hands of its run (in rank
+// order, or along the card lists; pairs' folds: in hand order), two in a word, and its hands' records.
+// It stays in registers while the block's nodes share the table and kind (resident schedule).
+template <typename P>
+struct TermLane {
+  TermRun<P> run;
+  uint32_t at[ScanPer<P>::n / 2];
+  uint4 rec[kTermHands];
+  __device__ __forceinline__ int hand(int e) const { return at[e / 2] >> (e & 1 ? 16 : 0) & 0xffffu; }
+  __device__ __forceinline__ uint4 record(int s, int) const { return rec[s]; }
+};
+
+// The same read from the staged table when it is used (one-node launch: each block has one node).
+template <typename P>
+struct TermStaged {
+  TermRun<P> run;
+  const uint16_t *list, *cards, *gs, *ge, *lo, *hi;  // list: the thread's run, or null (hand order)
+  __device__ __forceinline__ int hand(int e) const {
+    return e >= run.cnt ? 0 : list ? list[run.begin + e] : run.begin + e;
+  }
+  __device__ __forceinline__ uint4 record(int, int h) const {
+    return make_uint4(cards[h] | (uint32_t)gs[h] << 16, ge[h] | (uint32_t)lo[2 * h] << 16,
+                      hi[2 * h] | (uint32_t)lo[2 * h + 1] << 16, hi[2 * h + 1]);
+  }
+};
+
+template <typename P>
+__device__ __forceinline__ void term_lane_load(TermLane<P>& L, const GameDev& G, int table, bool show) {
+  const int H = G.n_hands, k = G.hand_size, tid = threadIdx.x;
+  if (!show && std::is_same<P, Single>::value) return;
+  const TermTab tt(H, k, G.deck);
+  const uint16_t* gt = G.term_tab + (size_t)table * tt.len;
+  L.run = TermRun<P>(H, k);
+#pragma unroll
+  for (int e = 0; e < ScanPer<P>::n; ++e) {
+    const int j = L.run.begin + e;
+    const uint32_t h = e >= L.run.cnt ? 0 : tid >= L.run.gp ? __ldg(gt + tt.clh + j) : show ? __ldg(gt + tt.perm + j) : j;
+    L.at[e / 2] = e & 1 ? L.at[e / 2] | h << 16 : h;
+  }
+#pragma unroll
+  for (int s = 0; s < kTermHands; ++s)
+    if (tid + s * kTermThreads < H) L.rec[s] = __ldg(G.term_rec + (size_t)table * H + tid + s * kTermThreads);
+}
+
+// Values at one node: q its reach row, ft the fold part of its board table (card lists, cards, list
+// offsets) and CP [k H + 1], Ps [H + 1] in shared memory; put(h, value) takes the results.
+template <typename P, typename LT, typename F>
+__device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int deck, bool show, uint64_t board, ff u,
+                                              const typename P::V* q, const uint16_t* ft, typename P::V* CP,
+                                              typename P::V* Ps, F put) {
+  using V = typename P::V;
+  using V1 = Vec<P, 1>;
+  constexpr bool single = std::is_same<P, Single>::value;
+  constexpr int gp = TermRun<P>::gp;
+  __shared__ VecAcc<P, 1> red[2][kTermThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint16_t* clh = ft;
+  const uint16_t* cards = ft + k * H;
+  const uint16_t* cloff = cards + H;
+  if constexpr (single) {
+    if (!show) {
+      // T: warp 0 keeps 32 lane-strided partial sums of q and combines them by a fixed xor tree; C[c]:
+      // one thread per card sums card c's list in list order
+      __shared__ float Cs[kMaxDeck], Ts;
+      if (tid < 32) {
+        float t = 0.f;
+#pragma unroll 8
+        for (int h = lane; h < H; h += 32) t = __fadd_rn(t, q[h]);
+        for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+        if (lane == 0) Ts = t;
+      } else if (tid - 32 < deck) {
+        const int c = tid - 32, end = cloff[c + 1];
+        float s = 0.f;
+#pragma unroll 8
+        for (int j = cloff[c]; j < end; ++j) s = __fadd_rn(s, q[clh[j]]);
+        Cs[c] = s;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int s = 0; s < kTermHands; ++s) {
+        const int h = tid + s * kTermThreads;
+        if (h < H) {
+          const unsigned cw = cards[h], c1 = cw & 0xffu, c2 = cw >> 8;
+          float m = __fsub_rn(Ts, Cs[c1]);
+          bool blocked = (board >> c1) & 1ull;
+          if (k == 2) {
+            m = __fadd_rn(__fsub_rn(m, Cs[c2]), q[h]);
+            blocked = blocked || ((board >> c2) & 1ull);
+          }
+          put(h, blocked ? 0.f : __fmul_rn(u.hi, m));
+        }
+      }
+      return;
+    }
+  }
+  {
+    V1 a[ScanPer<P>::n];
+    VecAcc<P, 1> x;
+#pragma unroll
+    for (int e = 0; e < ScanPer<P>::n; ++e) a[e].v[0] = q[L.hand(e)];
+    const int gtid = tid < gp ? tid : tid - gp;
+    scan_runs<P, 1>(a, L.run.cnt, red[tid >= gp], gtid, x);
+    __syncthreads();
+    if (tid < gp)
+      scan_write<P, 1, gp>(a, L.run.begin, L.run.cnt, H, red[0], gtid, x, reinterpret_cast<V1*>(Ps));
+    else
+      scan_write<P, 1, kTermThreads - gp>(a, L.run.begin, L.run.cnt, k * H, red[1], gtid, x, reinterpret_cast<V1*>(CP));
+  }
+  __syncthreads();
+  const V T = Ps[H], us = P::scale(u);
+#pragma unroll
+  for (int s = 0; s < kTermHands; ++s) {
+    const int h = tid + s * kTermThreads;
+    if (h < H) {
+      const uint4 r = L.record(s, h);
+      const unsigned c1 = r.x & 0xffu, c2 = (r.x >> 8) & 0xffu;
+      bool blocked = (board >> c1) & 1ull;
+      const V a0 = CP[cloff[c1]], z0 = CP[cloff[c1 + 1]];
+      V d;
+      if (show) {
+        V Wn = Ps[r.x >> 16], Ln = P::sub(T, Ps[r.y & 0xffffu]);
+        Wn = P::sub(Wn, P::sub(CP[r.y >> 16], a0));
+        Ln = P::sub(Ln, P::sub(z0, CP[r.z & 0xffffu]));
+        if (k == 2) {
+          blocked = blocked || ((board >> c2) & 1ull);
+          Wn = P::sub(Wn, P::sub(CP[r.z >> 16], CP[cloff[c2]]));
+          Ln = P::sub(Ln, P::sub(CP[cloff[c2 + 1]], CP[r.w & 0xffffu]));
+        }
+        d = P::sub(Wn, Ln);
+      } else {
+        d = P::sub(T, P::sub(z0, a0));
+        if (k == 2) {
+          blocked = blocked || ((board >> c2) & 1ull);
+          d = P::add(P::sub(d, P::sub(CP[cloff[c2 + 1]], CP[cloff[c2]])), q[h]);
+        }
+      }
+      put(h, blocked ? P::zero() : P::mul(us, d));
+    }
+  }
+}
+
+// The player of a block of the terminal launch and its item of n (grid: (player, item)).
+__device__ __forceinline__ int terminal_item(int n, int player_mask, int& i) {
+  if (player_mask != 3) {
+    i = player_mask == 1 ? 0 : 1;
+    return blockIdx.x;
+  }
+  i = (int)blockIdx.x >= n;
+  return blockIdx.x - i * n;
+}
+
+// Payoff for player i per unit of (opponent reach) x kappa at node n: the FP64 product as a pair
+// of FP32 rounded once on the host (FP32 values use its high part): no FP64 work per thread.
+__device__ __forceinline__ ff terminal_payoff(const GameDev& G, const NodeDev& nd, int n, int i) {
+  const bool neg = nd.type == kFold && nd.player == i;
+  return {neg ? -G.payoff_ff[2 * n] : G.payoff_ff[2 * n], neg ? -G.payoff_ff[2 * n + 1] : G.payoff_ff[2 * n + 1]};
+}
+
+// Terminal values (Stages 2-4), the one-node form for handles with few terminals.  One block per
+// (player, node): its board table comes in by a bulk (TMA) copy that starts before the launch waits
+// for its predecessor, the opponent's reach row by another after it.  A showdown below an all-in
+// run-out reads the run-out's reach row (src) and zeroes the hands holding a dealt card itself
+// (nobody acts below the run-out, so that is its reach).  The wait is bounded: on a timeout the
+// block sets *err, lets its copies drain and leaves.
+template <typename P>
+__global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __restrict__ games,
+                                                            const Work* __restrict__ work,
+                                                            const TermSrc* __restrict__ src, int n_work,
+                                                            int player_mask, int use_bar, int* err) {
+  using V = typename P::V;
+  int i;
+  const int first = terminal_item(n_work, player_mask, i), tid = threadIdx.x;
+  const GameDev& G = games[work[first].game];
+  const int n = work[first].unit, from = src[first].row[1 - i];
+  const NodeDev nd = G.nodes[n];
+  const int H = G.n_hands, k = G.hand_size;
+  const size_t stride = (size_t)G.hstride;
+  const TermTab tt(H, k, G.deck);
+  const bool show = nd.type == kShowdown;
+  const unsigned tab_bytes = (unsigned)(show ? tt.len : tt.fold_len) * 2u, q_bytes = (unsigned)(stride * sizeof(V));
+  const V* qsrc = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + (size_t)(1 - i) * G.n_nodes * stride;
+  V* dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + ((size_t)i * G.n_nodes + n) * stride;
+
+  extern __shared__ __align__(128) unsigned char smt[];
+  __shared__ __align__(8) uint64_t bar;
+  const uint16_t* tab = reinterpret_cast<const uint16_t*>(smt);  // [tt.len]
+  V* q = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);          // [hstride]
+  V* CP = q + stride;                                            // [k H + 1]
+  V* Ps = CP + (k * H + 1);                                      // [H + 1]
+  if (tid == 0) {
+    mbar_init(&bar, 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    mbar_arrive_expect_tx(&bar, tab_bytes + q_bytes);
+    bulk_copy_g2s(smt, G.term_tab + (size_t)(show ? nd.row : 0) * tt.len, tab_bytes, &bar);
+  }
+  pdl_wait();  // the reach rows come from the launch just before this one
+  pdl_trigger();
+  if (tid == 0) bulk_copy_g2s(q, qsrc + (size_t)term_src_node(from) * stride, q_bytes, &bar);
+  const ff u = terminal_payoff(G, nd, n, i);
+  TermStaged<P> L;
+  L.run = TermRun<P>(H, k);
+  L.list = tid >= L.run.gp ? tab + tt.clh : show ? tab + tt.perm : nullptr;
+  L.cards = tab + tt.cards, L.gs = tab + tt.gs, L.ge = tab + tt.ge, L.lo = tab + tt.lo, L.hi = tab + tt.hi;
+  const bool ok = tid >= 32 || mbar_wait_bounded(&bar, 0, g_first_wait_polls);  // one warp polls
+  if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
+    if (tid == 0) {
+      atomicExch(err, 1);
+      mbar_wait_bounded(&bar, 0);
+    }
+    __syncthreads();
+    return;
+  }
+  if (from < 0) {  // below an all-in run-out: its reach, without the hands holding a card dealt since
+    for (int h = tid; h < H; h += kTermThreads)
+      if (holds_board_card(L.cards, h, k, nd.board)) q[h] = P::zero();
+    __syncthreads();
+  }
+  terminal_node<P>(L, H, k, G.deck, show, nd.board, u, q, tab, CP, Ps, [&](int h, V v) { dst[h] = v; });
+}
+
+// ---- several nodes at once: the throughput form for handles whose terminals fill the GPU
+//
+// A group is up to NV nodes of one game, one kind (folds or showdowns) and one board table.  The
+// scan arrays of terminal_values become arrays of NV values (16 bytes), so each table entry and
+// each address is read and computed once for NV nodes and a gather is one 16-byte shared-memory
+// access.  Component v runs exactly the one-node form's operations in its order (the same runs
+// of entries per thread, the same combination of threads and warps), so the bits are the same.
+//
+// Blocks are persistent: two per SM, each walking its own contiguous stretch of the groups, so
+// that the board table is reloaded only when it changes, descriptors are staged once, and the
+// reach rows of the next group are in flight (bulk copies, two buffers) while the current one
+// is computed.  A showdown group takes three block barriers: rows landed; each thread has
+// gathered its run of entries into registers and summed it; the prefix sums are written.
+// Bound by random shared-memory gathers (5060 wavefronts a group of four, 45 % of the pipe's rate).
+// Measured against blocks that take their nodes one by one: exact turn 119 -> 88 us per player,
+// 256 rivers 132 -> 129, with one block per group and its descriptors read node by node 147.
 
 template <typename P, int NV>
 __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev* __restrict__ games,
@@ -1302,18 +1205,561 @@ __global__ void __launch_bounds__(kHandThreads, 1) k_hand(const GameDev* __restr
 }
 
 
+// ------------------------------------------------------------------ hand tiles
+//
+// The throughput form of the per-hand passes for handles of many subgames whose trees fit a
+// block's shared memory a few times per SM (batches of rivers).  One block owns W hands (32, 16
+// or 8: the most that fit) of one subgame and one player:
+//   A  the values of the tree's end nodes and the stored strategy come in by cp.async; the inner
+//      nodes' values (Stage 6) are computed level by level in shared memory;
+//   B  the regret and average update (Stage 7) of every row of the player: a flat loop over (row,
+//      hand) items with no order between them, four in flight a thread, so that the FP64 pipe
+//      (64 cycles a warp instruction and scheduler) and the R and S streams stay busy; the
+//      positive parts of the new regrets replace the strategy in shared memory;
+//   C  level by level from the root: regret matching of the player's nodes (Eq. rm) and the
+//      reach of their children (Stage 1), in the array of A.
+// R and S are read and written once, straight from registers; L2 is asked for their lines at the
+// start, before the launch waits for its predecessor.  The arithmetic is k_hand's, in its order.
+// Bound: the FP64 pipe (four operations a row and hand: 88 us on the batch below) and issue slots.
+// Measured, one player's update: 256 rivers, FP32 values 267 -> 180 us against the one-warp walk;
+// 64 rivers, pairs, Predictive CFR+ 321 -> 110 us.  Average pass 780 -> 167, best response 943 ->
+// 150 us (256 rivers, both players; k_hand before).
+
+constexpr int kTileThreads = 256;  // at most; 128 where the tiles are small (see create_impl)
+
+__host__ __device__ inline size_t tile_smem_bytes(int tab16, int n_nodes, int rows_max, int W, size_t es) {
+  return (size_t)tab16 * 16 + (size_t)(n_nodes + rows_max) * W * es;
+}
+
+// Copies rows of W values (count of them, row k of the source at row_at(k)) into the tile.
+template <typename V, typename F, typename T>
+__device__ __forceinline__ void tile_copy(V* tile, const V* __restrict__ src, size_t stride, int wlog, int count, F row_at,
+                                          T tile_at) {
+  const int pl = wlog + (sizeof(V) == 8 ? 3 : 2) - 4;  // log2 of a row's 16-byte pieces
+  for (int k = threadIdx.x; k < count << pl; k += blockDim.x) {
+    const int r = k >> pl, part = k & ((1 << pl) - 1);
+    cp_async<16>(reinterpret_cast<unsigned char*>(tile + (tile_at(r) << wlog)) + part * 16,
+                 reinterpret_cast<const unsigned char*>(src + (size_t)row_at(r) * stride) + part * 16);
+  }
+}
+
+// One lane's place in a tile: its column of the tile's arrays (node n or row r at [n << wlog]) and
+// the threads that walk the levels.
+struct TileLane {
+  const TileHead* head;
+  const uint16_t* tab;      // the table the head opens
+  const NodeDev* nodes;     // dealt cards of chance children
+  int p, wlog, slot, h, stride;
+  int group;                // threads taking part in the level walks: fewer wait less at their barriers
+  bool valid;               // a real hand
+  uint64_t hmask;           // its cards
+};
+
+// Barrier of the first `group` threads of the block.
+__device__ __forceinline__ void group_barrier(int group) {
+  if (group == (int)blockDim.x)
+    __syncthreads();
+  else
+    asm volatile("barrier.sync 1, %0;" ::"r"(group) : "memory");
+}
+
+// Phase A: the inner nodes' values from the deepest level up (Stage 6, Eq. backward; kModeBR: the
+// best response's), by the first `group` threads.  gv: the player's value rows; the values are
+// stored there when `store` is set, the root's always.
+template <int MODE, typename P>
+__device__ __forceinline__ void tile_values(const TileLane& T, typename P::V* val, const typename P::V* sg,
+                                            typename P::V* gv, bool store) {
+  using V = typename P::V;
+  const TileNode* inner = reinterpret_cast<const TileNode*>(T.tab + T.head->inner);
+  const uint16_t* level = T.tab + T.head->level;  // inner nodes of level l: [level[l], level[l + 1])
+  const int wlog = T.wlog, nslots = T.group >> wlog;
+  for (int l = T.head->levels - 1; l >= 0; --l) {
+    const int last = level[l + 1];
+    for (int k = level[l] + T.slot; k < last; k += nslots) {
+      const TileNode nd = inner[k];
+      const int A = nd.kids & 63, kind = nd.kids >> 6;
+      const V* c = val + (nd.first_kid << wlog);
+      V x;
+      if (MODE == kModeBR && kind == T.p) {
+        x = c[0];
+        for (int a = 1; a < A; ++a) x = P::vmax(x, c[a << wlog]);
+      } else {
+        typename P::Acc acc = P::acc0();
+        if (kind == 2) {  // children values carry the card probabilities; cards in the hand are out
+          for (int a = 0; a < A; ++a)
+            if (!((T.hmask >> T.nodes[nd.first_kid + a].deal) & 1ull)) P::acc(acc, c[a << wlog]);
+        } else if (kind != T.p) {
+#pragma unroll 4
+          for (int a = 0; a < A; ++a) P::acc(acc, c[a << wlog]);
+        } else {
+          const V* s = sg + (nd.row << wlog);
+#pragma unroll 4
+          for (int a = 0; a < A; ++a) P::acc_mul(acc, s[a << wlog], c[a << wlog]);
+        }
+        x = P::value(acc);
+      }
+      val[nd.id << wlog] = x;
+      if (T.valid && (store || l == 0)) gv[(size_t)nd.id * T.stride + T.h] = x;
+    }
+    group_barrier(T.group);
+  }
+}
+
+// tile_values for tiles of 8 hands in the latency forms, where a level is a few nodes and every
+// instruction of its chain counts: fixed offsets, the first four children loaded together (past a
+// node's last child they are not used; the tile ends with slack for them), and the next level's
+// node read before the barrier.
+constexpr int kTileSlack = 4;  // rows of slack behind a tile's strategy
+template <int MODE, typename P>
+__device__ __forceinline__ void tile_values8(const TileLane& T, typename P::V* val, const typename P::V* sg,
+                                             typename P::V* gv, bool store) {
+  using V = typename P::V;
+  const TileNode* inner = reinterpret_cast<const TileNode*>(T.tab + T.head->inner);
+  const uint16_t* level = T.tab + T.head->level;
+  const int nslots = T.group >> 3;
+  int l = T.head->levels - 1, first = level[l], last = level[l + 1];
+  TileNode nd = inner[min(first + T.slot, last - 1)];
+  for (;; --l) {
+    for (int k = first + T.slot; k < last;) {
+      const int A = nd.kids & 63, kind = nd.kids >> 6;
+      const V* c = val + nd.first_kid * 8;
+      V x;
+      if (kind == 2) {  // children values carry the card probabilities; cards in the hand are out
+        typename P::Acc acc = P::acc0();
+        for (int a = 0; a < A; ++a)
+          if (!((T.hmask >> T.nodes[nd.first_kid + a].deal) & 1ull)) P::acc(acc, c[a * 8]);
+        x = P::value(acc);
+      } else {
+        V cc[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) cc[e] = c[e * 8];
+        typename P::Acc acc = P::acc0();
+        if (kind != T.p) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (e < A) P::acc(acc, cc[e]);
+          for (int a = 4; a < A; ++a) P::acc(acc, c[a * 8]);
+          x = P::value(acc);
+        } else if (MODE == kModeBR) {
+          x = cc[0];
+#pragma unroll
+          for (int e = 1; e < 4; ++e)
+            if (e < A) x = P::vmax(x, cc[e]);
+          for (int a = 4; a < A; ++a) x = P::vmax(x, c[a * 8]);
+        } else {
+          const V* s = sg + nd.row * 8;
+          V ss[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ss[e] = s[e * 8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (e < A) P::acc_mul(acc, ss[e], cc[e]);
+          for (int a = 4; a < A; ++a) P::acc_mul(acc, s[a * 8], c[a * 8]);
+          x = P::value(acc);
+        }
+      }
+      val[nd.id * 8] = x;
+      if (T.valid && (store || l == 0)) gv[(size_t)nd.id * T.stride + T.h] = x;
+      k += nslots;
+      if (k < last) nd = inner[k];
+    }
+    if (l == 0) break;
+    last = first;
+    first = level[l - 1];
+    nd = inner[min(first + T.slot, last - 1)];
+    group_barrier(T.group);
+  }
+  group_barrier(T.group);
+}
+
+// Stage 7 of one row and hand (sign tests of FP64 values read the sign bit on the integer pipe): the
+// new R and S in place, rd the instantaneous regret (the next prediction of Predictive CFR+);
+// returns what regret matching takes.  rr: child value less node value; contrib: pi sigma(a).
+template <typename P, bool DCFR>
+__device__ __forceinline__ double tile_row(double& R, double& S, typename P::V rr, typename P::V contrib, const Discount& d,
+                                           int variant, double& rd) {
+  rd = P::to_double(rr);
+  const double c = P::to_double(contrib);
+  R += rd;
+  if constexpr (DCFR) {
+    R *= __double_as_longlong(R) > 0 ? d.dpos : d.dneg;
+    S = fma(S, d.dS, c);
+  } else {
+    if (variant == 2) R *= __double_as_longlong(R) > 0 ? d.dpos : d.dneg;
+    const bool plus = variant == 1 || variant == 3;  // CFR+, Predictive CFR+
+    if (plus && __double_as_longlong(R) < 0) R = 0.0;
+    S = fma(S, d.dS, plus ? d.wS * c : c);
+  }
+  return !DCFR && variant == 3 ? R + rd : R;  // Predictive CFR+ matches R + M
+}
+
+// Regret matching (Eq. rm) at a decision node of the player with NA actions from the positive parts
+// s, and the reach of its children c from the node's reach x (regret_match_n's operations).
+// put_sigma(row, value) and put_reach(node, value) take the results.
+template <typename P, int NA, typename FS, typename FR>
+__device__ __forceinline__ void tile_match(const TileNode& nd, const typename P::V* s, typename P::V* c, int wlog,
+                                           typename P::V x, FS put_sigma, FR put_reach) {
+  using V = typename P::V;
+  V y[NA], tot = P::zero();
+  int npos = 0;
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    y[a] = s[a << wlog];
+    npos += P::positive(y[a]);
+    tot = P::add(tot, y[a]);
+  }
+  const V inv = P::recip(tot);  // unused (and possibly not finite) unless npos > 1
+  const V uni = P::uniform(NA);
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    const V many = P::mul(y[a], inv);
+    y[a] = npos > 1 ? many : npos == 1 ? (P::positive(y[a]) ? P::one() : P::zero()) : uni;
+    put_sigma(nd.row + a, y[a]);
+    const V r = P::mul(x, y[a]);
+    c[a << wlog] = r;
+    put_reach(nd.first_kid + a, r);
+  }
+}
+
+// Phase C: regret matching and reach from the root down (rch[0] set) by the first `group` threads, over
+// the nodes that make new reach rows: the children of the player's decisions and of chance nodes
+// (every other node shares a row above it).
+template <typename P, typename FS, typename FR>
+__device__ __forceinline__ void tile_reach(const TileLane& T, typename P::V* rch, const typename P::V* sg, FS put_sigma,
+                                           FR put_reach) {
+  using V = typename P::V;
+  const TileNode* fwd = reinterpret_cast<const TileNode*>(T.tab + T.head->fwd[T.p]);
+  const uint16_t* flevel = T.tab + T.head->flevel[T.p];
+  const int wlog = T.wlog, nslots = T.group >> wlog, levels = T.head->flevels[T.p];
+  for (int l = 0; l < levels; ++l) {
+    const int last = flevel[l + 1];
+    for (int k = flevel[l] + T.slot; k < last; k += nslots) {
+      const TileNode nd = fwd[k];
+      const int A = nd.kids & 63;
+      const V x = rch[nd.id << wlog];
+      V* c = rch + (nd.first_kid << wlog);
+      const V* s = sg + (nd.row << wlog);
+      if (nd.kids >> 6 == 2) {
+        for (int a = 0; a < A; ++a) {
+          const V y = ((T.hmask >> T.nodes[nd.first_kid + a].deal) & 1ull) ? P::zero() : x;
+          c[a << wlog] = y;
+          put_reach(nd.first_kid + a, y);
+        }
+        continue;
+      }
+      switch (A) {
+        case 1: tile_match<P, 1>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 2: tile_match<P, 2>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 3: tile_match<P, 3>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 4: tile_match<P, 4>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 5: tile_match<P, 5>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 6: tile_match<P, 6>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 7: tile_match<P, 7>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        case 8: tile_match<P, 8>(nd, s, c, wlog, x, put_sigma, put_reach); break;
+        default: {  // up to kMaxActions
+          V tot = P::zero();
+          int npos = 0;
+          for (int a = 0; a < A; ++a) {
+            const V y = s[a << wlog];
+            npos += P::positive(y);
+            tot = P::add(tot, y);
+          }
+          const V inv = P::recip(tot), uni = P::uniform(A);
+          for (int a = 0; a < A; ++a) {
+            V y = s[a << wlog];
+            y = npos > 1 ? P::mul(y, inv) : npos == 1 ? (P::positive(y) ? P::one() : P::zero()) : uni;
+            put_sigma(nd.row + a, y);
+            const V r = P::mul(x, y);
+            c[a << wlog] = r;
+            put_reach(nd.first_kid + a, r);
+          }
+        }
+      }
+    }
+    group_barrier(T.group);
+  }
+}
+
+// tile_reach for tiles of 8 hands in the latency forms, as tile_values8.
+template <typename P, typename FS, typename FR>
+__device__ __forceinline__ void tile_reach8(const TileLane& T, typename P::V* rch, const typename P::V* sg, FS put_sigma,
+                                            FR put_reach) {
+  using V = typename P::V;
+  const TileNode* fwd = reinterpret_cast<const TileNode*>(T.tab + T.head->fwd[T.p]);
+  const uint16_t* flevel = T.tab + T.head->flevel[T.p];
+  const int nslots = T.group >> 3, levels = T.head->flevels[T.p];
+  if (levels == 0) return;
+  int first = 0, last = flevel[1];
+  TileNode nd = fwd[min(T.slot, last - 1)];
+  for (int l = 0;;) {
+    for (int k = first + T.slot; k < last;) {
+      const int A = nd.kids & 63;
+      const V x = rch[nd.id * 8];
+      V* c = rch + nd.first_kid * 8;
+      if (nd.kids >> 6 == 2) {
+        for (int a = 0; a < A; ++a) {
+          const V y = ((T.hmask >> T.nodes[nd.first_kid + a].deal) & 1ull) ? P::zero() : x;
+          c[a * 8] = y;
+          put_reach(nd.first_kid + a, y);
+        }
+      } else {
+        const V* s = sg + nd.row * 8;
+        V y[4], tot = P::zero();
+        int npos = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[e] = s[e * 8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e < A) npos += P::positive(y[e]), tot = P::add(tot, y[e]);
+        for (int a = 4; a < A; ++a) {
+          const V z = s[a * 8];
+          npos += P::positive(z), tot = P::add(tot, z);
+        }
+        const V inv = P::recip(tot), uni = P::uniform(A);  // inv is unused (and may not be finite) unless npos > 1
+        auto one = [&](int a, V z) {
+          const V many = P::mul(z, inv);
+          z = npos > 1 ? many : npos == 1 ? (P::positive(z) ? P::one() : P::zero()) : uni;
+          put_sigma(nd.row + a, z);
+          const V r = P::mul(x, z);
+          c[a * 8] = r;
+          put_reach(nd.first_kid + a, r);
+        };
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e < A) one(e, y[e]);
+        for (int a = 4; a < A; ++a) one(a, s[a * 8]);
+      }
+      k += nslots;
+      if (k < last) nd = fwd[k];
+    }
+    if (++l == levels) break;
+    first = last;
+    last = flevel[l + 1];
+    nd = fwd[min(first + T.slot, last - 1)];
+    group_barrier(T.group);
+  }
+  group_barrier(T.group);
+}
+
+// LAT: the latency form, for handles of few blocks (one subgame): R and S are staged in shared
+// memory with the strategy, before the launch waits for its predecessor, and every inner node's
+// value is stored (the level and wide schedules keep them readable).  Bound by the instruction latency
+// of a few warps per phase.  Measured, whole solves: Leduc (100 iterations, a launch per tree level
+// before) 14.0 -> 5.4 ms; 8 rivers of 403 hands 1.81 -> 1.50 ms (50 iterations).
+template <int MODE, typename P, bool DCFR, bool LAT>
+__global__ void __launch_bounds__(LAT ? 2 * kTileThreads : kTileThreads, LAT ? 2 : 4) k_tile(const GameDev* __restrict__ games,
+                                                       const Work* __restrict__ work, int n_work, int player_mask,
+                                                       int advance, int* iter, unsigned* done,
+                                                       const Discount* __restrict__ disc_tab, int variant) {
+  using V = typename P::V;
+  constexpr int kTileRows = LAT ? 1 : 4;  // (row, hand) items of phase B in flight per thread
+  extern __shared__ __align__(16) unsigned char smx[];
+  __shared__ Discount disc;
+  int p;
+  const Work wk = work[terminal_item(n_work, player_mask, p)];
+  const GameDev& G = games[wk.game];
+  const int wlog = G.tile_wlog, W = 1 << wlog, tid = threadIdx.x, w = tid & (W - 1), slot = tid >> wlog,
+            nslots = blockDim.x >> wlog;
+  const int h0 = wk.unit << wlog, h = h0 + w;  // < hstride: hstride is a multiple of 32 and W divides 32
+  const bool valid = h < G.n_hands;
+  const int N = G.n_nodes, stride = G.hstride, rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
+  const int tab16 = G.tile_tab16;
+  const TileHead* head = reinterpret_cast<const TileHead*>(smx);
+  const uint16_t* tab = reinterpret_cast<const uint16_t*>(smx);
+  const TileLane T{head, tab, G.nodes, p, wlog, slot, h, stride, LAT ? G.tile_group : (int)blockDim.x, valid,
+                   valid ? G.hand_mask[h] : 0ull};
+
+  // shared: the tile table, values / reach [N][W], strategy [rows][W], LAT: R and S [rows][W]
+  V* tval = reinterpret_cast<V*>(smx + (size_t)tab16 * 16);
+  V* tsg = tval + ((size_t)N << wlog);
+  double* tR = reinterpret_cast<double*>(tsg + ((size_t)nrows << wlog));
+  double* tS = tR + ((size_t)nrows << wlog);
+  V* val = tval + w;  // this lane's column: node n at val[n << wlog]
+  V* sg = tsg + w;    // row r at sg[r << wlog]
+  const size_t plane = (size_t)p * N * stride;
+  V* gv = static_cast<V*>(MODE == kModeBR ? G.cfv_br : G.cfv) + plane;
+  V* grch = static_cast<V*>(MODE == kModeAvg ? G.reach_bar : G.reach) + plane;
+  V* gsg = static_cast<V*>(MODE == kModeAvg ? G.sigbar : G.sigma) + (size_t)rb * stride;
+  double* gR = G.R + (size_t)rb * stride;
+  double* gS = G.S + (size_t)rb * stride;
+
+  // ---- what older launches wrote: the table, the strategy, and R and S (or their L2 lines)
+  for (int k = tid; k < tab16; k += blockDim.x)
+    reinterpret_cast<uint4*>(smx)[k] = __ldg(reinterpret_cast<const uint4*>(G.tile_tab) + k);
+  auto same = [](int r) { return r; };
+  if (MODE == kModeUpdate) {
+    if (tid == 0) disc = disc_tab[*iter];
+    tile_copy(tsg, static_cast<const V*>(gsg) + h0, (size_t)stride, wlog, nrows, same, same);
+  }
+  if (LAT) {
+    if (MODE == kModeUpdate || MODE == kModeInit) tile_copy(tR, static_cast<const double*>(gR) + h0, (size_t)stride, wlog, nrows, same, same);
+    if (MODE == kModeUpdate || MODE == kModeAvg) tile_copy(tS, static_cast<const double*>(gS) + h0, (size_t)stride, wlog, nrows, same, same);
+  } else if (MODE != kModeBR) {
+    const int ll = wlog == 5;  // lines of 16 doubles per row: 2, or 1
+    for (int k = tid; k < nrows << ll; k += blockDim.x) {
+      const size_t at = (size_t)(k >> ll) * stride + h0 + (k & ll) * 16;
+      if (MODE != kModeAvg) asm volatile("prefetch.global.L2 [%0];" ::"l"(gR + at));
+      if (MODE != kModeInit) asm volatile("prefetch.global.L2 [%0];" ::"l"(gS + at));
+    }
+  }
+  pdl_wait();  // terminal values come from the launch just before this one
+  pdl_trigger();
+  __syncthreads();
+
+  if (MODE == kModeUpdate || MODE == kModeBR) {
+    // ---- A: end values in, then inner values
+    const uint16_t* ends = tab + head->ends;
+    auto end = [&](int e) { return (int)ends[e]; };
+    tile_copy(tval, static_cast<const V*>(gv) + h0, (size_t)stride, wlog, head->n_ends, end, end);
+    cp_async_wait_all();
+    __syncthreads();
+    if (!LAT) {
+      tile_values<MODE, P>(T, val, sg, gv, MODE == kModeBR);
+    } else {
+      if (tid < T.group) {
+        if (wlog == 3) tile_values8<MODE, P>(T, val, sg, gv, true);
+        else tile_values<MODE, P>(T, val, sg, gv, true);
+      }
+      __syncthreads();
+    }
+  } else if (LAT) {
+    cp_async_wait_all();
+    __syncthreads();
+  }
+  if constexpr (MODE == kModeBR) {
+    // FP64 root sums of the tile's chunks, reduced by the game's last block as in k_hand
+    __shared__ int s_last;
+    __shared__ double red64[kHandThreads];
+    const int C = G.chunk;  // <= W
+    if (tid < W) {
+      double x = valid ? G.range64[(size_t)p * stride + h] * P::to_double(val[0]) : 0.0;
+      const unsigned mask = W == 32 ? 0xffffffffu : (1u << W) - 1u;
+      for (int o = C / 2; o > 0; o >>= 1) x += __shfl_down_sync(mask, x, o, C);
+      if (w % C == 0 && valid) G.br_partial[(size_t)p * G.n_chunks + h / C] = x;
+      __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+      const unsigned chunks = (unsigned)((min(h0 + W, G.n_hands) - h0 + C - 1) / C);
+      s_last = atomicAdd(G.br_done, chunks) + chunks == (unsigned)(2 * G.n_chunks);
+    }
+    __syncthreads();
+    if (s_last) {  // the sums of kHandThreads threads, as k_hand's last block forms them
+      __threadfence();
+      for (int q = 0; q < 2; ++q) {
+        for (int t = tid; t < kHandThreads; t += blockDim.x) {
+          double x = 0.0;
+          for (int c = t; c < G.n_chunks; c += kHandThreads) x += __ldcg(&G.br_partial[(size_t)q * G.n_chunks + c]);
+          red64[t] = x;
+        }
+        __syncthreads();
+        for (int o = kHandThreads / 2; o > 0; o >>= 1) {
+          for (int t = tid; t < o; t += blockDim.x) red64[t] += red64[t + o];
+          __syncthreads();
+        }
+        if (tid == 0) G.br_out[q] = red64[0];
+        __syncthreads();
+      }
+      if (tid == 0) *G.br_done = 0u;
+    }
+    return;
+  }
+
+  // ---- B: every row of the player
+  {
+    const TileRow* rowmap = reinterpret_cast<const TileRow*>(tab + head->rows[p]);
+    double* gM = G.M ? G.M + (size_t)rb * stride + h : nullptr;
+    const double* src = LAT ? (MODE == kModeAvg ? tS : tR) + w : (MODE == kModeAvg ? gS : gR) + h;
+    const double* srcS = LAT ? tS + w : gS + h;
+    const size_t rs = LAT ? (size_t)W : (size_t)stride;
+    for (int r0 = slot; r0 < nrows; r0 += kTileRows * nslots) {
+      double R[kTileRows], S[kTileRows];
+      V pi[kTileRows];
+      TileRow m[kTileRows];
+#pragma unroll
+      for (int e = 0; e < kTileRows; ++e) {
+        const int r = r0 + e * nslots;
+        if (r < nrows) {
+          R[e] = src[r * rs];
+          if (MODE == kModeUpdate) {
+            m[e] = rowmap[r];
+            S[e] = srcS[r * rs];
+            pi[e] = grch[(size_t)m[e].src * stride + h];
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < kTileRows; ++e) {
+        const int r = r0 + e * nslots;
+        if (r < nrows) {
+          double x = R[e];
+          if (MODE == kModeUpdate) {
+            double rd;
+            x = tile_row<P, DCFR>(R[e], S[e], P::sub(val[m[e].kid << wlog], val[m[e].node << wlog]),
+                                  P::mul(pi[e], sg[r << wlog]), disc, variant, rd);
+            if (valid) {
+              gR[(size_t)r * stride + h] = R[e];
+              gS[(size_t)r * stride + h] = S[e];
+              if (!DCFR && variant == 3) gM[(size_t)r * stride] = rd;
+            }
+          } else if (MODE == kModeInit && gM) {
+            x += gM[(size_t)r * stride];
+          }
+          sg[r << wlog] = __double_as_longlong(x) > 0 ? P::of_double(x) : P::zero();
+        }
+      }
+    }
+  }
+  __syncthreads();  // the positive parts are there, and the values have been read: their array takes the reach
+
+  // ---- C.  An update stores the reach rows it makes; the other passes every node's
+  if (tid < W) val[0] = valid ? static_cast<const V*>(G.range_v)[(size_t)p * stride + h] : P::zero();
+  __syncthreads();
+  auto put_sigma = [&](int r, V y) {
+    if (valid) gsg[(size_t)r * stride + h] = y;
+  };
+  auto put_reach = [&](int n, V y) {
+    if (MODE == kModeUpdate && valid) grch[(size_t)n * stride + h] = y;
+  };
+  if (!LAT) {
+    tile_reach<P>(T, val, sg, put_sigma, put_reach);
+  } else if (tid < T.group) {
+    if (wlog == 3) tile_reach8<P>(T, val, sg, put_sigma, put_reach);
+    else tile_reach<P>(T, val, sg, put_sigma, put_reach);
+  }
+  if (MODE != kModeUpdate) {
+    if (LAT) __syncthreads();
+    const uint16_t* all = tab + head->all[p];
+    for (int n = slot; valid && n < N; n += nslots) grch[(size_t)n * stride + h] = val[all[n] << wlog];
+  }
+
+  if (MODE == kModeUpdate && advance) {
+    if (LAT) __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      const unsigned prev = atomicAdd(done, 1u);
+      if (prev == gridDim.x - 1) {  // last block of the launch: every block has read *iter
+        *done = 0u;
+        *iter += 1;
+        __threadfence();
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ resident schedule
 //
 // The latency form of whole iterations, for handles whose hand chunks all fit the GPU at
 // once (a single subgame): one cooperative launch runs n iterations.  Block b owns hand chunk
 // b of both players and keeps its R, S, strategy and reach rows in shared memory for the whole
-// launch, beside the board table of the terminal nodes it evaluates.  An iteration's phases --
-// the terminal values of player i (Stages 2-4), then i's update (Stages 6, 7 and 1) -- each
-// read what the whole grid wrote in the phase before, so a grid barrier separates them.  What
-// crosses blocks (terminal values, reach rows) goes through global memory and is read past L1
-// (ld.global.cg), since another block of the same launch wrote it.  The arithmetic is that of
-// k_terminal and k_hand, and the global state left at the end is theirs: the level and
-// resident schedules give the same bits.
+// launch, beside what it needs of the board table of the terminal nodes it evaluates.  An
+// iteration's phases -- the terminal values of player i (Stages 2-4), then i's update (Stages 6, 7
+// and 1, as hand tiles) -- each read what the whole grid wrote in the phase before: values carrying
+// their iteration's stamp when updates alternate (below), the global rows with a grid barrier
+// between phases when both players update at once.  The arithmetic is that of k_terminal and
+// k_tile, and the global state left at the end is theirs: the level and resident schedules give
+// the same bits.  Bound by the latency of the chain of phases.  Measured on the 1081-hand river, FP32
+// values: 21.9 us an iteration with grid barriers and the per-hand kernel's passes, 16.4 now.
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
@@ -1361,128 +1807,207 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, i
 }
 
 __host__ __device__ inline size_t resident_term_bytes(int H, int k, int deck, int hstride, size_t es) {
-  return (size_t)TermTab(H, k, deck).len * 2 + (size_t)hstride * es + (size_t)(k * H + 1 + H + 1) * 8;
+  return (size_t)TermTab(H, k, deck).fold_len * 2 + ((size_t)hstride + (size_t)(k * H + 1 + H + 1)) * es;
 }
 
-// Shared memory of the resident kernel's hand region for one game (must match k_resident):
-// nodes, level offsets, per player the row -> node map and decision-node list, R, S, then the
-// values (one player at a time), and per player the reach and strategy.
-__host__ __device__ inline size_t resident_hand_bytes(int n_nodes, int n_levels, int rows_max, int W, size_t es) {
-  return round16((size_t)n_nodes * sizeof(NodeDev)) + round16((size_t)(n_levels + 1) * 4) +
-         4 * round16((size_t)rows_max * 4) + 4 * round16((size_t)rows_max * W * 8) +
-         round16((size_t)n_nodes * W * es) + 2 * round16((size_t)n_nodes * W * es) +
-         2 * round16((size_t)rows_max * W * es);
+// Shared memory of the resident kernel's hand region for one game (must match k_resident): the tile
+// table, per player R and S, the values (one player at a time), and per player reach and strategy.
+__host__ __device__ inline size_t resident_hand_bytes(int tab16, int n_nodes, int rows_max, int W, size_t es) {
+  return (size_t)tab16 * 16 + 4 * round16((size_t)rows_max * W * 8) + 3 * round16((size_t)n_nodes * W * es) +
+         2 * round16((size_t)rows_max * W * es) + (size_t)4 * W * es;  // slack for tile_values8's loads
 }
 
-// One terminal node of player i (Stages 2-4) in the resident kernel: the board table stays in
-// shared memory while the nodes the block evaluates read the same one (tab_game / tab_b name
-// it); the opponent's reach row is read past L1.  Ends with a block barrier.
+// What crosses blocks inside a launch of alternating updates goes as stamped words: a value and the
+// iteration's stamp in one 64-bit store (two for a pair), which a reader polls until the stamp is
+// there.  A value is then one store-to-load trip (770 cycles) away from its reader, where a grid
+// barrier takes about 2,900 (its release, 152 arrivals at one counter, the poll) and a load after it
+// another 400.  No word is overwritten before its readers are done: a terminal's values of player
+// i are rewritten once its block has read a whole reach row of the next update of the opponent, to
+// which every chunk contributes after having read those values; a reach row is rewritten once the
+// chunk has read the next values of every terminal of its subgame, whose blocks evaluate their
+// items in order, the opponent's of the iteration before among them.
+__device__ __forceinline__ void stamp_put(uint64_t* w, float v, uint32_t stamp) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"((uint64_t)stamp << 32 | __float_as_uint(v)) : "memory");
+}
+__device__ __forceinline__ void stamp_put(uint64_t* w, ff v, uint32_t stamp) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(w), "l"((uint64_t)stamp << 32 | __float_as_uint(v.hi)),
+               "l"((uint64_t)stamp << 32 | __float_as_uint(v.lo))
+               : "memory");
+}
+__device__ __forceinline__ bool stamp_get(const uint64_t* w, uint32_t stamp, float& v) {
+  uint64_t x;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w) : "memory");
+  v = __uint_as_float((uint32_t)x);
+  return (uint32_t)(x >> 32) == stamp;
+}
+__device__ __forceinline__ bool stamp_get(const uint64_t* w, uint32_t stamp, ff& v) {
+  uint64_t x, y;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(w) : "memory");
+  v = {__uint_as_float((uint32_t)x), __uint_as_float((uint32_t)y)};
+  return (uint32_t)(x >> 32) == stamp && (uint32_t)(y >> 32) == stamp;
+}
+// Bounded poll: false (and the error flag set) after `limit` polls, or once another block gave up.
+template <typename V>
+__device__ __forceinline__ bool stamp_wait(const uint64_t* w, uint32_t stamp, V& v, long limit, int* err) {
+  for (long k = 0; k < limit; ++k) {
+    if (stamp_get(w, stamp, v)) return true;
+    if ((k & 63) == 63 && ld_relaxed_s32(err) != 0) return false;
+  }
+  atomicExch(err, 1);
+  return false;
+}
+
+// A terminal node in the resident kernel: what does not change from iteration to iteration, kept
+// while the block's next item is the same node.
 template <typename P>
-__device__ __forceinline__ void resident_terminal(const GameDev* __restrict__ games, Work e, TermSrc ts, int i,
-                                                  unsigned char* smr, int& tab_game, int& tab_b) {
+struct ResidentTerm {
+  int item;  // its term_work entry, or -1
+  const GameDev* G;
+  int H, k, deck, N, stride, node, table;
+  bool show;
+  uint64_t board;
+  TermSrc src;
+  ff u[2];
+  int tab_game, tab_table, tab_show;  // what ft and lane hold
+  TermLane<P> lane;
+};
+
+// Values of player i at terminal item e (Stages 2-4).  The opponent's reach row comes from the global
+// rows (stamp 0: written by an earlier launch, or before a grid barrier) or, stamped, from xreach; the
+// values go to the global rows when `plain` is set, and stamped to xval when `put` is.  False when a
+// wait gave up.  Ends with a block barrier.
+template <typename P>
+__device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ games, const Work* __restrict__ term_work,
+                                                  const TermSrc* __restrict__ term_src, int e, int i, unsigned char* smr,
+                                                  ResidentTerm<P>& R, uint32_t stamp, uint32_t put, bool plain, long limit,
+                                                  int* err) {
   using V = typename P::V;
-  const GameDev& G = games[e.game];
-  const int n = e.unit, src = ts.row[1 - i];
-  const NodeDev nd = G.nodes[n];
-  const TermTab tt(G.n_hands, G.hand_size, G.deck);
-  const size_t stride = (size_t)G.hstride;
-  uint16_t* tab = reinterpret_cast<uint16_t*>(smr);
-  V* qs = reinterpret_cast<V*>(smr + (size_t)tt.len * 2);
-  ff* CP = reinterpret_cast<ff*>(smr + (size_t)tt.len * 2 + stride * sizeof(V));
-  ff* Psc = CP + (G.hand_size * G.n_hands + 1);
-  // a fold reads table 0, as in k_terminal (each table orders its per-card hand lists by its
-  // own board's ranks, so another table's lists would sum the same reach in another order)
-  const int b = nd.type == kShowdown ? nd.row : 0;
-  if (tab_game != e.game || tab_b != b) {  // len is a multiple of 8 entries: 16-byte pieces
-    const uint4* src4 = reinterpret_cast<const uint4*>(G.term_tab + (size_t)b * tt.len);
-    for (int k = threadIdx.x; k < tt.len / 8; k += blockDim.x) reinterpret_cast<uint4*>(tab)[k] = __ldg(src4 + k);
-    tab_game = e.game;
-    tab_b = b;
+  constexpr int words = (int)sizeof(V) / 4;  // stamped words per value
+  const int tid = threadIdx.x;
+  uint16_t* ft = reinterpret_cast<uint16_t*>(smr);
+  if (R.item != e) {
+    R.item = e;
+    const Work wk = term_work[e];
+    R.G = games + wk.game;
+    const NodeDev nd = R.G->nodes[wk.unit];
+    R.H = R.G->n_hands, R.k = R.G->hand_size, R.deck = R.G->deck, R.N = R.G->n_nodes, R.stride = R.G->hstride;
+    R.node = wk.unit;
+    R.src = term_src[e];
+    R.show = nd.type == kShowdown;
+    // a fold reads table 0, as in k_terminal (each table orders its per-card hand lists by its
+    // own board's ranks, so another table's lists would sum the same reach in another order)
+    R.table = R.show ? nd.row : 0;
+    R.board = nd.board;
+    for (int p = 0; p < 2; ++p) R.u[p] = terminal_payoff(*R.G, nd, wk.unit, p);
+    if (R.tab_game != wk.game || R.tab_table != R.table || R.tab_show != R.show) {
+      const TermTab tt(R.H, R.k, R.deck);
+      const uint4* gt = reinterpret_cast<const uint4*>(R.G->term_tab + (size_t)R.table * tt.len);
+      for (int x = tid; x < tt.fold_len / 8; x += kTermThreads) reinterpret_cast<uint4*>(ft)[x] = __ldg(gt + x);
+      term_lane_load(R.lane, *R.G, R.table, R.show);
+      R.tab_game = wk.game, R.tab_table = R.table, R.tab_show = R.show;
+    }
   }
-  {  // the row is a multiple of 128 bytes (hstride is a multiple of 32)
-    const uint4* q4 = reinterpret_cast<const uint4*>(static_cast<const V*>(G.reach) +
-                                                     ((size_t)(1 - i) * G.n_nodes + term_src_node(src)) * stride);
-    for (int k = threadIdx.x; k < (int)(stride * sizeof(V) / 16); k += blockDim.x)
-      reinterpret_cast<uint4*>(qs)[k] = __ldcg(q4 + k);
+  const int H = R.H, k = R.k, stride = R.stride, from = R.src.row[1 - i];
+  const TermTab tt(H, k, R.deck);
+  V* q = reinterpret_cast<V*>(smr + (size_t)tt.fold_len * 2);
+  V* CP = q + stride;
+  V* Ps = CP + (k * H + 1);
+  const size_t row = ((size_t)(1 - i) * R.N + term_src_node(from)) * stride;
+  bool ok = true;
+  if (stamp == 0) {
+    const V* src = static_cast<const V*>(R.G->reach) + row;
+    for (int h = tid; h < H; h += kTermThreads) q[h] = ld_cg(src + h);
+  } else {
+    const uint64_t* src = R.G->xreach + row * words;
+    V v[kTermHands];
+    bool got[kTermHands];
+#pragma unroll
+    for (int s = 0; s < kTermHands; ++s) {  // the first polls go out together
+      const int h = tid + s * kTermThreads;
+      got[s] = h >= H || (limit > 0 && stamp_get(src + (size_t)h * words, stamp, v[s]));
+    }
+#pragma unroll
+    for (int s = 0; s < kTermHands; ++s) {
+      const int h = tid + s * kTermThreads;
+      if (!got[s]) ok = stamp_wait(src + (size_t)h * words, stamp, v[s], limit, err) && ok;
+      if (h < H) q[h] = v[s];
+    }
   }
-  __syncthreads();
-  if (src < 0) {  // below an all-in run-out: zero the hands holding a card dealt on the way
-    for (int h = threadIdx.x; h < G.n_hands; h += blockDim.x)
-      if (holds_board_card(tab + tt.cards, h, G.hand_size, nd.board)) qs[h] = P::zero();
+  if (!__syncthreads_and(ok)) return false;
+  if (from < 0) {  // below an all-in run-out: zero the hands holding a card dealt on the way
+    for (int h = tid; h < H; h += kTermThreads)
+      if (holds_board_card(ft + tt.cards, h, k, R.board)) q[h] = P::zero();
     __syncthreads();
   }
-  const bool neg = nd.type == kFold && nd.player == i;
-  const ff u = {neg ? -G.payoff_ff[2 * n] : G.payoff_ff[2 * n], neg ? -G.payoff_ff[2 * n + 1] : G.payoff_ff[2 * n + 1]};
-  terminal_values<P>(G, nd, i, u, tt, tab, qs, CP, Psc,
-                     static_cast<V*>(G.cfv) + ((size_t)i * G.n_nodes + n) * stride);
+  const size_t out = ((size_t)i * R.N + R.node) * stride;
+  V* dst = static_cast<V*>(R.G->cfv) + out;
+  uint64_t* xdst = R.G->xval + out * words;
+  terminal_node<P>(R.lane, H, k, R.deck, R.show, R.board, R.u[i], q, ft, CP, Ps, [&](int h, V v) {
+    if (put) stamp_put(xdst + (size_t)h * words, v, put);
+    if (plain) dst[h] = v;
+  });
   __syncthreads();  // the row buffer and the scan arrays are free again
+  return true;
 }
 
 // n_iters iterations (alternating: terminal and update of player 0, then of player 1;
 // otherwise both players' terminals, then both updates).  Launched cooperatively, every block
-// resident: grid >= n_chunk_work.  sync[0] counts barrier arrivals, sync[1] blocks that have
+// resident: grid >= n_chunk_work.  Alternating updates pass values and reach as stamped words (the
+// stamps of iteration it of this launch are stamp0 + it + 1); simultaneous ones through the global
+// rows, a grid barrier between phases.  sync[0] counts barrier arrivals, sync[1] blocks that have
 // finished; the last block to finish resets both and advances *iter by n_iters.
 template <typename P>
 __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
     const GameDev* __restrict__ games, const Work* __restrict__ chunk_work, int n_chunk_work,
     const Work* __restrict__ term_work, const TermSrc* __restrict__ term_src, int n_term_work, int alternating,
     int n_iters, int* iter, const Discount* __restrict__ disc_tab, int variant, unsigned* sync, int* err,
-    unsigned term_bytes) {
+    unsigned term_bytes, uint32_t stamp0) {
   using V = typename P::V;
   constexpr size_t es = sizeof(V);
+  constexpr int words = (int)sizeof(V) / 4;
   extern __shared__ __align__(16) unsigned char smr[];
   const int tid = threadIdx.x;
   const bool owner = (int)blockIdx.x < n_chunk_work;
   const Work wk = owner ? chunk_work[blockIdx.x] : Work{0, 0};
   const GameDev& G = games[wk.game];
-  const int W = G.chunk, w = tid % W, slot = tid / W, nslots = kTermThreads / W;
+  const int wlog = G.tile_wlog, W = 1 << wlog, w = tid & (W - 1), slot = tid >> wlog, nslots = kTermThreads >> wlog;
   const int h = wk.unit * W + w;  // < hstride
   const bool valid = owner && h < G.n_hands;
-  const int N = G.n_nodes, L = G.n_levels;
-  const size_t stride = (size_t)G.hstride;
+  const int N = G.n_nodes, stride = G.hstride, tab16 = G.tile_tab16;
   const int rows_max = max(G.row_begin[1] - G.row_begin[0], G.row_begin[2] - G.row_begin[1]);
-  const uint64_t hmask = valid ? G.hand_mask[h] : 0ull;
 
-  // hand region (see resident_hand_bytes), after the terminal region
+  // hand region (see resident_hand_bytes), after the terminal region; columns of this lane
   unsigned char* cur = smr + term_bytes;
-  NodeDev* snodes = reinterpret_cast<NodeDev*>(cur);
-  cur += round16((size_t)N * sizeof(NodeDev));
-  int* sls = reinterpret_cast<int*>(cur);
-  cur += round16((size_t)(L + 1) * 4);
-  const size_t ri = round16((size_t)rows_max * 4), rd8 = round16((size_t)rows_max * W * 8);
-  int* srow[2] = {reinterpret_cast<int*>(cur), reinterpret_cast<int*>(cur + ri)};
-  cur += 2 * ri;
-  int* sdec[2] = {reinterpret_cast<int*>(cur), reinterpret_cast<int*>(cur + ri)};
-  cur += 2 * ri;
-  double* sR[2] = {reinterpret_cast<double*>(cur), reinterpret_cast<double*>(cur + rd8)};
+  unsigned char* stab = cur;
+  cur += (size_t)tab16 * 16;
+  const size_t rd8 = round16((size_t)rows_max * W * 8);
+  double* sR[2] = {reinterpret_cast<double*>(cur) + w, reinterpret_cast<double*>(cur + rd8) + w};
   cur += 2 * rd8;
-  double* sS[2] = {reinterpret_cast<double*>(cur), reinterpret_cast<double*>(cur + rd8)};
+  double* sS[2] = {reinterpret_cast<double*>(cur) + w, reinterpret_cast<double*>(cur + rd8) + w};
   cur += 2 * rd8;
   const size_t nv = round16((size_t)N * W * es), rv = round16((size_t)rows_max * W * es);
-  V* sv = reinterpret_cast<V*>(cur);
+  V* val = reinterpret_cast<V*>(cur) + w;
   cur += nv;
-  V* srch[2] = {reinterpret_cast<V*>(cur), reinterpret_cast<V*>(cur + nv)};
+  V* srch[2] = {reinterpret_cast<V*>(cur) + w, reinterpret_cast<V*>(cur + nv) + w};
   cur += 2 * nv;
-  V* ssg[2] = {reinterpret_cast<V*>(cur), reinterpret_cast<V*>(cur + rv)};
+  V* ssg[2] = {reinterpret_cast<V*>(cur) + w, reinterpret_cast<V*>(cur + rv) + w};
+  const TileHead* head = reinterpret_cast<const TileHead*>(stab);
+  const uint16_t* tab = reinterpret_cast<const uint16_t*>(stab);
 
   // ---- stage the tree and the chunk's state of both players (written by earlier launches)
   if (owner) {
-    const int4* gn = reinterpret_cast<const int4*>(G.nodes);
-    for (int k = tid; k < 2 * N; k += kTermThreads) reinterpret_cast<int4*>(snodes)[k] = __ldg(gn + k);
-    for (int k = tid; k <= L; k += kTermThreads) sls[k] = G.level_start[k];
+    for (int k = tid; k < tab16; k += kTermThreads)
+      reinterpret_cast<uint4*>(stab)[k] = __ldg(reinterpret_cast<const uint4*>(G.tile_tab) + k);
     for (int p = 0; p < 2; ++p) {
       const int rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
-      const int db = G.dec_begin[p], ndec = G.dec_begin[p + 1] - db;
-      for (int k = tid; k < nrows; k += kTermThreads) srow[p][k] = G.row_node[rb + k];
-      for (int k = tid; k < ndec; k += kTermThreads) sdec[p][k] = G.dec_nodes[db + k];
       for (int r = slot; r < nrows; r += nslots) {
         const size_t g = (size_t)(rb + r) * stride + h;
-        sR[p][r * W + w] = G.R[g];
-        sS[p][r * W + w] = G.S[g];
-        ssg[p][r * W + w] = static_cast<const V*>(G.sigma)[g];
+        sR[p][r << wlog] = G.R[g];
+        sS[p][r << wlog] = G.S[g];
+        ssg[p][r << wlog] = static_cast<const V*>(G.sigma)[g];
       }
       const V* grch = static_cast<const V*>(G.reach) + (size_t)p * N * stride + h;
-      for (int n = slot; n < N; n += nslots) srch[p][n * W + w] = grch[(size_t)n * stride];
+      for (int n = slot; n < N; n += nslots) srch[p][n << wlog] = grch[(size_t)n * stride];
     }
   }
   __syncthreads();
@@ -1491,46 +2016,95 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
   const int steps = alternating ? 2 : 1;
   unsigned nbar = 0;
   bool ok = true;
-  int tab_game = -1, tab_b = -1;
+  ResidentTerm<P> term;
+  term.item = term.tab_game = term.tab_table = term.tab_show = -1;
   for (int it = 0; it < n_iters && ok; ++it) {
     const Discount d = disc_tab[it0 + it];
+    const bool last = it == n_iters - 1;
+    const uint32_t stamp = stamp0 + (uint32_t)it + 1u;
     for (int step = 0; step < steps && ok; ++step) {
       const int pm = alternating ? 1 << step : 3;
       const int p0 = pm == 2 ? 1 : 0, np = pm == 3 ? 2 : 1;
+      const long limit = it == 0 ? g_first_wait_polls : kWaitLimit;
       // ---- terminal values of the player(s) of this step (Stages 2-4)
-      for (int item = blockIdx.x; item < np * n_term_work; item += gridDim.x) {
-        const int e = item % n_term_work;
-        resident_terminal<P>(games, term_work[e], term_src[e], p0 + item / n_term_work, smr, tab_game, tab_b);
+      for (int item = blockIdx.x; item < np * n_term_work && ok; item += gridDim.x) {
+        const int e = item % n_term_work, i = p0 + item / n_term_work;
+        // player 0's first terminals read what the launch before left
+        const uint32_t from = !alternating || (it == 0 && step == 0) ? 0u : step == 0 ? stamp - 1u : stamp;
+        ok = resident_terminal<P>(games, term_work, term_src, e, i, smr, term, from, alternating ? stamp : 0u,
+                                  !alternating || last, limit, err);
       }
-      ++nbar;
-      ok = grid_barrier(&sync[0], nbar * gridDim.x, err, nbar == 1 ? g_first_wait_polls : kWaitLimit);
       if (!ok) break;
+      if (!alternating) {
+        ++nbar;
+        ok = grid_barrier(&sync[0], nbar * gridDim.x, err, nbar == 1 ? g_first_wait_polls : kWaitLimit);
+        if (!ok) break;
+      }
       // ---- the update of the chunk's hands (Stages 6, 7, then 1 with the new strategy)
       if (owner) {
-        for (int p = p0; p < p0 + np; ++p) {
+        for (int p = p0; p < p0 + np && ok; ++p) {
           const int rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
-          const int ndec = G.dec_begin[p + 1] - G.dec_begin[p];
-          V* gv = static_cast<V*>(G.cfv) + (size_t)p * N * stride + h;
-          V* grch = static_cast<V*>(G.reach) + (size_t)p * N * stride + h;
-          const Col<V> v{sv + w, (size_t)W};
-          for (int n = slot; n < N; n += nslots) v[n] = ld_cg(gv + (size_t)n * stride);
+          const TileLane T{head, tab, G.nodes, p, wlog, slot, h, stride, G.tile_group, valid,
+                           valid ? G.hand_mask[h] : 0ull};
+          const size_t plane = (size_t)p * N * stride;
+          V* gv = static_cast<V*>(G.cfv) + plane;
+          V* grch = static_cast<V*>(G.reach) + plane;
+          const uint64_t* xv = G.xval + plane * words;
+          uint64_t* xr = G.xreach + plane * words;
+          const uint16_t* ends = tab + head->ends;
+          bool got = true;
+          for (int e = slot; e < head->n_ends; e += nslots) {
+            const int n = ends[e];
+            const size_t at = (size_t)n * stride + h;
+            V x = P::zero();
+            if (!alternating) x = ld_cg(gv + at);
+            else if (valid) got = stamp_wait(xv + at * words, stamp, x, limit, err) && got;
+            val[n << wlog] = x;
+          }
+          ok = __syncthreads_and(got);
+          if (!ok) break;
+          // A: later iterations of the launch overwrite the inner values, so only the last stores them
+          if (tid < T.group) {
+            if (wlog == 3) tile_values8<kModeUpdate, P>(T, val, ssg[p], gv, last);
+            else tile_values<kModeUpdate, P>(T, val, ssg[p], gv, last);
+          }
           __syncthreads();
-          const HandView<P> hv{snodes, sls, srow[p], sdec[p], L, ndec, nrows, rb, p, slot, nslots, valid, true, hmask,
-                               v, Col<V>{srch[p] + w, (size_t)W}, Col<V>{ssg[p] + w, (size_t)W},
-                               Col<double>{sR[p] + w, (size_t)W}, Col<double>{sS[p] + w, (size_t)W}};
-          hand_backward<kModeUpdate, P>(hv);
-          if (valid)
-            for (int n = slot; n < N; n += nslots) gv[(size_t)n * stride] = v[n];
-          hand_rows<kModeUpdate, P>(hv, d, variant, hv.Rc, hv.Sc, true,
-                                    Col<double>{G.M ? G.M + (size_t)rb * stride + h : nullptr, stride});
-          hand_rm<P>(hv);
-          hand_forward<P>(hv, valid ? static_cast<const V*>(G.range_v)[(size_t)p * stride + h] : P::zero());
-          if (valid)  // the opponent's terminal values read these rows
-            for (int n = slot; n < N; n += nslots) grch[(size_t)n * stride] = hv.rch[n];
+          // B
+          const TileRow* rowmap = reinterpret_cast<const TileRow*>(tab + head->rows[p]);
+          for (int r = slot; r < nrows; r += nslots) {
+            const TileRow m = rowmap[r];
+            double rd, R = sR[p][r << wlog], S = sS[p][r << wlog];
+            const double x = tile_row<P, false>(R, S, P::sub(val[m.kid << wlog], val[m.node << wlog]),
+                                                P::mul(srch[p][m.src << wlog], ssg[p][r << wlog]), d, variant, rd);
+            sR[p][r << wlog] = R;
+            sS[p][r << wlog] = S;
+            if (variant == 3 && valid) G.M[(size_t)(rb + r) * stride + h] = rd;
+            ssg[p][r << wlog] = __double_as_longlong(x) > 0 ? P::of_double(x) : P::zero();
+          }
+          __syncthreads();
+          // C: the opponent's terminal values read the new reach rows (the root's never changes, but its
+          // stamp tells that this update is done)
+          auto put_reach = [&](int n, V y) {
+            if (!valid) return;
+            const size_t at = (size_t)n * stride + h;
+            if (alternating) stamp_put(xr + at * words, y, stamp);
+            if (!alternating || last) grch[at] = y;
+          };
+          if (tid < W) put_reach(0, srch[p][0]);
+          auto put_sigma = [&](int r, V y) { ssg[p][r << wlog] = y; };
+          if (tid < T.group) {
+            if (wlog == 3) tile_reach8<P>(T, srch[p], ssg[p], put_sigma, put_reach);
+            else tile_reach<P>(T, srch[p], ssg[p], put_sigma, put_reach);
+          }
+          if (np == 2) __syncthreads();  // the values are free for the other player
         }
       }
-      ++nbar;
-      ok = grid_barrier(&sync[0], nbar * gridDim.x, err, kWaitLimit);
+      if (!alternating) {
+        ++nbar;
+        ok = ok && grid_barrier(&sync[0], nbar * gridDim.x, err, kWaitLimit);
+      } else {
+        __syncthreads();  // the strategy and reach rows of this update are in place
+      }
     }
   }
 
@@ -1540,9 +2114,9 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
       const int rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
       for (int r = slot; r < nrows; r += nslots) {
         const size_t g = (size_t)(rb + r) * stride + h;
-        G.R[g] = sR[p][r * W + w];
-        G.S[g] = sS[p][r * W + w];
-        static_cast<V*>(G.sigma)[g] = ssg[p][r * W + w];
+        G.R[g] = sR[p][r << wlog];
+        G.S[g] = sS[p][r << wlog];
+        static_cast<V*>(G.sigma)[g] = ssg[p][r << wlog];
       }
     }
   }
@@ -2071,321 +2645,6 @@ __global__ void __launch_bounds__(kStreamWarps * 32) k_stream_update(
   }
 }
 
-// ------------------------------------------------------------------ hand tiles
-//
-// The throughput form of the per-hand passes for handles of many subgames whose trees fit a
-// block's shared memory a few times per SM (batches of rivers).  One block owns W hands (32, 16
-// or 8: the most that fit) of one subgame and one player:
-//   A  the values of the tree's end nodes and the stored strategy come in by cp.async; the inner
-//      nodes' values (Stage 6) are computed level by level in shared memory;
-//   B  the regret and average update (Stage 7) of every row of the player: a flat loop over (row,
-//      hand) items with no order between them, four in flight a thread, so that the FP64 pipe
-//      (64 cycles a warp instruction and scheduler) and the R and S streams stay busy; the
-//      positive parts of the new regrets replace the strategy in shared memory;
-//   C  level by level from the root: regret matching of the player's nodes (Eq. rm) and the
-//      reach of their children (Stage 1), in the array of A.
-// R and S are read and written once, straight from registers; L2 is asked for their lines at the
-// start, before the launch waits for its predecessor.  The arithmetic is k_hand's, in its order.
-// Bound: the FP64 pipe (four operations a row and hand: 88 us on the batch below) and issue slots.
-// Measured, one player's update: 256 rivers, FP32 values 267 -> 180 us against the one-warp walk;
-// 64 rivers, pairs, Predictive CFR+ 321 -> 110 us.  Average pass 780 -> 167, best response 943 ->
-// 150 us (256 rivers, both players; k_hand before).
-
-constexpr int kTileThreads = 256;  // at most; 128 where the tiles are small (see create_impl)
-constexpr int kTileRows = 4;       // (row, hand) items of phase B in flight per thread
-
-__host__ __device__ inline size_t tile_smem_bytes(int tab16, int n_nodes, int rows_max, int W, size_t es) {
-  return (size_t)tab16 * 16 + (size_t)(n_nodes + rows_max) * W * es;
-}
-
-// Copies rows of W values (count of them, row k of the source at row_at(k)) into the tile.
-template <typename V, typename F, typename T>
-__device__ __forceinline__ void tile_copy(V* tile, const V* __restrict__ src, size_t stride, int wlog, int count, F row_at,
-                                          T tile_at) {
-  const int pl = wlog + (sizeof(V) == 8 ? 3 : 2) - 4;  // log2 of a row's 16-byte pieces
-  for (int k = threadIdx.x; k < count << pl; k += blockDim.x) {
-    const int r = k >> pl, part = k & ((1 << pl) - 1);
-    cp_async<16>(reinterpret_cast<unsigned char*>(tile + (tile_at(r) << wlog)) + part * 16,
-                 reinterpret_cast<const unsigned char*>(src + (size_t)row_at(r) * stride) + part * 16);
-  }
-}
-
-// Regret matching (Eq. rm) at a decision node of the player with NA actions from the positive parts
-// s, and the reach of its children from the node's reach x (regret_match_n's operations).
-template <typename P, int NA>
-__device__ __forceinline__ void tile_match(const typename P::V* s, typename P::V* c, int wlog, typename P::V x,
-                                           typename P::V* __restrict__ gs, typename P::V* __restrict__ gc, int stride,
-                                           bool store_reach, bool valid) {
-  using V = typename P::V;
-  V y[NA], tot = P::zero();
-  int npos = 0;
-#pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    y[a] = s[a << wlog];
-    npos += P::positive(y[a]);
-    tot = P::add(tot, y[a]);
-  }
-  const V inv = P::recip(tot);  // unused (and possibly not finite) unless npos > 1
-  const V uni = P::uniform(NA);
-#pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    const V many = P::mul(y[a], inv);
-    y[a] = npos > 1 ? many : npos == 1 ? (P::positive(y[a]) ? P::one() : P::zero()) : uni;
-    const V r = P::mul(x, y[a]);
-    c[a << wlog] = r;
-    if (valid) {
-      gs[(size_t)a * stride] = y[a];
-      if (store_reach) gc[(size_t)a * stride] = r;
-    }
-  }
-}
-
-template <int MODE, typename P, bool DCFR>
-__global__ void __launch_bounds__(kTileThreads, 4) k_tile(const GameDev* __restrict__ games,
-                                                       const Work* __restrict__ work, int n_work, int player_mask,
-                                                       int advance, int* iter, unsigned* done,
-                                                       const Discount* __restrict__ disc_tab, int variant) {
-  using V = typename P::V;
-  extern __shared__ __align__(16) unsigned char smx[];
-  __shared__ Discount disc;
-  int p;
-  const Work wk = work[terminal_item(n_work, player_mask, p)];
-  const GameDev& G = games[wk.game];
-  const int wlog = G.tile_wlog, W = 1 << wlog, tid = threadIdx.x, w = tid & (W - 1), slot = tid >> wlog,
-            nslots = blockDim.x >> wlog;
-  const int h0 = wk.unit << wlog, h = h0 + w;  // < hstride: hstride is a multiple of 32 and W divides 32
-  const bool valid = h < G.n_hands;
-  const int N = G.n_nodes, stride = G.hstride, rb = G.row_begin[p], nrows = G.row_begin[p + 1] - rb;
-  const uint64_t hmask = valid ? G.hand_mask[h] : 0ull;
-  const int tab16 = G.tile_tab16;
-
-  // shared: the tile table, values / reach [N][W], strategy [rows][W]
-  V* tval = reinterpret_cast<V*>(smx + (size_t)tab16 * 16);
-  V* val = tval + w;                 // this lane's column: node n at val[n << wlog]
-  V* sg = val + ((size_t)N << wlog);  // row r at sg[r << wlog]
-  const size_t plane = (size_t)p * N * stride;
-  V* gv = static_cast<V*>(MODE == kModeBR ? G.cfv_br : G.cfv) + plane;
-  V* grch = static_cast<V*>(MODE == kModeAvg ? G.reach_bar : G.reach) + plane;
-  V* gsg = static_cast<V*>(MODE == kModeAvg ? G.sigbar : G.sigma) + (size_t)rb * stride;
-  double* gR = G.R + (size_t)rb * stride;
-  double* gS = G.S + (size_t)rb * stride;
-
-  // ---- what older launches wrote: the table, the strategy, and L2 lines of R and S
-  for (int k = tid; k < tab16; k += blockDim.x)
-    reinterpret_cast<uint4*>(smx)[k] = __ldg(reinterpret_cast<const uint4*>(G.tile_tab) + k);
-  if (MODE == kModeUpdate) {
-    if (tid == 0) disc = disc_tab[*iter];
-    auto same = [](int r) { return r; };
-    tile_copy(tval + ((size_t)N << wlog), gsg + h0, (size_t)stride, wlog, nrows, same, same);
-  }
-  if (MODE != kModeBR) {
-    const int ll = wlog == 5;  // lines of 16 doubles per row: 2, or 1
-    for (int k = tid; k < nrows << ll; k += blockDim.x) {
-      const size_t at = (size_t)(k >> ll) * stride + h0 + (k & ll) * 16;
-      if (MODE != kModeAvg) asm volatile("prefetch.global.L2 [%0];" ::"l"(gR + at));
-      if (MODE != kModeInit) asm volatile("prefetch.global.L2 [%0];" ::"l"(gS + at));
-    }
-  }
-  pdl_wait();  // terminal values come from the launch just before this one
-  pdl_trigger();
-  __syncthreads();
-  const TileHead* head = reinterpret_cast<const TileHead*>(smx);
-  const uint16_t* tab = reinterpret_cast<const uint16_t*>(smx);
-  const TileNode* inner = reinterpret_cast<const TileNode*>(tab + head->inner);
-  const uint16_t* level = tab + head->level;  // inner nodes of level l: [level[l], level[l + 1])
-  const int L = head->levels;
-
-  if (MODE == kModeUpdate || MODE == kModeBR) {
-    // ---- A: end values in, then inner values from the deepest level up
-    const uint16_t* ends = tab + head->ends;
-    auto end = [&](int e) { return (int)ends[e]; };
-    tile_copy(tval, static_cast<const V*>(gv) + h0, (size_t)stride, wlog, head->n_ends, end, end);
-    cp_async_wait_all();
-    __syncthreads();
-    for (int l = L - 1; l >= 0; --l) {
-      const int last = level[l + 1];
-      for (int k = level[l] + slot; k < last; k += nslots) {
-        const TileNode nd = inner[k];
-        const int A = nd.kids & 63, kind = nd.kids >> 6;
-        const V* c = val + (nd.first_kid << wlog);
-        V x;
-        if (MODE == kModeBR && kind == p) {
-          x = c[0];
-          for (int a = 1; a < A; ++a) x = P::vmax(x, c[a << wlog]);
-        } else {
-          typename P::Acc acc = P::acc0();
-          if (kind == 2) {  // children values carry the card probabilities; cards in the hand are out
-            for (int a = 0; a < A; ++a)
-              if (!((hmask >> G.nodes[nd.first_kid + a].deal) & 1ull)) P::acc(acc, c[a << wlog]);
-          } else if (kind != p) {
-#pragma unroll 4
-            for (int a = 0; a < A; ++a) P::acc(acc, c[a << wlog]);
-          } else {
-            const V* s = sg + (nd.row << wlog);
-#pragma unroll 4
-            for (int a = 0; a < A; ++a) P::acc_mul(acc, s[a << wlog], c[a << wlog]);
-          }
-          x = P::value(acc);
-        }
-        val[nd.id << wlog] = x;
-        if (valid && (MODE == kModeBR || l == 0)) gv[(size_t)nd.id * stride + h] = x;
-      }
-      __syncthreads();
-    }
-  }
-  if constexpr (MODE == kModeBR) {
-    // FP64 root sums of the tile's chunks, reduced by the game's last block as in k_hand
-    __shared__ int s_last;
-    __shared__ double red64[kHandThreads];
-    const int C = G.chunk;  // <= W
-    if (tid < W) {
-      double x = valid ? G.range64[(size_t)p * stride + h] * P::to_double(val[0]) : 0.0;
-      const unsigned mask = W == 32 ? 0xffffffffu : (1u << W) - 1u;
-      for (int o = C / 2; o > 0; o >>= 1) x += __shfl_down_sync(mask, x, o, C);
-      if (w % C == 0 && valid) G.br_partial[(size_t)p * G.n_chunks + h / C] = x;
-      __threadfence();
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const unsigned chunks = (unsigned)((min(h0 + W, G.n_hands) - h0 + C - 1) / C);
-      s_last = atomicAdd(G.br_done, chunks) + chunks == (unsigned)(2 * G.n_chunks);
-    }
-    __syncthreads();
-    if (s_last) {  // the sums of kHandThreads threads, as k_hand's last block forms them
-      __threadfence();
-      for (int q = 0; q < 2; ++q) {
-        for (int t = tid; t < kHandThreads; t += blockDim.x) {
-          double x = 0.0;
-          for (int c = t; c < G.n_chunks; c += kHandThreads) x += __ldcg(&G.br_partial[(size_t)q * G.n_chunks + c]);
-          red64[t] = x;
-        }
-        __syncthreads();
-        for (int o = kHandThreads / 2; o > 0; o >>= 1) {
-          for (int t = tid; t < o; t += blockDim.x) red64[t] += red64[t + o];
-          __syncthreads();
-        }
-        if (tid == 0) G.br_out[q] = red64[0];
-        __syncthreads();
-      }
-      if (tid == 0) *G.br_done = 0u;
-    }
-    return;
-  }
-
-  // ---- B: every row of the player (sign tests of FP64 values read the sign bit on the integer pipe)
-  {
-    const TileRow* rowmap = reinterpret_cast<const TileRow*>(tab + head->rows[p]);
-    double* gM = G.M ? G.M + (size_t)rb * stride + h : nullptr;
-    const double* src = (MODE == kModeAvg ? gS : gR) + h;
-    for (int r0 = slot; r0 < nrows; r0 += kTileRows * nslots) {
-      double R[kTileRows], S[kTileRows];
-      V pi[kTileRows];
-      TileRow m[kTileRows];
-#pragma unroll
-      for (int e = 0; e < kTileRows; ++e) {
-        const int r = r0 + e * nslots;
-        if (r < nrows) {
-          R[e] = src[(size_t)r * stride];
-          if (MODE == kModeUpdate) {
-            m[e] = rowmap[r];
-            S[e] = gS[(size_t)r * stride + h];
-            pi[e] = grch[(size_t)m[e].src * stride + h];
-          }
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < kTileRows; ++e) {
-        const int r = r0 + e * nslots;
-        if (r < nrows) {
-          double x = R[e];
-          if (MODE == kModeUpdate) {
-            const V rr = P::sub(val[m[e].kid << wlog], val[m[e].node << wlog]);  // instantaneous regret
-            const double rd = P::to_double(rr);
-            const double contrib = P::to_double(P::mul(pi[e], sg[r << wlog]));  // pi_i(I) sigma(I, a)
-            x += rd;
-            double sn;
-            if constexpr (DCFR) {
-              x *= __double_as_longlong(x) > 0 ? disc.dpos : disc.dneg;
-              sn = fma(S[e], disc.dS, contrib);
-            } else {
-              if (variant != 0 && __double_as_longlong(x) < 0) x = 0.0;  // CFR+, Predictive CFR+
-              sn = fma(S[e], disc.dS, variant != 0 ? disc.wS * contrib : contrib);
-            }
-            if (valid) {
-              gR[(size_t)r * stride + h] = x;
-              gS[(size_t)r * stride + h] = sn;
-            }
-            if (!DCFR && variant == 3) {
-              if (valid) gM[(size_t)r * stride] = rd;  // the prediction of the next regret
-              x += rd;                                 // Predictive CFR+ matches R + M
-            }
-          } else if (MODE == kModeInit && gM) {
-            x += gM[(size_t)r * stride];
-          }
-          sg[r << wlog] = __double_as_longlong(x) > 0 ? P::of_double(x) : P::zero();
-        }
-      }
-    }
-  }
-  __syncthreads();  // the positive parts are there, and the values have been read: their array takes the reach
-
-  // ---- C: regret matching and reach from the root down, over the nodes that make new rows: the
-  // children of the player's decisions and of chance nodes (every other node shares a row above
-  // it).  An update stores those rows; the other passes every node's
-  if (tid < W) val[0] = valid ? static_cast<const V*>(G.range_v)[(size_t)p * stride + h] : P::zero();
-  __syncthreads();
-  const TileNode* fwd = reinterpret_cast<const TileNode*>(tab + head->fwd[p]);
-  const uint16_t* flevel = tab + head->flevel[p];
-  for (int l = 0; l < head->flevels[p]; ++l) {
-    const int last = flevel[l + 1];
-    for (int k = flevel[l] + slot; k < last; k += nslots) {
-      const TileNode nd = fwd[k];
-      const int A = nd.kids & 63;
-      const V x = val[nd.id << wlog];
-      V* c = val + (nd.first_kid << wlog);
-      V* gc = grch + (size_t)nd.first_kid * stride + h;
-      const V* s = sg + (nd.row << wlog);
-      V* gs = gsg + (size_t)nd.row * stride + h;
-      if (nd.kids >> 6 == 2) {
-        for (int a = 0; a < A; ++a) {
-          const V y = ((hmask >> G.nodes[nd.first_kid + a].deal) & 1ull) ? P::zero() : x;
-          c[a << wlog] = y;
-          if (MODE == kModeUpdate && valid) gc[(size_t)a * stride] = y;
-        }
-        continue;
-      }
-      constexpr bool upd = MODE == kModeUpdate;
-      switch (A) {
-        case 1: tile_match<P, 1>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 2: tile_match<P, 2>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 3: tile_match<P, 3>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 4: tile_match<P, 4>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 5: tile_match<P, 5>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 6: tile_match<P, 6>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        case 7: tile_match<P, 7>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-        default: tile_match<P, 8>(s, c, wlog, x, gs, gc, stride, upd, valid); break;
-      }
-    }
-    __syncthreads();
-  }
-  if (MODE != kModeUpdate && valid) {
-    const uint16_t* all = tab + head->all[p];
-    for (int n = slot; n < N; n += nslots) grch[(size_t)n * stride + h] = val[all[n] << wlog];
-  }
-
-  if (MODE == kModeUpdate && advance) {
-    if (tid == 0) {
-      __threadfence();
-      const unsigned prev = atomicAdd(done, 1u);
-      if (prev == gridDim.x - 1) {  // last block of the launch: every block has read *iter
-        *done = 0u;
-        *iter += 1;
-        __threadfence();
-      }
-    }
-  }
-}
-
 // sigma = RM(R) at every decision node of every game (current strategy, for read-back when
 // the update launches do not store it).
 template <typename P>
@@ -2652,19 +2911,20 @@ size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es)
 size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv) {
   const TermTab tt(n_hands, hand_size, deck);
   const size_t scan = (size_t)(hand_size * n_hands + 1 + n_hands + 1);
-  if (nv == 1) return (size_t)tt.len * 2 + (size_t)hstride * es + scan * sizeof(ff);
+  if (nv == 1) return (size_t)tt.len * 2 + (size_t)hstride * es + scan * es;
   return kTermSegment * sizeof(TermGroup) + (size_t)tt.fold_len * 2 + 2 * (size_t)nv * hstride * es + scan * nv * es;
 }
 
-size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es) {
-  return tile_smem_bytes(tab16, n_nodes, rows_max, W, es);
+size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es, int staged) {
+  const size_t slack = staged ? (size_t)kTileSlack * W * es : 0;
+  return tile_smem_bytes(tab16, n_nodes, rows_max, W, es) + (staged ? (size_t)2 * rows_max * W * 8 : 0) + slack;
 }
 
 size_t resident_term_size(int n_hands, int hand_size, int deck, int hstride, size_t es) {
   return round16(resident_term_bytes(n_hands, hand_size, deck, hstride, es));
 }
-size_t resident_hand_size(int n_nodes, int n_levels, int rows_max, int W, size_t es) {
-  return resident_hand_bytes(n_nodes, n_levels, rows_max, W, es);
+size_t resident_hand_size(int tab16, int n_nodes, int rows_max, int W, size_t es) {
+  return resident_hand_bytes(tab16, n_nodes, rows_max, W, es);
 }
 int resident_blocks_per_sm(int precision, size_t smem) {
   int n = 0;
@@ -2703,11 +2963,15 @@ static cudaError_t configure_precision() {
   if (e == cudaSuccess) e = configure_one(k_terminal_vec<P, 2>, 200 * 1024);
   if (e == cudaSuccess && sizeof(typename P::V) == 4) e = configure_one(k_terminal_vec<Single, 4>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_average_rows<P>, 0);
-  if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false>, kTileSmem);
-  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false>, kTileSmem);
-  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, true>, kTileSmem);
-  if (e == cudaSuccess) e = configure_one(k_tile<kModeAvg, P, false>, kTileSmem);
-  if (e == cudaSuccess) e = configure_one(k_tile<kModeBR, P, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, true, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeAvg, P, false, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeBR, P, false, false>, kTileSmem);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false, true>, kTileSmemStaged);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false, true>, kTileSmemStaged);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeAvg, P, false, true>, kTileSmemStaged);
+  if (e == cudaSuccess) e = configure_one(k_tile<kModeBR, P, false, true>, kTileSmemStaged);
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 1>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 2>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_current_rows<P>, 0);
@@ -2866,18 +3130,21 @@ int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advanc
   return back + 1;
 }
 
-template <int MODE>
-static int launch_tile(const LaunchCtx& c, int player_mask, int advance, void* stream, bool pdl) {
+template <int MODE, typename P>
+static cudaError_t launch_tile_p(const LaunchCtx& c, int player_mask, int advance, void* stream, bool pdl) {
   auto go = [&](auto kernel) {
     return launch_kernel(kernel, c.n_tile_work * (player_mask == 3 ? 2 : 1), c.tile_threads, c.smem_tile, stream, pdl,
                          c.games, c.tile_work, c.n_tile_work, player_mask, advance, c.iter, c.done, c.disc, c.variant);
   };
   constexpr bool upd = MODE == kModeUpdate;  // the other passes do not depend on the variant
-  cudaError_t e;
-  if (c.precision == kPrecisionSingle)
-    e = upd && c.variant == 2 ? go(k_tile<MODE, Single, upd>) : go(k_tile<MODE, Single, false>);
-  else
-    e = upd && c.variant == 2 ? go(k_tile<MODE, Pairs, upd>) : go(k_tile<MODE, Pairs, false>);
+  if (c.tile_staged) return go(k_tile<MODE, P, false, true>);
+  return upd && c.variant == 2 ? go(k_tile<MODE, P, upd, false>) : go(k_tile<MODE, P, false, false>);
+}
+
+template <int MODE>
+static int launch_tile(const LaunchCtx& c, int player_mask, int advance, void* stream, bool pdl) {
+  const cudaError_t e = c.precision == kPrecisionSingle ? launch_tile_p<MODE, Single>(c, player_mask, advance, stream, pdl)
+                                                        : launch_tile_p<MODE, Pairs>(c, player_mask, advance, stream, pdl);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_tile failed: %s\n", cudaGetErrorString(e));
     return -1;
@@ -2886,8 +3153,8 @@ static int launch_tile(const LaunchCtx& c, int player_mask, int advance, void* s
 }
 
 int launch_init(const LaunchCtx& c, void* stream) {
-  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeInit, 3, 0, stream);
   if (c.n_tile_work > 0) return launch_tile<kModeInit>(c, 3, 0, stream, false);
+  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeInit, 3, 0, stream);
   return launch_hand<kModeInit>(c, 3, 0, stream, false);
 }
 template <typename P, int HP>
@@ -2908,7 +3175,7 @@ static int launch_stream_p(const LaunchCtx& c, int player_mask, int advance, voi
 }
 
 int launch_update(const LaunchCtx& c, int player_mask, int advance, void* stream) {
-  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeUpdate, player_mask, advance, stream);
+  if (c.n_tile_work == 0 && c.schedule == kScheduleWide) return launch_wide_pass(c, kModeUpdate, player_mask, advance, stream);
   if (c.n_tile_work > 0) return launch_tile<kModeUpdate>(c, player_mask, advance, stream, c.pdl != 0);
   if (c.schedule == kScheduleStream)
     return c.precision == kPrecisionSingle
@@ -2927,13 +3194,13 @@ int launch_current_rows(const LaunchCtx& c, void* stream) {
   return check_launch("k_current_rows");
 }
 int launch_avg_reach(const LaunchCtx& c, void* stream) {
-  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeAvg, 3, 0, stream);
   if (c.n_tile_work > 0) return launch_tile<kModeAvg>(c, 3, 0, stream, false);
+  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeAvg, 3, 0, stream);
   return launch_hand<kModeAvg>(c, 3, 0, stream, false);
 }
 int launch_br(const LaunchCtx& c, void* stream) {
-  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeBR, 3, 0, stream);
   if (c.n_tile_work > 0) return launch_tile<kModeBR>(c, 3, 0, stream, c.pdl != 0);
+  if (c.schedule == kScheduleWide) return launch_wide_pass(c, kModeBR, 3, 0, stream);
   return launch_hand<kModeBR>(c, 3, 0, stream, c.pdl != 0);
 }
 
@@ -2964,7 +3231,7 @@ int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stre
 // One cooperative launch: every block is resident at once, which the grid barriers need
 // (the launch fails rather than run a grid that does not fit).
 template <typename P>
-static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stream) {
+static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c.resident_grid);
   cfg.blockDim = dim3(kTermThreads);
@@ -2977,12 +3244,12 @@ static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stre
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_resident<P>, c.games, c.chunk_work, c.n_chunk_work, c.term_work,
                             c.term_src, c.n_term_work, c.alternating, n_iters, c.iter,
-                            c.disc, c.variant, c.resident_sync, c.err, c.resident_term);
+                            c.disc, c.variant, c.resident_sync, c.err, c.resident_term, stamp0);
 }
 
-int launch_resident(const LaunchCtx& c, int n_iters, void* stream) {
-  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single>(c, n_iters, stream)
-                                                        : launch_resident_p<Pairs>(c, n_iters, stream);
+int launch_resident(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream) {
+  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single>(c, n_iters, stamp0, stream)
+                                                        : launch_resident_p<Pairs>(c, n_iters, stamp0, stream);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_resident failed: %s\n", cudaGetErrorString(e));
     return -1;

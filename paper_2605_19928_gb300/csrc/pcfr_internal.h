@@ -104,6 +104,7 @@ struct alignas(8) TileRow {  // a row's child node, its decision node, and the n
 
 constexpr int kTileSmemSmall = 26 * 1024;  // shared memory of a block of 128 threads: eight fit an SM
 constexpr int kTileSmem = 53 * 1024;       // of a block of 256 threads: four fit
+constexpr int kTileSmemStaged = 200 * 1024;  // of the latency form, at most
 
 // One node of the stream schedule's program (pre-order), 16 bytes.  Offsets are in
 // elements of a per-hand array (multiples of hstride).
@@ -169,6 +170,7 @@ struct GameDev {
   const uint16_t* tile_tab;    // hand tiles: TileHead and its lists (null: the handle does not use them)
   int tile_tab16;              // its length in 16-byte units
   int tile_wlog;               // log2 of the hands per tile
+  int tile_group;              // threads that walk its levels in the latency form and k_resident
   const int32_t* chunks;       // load chunks of the stream schedule (see stream_tables)
   int chunk_off[4], chunk_count[4];
   const uint32_t* units;       // loads of the stream schedule, in the order the passes use them
@@ -183,6 +185,8 @@ struct GameDev {
   void* reach_bar;
   void* cfv;
   void* cfv_br;
+  uint64_t* xval;              // resident schedule, alternating: stamped values [2][n_nodes][hstride][sizeof(V) / 4]
+  uint64_t* xreach;            // and stamped reach rows, laid out alike
   double* br_partial;          // [2][n_chunks] per-block sums of r_i(h) v*_i(root, h)
   double* br_out;              // [2]
   unsigned* br_done;           // blocks of the best-response pass that have finished
@@ -253,10 +257,11 @@ struct LaunchCtx {
   const Work* warp_work;       // device [n_warp_work]: (game, first group of 32 hands) of each
                                // block of the stream schedule, largest trees first
   int n_warp_work;
-  const Work* tile_work;       // device [n_tile_work]: (game, tile), largest trees first; the stream
-  int n_tile_work;             // schedule's passes run as k_tile when there are any
+  const Work* tile_work;       // device [n_tile_work]: (game, tile), largest trees first; the per-hand
+  int n_tile_work;             // passes run as k_tile when there are any
   size_t smem_tile;            // dynamic shared memory of k_tile
   int tile_threads;            // its threads per block
+  int tile_staged;             // its latency form (R and S staged; level and wide schedules)
   int stream_depth;            // stack slots per lane of the stream schedule
   int stream_prog;             // nodes of the largest tree, if its program is staged in shared
                                // memory; 0 = read from global memory
@@ -301,14 +306,15 @@ int configure_kernels();  // once per process, before the first launch
 // Polls of the terminal kernel's first bulk-copy wait on the current device (< 0: the
 // default limit); for tests of the timeout path.  Returns 0 or -1.
 int set_first_wait_polls(long polls);
-// Shared memory of k_tile for one game (tab16: its table in 16-byte units).
-size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es);
+// Shared memory of k_tile for one game (tab16: its table in 16-byte units; staged: its latency form).
+size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es, int staged);
 // Resident schedule: shared memory of its two regions for one game, the blocks of k_resident
-// one SM holds with `smem` bytes (0 if none), and the cooperative launch of n_iters iterations.
+// one SM holds with `smem` bytes (0 if none), and the cooperative launch of n_iters iterations (its stamps are stamp0 + 1 ..
+// stamp0 + n_iters, none of which the handle used before).
 size_t resident_term_size(int n_hands, int hand_size, int deck, int hstride, size_t es);
-size_t resident_hand_size(int n_nodes, int n_levels, int rows_max, int W, size_t es);
+size_t resident_hand_size(int tab16, int n_nodes, int rows_max, int W, size_t es);
 int resident_blocks_per_sm(int precision, size_t smem);
-int launch_resident(const LaunchCtx& c, int n_iters, void* stream);
+int launch_resident(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream);
 // Dense layer of the leaf network (leafnet.cu): C[M][N] = act(A[M][K] B[N][K]^T + bias), BF16
 // A and B, FP32 accumulation, C in BF16 (out_f32 = 0) or FP32; N a multiple of 128, K of 64.
 // Returns 0, -1 (launch failed), -2 (bad shape or alignment), -3 (no tensor-map encoder).

@@ -712,7 +712,6 @@ std::vector<uint16_t> tile_table(const HostGame& g) {
         ends.push_back((uint16_t)n);
         continue;
       }
-      if (nd.type == kDecision && nd.n_kids > kStreamMaxActions) return {};
       TileNode t{};
       t.id = (uint16_t)n;
       t.first_kid = (uint16_t)nd.first_kid;
@@ -780,6 +779,16 @@ std::vector<uint16_t> tile_table(const HostGame& g) {
   memcpy(out.data(), &head, sizeof head);
   out.resize((out.size() + 7) / 8 * 8, 0);
   return out;
+}
+
+int tile_walkers(const HostGame& g, int W) {
+  int widest = 1;
+  for (size_t l = 0; l + 1 < g.level_start.size(); ++l) {
+    int cnt = 0;
+    for (int n = g.level_start[l]; n < g.level_start[l + 1]; ++n) cnt += !is_terminal(g.nodes[(size_t)n]);
+    widest = std::max(widest, cnt);
+  }
+  return std::min((widest * W + 31) / 32 * 32, 256);
 }
 
 void plan_runouts(const HostGame& h, RunoutPlan& r) {

@@ -87,10 +87,14 @@ std::vector<int32_t> stream_tables(const HostGame& g, const std::vector<int32_t>
                                    int chunk_off[4], int chunk_count[4]);
 
 // The hand-tile table of one subgame (TileHead and its lists, pcfr_internal.h), or empty when its
-// tree does not suit them (node or row ids beyond 16 bits, more actions than a tile's rows hold).
+// tree does not suit them (node or row ids beyond 16 bits).
 // Nodes of one level are ordered by kind and action count, so that the slots sharing a warp take the
 // same path; their order changes no result.
 std::vector<uint16_t> tile_table(const HostGame& g);
+
+// Threads that walk the levels of a tile of W hands in the latency form: enough for the widest level in
+// one step, a multiple of 32 from 32 to 256.
+int tile_walkers(const HostGame& g, int W);
 
 // All-in run-outs of one game evaluated by win-minus-loss tables (runout.h): a run-out's top
 // is a chance node below a decision whose subtree holds only chance and showdown nodes, all of

@@ -72,6 +72,32 @@ def test_stream_schedule_and_terminal_groups_keep_the_bits(case, variant, altern
 
 
 @pytest.mark.parametrize("precision", ["single", "pairs"])
+@pytest.mark.parametrize("variant,alternating", [("dcfr", True), ("pcfr+", False), ("cfr+", True)])
+def test_latency_forms_keep_the_bits(variant, alternating, precision):
+    """The staged tiles (4 hands or more) and the resident schedule's phases against the per-hand
+    kernel (chunks of 2 hands take it), with 12 actions at a node, and trees wider than a block."""
+    many = tuple(0.2 * k for k in range(1, 11)) + (ALL_IN,)
+    for specs in ([river(19, 41, bet_sizes=many, max_raises=1, stack=800.0)],
+                  [river(45, 43, bet_sizes=(0.33, 0.5, 0.75, 1.0, ALL_IN), max_raises=3, stack=900.0)],
+                  [synth.leduc()], [river(27, 45), synth.kuhn()], BATCHES["turns"]()[:2]):
+        kw = dict(alternating=alternating, precision=precision)
+        want = _solve(specs, capi.make_opts(variant, schedule="level", chunk_hands=2, **kw))
+        runs = [("level", 4), ("level", 8), ("level", 32), ("resident", 1), ("resident", 8)]
+        if len(specs) == 1 and specs[0].bet_sizes != many:
+            runs.append(("wide", 8))
+        for schedule, chunk in runs:
+            try:
+                got = _solve(specs, capi.make_opts(variant, schedule=schedule, chunk_hands=chunk, **kw))
+            except capi.CfrError as e:
+                assert schedule == "resident" and e.code == capi.CFR_EINVAL  # too large for shared memory
+                continue
+            for x, y in zip([*got[0], *got[3]], [*want[0], *want[3]], strict=True):
+                assert np.array_equal(x, y), (schedule, chunk)
+            assert np.allclose(got[1], want[1], rtol=1e-13, atol=1e-15)  # FP64 root sums over other chunks
+            assert np.allclose(got[2], want[2], rtol=1e-13, atol=1e-15)
+
+
+@pytest.mark.parametrize("precision", ["single", "pairs"])
 def test_many_groups_per_block(precision):
     """Stretches of several groups over games of different hand counts (shared memory laid out anew)."""
     specs = [river(40 + 29 * k % 170, 100 + k, stack=100.0 + 37.0 * k, max_raises=2 + k % 2) for k in range(70)]
