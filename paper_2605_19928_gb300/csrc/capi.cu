@@ -59,8 +59,9 @@ struct cfr_tree {
   Work* d_term_segments = nullptr;
   Work* d_warp_work = nullptr;
   Work* d_tile_work = nullptr;
-  int32_t* d_wide_inner = nullptr;  // wide schedule: inner node ids, level by level
-  int32_t* d_wide_fwd = nullptr;    // wide schedule: nodes whose reach is stored, level by level
+  WideNode* d_wide_inner = nullptr;                // wide schedule: inner nodes, level by level
+  WideReach* d_wide_fwd[2] = {nullptr, nullptr};   // per player: nodes that make new reach rows, by depth
+  int32_t* d_reach_row[2] = {nullptr, nullptr};    // run-out tables: HostGame::reach_row
   TermSrc* d_term_src = nullptr;    // reach rows of each terminal work entry
   // all-in run-outs evaluated by win-minus-loss tables (runout_tables; none: all zero)
   RunoutItem* d_ro_items = nullptr;   // top nodes, sorted by table
@@ -69,7 +70,7 @@ struct cfr_tree {
   int ro_n8 = 0, ro_n16 = 0;          // groups of tops on uint8 / uint16 tables
   RunoutTable* d_ro_tables = nullptr;
   unsigned char* d_ro_pool = nullptr;
-  std::vector<int> wide_inner_off, wide_fwd_off;
+  std::vector<int> wide_inner_off, wide_fwd_off[2];
   int* d_iter = nullptr;
   unsigned* d_done = nullptr;
   unsigned* d_res_sync = nullptr;   // resident schedule: barrier and exit counters
@@ -160,7 +161,8 @@ int launch_terminals(const cfr_tree* t, int player_mask, int use_bar, cudaStream
   if (t->ro_n8 + t->ro_n16 == 0) return 0;
   const HostGame& h = t->host[0];
   return launch_runout_values(t->ctx.games, t->d_ro_items, t->d_ro_groups8, t->ro_n8, t->d_ro_groups16, t->ro_n16,
-                              t->d_ro_tables, t->d_ro_pool, h.n_hands, player_mask, use_bar, s);
+                              t->d_ro_tables, t->d_ro_pool, t->ctx.reach_row[0], t->ctx.reach_row[1], h.n_hands, player_mask,
+                              use_bar, s);
 }
 
 // Kernels one terminal stage launches.
@@ -656,24 +658,48 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
                                   " blocks fit)");
     }
   }
-  if (schedule == kScheduleWide) {  // per level: the inner nodes, and the nodes whose reach is stored
+  if (schedule == kScheduleWide && !tiles) {  // per level: the inner nodes; per player: the nodes with new reach rows
     const HostGame& h = t->host[0];
-    const int L = (int)h.level_start.size() - 1;
+    const int L = (int)h.level_start.size() - 1, N = (int)h.nodes.size();
     t->wide_inner_off.assign(1, 0);
-    t->wide_fwd_off.assign(1, 0);
-    std::vector<int32_t> inner, fwd;
+    std::vector<WideNode> inner;
     for (int l = 0; l < L; ++l) {
       for (int n = h.level_start[l]; n < h.level_start[l + 1]; ++n) {
+        const NodeDev& nd = h.nodes[(size_t)n];
         const bool tabled = !ro.top.empty() && (ro.top[(size_t)n] || ro.inside[(size_t)n]);
-        if (!is_end(h.nodes[(size_t)n].type) && !tabled) inner.push_back(n);
-        if (h.reach_src[(size_t)n] == n) fwd.push_back(n);
+        if (is_end(nd.type) || tabled) continue;
+        const uint32_t kind = nd.type == kChance ? 2 : nd.player;
+        inner.push_back({(uint32_t)n | (uint32_t)nd.n_kids << 24 | kind << 30, nd.first_kid, nd.row,
+                         kind < 2 ? h.reach_row[kind][(size_t)n] : 0});
       }
       t->wide_inner_off.push_back((int)inner.size());
-      t->wide_fwd_off.push_back((int)fwd.size());
     }
-    if ((rc = upload(t, inner, &t->d_wide_inner)) || (rc = upload(t, fwd, &t->d_wide_fwd))) {
+    if ((rc = upload(t, inner, &t->d_wide_inner))) {
       delete t;
       return rc;
+    }
+    for (int p = 0; p < 2; ++p) {
+      std::vector<int> depth((size_t)N, 0);
+      std::vector<std::vector<WideReach>> by(1);
+      by[0].push_back({0, -1, -1, -1});
+      for (int n = 1; n < N; ++n) {
+        const NodeDev& nd = h.nodes[(size_t)n];
+        const int src = h.reach_row[p][(size_t)nd.parent];
+        if (h.reach_row[p][(size_t)n] != n) continue;
+        const size_t d = (size_t)(depth[(size_t)n] = depth[(size_t)src] + 1);
+        if (by.size() <= d) by.resize(d + 1);
+        by[d].push_back({n, src, nd.aplayer == p ? nd.arow : -1, nd.deal == kNoCard ? -1 : nd.deal});
+      }
+      std::vector<WideReach> fwd;
+      t->wide_fwd_off[p].assign(1, 0);
+      for (const auto& l : by) {
+        fwd.insert(fwd.end(), l.begin(), l.end());
+        t->wide_fwd_off[p].push_back((int)fwd.size());
+      }
+      if ((rc = upload(t, fwd, &t->d_wide_fwd[p])) || (o.runout_tables && (rc = upload(t, h.reach_row[p], &t->d_reach_row[p])))) {
+        delete t;
+        return rc;
+      }
     }
   }
 
@@ -981,14 +1007,20 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const long items = (long)term_work.size() * (o.alternating ? 1 : 2);
     c.resident_grid = (int)std::max<long>(chunk_work.size(), std::min<long>(items, n_sms));
   }
-  if (schedule == kScheduleWide) {
+  if (schedule == kScheduleWide && !tiles) {
     const HostGame& h = t->host[0];
     c.wide_levels = (int)t->wide_inner_off.size() - 1;
     c.wide_inner_off = t->wide_inner_off.data();
     c.wide_inner = t->d_wide_inner;
-    c.wide_fwd_off = t->wide_fwd_off.data();
-    c.wide_fwd = t->d_wide_fwd;
-    c.wide_stride = h.hstride;
+    for (int p = 0; p < 2; ++p) {
+      c.wide_fwd_levels[p] = (int)t->wide_fwd_off[p].size() - 1;
+      c.wide_fwd_off[p] = t->wide_fwd_off[p].data();
+      c.wide_fwd[p] = t->d_wide_fwd[p];
+      c.reach_row[p] = t->d_reach_row[p];
+    }
+    const int pairs = (h.n_hands + 1) / 2;  // two hands a thread, blocks of even size
+    c.wide_segments = (pairs + 255) / 256;
+    c.wide_threads = ((pairs + c.wide_segments - 1) / c.wide_segments + 31) / 32 * 32;
     int dmax = 0;
     for (int p = 0; p < 2; ++p) {
       int cnt = 0;

@@ -2700,168 +2700,235 @@ __global__ void k_average_rows(const GameDev* __restrict__ games, int n_games) {
 
 // ------------------------------------------------------------------ wide schedule
 //
-// For one tree too large to stage in shared memory, each pass of the per-hand kernel
-// becomes one launch per level in which every thread owns one (node, hand) pair: the hand
-// index is the fastest-moving coordinate, so each warp reads and writes 32 consecutive
-// entries of a row, and a level of n nodes runs n x hstride threads at once instead of
-// stepping through its nodes in a few blocks.  The arithmetic per (node, hand) -- the order
-// of every sum over children, regret matching, the Stage 7 update -- is the per-hand
-// kernel's, so the schedules agree bit for bit.
+// For one tree too large to stage in shared memory, each pass of the per-hand kernel becomes one
+// launch per level over all of that level's (node, hand) pairs.  A block takes one node (or, when
+// its hands are more than 512, an even share of them), two consecutive hands a thread: the node's
+// description is one 16-byte load, branches are the block's, and rows are read and written 16
+// bytes a thread (FP64) or 8 (FP32 values).  The arithmetic per (node, hand) -- the order of every
+// sum over children, regret matching, the Stage 7 update -- is the per-hand kernel's, so the
+// schedules agree bit for bit.  Bound by DRAM where a level holds many nodes and by the launches'
+// latency where it does not.  Measured, one player's update with FP32 values: exact turn 355 -> 225 us,
+// learned flop 204 -> 144 us against one thread per (node, hand) that found its node by division
+// and stored every node's reach; average pass of the turn 278 -> 143, best response 192 -> 110.
+// Three blocks of 85 registers per SM (nodes of six actions and more spill) beat two without
+// spills (253 us).
 
-constexpr int kWideThreads = 256;
+constexpr int kWideThreads = 256;  // at most; LaunchCtx::wide_threads
+
+template <typename P>
+struct alignas(2 * sizeof(typename P::V)) V2 {  // two consecutive hands' values
+  typename P::V v[2];
+};
+
+// Two hands of a row; `both`: the second exists (it is not stored otherwise).
+template <typename T2, typename T>
+__device__ __forceinline__ T2 load2(const T* p) { return *reinterpret_cast<const T2*>(p); }
+template <typename P>
+__device__ __forceinline__ void store2(typename P::V* p, const V2<P>& x, bool both) {
+  if (both) *reinterpret_cast<V2<P>*>(p) = x;
+  else p[0] = x.v[0];
+}
+__device__ __forceinline__ void store2(double* p, double2 x, bool both) {
+  if (both) *reinterpret_cast<double2*>(p) = x;
+  else p[0] = x.x;
+}
+
+// The update at one of the player's decision nodes with NA actions, for two hands: the value under
+// the current strategy, then Stage 7 and the new strategy RM(R') (Eq. rm).
+template <typename P, int NA>
+__device__ __forceinline__ V2<P> wide_decision(const typename P::V* __restrict__ c, typename P::V* __restrict__ sgp,
+                                               const typename P::V* __restrict__ pip, double* __restrict__ Rp,
+                                               double* __restrict__ Sp, double* __restrict__ Mp, size_t S,
+                                               const Discount& d, int variant, bool both) {
+  using V = typename P::V;
+  V2<P> cc[NA], sg[NA];
+  double2 R[NA], Sv[NA];
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    cc[a] = load2<V2<P>>(c + (size_t)a * S);
+    sg[a] = load2<V2<P>>(sgp + (size_t)a * S);
+    R[a] = load2<double2>(Rp + (size_t)a * S);
+    Sv[a] = load2<double2>(Sp + (size_t)a * S);
+  }
+  const V2<P> pi = load2<V2<P>>(pip);
+  V2<P> val;
+  const bool plus = variant == 1 || variant == 3;  // CFR+, Predictive CFR+
+  double2 rd[NA];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    typename P::Acc acc = P::acc0();
+#pragma unroll
+    for (int a = 0; a < NA; ++a) P::acc_mul(acc, sg[a].v[j], cc[a].v[j]);
+    val.v[j] = P::value(acc);
+    double Rm[NA];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      const double r = P::to_double(P::sub(cc[a].v[j], val.v[j]));                // instantaneous regret
+      const double contrib = P::to_double(P::mul(pi.v[j], sg[a].v[j]));          // pi_i(I) sigma(I, a)
+      double x = (j ? R[a].y : R[a].x) + r;
+      if (variant == 2) x *= __double_as_longlong(x) > 0 ? d.dpos : d.dneg;
+      if (plus && __double_as_longlong(x) < 0) x = 0.0;
+      const double sn = fma(j ? Sv[a].y : Sv[a].x, d.dS, plus ? d.wS * contrib : contrib);
+      (j ? R[a].y : R[a].x) = x;
+      (j ? Sv[a].y : Sv[a].x) = sn;
+      (j ? rd[a].y : rd[a].x) = r;
+      Rm[a] = variant == 3 ? x + r : x;  // Predictive CFR+ matches R + M
+    }
+    V y[NA];
+    regret_match_n<P, NA>(Rm, y);
+#pragma unroll
+    for (int a = 0; a < NA; ++a) sg[a].v[j] = y[a];
+  }
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    store2(Rp + (size_t)a * S, R[a], both);
+    store2(Sp + (size_t)a * S, Sv[a], both);
+    if (variant == 3) store2(Mp + (size_t)a * S, rd[a], both);  // the prediction of the next regret
+    store2<P>(sgp + (size_t)a * S, sg[a], both);
+  }
+  return val;
+}
 
 // Bottom-up step at the inner nodes of one level (Stage 6, Eq. backward) for player p =
 // blockIdx.y when both players are in the launch.  kModeUpdate: at p's decision nodes also
 // the regrets, the Stage 7 update of R and S and the new strategy RM(R') (Eq. rm);
 // kModeBR: the best-response value max_a v(child a) at p's decision nodes.
 template <int MODE, typename P>
-__global__ void __launch_bounds__(kWideThreads, 4) k_wide_back(const GameDev* __restrict__ games,
-                                                            const int32_t* __restrict__ inner, int cnt,
+__global__ void __launch_bounds__(kWideThreads, 3) k_wide_back(const GameDev* __restrict__ games,
+                                                            const WideNode* __restrict__ inner, int segments,
                                                             int player_mask, const int* __restrict__ iter,
                                                             const Discount* __restrict__ disc_tab, int variant) {
   using V = typename P::V;
+  const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
+  const WideNode w = inner[blockIdx.x / (unsigned)segments];
+  const int h = 2 * ((int)(blockIdx.x % (unsigned)segments) * (int)blockDim.x + (int)threadIdx.x);
   pdl_wait();
   pdl_trigger();
   const GameDev& G = games[0];
-  const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
-  const size_t S = (size_t)G.hstride;
-  const size_t e = (size_t)blockIdx.x * kWideThreads + threadIdx.x;
-  if (e >= (size_t)cnt * S) return;
-  const int n = inner[e / S], h = (int)(e % S);
   if (h >= G.n_hands) return;
-  const NodeDev nd = G.nodes[n];
-  const size_t N = (size_t)G.n_nodes;
+  const bool both = h + 1 < G.n_hands;
+  const size_t S = (size_t)G.hstride, N = (size_t)G.n_nodes;
   V* v = static_cast<V*>(MODE == kModeBR ? G.cfv_br : G.cfv) + (size_t)p * N * S + h;
-  const int A = nd.n_kids, k0 = nd.first_kid;
-  V val;
-  if (MODE == kModeBR && nd.type == kDecision && nd.player == p) {
-    val = v[(size_t)k0 * S];
-    for (int a = 1; a < A; ++a) val = P::vmax(val, v[(size_t)(k0 + a) * S]);
-    v[(size_t)n * S] = val;
-    return;
-  }
-  if (nd.type == kChance) {
+  const int n = w.node(), A = w.kids(), kind = w.kind();
+  const V* c = v + (size_t)w.first_kid * S;
+  V2<P> val;
+  if (kind == 2) {
     // children values already carry the card probabilities; cards in the hand are out
-    const uint64_t hmask = G.hand_mask[h];
-    typename P::Acc acc = P::acc0();
-    for (int a = 0; a < A; ++a)
-      if (!((hmask >> G.nodes[k0 + a].deal) & 1ull)) P::acc(acc, v[(size_t)(k0 + a) * S]);
-    v[(size_t)n * S] = P::value(acc);
-    return;
-  }
-  if (nd.player != p || MODE == kModeBR) {
-    typename P::Acc acc = P::acc0();
-    for (int a = 0; a < A; ++a) P::acc(acc, v[(size_t)(k0 + a) * S]);
-    v[(size_t)n * S] = P::value(acc);
-    return;
-  }
-  // p's decision node: value under the current strategy, then the Stage 7 update
-  V* sgp = static_cast<V*>(G.sigma) + (size_t)nd.row * S + h;
-  V c[kStreamMaxActions], sg[kStreamMaxActions];
-  typename P::Acc acc = P::acc0();
-#pragma unroll
-  for (int a = 0; a < kStreamMaxActions; ++a)
-    if (a < A) {
-      c[a] = v[(size_t)(k0 + a) * S];
-      sg[a] = sgp[(size_t)a * S];
-      P::acc_mul(acc, sg[a], c[a]);
+    const uint64_t m0 = G.hand_mask[h], m1 = both ? G.hand_mask[h + 1] : 0ull;
+    typename P::Acc a0 = P::acc0(), a1 = P::acc0();
+    for (int a = 0; a < A; ++a) {
+      const int deal = G.nodes[w.first_kid + a].deal;
+      const V2<P> x = load2<V2<P>>(c + (size_t)a * S);
+      if (!((m0 >> deal) & 1ull)) P::acc(a0, x.v[0]);
+      if (!((m1 >> deal) & 1ull)) P::acc(a1, x.v[1]);
     }
-  val = P::value(acc);
-  v[(size_t)n * S] = val;
-  const Discount d = disc_tab[*iter];
-  const V pi = static_cast<const V*>(G.reach)[((size_t)p * N + n) * S + h];
-  double* Rp = G.R + (size_t)nd.row * S + h;
-  double* Sp = G.S + (size_t)nd.row * S + h;
-  double* Mp = variant == 3 ? G.M + (size_t)nd.row * S + h : nullptr;
-  double Rm[kStreamMaxActions];
-#pragma unroll
-  for (int a = 0; a < kStreamMaxActions; ++a) {
-    Rm[a] = 0.0;
-    if (a < A) {
-      const V rr = P::sub(c[a], val);                          // instantaneous regret
-      const double contrib = P::to_double(P::mul(pi, sg[a]));  // pi_i(I) sigma(I, a)
-      const double rd = P::to_double(rr);
-      double x = Rp[(size_t)a * S] + rd;
-      if (variant == 2) x *= __double_as_longlong(x) > 0 ? d.dpos : d.dneg;
-      if ((variant == 1 || variant == 3) && __double_as_longlong(x) < 0) x = 0.0;  // CFR+, Predictive CFR+
-      const double sn = fma(Sp[(size_t)a * S], d.dS, (variant == 1 || variant == 3) ? d.wS * contrib : contrib);
-      Rp[(size_t)a * S] = x;
-      Sp[(size_t)a * S] = sn;
-      Rm[a] = x;
-      if (variant == 3) {
-        Mp[(size_t)a * S] = rd;  // the prediction of the next regret
-        Rm[a] = x + rd;          // Predictive CFR+ matches R + M
-      }
+    val.v[0] = P::value(a0), val.v[1] = P::value(a1);
+  } else if (kind != p) {
+    typename P::Acc a0 = P::acc0(), a1 = P::acc0();
+#pragma unroll 4
+    for (int a = 0; a < A; ++a) {
+      const V2<P> x = load2<V2<P>>(c + (size_t)a * S);
+      P::acc(a0, x.v[0]);
+      P::acc(a1, x.v[1]);
+    }
+    val.v[0] = P::value(a0), val.v[1] = P::value(a1);
+  } else if (MODE == kModeBR) {
+    val = load2<V2<P>>(c);
+    for (int a = 1; a < A; ++a) {
+      const V2<P> x = load2<V2<P>>(c + (size_t)a * S);
+      val.v[0] = P::vmax(val.v[0], x.v[0]);
+      val.v[1] = P::vmax(val.v[1], x.v[1]);
+    }
+  } else {
+    const size_t at = (size_t)w.row * S + h;
+    V* sg = static_cast<V*>(G.sigma) + at;
+    const V* pi = static_cast<const V*>(G.reach) + ((size_t)p * N + w.src) * S + h;
+    double* Mp = G.M ? G.M + at : nullptr;
+    const Discount d = disc_tab[*iter];
+    switch (A) {  // the block's, at most kStreamMaxActions
+      case 1: val = wide_decision<P, 1>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 2: val = wide_decision<P, 2>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 3: val = wide_decision<P, 3>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 4: val = wide_decision<P, 4>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 5: val = wide_decision<P, 5>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 6: val = wide_decision<P, 6>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      case 7: val = wide_decision<P, 7>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
+      default: val = wide_decision<P, 8>(c, sg, pi, G.R + at, G.S + at, Mp, S, d, variant, both); break;
     }
   }
-  V sn[kStreamMaxActions];
-  regret_match<P>(Rm, A, sn);
-#pragma unroll
-  for (int a = 0; a < kStreamMaxActions; ++a)
-    if (a < A) sgp[(size_t)a * S] = sn[a];
+  store2<P>(v + (size_t)n * S, val, both);
 }
 
-// Strategy rows of player p (blockIdx.y when both): RM(R) (+ M for Predictive CFR+) into
-// sigma (avg = 0), or the average S / sum S into sigbar (avg = 1), as the per-hand kernel
-// computes them: positive parts in the value type, their sum in action order.
+// Strategy rows of player p = blockIdx.y: RM(R) (+ M for Predictive CFR+) into sigma (avg = 0), or the
+// average S / sum S into sigbar (avg = 1), as the per-hand kernel computes them: positive parts in
+// the value type, their sum in action order.
 template <typename P>
-__global__ void __launch_bounds__(kWideThreads) k_wide_rows(const GameDev* __restrict__ games, int player_mask,
-                                                            int avg) {
+__global__ void __launch_bounds__(kWideThreads) k_wide_rows(const GameDev* __restrict__ games, int segments, int avg) {
   using V = typename P::V;
   pdl_wait();
   pdl_trigger();
   const GameDev& G = games[0];
-  const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
-  const size_t S = (size_t)G.hstride;
+  const int p = blockIdx.y, k = (int)(blockIdx.x / (unsigned)segments);
   const int db = G.dec_begin[p], ndec = G.dec_begin[p + 1] - db;
-  const size_t e = (size_t)blockIdx.x * kWideThreads + threadIdx.x;
-  if (e >= (size_t)ndec * S) return;
-  const int h = (int)(e % S);
-  if (h >= G.n_hands) return;
-  const NodeDev nd = G.nodes[G.dec_nodes[db + (int)(e / S)]];
-  double x[kStreamMaxActions];
-  load_rows((avg ? G.S : G.R) + (size_t)nd.row * S + h, S, nd.n_kids, x);
-  if (!avg && G.M) {
-    double m[kStreamMaxActions];
-    load_rows(G.M + (size_t)nd.row * S + h, S, nd.n_kids, m);
+  const int h0 = 2 * ((int)(blockIdx.x % (unsigned)segments) * (int)blockDim.x + (int)threadIdx.x);
+  if (k >= ndec || h0 >= G.n_hands) return;
+  const size_t S = (size_t)G.hstride;
+  const NodeDev nd = G.nodes[G.dec_nodes[db + k]];
+  for (int h = h0; h < min(h0 + 2, G.n_hands); ++h) {
+    double x[kStreamMaxActions];
+    load_rows((avg ? G.S : G.R) + (size_t)nd.row * S + h, S, nd.n_kids, x);
+    if (!avg && G.M) {
+      double m[kStreamMaxActions];
+      load_rows(G.M + (size_t)nd.row * S + h, S, nd.n_kids, m);
 #pragma unroll
-    for (int a = 0; a < kStreamMaxActions; ++a) x[a] += m[a];
+      for (int a = 0; a < kStreamMaxActions; ++a) x[a] += m[a];
+    }
+    V sg[kStreamMaxActions];
+    regret_match<P>(x, nd.n_kids, sg);
+    V* out = static_cast<V*>(avg ? G.sigbar : G.sigma) + (size_t)nd.row * S + h;
+#pragma unroll
+    for (int a = 0; a < kStreamMaxActions; ++a)
+      if (a < nd.n_kids) out[(size_t)a * S] = sg[a];
   }
-  V sg[kStreamMaxActions];
-  regret_match<P>(x, nd.n_kids, sg);
-  V* out = static_cast<V*>(avg ? G.sigbar : G.sigma) + (size_t)nd.row * S + h;
-#pragma unroll
-  for (int a = 0; a < kStreamMaxActions; ++a)
-    if (a < nd.n_kids) out[(size_t)a * S] = sg[a];
 }
 
-// Top-down step at the nodes of one level whose reach is stored (list[0 .. cnt)) (Stages
-// 1-2): p's reach is the parent's times p's probability of the action, and zero for hands
-// holding a dealt card.  Level 0 (the root) takes p's range.
+// Top-down step (Stages 1-2) of player p = blockIdx.y (or the one of the launch) over the nodes that
+// make new reach rows at one depth: its row is the one above it times p's probability of the
+// action, or without the hands holding the dealt card.  The root takes p's range.
 template <typename P>
 __global__ void __launch_bounds__(kWideThreads) k_wide_fwd(const GameDev* __restrict__ games,
-                                                           const int32_t* __restrict__ list, int cnt,
+                                                           const WideReach* __restrict__ list0, int cnt0,
+                                                           const WideReach* __restrict__ list1, int cnt1, int segments,
                                                            int player_mask, int avg) {
   using V = typename P::V;
+  const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
+  const int k = (int)(blockIdx.x / (unsigned)segments);
+  const int h = 2 * ((int)(blockIdx.x % (unsigned)segments) * (int)blockDim.x + (int)threadIdx.x);
+  if (k >= (p ? cnt1 : cnt0)) return;  // (a launch's blocks may leave before its trigger)
+  const WideReach w = (p ? list1 : list0)[k];
   pdl_wait();
   pdl_trigger();
   const GameDev& G = games[0];
-  const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
-  const size_t S = (size_t)G.hstride;
-  const size_t e = (size_t)blockIdx.x * kWideThreads + threadIdx.x;
-  if (e >= (size_t)cnt * S) return;
-  const int n = list[e / S], h = (int)(e % S);
   if (h >= G.n_hands) return;
+  const bool both = h + 1 < G.n_hands;
+  const size_t S = (size_t)G.hstride;
   V* rch = static_cast<V*>(avg ? G.reach_bar : G.reach) + (size_t)p * G.n_nodes * S + h;
-  if (n == 0) {
-    rch[0] = static_cast<const V*>(G.range_v)[(size_t)p * S + h];
-    return;
+  V2<P> x;
+  if (w.src < 0) {
+    x = load2<V2<P>>(static_cast<const V*>(G.range_v) + (size_t)p * S + h);
+  } else {
+    x = load2<V2<P>>(rch + (size_t)w.src * S);
+    if (w.arow >= 0) {
+      const V2<P> s = load2<V2<P>>(static_cast<const V*>(avg ? G.sigbar : G.sigma) + (size_t)w.arow * S + h);
+      x.v[0] = P::mul(x.v[0], s.v[0]);
+      x.v[1] = P::mul(x.v[1], s.v[1]);
+    }
+    if (w.deal >= 0) {
+      if ((G.hand_mask[h] >> w.deal) & 1ull) x.v[0] = P::zero();
+      if (both && ((G.hand_mask[h + 1] >> w.deal) & 1ull)) x.v[1] = P::zero();
+    }
   }
-  const NodeDev nd = G.nodes[n];
-  V x = rch[(size_t)nd.parent * S];
-  if (nd.aplayer == p) x = P::mul(x, static_cast<const V*>(avg ? G.sigbar : G.sigma)[(size_t)nd.arow * S + h]);
-  if (nd.deal != kNoCard && ((G.hand_mask[h] >> nd.deal) & 1ull)) x = P::zero();
-  rch[(size_t)n * S] = x;
+  store2<P>(rch + (size_t)w.node * S, x, both);
 }
 
 // FP64 root sums of the best response, one block per player: sum_h r_p(h) v*_p(root, h),
@@ -3038,14 +3105,12 @@ static int launch_hand(const LaunchCtx& c, int player_mask, int advance, void* s
 
 // ---- wide schedule: a pass is a sequence of per-level launches (host loop over levels)
 
-static unsigned wide_blocks(size_t items) { return (unsigned)((items + kWideThreads - 1) / kWideThreads); }
-
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_wide(void (*kernel)(KArgs...), unsigned blocks, int players, void* stream, bool pdl,
+static cudaError_t launch_wide(void (*kernel)(KArgs...), unsigned blocks, int players, int threads, void* stream, bool pdl,
                                Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks, (unsigned)players);
-  cfg.blockDim = dim3(kWideThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -3058,27 +3123,32 @@ static cudaError_t launch_wide(void (*kernel)(KArgs...), unsigned blocks, int pl
 template <int MODE, typename P>
 static cudaError_t wide_backward(const LaunchCtx& c, int player_mask, void* stream) {
   const int players = player_mask == 3 ? 2 : 1;
-  const size_t S = (size_t)c.wide_stride;
   for (int l = c.wide_levels - 1; l >= 0; --l) {
     const int cnt = c.wide_inner_off[l + 1] - c.wide_inner_off[l];
     if (cnt == 0) continue;
     const cudaError_t e =
-        launch_wide(k_wide_back<MODE, P>, wide_blocks((size_t)cnt * S), players, stream, c.pdl != 0, c.games,
-                    c.wide_inner + c.wide_inner_off[l], cnt, player_mask, c.iter, c.disc, c.variant);
+        launch_wide(k_wide_back<MODE, P>, (unsigned)cnt * c.wide_segments, players, c.wide_threads, stream, c.pdl != 0,
+                    c.games, c.wide_inner + c.wide_inner_off[l], c.wide_segments, player_mask, c.iter, c.disc, c.variant);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
+// The nodes of depth d of the players in the mask that make new reach rows.
+static int wide_fwd_count(const LaunchCtx& c, int p, int d) {
+  return d < c.wide_fwd_levels[p] ? c.wide_fwd_off[p][d + 1] - c.wide_fwd_off[p][d] : 0;
+}
+
 template <typename P>
 static cudaError_t wide_forward(const LaunchCtx& c, int player_mask, int avg, int first_level, void* stream) {
   const int players = player_mask == 3 ? 2 : 1;
-  const size_t S = (size_t)c.wide_stride;
-  for (int l = first_level; l < c.wide_levels; ++l) {
-    const int a0 = c.wide_fwd_off[l], cnt = c.wide_fwd_off[l + 1] - a0;
+  for (int d = first_level; d < c.wide_fwd_levels[0] || d < c.wide_fwd_levels[1]; ++d) {
+    const int c0 = player_mask & 1 ? wide_fwd_count(c, 0, d) : 0, c1 = player_mask & 2 ? wide_fwd_count(c, 1, d) : 0;
+    const int cnt = c0 > c1 ? c0 : c1;
     if (cnt == 0) continue;
-    const cudaError_t e = launch_wide(k_wide_fwd<P>, wide_blocks((size_t)cnt * S), players, stream, c.pdl != 0,
-                                      c.games, c.wide_fwd + a0, cnt, player_mask, avg);
+    const cudaError_t e = launch_wide(k_wide_fwd<P>, (unsigned)cnt * c.wide_segments, players, c.wide_threads, stream,
+                                      c.pdl != 0, c.games, c.wide_fwd[0] + (c0 ? c.wide_fwd_off[0][d] : 0), c0,
+                                      c.wide_fwd[1] + (c1 ? c.wide_fwd_off[1][d] : 0), c1, c.wide_segments, player_mask, avg);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -3087,8 +3157,8 @@ static cudaError_t wide_forward(const LaunchCtx& c, int player_mask, int avg, in
 template <typename P>
 static cudaError_t wide_rows(const LaunchCtx& c, int avg, void* stream) {
   // rows of both players: the larger player's decision-node count sizes the grid
-  return launch_wide(k_wide_rows<P>, wide_blocks((size_t)c.wide_max_dec * c.wide_stride), 2, stream, c.pdl != 0,
-                     c.games, 3, avg);
+  return launch_wide(k_wide_rows<P>, (unsigned)c.wide_max_dec * c.wide_segments, 2, c.wide_threads, stream, c.pdl != 0,
+                     c.games, c.wide_segments, avg);
 }
 
 template <typename P>
@@ -3097,14 +3167,14 @@ static int wide_pass(const LaunchCtx& c, int which, int player_mask, int advance
   if (which == kModeUpdate) {
     e = wide_backward<kModeUpdate, P>(c, player_mask, stream);
     if (e == cudaSuccess) e = wide_forward<P>(c, player_mask, 0, 1, stream);
-    if (e == cudaSuccess && advance) e = launch_wide(k_wide_advance, 1, 1, stream, c.pdl != 0, c.iter);
+    if (e == cudaSuccess && advance) e = launch_wide(k_wide_advance, 1, 1, 1, stream, c.pdl != 0, c.iter);
   } else if (which == kModeInit || which == kModeAvg) {
     const int avg = which == kModeAvg;
     e = wide_rows<P>(c, avg, stream);
     if (e == cudaSuccess) e = wide_forward<P>(c, 3, avg, 0, stream);
   } else {  // kModeBR
     e = wide_backward<kModeBR, P>(c, 3, stream);
-    if (e == cudaSuccess) e = launch_wide(k_wide_root<P>, 2, 1, stream, c.pdl != 0, c.games);
+    if (e == cudaSuccess) e = launch_wide(k_wide_root<P>, 2, 1, kWideThreads, stream, c.pdl != 0, c.games);
   }
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of a wide-schedule kernel failed: %s\n", cudaGetErrorString(e));
@@ -3120,12 +3190,10 @@ static int launch_wide_pass(const LaunchCtx& c, int which, int player_mask, int 
 
 int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advance) {
   int back = 0, fwd = 0;
-  for (int l = 0; l < c.wide_levels; ++l) {
-    back += c.wide_inner_off[l + 1] > c.wide_inner_off[l];
-    fwd += c.wide_fwd_off[l + 1] > c.wide_fwd_off[l];
-  }
-  (void)player_mask;
-  if (which == kModeUpdate) return back + (fwd - 1) + (advance ? 1 : 0);
+  for (int l = 0; l < c.wide_levels; ++l) back += c.wide_inner_off[l + 1] > c.wide_inner_off[l];
+  for (int d = which == kModeUpdate; d < c.wide_fwd_levels[0] || d < c.wide_fwd_levels[1]; ++d)
+    fwd += (player_mask & 1 && wide_fwd_count(c, 0, d)) || (player_mask & 2 && wide_fwd_count(c, 1, d));
+  if (which == kModeUpdate) return back + fwd + (advance ? 1 : 0);
   if (which == kModeInit || which == kModeAvg) return 1 + fwd;
   return back + 1;
 }

@@ -218,6 +218,22 @@ struct alignas(16) TermGroup {
 static_assert(sizeof(TermGroup) == 160, "TermGroup is 160 bytes");
 constexpr int kTermSegment = 16;  // groups a block of the grouped terminal launch walks at most
 
+// Wide schedule: an inner node, and a node that makes a new reach row of one player.
+struct alignas(16) WideNode {
+  uint32_t id;        // node | children << 24 | (player, or 2 for a chance node) << 30
+  int32_t first_kid;
+  int32_t row;        // decision: first row
+  int32_t src;        // decision: node whose reach row of its player stands for its own
+  __host__ __device__ int node() const { return (int)(id & 0xffffffu); }
+  __host__ __device__ int kids() const { return (int)(id >> 24 & 63u); }
+  __host__ __device__ int kind() const { return (int)(id >> 30); }
+};
+struct alignas(16) WideReach {
+  int32_t node, src;  // src: node whose row it derives from (-1: the root, from the range)
+  int32_t arow;       // row of the player's action that leads here, or -1
+  int32_t deal;       // dealt card, or -1
+};
+
 struct Work {
   int game;
   int unit;  // chunk index (per-hand passes) or node id (terminal pass)
@@ -243,6 +259,7 @@ struct LaunchCtx {
   const Work* term_segments;      // device [n_term_segments]: (first group, count), one block's
   int n_term_segments;
   const TermSrc* term_src;     // device [n_term_work]: reach rows of each terminal
+  const int32_t* reach_row[2]; // device [n_nodes] (run-out tables): HostGame::reach_row
   int* iter;                   // device: iterations completed
   unsigned* done;              // device: block arrival counter
   int* err;                    // device: nonzero after a bounded wait gave up
@@ -269,14 +286,16 @@ struct LaunchCtx {
   int stream_units;            // load descriptors staged per block (0 when the program is not)
   int stream_hp;               // hands per lane of the stream schedule (1 or 2): a warp owns 32 * stream_hp
   // wide schedule (one game): level l's inner nodes are wide_inner[wide_inner_off[l] ..
-  // wide_inner_off[l + 1]), the nodes whose reach is stored wide_fwd[wide_fwd_off[l] ..
-  // wide_fwd_off[l + 1]) (all but the run-out nodes that read their source's reach)
+  // wide_inner_off[l + 1]); per player, the nodes that make new reach rows at depth d (0: the root) are
+  // wide_fwd[p][wide_fwd_off[p][d] .. wide_fwd_off[p][d + 1])
   int wide_levels;             // number of levels
   const int* wide_inner_off;   // host [wide_levels + 1]
-  const int32_t* wide_inner;   // device: inner node ids, level by level
-  const int* wide_fwd_off;     // host [wide_levels + 1]
-  const int32_t* wide_fwd;     // device: node ids, level by level
-  int wide_stride;             // hstride of the game
+  const WideNode* wide_inner;  // device, level by level
+  int wide_fwd_levels[2];
+  const int* wide_fwd_off[2];  // host [wide_fwd_levels + 1]
+  const WideReach* wide_fwd[2];  // device
+  int wide_segments;           // blocks per node, and
+  int wide_threads;            // threads of each (two hands a thread)
   int wide_max_dec;            // decision nodes of the player who has more
   // resident schedule (cfr_iterate only; the other passes use the level schedule's kernels)
   int resident;                // cfr_iterate runs k_resident

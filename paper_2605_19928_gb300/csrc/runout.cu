@@ -130,14 +130,15 @@ __device__ __forceinline__ void runout_step(const Row4<T>& row, const ulonglong2
 template <typename T, int kTops>
 __device__ __forceinline__ void runout_tops(const GameDev& G, const RunoutItem* __restrict__ items, int count,
                                             const T* __restrict__ table, int h0, const float* __restrict__ reach,
-                                            float* __restrict__ out, ulonglong2* qs) {
+                                            const int32_t* __restrict__ reach_row, float* __restrict__ out,
+                                            ulonglong2* qs) {
   const int H = G.n_hands, tid = threadIdx.x;
   const size_t S = (size_t)G.hstride;
   const uint32_t ld = (uint32_t)S;
   uint32_t at = h0 < H ? (uint32_t)h0 : 0u;  // a thread past the hands computes hand 0's and drops them
   const float* src[kTops];
 #pragma unroll
-  for (int g = 0; g < kTops; ++g) src[g] = reach + (size_t)items[g < count ? g : 0].node * S;
+  for (int g = 0; g < kTops; ++g) src[g] = reach + (size_t)reach_row[items[g < count ? g : 0].node] * S;
   f32x2 acc[kTops][2];
 #pragma unroll
   for (int g = 0; g < kTops; ++g) acc[g][0] = acc[g][1] = 0ull;
@@ -206,7 +207,9 @@ __global__ void __launch_bounds__(kValueThreads) k_runout_values(const GameDev* 
                                                                  const RunoutGroup* __restrict__ groups8,
                                                                  const RunoutGroup* __restrict__ groups16, int n16,
                                                                  const RunoutTable* __restrict__ tables,
-                                                                 const unsigned char* __restrict__ pool, int hand_blocks,
+                                                                 const unsigned char* __restrict__ pool,
+                                                                 const int32_t* __restrict__ row0,
+                                                                 const int32_t* __restrict__ row1, int hand_blocks,
                                                                  int player_mask, int use_bar) {
   __shared__ __align__(16) ulonglong2 qs[2 * kChunk * kTops8 / 2];
   const GameDev& G = games[0];
@@ -223,12 +226,12 @@ __global__ void __launch_bounds__(kValueThreads) k_runout_values(const GameDev* 
     const int first = (b % kSubs16) * kTops16, count = min(gr.count - first, kTops16);
     if (count > 0)
       runout_tops<uint16_t, kTops16>(G, items + gr.item0 + first, count,
-                                     reinterpret_cast<const uint16_t*>(pool + tables[gr.table].offset), h0, reach, out, qs);
+                                     reinterpret_cast<const uint16_t*>(pool + tables[gr.table].offset), h0, reach, i ? row0 : row1, out, qs);
   } else {
     b -= blocks16;
     const int h0 = 4 * ((b % hand_blocks) * kValueThreads + (int)threadIdx.x);
     const RunoutGroup gr = groups8[b / hand_blocks];
-    runout_tops<uint8_t, kTops8>(G, items + gr.item0, gr.count, pool + tables[gr.table].offset, h0, reach, out, qs);
+    runout_tops<uint8_t, kTops8>(G, items + gr.item0, gr.count, pool + tables[gr.table].offset, h0, reach, i ? row0 : row1, out, qs);
   }
 }
 
@@ -245,12 +248,13 @@ int launch_runout_build(const RunoutTable* tables, int n_tables, const RunoutBoa
 
 int launch_runout_values(const GameDev* games, const RunoutItem* items, const RunoutGroup* groups8, int n8,
                          const RunoutGroup* groups16, int n16, const RunoutTable* tables, const unsigned char* pool,
-                         int n_hands, int player_mask, int use_bar, void* stream) {
+                         const int32_t* row0, const int32_t* row1, int n_hands, int player_mask, int use_bar,
+                         void* stream) {
   if (n8 + n16 == 0) return 0;
   const int hand_blocks = (n_hands + 4 * kValueThreads - 1) / (4 * kValueThreads);
   const dim3 grid((unsigned)((n16 * kSubs16 + n8) * hand_blocks), player_mask == 3 ? 2u : 1u);
   k_runout_values<<<grid, kValueThreads, 0, (cudaStream_t)stream>>>(games, items, groups8, groups16, n16, tables, pool,
-                                                                   hand_blocks, player_mask, use_bar);
+                                                                   row0, row1, hand_blocks, player_mask, use_bar);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -56,9 +56,11 @@ int launch_runout_build(const RunoutTable* tables, int n_tables, const RunoutBoa
 // Values of the players in player_mask (1, 2 or 3) at every run-out top node of game 0, from
 // the opponent's reach (use_bar: the average-strategy reach, into cfv_br), FP32 values.  The
 // groups8 use uint8 tables, groups16 uint16 ones; items are the top nodes, sorted by table.
-// One launch (none without groups).
+// row0 / row1: per player, the node whose reach row stands for each node's.  One launch (none without
+// groups).
 int launch_runout_values(const GameDev* games, const RunoutItem* items, const RunoutGroup* groups8, int n8,
                          const RunoutGroup* groups16, int n16, const RunoutTable* tables, const unsigned char* pool,
-                         int n_hands, int player_mask, int use_bar, void* stream);
+                         const int32_t* row0, const int32_t* row1, int n_hands, int player_mask, int use_bar,
+                         void* stream);
 
 }  // namespace pcfr
