@@ -94,6 +94,7 @@ struct cfr_tree {
   std::vector<LeafDev> leaf_host;
   std::vector<int> leaf_col;    // network column of each card-pair slot (hand order, or the slot)
   bool leaf_net_set = false;
+  bool leaf_half = false;         // iterations have computed one player's network outputs at a time
   int64_t launches = 0;         // kernels launched (graph replays included)
   int64_t device_bytes = 0;
   int64_t h2d_bytes = 0;
@@ -1057,13 +1058,14 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
 }
 
 // Depth-limit leaves (Stage 5): network inputs from both players' reach at the leaves, the
-// four dense layers, then the leaf values of player 0, player 1 or both (mask 1, 2, 3).
+// four dense layers (the last for those players' outputs only), then the leaf values of player 0,
+// player 1 or both (mask 1, 2, 3).
 // Launches 1 + 4 + (1 or 2) kernels; none without leaves.
 int enqueue_leaves(cfr_tree* t, int player_mask, int use_bar, cudaStream_t s) {
   const LeafCtx& L = t->leaf;
   if (L.n_leaves == 0) return 0;
   const LaunchCtx& c = t->ctx;
-  if (launch_leaf_inputs(c, L, use_bar, s) || launch_leaf_net(c, L, s)) return -1;
+  if (launch_leaf_inputs(c, L, use_bar, s) || launch_leaf_net(c, L, player_mask, s)) return -1;
   for (int p = 0; p < 2; ++p)
     if (((player_mask >> p) & 1) && launch_leaf_values(c, L, p, use_bar, s)) return -1;
   return 0;
@@ -1167,6 +1169,7 @@ int cfr_iterate(cfr_tree* t, int n_iters) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
   }
   t->state_gen += 1;
+  if (t->leaf.n_leaves > 0 && t->opts.alternating) t->leaf_half = true;
   if (t->ctx.resident) {  // one cooperative launch per 2^20 iterations (its barrier count stays in 32 bits)
     for (int done = 0; done < n_iters; done += 1 << 20) {
       const int n = std::min(n_iters - done, 1 << 20);
@@ -1569,6 +1572,10 @@ int cfr_read_leaf_rows(cfr_tree* t, int what, int row0, int n_rows, void* out) {
   std::vector<unsigned char> raw((size_t)n_rows * width * es);
   const unsigned char* src = what == 0 ? static_cast<const unsigned char*>(t->leaf.X)
                                        : reinterpret_cast<const unsigned char*>(t->leaf.Y);
+  if (what == 1 && t->leaf_half && n_rows) {  // both players' outputs, from the last evaluation's hidden rows
+    if (launch_leaf_outputs(t->ctx, t->leaf, 3, t->stream) != 0) return fail(CFR_ECUDA, "leaf launch failed");
+    t->launches += 1;
+  }
   if (n_rows)
     CK(cudaMemcpyAsync(raw.data(), src + (size_t)row0 * width * es, raw.size(), cudaMemcpyDeviceToHost, t->stream));
   CK(cudaStreamSynchronize(t->stream));

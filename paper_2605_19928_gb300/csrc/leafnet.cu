@@ -2,19 +2,21 @@
 // Section 4.3): C = act(A B^T + bias) with A the [M][K] BF16 activations, B the [N][K] BF16
 // weights (both K-major), FP32 accumulation on the 5th-generation tensor cores.
 //
-// A persistent kernel, one CTA per SM, walks 128 x BN tiles of C (BN = 256, 192 or 128,
-// the largest that divides N; the N tiles of one block of rows are consecutive so that the
-// CTAs reading that block of A run together and share it through L2):
-//   * one lane of warp 0 streams 128 x 64 tiles of A and BN x 64 tiles of B into a 4-stage
-//     ring of shared memory with TMA (128-byte swizzle, the layout the MMA descriptors below
-//     describe);
-//   * one lane of warp 1 issues tcgen05.mma (M 128, N BN, K 16 per instruction, four per
-//     64-wide stage) into one of two TMEM accumulators, commits each stage back to its
-//     "empty" barrier and each finished tile to its accumulator's "full" barrier;
-//   * eight warps each read half the columns of one 32-lane quarter of the finished
-//     accumulator with tcgen05.ld, add the bias, apply GELU (hidden layers), store BF16 (or
-//     FP32, staged in shared memory and written by bulk tensor stores) and hand the
-//     accumulator back, so a tile's epilogue runs while the next tile's MMAs fill the other.
+// A persistent kernel, one pair of CTAs (a cluster of two SMs) per 256 x BN tile of C at a time
+// (BN a multiple of 32 up to 256, see gemm_bn; the N tiles of one block of rows are consecutive so
+// that the pairs reading that block of A run together and share it through L2):
+//   * in each CTA one lane of warp 0 streams its 128 x 64 half of the tile's A rows and its BN / 2 x
+//     64 half of the tile's B rows into a ring of shared memory with TMA (128-byte swizzle, the
+//     layout the MMA descriptors below describe); both CTAs' copies count at the first CTA's
+//     "full" barriers;
+//   * in the first CTA one lane of warp 1 issues tcgen05.mma for the pair (cta_group::2: M 256, N
+//     BN, K 16 per instruction, four per 64-wide stage) into one of two TMEM accumulators, each
+//     CTA's TMEM holding its own 128 rows, commits each stage back to both CTAs' "empty"
+//     barriers and each finished tile to both CTAs' "full accumulator" barriers;
+//   * in each CTA eight warps each take every other 32-column block of one 32-lane quarter of the
+//     finished accumulator with tcgen05.ld, add the bias, apply GELU (hidden layers), stage the
+//     block in shared memory and write it by bulk tensor stores, two in flight a warp; then they
+//     hand the accumulator back, so a tile's epilogue runs while the next tile's MMAs fill the other.
 // Every mbarrier wait is bounded; a wait that gives up sets *err, the CTA stops issuing,
 // waits for the copies and MMAs it has in flight and frees its TMEM.
 #include <cuda.h>
@@ -29,13 +31,14 @@ namespace pcfr {
 
 namespace {
 
-constexpr int kBM = 128, kBK = 64, kStages = 4, kBNMax = 256;
-constexpr int kATile = kBM * kBK * 2;        // 16 KB: one A stage
-constexpr int kBTileMax = kBNMax * kBK * 2;  // 32 KB: one B stage of the widest tile
-constexpr int kEpiWarps = 8;                 // two per TMEM lane quarter, each half the columns
-constexpr int kStageBufs = 8 / kEpiWarps;    // 4 KB output staging blocks per epilogue warp (32 KB in all)
+constexpr int kBM = 128, kBK = 64, kBNMax = 256;  // rows of C per CTA, a pair's tile has 2 kBM
+constexpr int kATile = kBM * kBK * 2;            // 16 KB: one A stage
+constexpr int kRingBytes = 160 * 1024;           // stages of A and B: 5 of the widest tile's 32 KB
+constexpr int kMaxStages = 8;
+constexpr int kEpiWarps = 8;                     // two per TMEM lane quarter
+constexpr int kStageBufs = 2, kStageBuf = 4096;  // output staging blocks per epilogue warp
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, then the epilogue warps
-constexpr int kTmemCols = 512;               // two accumulators of up to 256 columns
+constexpr int kTmemCols = 512;                   // two accumulators of up to 256 columns
 constexpr long kGemmWaitLimit = 1l << 22;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -61,12 +64,32 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
     if (bar_try_wait(bar, parity)) return true;
   return false;
 }
+// The same for a barrier at which the other CTA's threads arrive.
+__device__ __forceinline__ bool bar_wait_cluster(uint64_t* bar, uint32_t parity) {
+  for (long k = 0; k < kGemmWaitLimit; ++k) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+// The address of the pair's first CTA's copy of a shared variable.
+__device__ __forceinline__ uint32_t of_first_cta(const void* p) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_addr(p)));
+  return a;
+}
+// One box into this CTA's shared memory, counted at the barrier `bar` of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], "
+      "[%4];" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
 
@@ -85,30 +108,43 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
 }
 
 // Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, both K-major, N = bn,
-// M = kBM.
+// M = 2 kBM (the pair's).
 __host__ __device__ constexpr uint32_t instr_desc(int bn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(2 * kBM >> 4) << 24);
 }
 
+// The pair's MMA: descriptors and TMEM address are offsets that both CTAs apply to their own memory.
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// One arrival at this CTA's barrier, or at the same barrier of both CTAs, when the MMAs so far are done.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
                : "memory");
+}
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_addr(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 
-__device__ __forceinline__ uint16_t to_bf16(float x) {  // round to nearest even (finite inputs)
-  uint32_t u = __float_as_uint(x);
-  u += 0x7fffu + ((u >> 16) & 1u);
-  return (uint16_t)(u >> 16);
+// Two floats to BF16 (round to nearest even), lo in the low half.
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
 }
 
 // Hint: bring one box of the tensor into L2 (no shared memory, no barrier; a box past the
@@ -128,195 +164,226 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-__device__ __forceinline__ void bar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+// 32 columns of this warp's 32 accumulator lanes, one lane a thread; the values are there after
+// tmem_wait (which names them, so that their uses stay behind it).
+__device__ __forceinline__ void tmem_load(uint32_t (&v)[32], uint32_t addr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(addr));
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+               :
+               : "memory");
+}
+// One arrival at the barrier `bar` of either CTA of the pair.
+__device__ __forceinline__ void bar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
+// Columns [n_begin, n_begin + n_nt bn) of C.  A pair's tile needs 32 KB of A and B per CTA for the MMAs
+// that take 48 KB as a 128 x 256 tile of one CTA.  The MMAs alone, without loads and epilogue, take
+// 89 us on 49,392 rows of layer 1 (six rounds of tiles where 5.1 would do); the epilogue's GELU and
+// the loads behind it make that 118 us (115 as one-CTA tiles).  The 512-wide layers of K = 512 are bound
+// by GELU's instructions: 60 -> 50 us at 49,392 rows.  The output layer is bound by its FP32 stores
+// (12,528 rows: 43.2 -> 39.1 us) and, in an update of one player, computes that player's half.  A
+// turn's 624 rows spread over narrow tiles: 24.2 -> 19.5 us (layer 1), 14.0 -> 8.5 (512 x 512).
+template <bool F32, bool ACT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                const __grid_constant__ CUtensorMap map_c, const float* __restrict__ bias, void* __restrict__ out,
-                int M, int N, int K, int bn, int act, int out_f32, int* err) {
-  extern __shared__ __align__(1024) unsigned char smg[];
-  // 1024-byte aligned stage buffers: A stages, then B stages
+                const __grid_constant__ CUtensorMap map_c, const float* __restrict__ bias, int M, int n_begin, int n_nt,
+                int kb_count, int bn, int stages, int* err) {
+  extern __shared__ __align__(128) unsigned char smg[];
+  // 1024-byte aligned: the ring (A then B of each stage), the epilogue's staging blocks, its bias rows
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smg) + 1023) & ~(uintptr_t)1023);
-  unsigned char* sa = base;
-  unsigned char* sb = base + kStages * kATile;
-  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], mma_done;
+  __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], mma_done;
   __shared__ uint32_t tmem_base;
-  __shared__ volatile int failed;  // set by any role whose bounded wait gave up; the others poll it
+  __shared__ volatile int failed;  // set by any role whose bounded wait gave up; the CTA's others poll it
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_nt = N / bn, n_tiles = n_nt * ((M + kBM - 1) / kBM), kb_count = K / kBK;
-  const uint32_t b_bytes = (uint32_t)bn * kBK * 2;
+  const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  const int n_tiles = n_nt * ((M + 2 * kBM - 1) / (2 * kBM));
+  const uint32_t stage_bytes = kATile + (uint32_t)bn / 2 * kBK * 2;  // multiples of 1024
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < stages; ++s) {
       bar_init(&full[s], 1);
       bar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
-      bar_init(&acc_full[b], 1);   // one tcgen05.commit per finished tile
-      bar_init(&acc_empty[b], kEpiWarps);  // one arrival per epilogue warp
+      bar_init(&acc_full[b], 1);               // one tcgen05.commit per finished tile
+      bar_init(&acc_empty[b], 2 * kEpiWarps);  // one arrival per epilogue warp of the pair
     }
     bar_init(&mma_done, 1);
     failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
                  "r"(kTmemCols)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  cluster_sync();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_base;
+  const uint32_t tmem = tmem_base;  // all of TMEM: the same address in both CTAs
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer
-      int it = 0;
-      for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
-        const int m0 = (tile / n_nt) * kBM, n0 = (tile % n_nt) * bn;
-        const int next = tile + (int)gridDim.x, m0_next = (next / n_nt) * kBM;
+      int s = 0, round = 0, it = 0;
+      for (int tile = pair; tile < n_tiles && !failed; tile += pairs) {
+        const int m0 = (tile / n_nt) * 2 * kBM + rank * kBM, n0 = n_begin + (tile % n_nt) * bn + rank * (bn / 2);
+        const int next = tile + pairs, m0_next = (next / n_nt) * 2 * kBM + rank * kBM;
         for (int kb = 0; kb < kb_count; ++kb, ++it) {
-          const int s = it % kStages;
-          // the A box a full ring ahead (into the CTA's next tile near the end) goes to L2
+          // the A box a full ring ahead (into the pair's next tile near the end) goes to L2
           // now, so that its load, issued when a stage frees up, waits on L2 rather than DRAM
-          if (kb + kStages < kb_count)
-            tma_prefetch_2d(&map_a, (kb + kStages) * kBK, m0);
-          else if (next < n_tiles && kb + kStages - kb_count < kb_count)
-            tma_prefetch_2d(&map_a, (kb + kStages - kb_count) * kBK, m0_next);
-          if (!bar_wait(&empty[s], ((uint32_t)(it / kStages) & 1u) ^ 1u)) {
+          if (kb + stages < kb_count)
+            tma_prefetch_2d(&map_a, (kb + stages) * kBK, m0);
+          else if (next < n_tiles && kb + stages - kb_count < kb_count)
+            tma_prefetch_2d(&map_a, (kb + stages - kb_count) * kBK, m0_next);
+          if (!bar_wait(&empty[s], ((uint32_t)round & 1u) ^ 1u)) {
             failed = 1;
             break;
           }
-          bar_expect_tx(&full[s], kATile + b_bytes);
-          tma_load_2d(sa + s * kATile, &map_a, kb * kBK, m0, &full[s]);
-          tma_load_2d(sb + s * kBTileMax, &map_b, kb * kBK, n0, &full[s]);
+          unsigned char* sa = base + s * stage_bytes;
+          if (rank == 0) bar_expect_tx(&full[s], 2 * stage_bytes);
+          const uint32_t bar = of_first_cta(&full[s]);
+          tma_load_2d(sa, &map_a, kb * kBK, m0, bar);
+          tma_load_2d(sa + kATile, &map_b, kb * kBK, n0, bar);
+          if (++s == stages) s = 0, ++round;
         }
       }
-      // the copies of the last round of each stage have landed before the CTA can leave
-      for (int j = it - 1; j >= 0 && j >= it - kStages; --j) bar_wait(&full[j % kStages], (uint32_t)(j / kStages) & 1u);
+      // both CTAs' copies of the last round of each stage have landed before the pair leaves (its
+      // second CTA waits for the first at the end)
+      if (rank == 0)
+        for (int j = it - 1; j >= 0 && j >= it - stages; --j) bar_wait(&full[j % stages], (uint32_t)(j / stages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {  // MMA issuer
+    if (lane == 0 && rank == 0) {  // MMA issuer of the pair
       const uint32_t idesc = instr_desc(bn);
-      int it = 0, lt = 0;
-      for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x, ++lt) {
+      int s = 0, round = 0, lt = 0;
+      for (int tile = pair; tile < n_tiles && !failed; tile += pairs, ++lt) {
         const int acc = lt & 1;
-        if (!bar_wait(&acc_empty[acc], ((uint32_t)(lt >> 1) & 1u) ^ 1u)) {  // the epilogue has drained it
+        if (!bar_wait_cluster(&acc_empty[acc], ((uint32_t)(lt >> 1) & 1u) ^ 1u)) {  // the epilogues have drained it
           failed = 1;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem + (uint32_t)(acc * kBNMax);
         bool ok = true;
-        for (int kb = 0; kb < kb_count; ++kb, ++it) {
-          const int s = it % kStages;
-          if (!bar_wait(&full[s], (uint32_t)(it / kStages) & 1u)) {
+        for (int kb = 0; kb < kb_count; ++kb) {
+          if (!bar_wait(&full[s], (uint32_t)round & 1u)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_addr(sa + s * kATile), b0 = smem_addr(sb + s * kBTileMax);
+          const uint32_t a0 = smem_addr(base + s * stage_bytes), b0 = a0 + kATile;
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)
             mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(&empty[s]);  // the stage is free once these MMAs have read it
+          mma_commit_pair(&empty[s]);  // the stage is free once these MMAs have read it
+          if (++s == stages) s = 0, ++round;
         }
         if (!ok) {
           failed = 1;
           break;
         }
-        mma_commit(&acc_full[acc]);  // the tile's accumulator is complete
+        mma_commit_pair(&acc_full[acc]);  // the tile's accumulator is complete
       }
       mma_commit(&mma_done);  // every MMA issued above has completed
       bar_wait(&mma_done, 0);
     }
     __syncwarp();
-  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, columns of part
-            // (w - 2) / 4 of the tile
-    constexpr int parts = kEpiWarps / 4;  // warps per lane quarter, each a share of the columns
-    const int q = warp & 3, part = (warp - 2) >> 2;
-    const int c_begin = part * (bn / parts), c_end = c_begin + bn / parts;
-    // FP32 output: 32 x 32 staging blocks in the TMA store's 128-byte-swizzled layout
-    // (16-byte chunk j of row r at chunk j ^ (r % 8)), each written by the warp and stored by
-    // one bulk tensor copy
-    unsigned char* stage = sb + kStages * kBTileMax + (size_t)(warp - 2) * kStageBufs * 4096;
-    int cc = 0;  // 32-column blocks this warp has staged
+  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, every other 32-column
+            // block, from its part (w - 2) / 4 on (the parts take turns to start, as the count may be odd)
+    const int q = warp & 3, part = (warp - 2) >> 2, blocks = bn / 32;
+    // staging blocks of 32 rows x 32 columns in the bulk store's swizzled layout: 16-byte chunk j of row
+    // r at chunk j ^ (r % 8) (FP32, 128-byte rows) or j ^ (r / 2 % 4) (BF16, 64-byte rows)
+    unsigned char* stage = base + kRingBytes + (size_t)(warp - 2) * kStageBufs * kStageBuf;
+    float* sbias = reinterpret_cast<float*>(base + kRingBytes + kEpiWarps * kStageBufs * kStageBuf) + (warp - 2) * 32;
+    int cc = 0;  // blocks this warp has staged
     int lt = 0;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++lt) {
+    // one block: its values v and bias (lane's column) to the staging block, and from there to C
+    auto put = [&](const uint32_t (&v)[32], float bias_lane, int col, int row) {
+      unsigned char* buf = stage + (cc & 1) * kStageBuf;
+      if (cc >= kStageBufs && lane == 0)  // the store that last read this block has finished reading it
+        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      __syncwarp();  // (and the last block's bias has been read)
+      sbias[lane] = bias_lane;
+      __syncwarp();
+      constexpr int per = F32 ? 4 : 8;  // values of a 16-byte chunk
+#pragma unroll
+      for (int j = 0; j < 32 / per; ++j) {
+        float y[per];
+#pragma unroll
+        for (int e = 0; e < per; e += 4) {
+          const float4 bv = *reinterpret_cast<const float4*>(sbias + per * j + e);
+          y[e] = __uint_as_float(v[per * j + e]) + bv.x;
+          y[e + 1] = __uint_as_float(v[per * j + e + 1]) + bv.y;
+          y[e + 2] = __uint_as_float(v[per * j + e + 2]) + bv.z;
+          y[e + 3] = __uint_as_float(v[per * j + e + 3]) + bv.w;
+        }
+        if (ACT) {
+#pragma unroll
+          for (int e = 0; e < per; ++e) y[e] = gelu(y[e]);
+        }
+        if constexpr (F32)
+          *reinterpret_cast<float4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(y[0], y[1], y[2], y[3]);
+        else
+          *reinterpret_cast<uint4*>(buf + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+              make_uint4(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]), pack_bf16x2(y[4], y[5]), pack_bf16x2(y[6], y[7]));
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the bulk copy
+      __syncwarp();
+      if (lane == 0) tma_store_2d(&map_c, col, row, buf);  // rows past M are clipped
+      ++cc;
+    };
+    for (int tile = pair; tile < n_tiles; tile += pairs, ++lt) {
       const int acc = lt & 1;
+      const int row0 = (tile / n_nt) * 2 * kBM + rank * kBM + q * 32, n0 = n_begin + (tile % n_nt) * bn;
+      const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBNMax);
+      const int last = row0 < M ? blocks : 0;
+      int b = (part + lt) & 1;
+      // a block's bias and accumulator values are asked for before the block in front of it is worked on
+      auto bias_at = [&](int blk) { return bias && blk < last ? __ldg(bias + n0 + blk * 32 + lane) : 0.f; };
+      float b0 = bias_at(b), b1;
       const bool ok = bar_wait(&acc_full[acc], (uint32_t)(lt >> 1) & 1u);
       if (!__all_sync(0xffffffffu, ok) || failed) {
         if (lane == 0) failed = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int m0 = (tile / n_nt) * kBM, n0 = (tile % n_nt) * bn;
-      const int row = m0 + q * 32 + lane;
-      for (int c0 = c_begin; c0 < c_end; c0 += 32) {
-        uint32_t v[32];
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBNMax + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-            "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-              "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int col = n0 + c0;
-        if (out_f32) {
-          unsigned char* buf = stage + (cc % kStageBufs) * 4096;
-          if (cc >= kStageBufs) {  // the store that last read this block has finished reading it
-            if (lane == 0) {
-              if (kStageBufs == 2)
-                asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-              else
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            }
-            __syncwarp();
-          }
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            float y[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              y[e] = __uint_as_float(v[4 * j + e]) + (bias ? bias[col + 4 * j + e] : 0.f);
-              if (act) y[e] = gelu(y[e]);
-            }
-            *reinterpret_cast<float4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(y[0], y[1], y[2], y[3]);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the bulk copy
-          __syncwarp();
-          if (lane == 0) tma_store_2d(&map_c, col, m0 + q * 32, buf);  // rows past M are clipped
-          ++cc;
-        } else if (row < M) {
-          float y[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            y[j] = __uint_as_float(v[j]) + (bias ? bias[col + j] : 0.f);
-            if (act) y[j] = gelu(y[j]);
-          }
-          {
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(out) + (size_t)row * N + col);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              uint32_t w[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                w[e] = (uint32_t)to_bf16(y[8 * j + 2 * e]) | ((uint32_t)to_bf16(y[8 * j + 2 * e + 1]) << 16);
-              dst[j] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-          }
-        }
+      auto drained = [&] {  // this warp's part of the accumulator is in registers: it is free
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) bar_arrive_cluster(of_first_cta(&acc_empty[acc]));
+      };
+      uint32_t v0[32], v1[32];
+      if (b < last) tmem_load(v0, taddr + (uint32_t)(b * 32));
+      while (b + 2 < last) {
+        tmem_wait(v0);
+        tmem_load(v1, taddr + (uint32_t)(b * 32 + 64));
+        b1 = bias_at(b + 2);
+        put(v0, b0, n0 + b * 32, row0);
+        tmem_wait(v1);
+        if (b + 4 < last) tmem_load(v0, taddr + (uint32_t)(b * 32 + 128));
+        else drained();
+        b0 = bias_at(b + 4);
+        put(v1, b1, n0 + b * 32 + 64, row0);
+        b += 4;
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) bar_arrive(&acc_empty[acc]);  // this quarter of the accumulator is free
+      if (b < last) {  // an odd last block
+        tmem_wait(v0);
+        drained();
+        put(v0, b0, n0 + b * 32, row0);
+      } else if (last <= ((part + lt) & 1)) {  // none at all
+        drained();
+      }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // every store has completed
     __syncwarp();
@@ -324,9 +391,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (failed && threadIdx.x == 0) atomicExch(err, 1);
+  cluster_sync();  // neither CTA leaves while the other may still signal its barriers
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
@@ -348,18 +416,18 @@ EncodeTiled encoder() {
   return fn;
 }
 
-// Row-major [rows][cols] FP32 matrix, 32 x 32 boxes with 128-byte swizzle (the epilogue's
-// bulk stores).
-bool encode_out_f32(CUtensorMap* map, void* ptr, int rows, int cols) {
+// Row-major [rows][cols] FP32 or BF16 matrix, 32 x 32 boxes with a swizzle of a box row's width
+// (the epilogue's bulk stores).
+bool encode_out(CUtensorMap* map, void* ptr, int rows, int cols, int f32) {
   EncodeTiled fn = encoder();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+  const cuuint64_t strides[1] = {(cuuint64_t)cols * (f32 ? 4 : 2)};
   const cuuint32_t box[2] = {32, 32};
   const cuuint32_t estr[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-         CUDA_SUCCESS;
+  return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Row-major [rows][cols] BF16 matrix, box_rows x 64 boxes with 128-byte swizzle.
@@ -377,39 +445,65 @@ bool encode(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows)
 
 }  // namespace
 
-// stages of A and B, the epilogue warps' 4 KB output staging blocks, alignment slack
-size_t gemm_smem_bytes() { return (size_t)kStages * (kATile + kBTileMax) + kEpiWarps * kStageBufs * 4096 + 1024; }
+// the ring, the epilogue warps' staging blocks and bias rows, alignment slack
+size_t gemm_smem_bytes() { return (size_t)kRingBytes + kEpiWarps * (kStageBufs * kStageBuf + 128) + 1024; }
 
 int configure_gemm() {
-  return cudaFuncSetAttribute(k_gemm_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem_bytes()) ==
-                 cudaSuccess
-             ? 0
-             : -1;
+  const int smem = (int)gemm_smem_bytes();
+  for (auto k : {k_gemm_bf16<false, false>, k_gemm_bf16<false, true>, k_gemm_bf16<true, false>, k_gemm_bf16<true, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return -1;
+  return 0;
 }
 
-int launch_gemm_bf16(const void* A, const void* B, const float* bias, void* C, int M, int N, int K, int act,
-                     int out_f32, int* err, void* stream) {
+// Width of the tiles of n columns: the one whose rounds of tiles over the pairs take least by this
+// count of cycles.  A tile's fill is its loads (256 + bn bytes of A and B a row of 64, at 64 bytes a
+// cycle) or its MMAs, its drain about 20 cycles a column; the last drain is not covered by a fill.
+// A few rows (a turn's 13 leaves have 624) thus spread over narrow tiles, many take 256-wide ones.
+static int gemm_bn(int M, int n, int kb_count, int pairs) {
+  int best = 0;
+  double best_cost = 0;
+  for (int bn = 32; bn <= kBNMax; bn += 32) {
+    if (n % bn) continue;
+    const long tiles = (long)(n / bn) * ((M + 2 * kBM - 1) / (2 * kBM)), rounds = (tiles + pairs - 1) / pairs;
+    const double fill = (double)kb_count * (256 + bn > 2 * bn ? 256 + bn : 2 * bn), drain = 20.0 * bn;
+    const double cost = (double)rounds * (fill > drain ? fill : drain) + drain;
+    if (best == 0 || cost < best_cost) best = bn, best_cost = cost;
+  }
+  return best;
+}
+
+// Columns [n_begin, n_begin + n_cols) of C (a multiple of 32 of them; n_begin a multiple of 8, of 4
+// with FP32 output: a bulk store starts on a 16-byte boundary).
+static int launch_gemm_cols(const void* A, const void* B, const float* bias, void* C, int M, int N, int K, int n_begin,
+                            int n_cols, int act, int out_f32, int* err, void* stream) {
   if (M <= 0 || N <= 0 || K <= 0 || N % 128 || K % kBK) return -2;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15) return -2;
-  const int bn = N % 256 == 0 ? 256 : N % 192 == 0 ? 192 : 128;  // the widest tile that divides N
-  const long tiles = (long)(N / bn) * ((M + kBM - 1) / kBM);
-  if (tiles > (1l << 30)) return -2;
-  CUtensorMap ma, mb, mc = {};
-  if (!encode(&ma, A, M, K, kBM) || !encode(&mb, B, N, K, bn)) return -3;
-  if (out_f32 && !encode_out_f32(&mc, C, M, N)) return -3;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 2)
     return -1;
-  const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);  // persistent: one CTA per SM
-  k_gemm_bf16<<<grid, kGemmThreads, gemm_smem_bytes(), (cudaStream_t)stream>>>(ma, mb, mc, bias, C, M, N, K, bn,
-                                                                               act, out_f32, err);
+  const int bn = gemm_bn(M, n_cols, K / kBK, sms / 2);
+  const long tiles = (long)(n_cols / bn) * ((M + 2 * kBM - 1) / (2 * kBM));
+  if (tiles > (1l << 29)) return -2;
+  CUtensorMap ma, mb, mc;
+  if (!encode(&ma, A, M, K, kBM) || !encode(&mb, B, N, K, bn / 2) || !encode_out(&mc, C, M, N, out_f32)) return -3;
+  const int pairs = (int)(tiles < sms / 2 ? tiles : sms / 2);  // persistent: one CTA per SM
+  const int stage = kATile + bn * kBK, stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
+  auto* kernel = out_f32 ? (act ? k_gemm_bf16<true, true> : k_gemm_bf16<true, false>)
+                         : (act ? k_gemm_bf16<false, true> : k_gemm_bf16<false, false>);
+  kernel<<<2 * pairs, kGemmThreads, gemm_smem_bytes(), (cudaStream_t)stream>>>(ma, mb, mc, bias, M, n_begin, n_cols / bn,
+                                                                               K / kBK, bn, stages, err);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_gemm_bf16 failed: %s\n", cudaGetErrorString(e));
     return -1;
   }
   return 0;
+}
+
+int launch_gemm_bf16(const void* A, const void* B, const float* bias, void* C, int M, int N, int K, int act,
+                     int out_f32, int* err, void* stream) {
+  return launch_gemm_cols(A, B, bias, C, M, N, K, 0, N, act, out_f32, err, stream);
 }
 
 // ------------------------------------------------------------------ leaf inputs and values
@@ -472,13 +566,6 @@ __device__ __forceinline__ int river_card(uint64_t board, int k) {
   for (int n = -1; c < 51; ++c)
     if (!((board >> c) & 1ull) && ++n == k) break;
   return c;
-}
-
-// Two floats to BF16 (round to nearest even), lo in the low half.
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  uint32_t d;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-  return d;
 }
 
 __device__ __forceinline__ float warp_sum_f32(float x) {
@@ -773,13 +860,24 @@ int launch_leaf_inputs(const LaunchCtx& c, const LeafCtx& L, int use_bar, void* 
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_leaf_net(const LaunchCtx& c, const LeafCtx& L, void* stream) {
+// The output layer's columns of each player: six 224-wide tiles that cover the player's 1326, player
+// 1's opening 18 columns early (16-byte aligned) so as to end with its last.
+constexpr int kLeafHalf = 1344, kLeafHalfBegin[2] = {0, 2 * kLeafSlots - kLeafHalf};
+static_assert(kLeafHalf >= kLeafSlots && kLeafHalfBegin[1] % 4 == 0 && kLeafHalf % 224 == 0, "a player's output columns");
+
+int launch_leaf_outputs(const LaunchCtx& c, const LeafCtx& L, int player_mask, void* stream) {
+  const int rows = L.n_leaves * kLeafCards;
+  const int begin = player_mask == 3 ? 0 : kLeafHalfBegin[player_mask - 1], cols = player_mask == 3 ? kLeafOut : kLeafHalf;
+  return launch_gemm_cols(L.H3, L.W[3], L.b[3], L.Y, rows, kLeafOut, kLeafHidden, begin, cols, 0, 1, c.err, stream) ? -1 : 0;
+}
+
+int launch_leaf_net(const LaunchCtx& c, const LeafCtx& L, int player_mask, void* stream) {
   if (L.n_leaves == 0) return 0;
   const int rows = L.n_leaves * kLeafCards;
   if (launch_gemm_bf16(L.X, L.W[0], L.b[0], L.H1, rows, kLeafHidden, kLeafIn, 1, 0, c.err, stream) ||
       launch_gemm_bf16(L.H1, L.W[1], L.b[1], L.H2, rows, kLeafHidden, kLeafHidden, 1, 0, c.err, stream) ||
       launch_gemm_bf16(L.H2, L.W[2], L.b[2], L.H3, rows, kLeafHidden, kLeafHidden, 1, 0, c.err, stream) ||
-      launch_gemm_bf16(L.H3, L.W[3], L.b[3], L.Y, rows, kLeafOut, kLeafHidden, 0, 1, c.err, stream))
+      launch_leaf_outputs(c, L, player_mask, stream))
     return -1;
   return 0;
 }

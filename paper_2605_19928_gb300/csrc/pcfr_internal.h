@@ -380,10 +380,12 @@ struct LeafCtx {
                            // read and write them coalesced; 0: slot order
 };
 
-// Leaf values of player i (use_bar: against the average strategy, into cfv_br) or, with
-// player -1, only the network (both players' inputs and the four layers).
+// The network's input rows (use_bar: of the average strategy), its four layers -- the last for the
+// outputs of player 0, player 1 or both (mask 1, 2, 3) -- and the leaf values of player i (use_bar:
+// into cfv_br).  launch_leaf_outputs is the last layer alone, from the hidden rows L.H3.
 int launch_leaf_inputs(const LaunchCtx& c, const LeafCtx& L, int use_bar, void* stream);
-int launch_leaf_net(const LaunchCtx& c, const LeafCtx& L, void* stream);
+int launch_leaf_net(const LaunchCtx& c, const LeafCtx& L, int player_mask, void* stream);
+int launch_leaf_outputs(const LaunchCtx& c, const LeafCtx& L, int player_mask, void* stream);
 int launch_leaf_values(const LaunchCtx& c, const LeafCtx& L, int player, int use_bar, void* stream);
 // Dynamic shared memory of one stream-schedule block: the staged program (prog_nodes nodes)
 // and one player's load descriptors (prog_units), and per lane a prefetch ring of 2 x half
