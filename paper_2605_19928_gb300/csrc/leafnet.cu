@@ -13,10 +13,10 @@
 //     BN, K 16 per instruction, four per 64-wide stage) into one of two TMEM accumulators, each
 //     CTA's TMEM holding its own 128 rows, commits each stage back to both CTAs' "empty"
 //     barriers and each finished tile to both CTAs' "full accumulator" barriers;
-//   * in each CTA eight warps each take every other 32-column block of one 32-lane quarter of the
+//   * in each CTA sixteen warps each take every fourth 32-column block of one 32-lane quarter of the
 //     finished accumulator with tcgen05.ld, add the bias, apply GELU (hidden layers), stage the
-//     block in shared memory and write it by bulk tensor stores, two in flight a warp; then they
-//     hand the accumulator back, so a tile's epilogue runs while the next tile's MMAs fill the other.
+//     block in shared memory and write it by bulk tensor stores; the accumulator is handed back as
+//     soon as it is in registers, so a tile's epilogue runs while the next tile's MMAs fill the other.
 // Every mbarrier wait is bounded; a wait that gives up sets *err, the CTA stops issuing,
 // waits for the copies and MMAs it has in flight and frees its TMEM.
 #include <cuda.h>
@@ -35,8 +35,9 @@ constexpr int kBM = 128, kBK = 64, kBNMax = 256;  // rows of C per CTA, a pair's
 constexpr int kATile = kBM * kBK * 2;            // 16 KB: one A stage
 constexpr int kRingBytes = 160 * 1024;           // stages of A and B: 5 of the widest tile's 32 KB
 constexpr int kMaxStages = 8;
-constexpr int kEpiWarps = 8;                     // two per TMEM lane quarter
-constexpr int kStageBufs = 2, kStageBuf = 4096;  // output staging blocks per epilogue warp
+constexpr int kEpiWarps = 16;                    // four per TMEM lane quarter
+constexpr int kEpiParts = kEpiWarps / 4;
+constexpr int kStageBytes = 4096;                // output staging per epilogue warp: one FP32 block, two BF16 blocks
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, then the epilogue warps
 constexpr int kTmemCols = 512;                   // two accumulators of up to 256 columns
 constexpr long kGemmWaitLimit = 1l << 22;
@@ -186,19 +187,20 @@ __device__ __forceinline__ void bar_arrive_cluster(uint32_t bar) {
 
 // Columns [n_begin, n_begin + n_nt bn) of C.  A pair's tile needs 32 KB of A and B per CTA for the MMAs
 // that take 48 KB as a 128 x 256 tile of one CTA.  The MMAs alone, without loads and epilogue, take
-// 89 us on 49,392 rows of layer 1 (six rounds of tiles where 5.1 would do); the epilogue's GELU and
-// the loads behind it make that 118 us (115 as one-CTA tiles).  The 512-wide layers of K = 512 are bound
-// by GELU's instructions: 60 -> 50 us at 49,392 rows.  The output layer is bound by its FP32 stores
-// (12,528 rows: 43.2 -> 39.1 us) and, in an update of one player, computes that player's half.  A
-// turn's 624 rows spread over narrow tiles: 24.2 -> 19.5 us (layer 1), 14.0 -> 8.5 (512 x 512).
+// 89 us on 49,392 rows of layer 1 (six rounds of tiles where 5.1 would do); GELU and the loads make
+// that 118 us (115 as one-CTA tiles).  The 512-wide layers of K = 512 are bound by GELU's
+// instructions: 60 us at 49,392 rows as one-CTA tiles, 50 with eight epilogue warps, 46 with sixteen
+// (half the registers each).  The output layer is bound by its FP32 stores (12,528 rows: 43.2 ->
+// 38.5 us) and, in an update of one player, computes that player's half.  A turn's 624 rows spread
+// over narrow tiles and the launches' prologues overlap (programmatic dependent launch): 24.2 -> 19.2
+// us (layer 1), 14.0 -> 7.5 (512 x 512).
 template <bool F32, bool ACT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_c, const float* __restrict__ bias, int M, int n_begin, int n_nt,
                 int kb_count, int bn, int stages, int* err) {
-  extern __shared__ __align__(128) unsigned char smg[];
-  // 1024-byte aligned: the ring (A then B of each stage), the epilogue's staging blocks, its bias rows
-  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smg) + 1023) & ~(uintptr_t)1023);
+  // the ring (A then B of each stage, 1024-byte aligned), the epilogue's staging blocks, its bias rows
+  extern __shared__ __align__(1024) unsigned char base[];
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], mma_done;
   __shared__ uint32_t tmem_base;
   __shared__ volatile int failed;  // set by any role whose bounded wait gave up; the CTA's others poll it
@@ -231,6 +233,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   cluster_sync();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;  // all of TMEM: the same address in both CTAs
+  // A and the bias may come from the launch just before this one (programmatic dependent launch)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer
@@ -299,20 +304,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       bar_wait(&mma_done, 0);
     }
     __syncwarp();
-  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, every other 32-column
-            // block, from its part (w - 2) / 4 on (the parts take turns to start, as the count may be odd)
+  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, every fourth 32-column
+            // block, from its part (w - 2) / 4 on (the parts take turns, as the count may be uneven)
     const int q = warp & 3, part = (warp - 2) >> 2, blocks = bn / 32;
     // staging blocks of 32 rows x 32 columns in the bulk store's swizzled layout: 16-byte chunk j of row
     // r at chunk j ^ (r % 8) (FP32, 128-byte rows) or j ^ (r / 2 % 4) (BF16, 64-byte rows)
-    unsigned char* stage = base + kRingBytes + (size_t)(warp - 2) * kStageBufs * kStageBuf;
-    float* sbias = reinterpret_cast<float*>(base + kRingBytes + kEpiWarps * kStageBufs * kStageBuf) + (warp - 2) * 32;
+    unsigned char* stage = base + kRingBytes + (size_t)(warp - 2) * kStageBytes;
+    float* sbias = reinterpret_cast<float*>(base + kRingBytes + kEpiWarps * kStageBytes) + (warp - 2) * 32;
     int cc = 0;  // blocks this warp has staged
     int lt = 0;
     // one block: its values v and bias (lane's column) to the staging block, and from there to C
     auto put = [&](const uint32_t (&v)[32], float bias_lane, int col, int row) {
-      unsigned char* buf = stage + (cc & 1) * kStageBuf;
-      if (cc >= kStageBufs && lane == 0)  // the store that last read this block has finished reading it
-        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      unsigned char* buf = stage + (F32 ? 0 : (cc & 1) * (kStageBytes / 2));
+      if (lane == 0) {  // the store that last read this block has finished reading it
+        if (F32)
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        else
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      }
       __syncwarp();  // (and the last block's bias has been read)
       sbias[lane] = bias_lane;
       __syncwarp();
@@ -348,10 +357,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       const int row0 = (tile / n_nt) * 2 * kBM + rank * kBM + q * 32, n0 = n_begin + (tile % n_nt) * bn;
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBNMax);
       const int last = row0 < M ? blocks : 0;
-      int b = (part + lt) & 1;
-      // a block's bias and accumulator values are asked for before the block in front of it is worked on
+      int b = (part + lt) % kEpiParts;
       auto bias_at = [&](int blk) { return bias && blk < last ? __ldg(bias + n0 + blk * 32 + lane) : 0.f; };
-      float b0 = bias_at(b), b1;
+      float bias_lane = bias_at(b);
       const bool ok = bar_wait(&acc_full[acc], (uint32_t)(lt >> 1) & 1u);
       if (!__all_sync(0xffffffffu, ok) || failed) {
         if (lane == 0) failed = 1;
@@ -363,26 +371,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         __syncwarp();
         if (lane == 0) bar_arrive_cluster(of_first_cta(&acc_empty[acc]));
       };
-      uint32_t v0[32], v1[32];
-      if (b < last) tmem_load(v0, taddr + (uint32_t)(b * 32));
-      while (b + 2 < last) {
-        tmem_wait(v0);
-        tmem_load(v1, taddr + (uint32_t)(b * 32 + 64));
-        b1 = bias_at(b + 2);
-        put(v0, b0, n0 + b * 32, row0);
-        tmem_wait(v1);
-        if (b + 4 < last) tmem_load(v0, taddr + (uint32_t)(b * 32 + 128));
-        else drained();
-        b0 = bias_at(b + 4);
-        put(v1, b1, n0 + b * 32 + 64, row0);
-        b += 4;
-      }
-      if (b < last) {  // an odd last block
-        tmem_wait(v0);
-        drained();
-        put(v0, b0, n0 + b * 32, row0);
-      } else if (last <= ((part + lt) & 1)) {  // none at all
-        drained();
+      if (b >= last) drained();  // no block of this tile
+      for (; b < last; b += kEpiParts) {
+        uint32_t v[32];
+        tmem_load(v, taddr + (uint32_t)(b * 32));
+        const float next = bias_at(b + kEpiParts);
+        tmem_wait(v);
+        if (b + kEpiParts >= last) drained();
+        put(v, bias_lane, n0 + b * 32, row0);
+        bias_lane = next;
       }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // every store has completed
@@ -445,8 +442,8 @@ bool encode(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows)
 
 }  // namespace
 
-// the ring, the epilogue warps' staging blocks and bias rows, alignment slack
-size_t gemm_smem_bytes() { return (size_t)kRingBytes + kEpiWarps * (kStageBufs * kStageBuf + 128) + 1024; }
+// the ring, the epilogue warps' staging blocks and bias rows
+size_t gemm_smem_bytes() { return (size_t)kRingBytes + kEpiWarps * (kStageBytes + 128); }
 
 int configure_gemm() {
   const int smem = (int)gemm_smem_bytes();
@@ -491,9 +488,17 @@ static int launch_gemm_cols(const void* A, const void* B, const float* bias, voi
   const int stage = kATile + bn * kBK, stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
   auto* kernel = out_f32 ? (act ? k_gemm_bf16<true, true> : k_gemm_bf16<true, false>)
                          : (act ? k_gemm_bf16<false, true> : k_gemm_bf16<false, false>);
-  kernel<<<2 * pairs, kGemmThreads, gemm_smem_bytes(), (cudaStream_t)stream>>>(ma, mb, mc, bias, M, n_begin, n_cols / bn,
-                                                                               K / kBK, bn, stages, err);
-  const cudaError_t e = cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * pairs));
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = gemm_smem_bytes();
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, ma, mb, mc, bias, M, n_begin, n_cols / bn, K / kBK, bn, stages, err);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_gemm_bf16 failed: %s\n", cudaGetErrorString(e));
     return -1;
