@@ -73,7 +73,7 @@ struct cfr_tree {
   std::vector<int> wide_inner_off, wide_fwd_off[2];
   int* d_iter = nullptr;
   unsigned* d_done = nullptr;
-  unsigned* d_res_sync = nullptr;   // resident schedule: barrier and exit counters
+  unsigned* d_res_sync = nullptr;   // resident schedule: barrier and exit counters, the last stamp
   int* d_err = nullptr;
   Discount* d_disc = nullptr;
   int disc_capacity = 0;
@@ -86,7 +86,6 @@ struct cfr_tree {
   cfr_solver_opts opts{};
   LaunchCtx ctx{};
   int iters_done = 0;
-  uint32_t resident_stamp = 0;  // resident schedule: the last stamp its launches have used
   int64_t state_gen = 0;        // bumped whenever R or S may change
   int64_t avg_gen = -1;         // state_gen for which sigbar holds k_average_rows' output
   int64_t cur_gen = -1;         // state_gen for which sigma holds RM(R) (stream schedule)
@@ -959,7 +958,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       (rc = upload(t, term_groups, &t->d_term_groups)) || (rc = upload(t, term_segments, &t->d_term_segments)) ||
       (rc = upload(t, tile_work, &t->d_tile_work)) ||
       (rc = zeros(t, 1, &t->d_iter)) ||
-      (rc = zeros(t, 1, &t->d_done)) || (rc = zeros(t, 1, &t->d_err)) || (rc = zeros(t, 2, &t->d_res_sync)) ||
+      (rc = zeros(t, 1, &t->d_done)) || (rc = zeros(t, 1, &t->d_err)) || (rc = zeros(t, 3, &t->d_res_sync)) ||
       (rc = upload(t, discount_table(o, kDiscountCapacity), &t->d_disc))) {
     delete t;
     return rc;
@@ -1173,16 +1172,7 @@ int cfr_iterate(cfr_tree* t, int n_iters) {
   if (t->ctx.resident) {  // one cooperative launch per 2^20 iterations (its barrier count stays in 32 bits)
     for (int done = 0; done < n_iters; done += 1 << 20) {
       const int n = std::min(n_iters - done, 1 << 20);
-      if (t->resident_stamp > 0xffffffffu - (uint32_t)n) {  // the stamps start again: clear the old ones
-        for (const GameDev& d : t->dev) {
-          const size_t bytes = (size_t)2 * d.n_nodes * d.hstride * (t->opts.precision == CFR_PRECISION_SINGLE ? 8 : 16);
-          if (d.xval) CK(cudaMemsetAsync(d.xval, 0, bytes, t->stream));
-          if (d.xreach) CK(cudaMemsetAsync(d.xreach, 0, bytes, t->stream));
-        }
-        t->resident_stamp = 0;
-      }
-      if (launch_resident(t->ctx, n, t->resident_stamp, t->stream) != 0) return fail(CFR_ECUDA, "resident launch failed");
-      t->resident_stamp += (uint32_t)n;
+      if (launch_resident(t->ctx, n, t->stream) != 0) return fail(CFR_ECUDA, "resident launch failed");
       t->launches += 1;
     }
     t->iters_done += n_iters;

@@ -1873,14 +1873,14 @@ struct ResidentTerm {
 };
 
 // Values of player i at terminal item e (Stages 2-4).  The opponent's reach row comes from the global
-// rows (stamp 0: written by an earlier launch, or before a grid barrier) or, stamped, from xreach; the
-// values go to the global rows when `plain` is set, and stamped to xval when `put` is.  False when a
-// wait gave up.  Ends with a block barrier.
+// rows (written by an earlier launch, or before a grid barrier) or, when `get` is set, with the stamp
+// `from_stamp` from xreach; the values go to the global rows when `plain` is set, and with the stamp
+// `stamp` to xval when `put` is.  False when a wait gave up.  Ends with a block barrier.
 template <typename P>
 __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ games, const Work* __restrict__ term_work,
                                                   const TermSrc* __restrict__ term_src, int e, int i, unsigned char* smr,
-                                                  ResidentTerm<P>& R, uint32_t stamp, uint32_t put, bool plain, long limit,
-                                                  int* err) {
+                                                  ResidentTerm<P>& R, bool get, uint32_t from_stamp, bool put,
+                                                  uint32_t stamp, bool plain, long limit, int* err) {
   using V = typename P::V;
   constexpr int words = (int)sizeof(V) / 4;  // stamped words per value
   const int tid = threadIdx.x;
@@ -1914,7 +1914,7 @@ __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ ga
   V* Ps = CP + (k * H + 1);
   const size_t row = ((size_t)(1 - i) * R.N + term_src_node(from)) * stride;
   bool ok = true;
-  if (stamp == 0) {
+  if (!get) {
     const V* src = static_cast<const V*>(R.G->reach) + row;
     for (int h = tid; h < H; h += kTermThreads) q[h] = ld_cg(src + h);
   } else {
@@ -1924,12 +1924,12 @@ __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ ga
 #pragma unroll
     for (int s = 0; s < kTermHands; ++s) {  // the first polls go out together
       const int h = tid + s * kTermThreads;
-      got[s] = h >= H || (limit > 0 && stamp_get(src + (size_t)h * words, stamp, v[s]));
+      got[s] = h >= H || (limit > 0 && stamp_get(src + (size_t)h * words, from_stamp, v[s]));
     }
 #pragma unroll
     for (int s = 0; s < kTermHands; ++s) {
       const int h = tid + s * kTermThreads;
-      if (!got[s]) ok = stamp_wait(src + (size_t)h * words, stamp, v[s], limit, err) && ok;
+      if (!got[s]) ok = stamp_wait(src + (size_t)h * words, from_stamp, v[s], limit, err) && ok;
       if (h < H) q[h] = v[s];
     }
   }
@@ -1943,7 +1943,7 @@ __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ ga
   V* dst = static_cast<V*>(R.G->cfv) + out;
   uint64_t* xdst = R.G->xval + out * words;
   terminal_node<P>(R.lane, H, k, R.deck, R.show, R.board, R.u[i], q, ft, CP, Ps, [&](int h, V v) {
-    if (put) stamp_put(xdst + (size_t)h * words, v, put);
+    if (put) stamp_put(xdst + (size_t)h * words, v, stamp);
     if (plain) dst[h] = v;
   });
   __syncthreads();  // the row buffer and the scan arrays are free again
@@ -1953,15 +1953,17 @@ __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ ga
 // n_iters iterations (alternating: terminal and update of player 0, then of player 1;
 // otherwise both players' terminals, then both updates).  Launched cooperatively, every block
 // resident: grid >= n_chunk_work.  Alternating updates pass values and reach as stamped words (the
-// stamps of iteration it of this launch are stamp0 + it + 1); simultaneous ones through the global
+// stamp of iteration it of this launch is sync[2] + it + 1); simultaneous ones through the global
 // rows, a grid barrier between phases.  sync[0] counts barrier arrivals, sync[1] blocks that have
-// finished; the last block to finish resets both and advances *iter by n_iters.
+// finished; the last block to finish resets both and advances *iter and sync[2] by n_iters.  The
+// stamps are counted on the device, over the handle's life, so that a launch replayed from a
+// captured graph takes new ones too; every word is rewritten every iteration, so they may wrap.
 template <typename P>
 __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
     const GameDev* __restrict__ games, const Work* __restrict__ chunk_work, int n_chunk_work,
     const Work* __restrict__ term_work, const TermSrc* __restrict__ term_src, int n_term_work, int alternating,
     int n_iters, int* iter, const Discount* __restrict__ disc_tab, int variant, unsigned* sync, int* err,
-    unsigned term_bytes, uint32_t stamp0) {
+    unsigned term_bytes) {
   using V = typename P::V;
   constexpr size_t es = sizeof(V);
   constexpr int words = (int)sizeof(V) / 4;
@@ -2012,7 +2014,8 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
   }
   __syncthreads();
 
-  const int it0 = *iter;  // written only by the last block to finish
+  const int it0 = *iter;             // written only by the last block to finish
+  const uint32_t stamp0 = sync[2];  // too
   const int steps = alternating ? 2 : 1;
   unsigned nbar = 0;
   bool ok = true;
@@ -2030,9 +2033,8 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
       for (int item = blockIdx.x; item < np * n_term_work && ok; item += gridDim.x) {
         const int e = item % n_term_work, i = p0 + item / n_term_work;
         // player 0's first terminals read what the launch before left
-        const uint32_t from = !alternating || (it == 0 && step == 0) ? 0u : step == 0 ? stamp - 1u : stamp;
-        ok = resident_terminal<P>(games, term_work, term_src, e, i, smr, term, from, alternating ? stamp : 0u,
-                                  !alternating || last, limit, err);
+        ok = resident_terminal<P>(games, term_work, term_src, e, i, smr, term, alternating && (it > 0 || step > 0),
+                                  step == 0 ? stamp - 1u : stamp, alternating != 0, stamp, !alternating || last, limit, err);
       }
       if (!ok) break;
       if (!alternating) {
@@ -2126,6 +2128,7 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
     if (atomicAdd(&sync[1], 1u) == gridDim.x - 1) {  // every other block has left its waits
       sync[0] = 0u;
       sync[1] = 0u;
+      sync[2] = stamp0 + (uint32_t)n_iters;
       *iter += n_iters;
       __threadfence();
     }
@@ -3299,7 +3302,7 @@ int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stre
 // One cooperative launch: every block is resident at once, which the grid barriers need
 // (the launch fails rather than run a grid that does not fit).
 template <typename P>
-static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream) {
+static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c.resident_grid);
   cfg.blockDim = dim3(kTermThreads);
@@ -3312,12 +3315,12 @@ static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, uint32_t s
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_resident<P>, c.games, c.chunk_work, c.n_chunk_work, c.term_work,
                             c.term_src, c.n_term_work, c.alternating, n_iters, c.iter,
-                            c.disc, c.variant, c.resident_sync, c.err, c.resident_term, stamp0);
+                            c.disc, c.variant, c.resident_sync, c.err, c.resident_term);
 }
 
-int launch_resident(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream) {
-  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single>(c, n_iters, stamp0, stream)
-                                                        : launch_resident_p<Pairs>(c, n_iters, stamp0, stream);
+int launch_resident(const LaunchCtx& c, int n_iters, void* stream) {
+  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single>(c, n_iters, stream)
+                                                        : launch_resident_p<Pairs>(c, n_iters, stream);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_resident failed: %s\n", cudaGetErrorString(e));
     return -1;

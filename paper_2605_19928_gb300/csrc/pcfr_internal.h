@@ -302,7 +302,7 @@ struct LaunchCtx {
   int resident_grid;           // blocks of the cooperative launch (>= n_chunk_work)
   size_t smem_resident;        // its dynamic shared memory: terminal region, then hand region
   unsigned resident_term;      // bytes of the terminal region
-  unsigned* resident_sync;     // device [2]: barrier arrivals, blocks finished (zero between launches)
+  unsigned* resident_sync;     // device [3]: barrier arrivals, blocks finished (zero between launches), the last stamp used
   int alternating;
 };
 
@@ -328,12 +328,11 @@ int set_first_wait_polls(long polls);
 // Shared memory of k_tile for one game (tab16: its table in 16-byte units; staged: its latency form).
 size_t tile_smem_size(int tab16, int n_nodes, int rows_max, int W, size_t es, int staged);
 // Resident schedule: shared memory of its two regions for one game, the blocks of k_resident
-// one SM holds with `smem` bytes (0 if none), and the cooperative launch of n_iters iterations (its stamps are stamp0 + 1 ..
-// stamp0 + n_iters, none of which the handle used before).
+// one SM holds with `smem` bytes (0 if none), and the cooperative launch of n_iters iterations.
 size_t resident_term_size(int n_hands, int hand_size, int deck, int hstride, size_t es);
 size_t resident_hand_size(int tab16, int n_nodes, int rows_max, int W, size_t es);
 int resident_blocks_per_sm(int precision, size_t smem);
-int launch_resident(const LaunchCtx& c, int n_iters, uint32_t stamp0, void* stream);
+int launch_resident(const LaunchCtx& c, int n_iters, void* stream);
 // Dense layer of the leaf network (leafnet.cu): C[M][N] = act(A[M][K] B[N][K]^T + bias), BF16
 // A and B, FP32 accumulation, C in BF16 (out_f32 = 0) or FP32; N a multiple of 128, K of 64.
 // Returns 0, -1 (launch failed), -2 (bad shape or alignment), -3 (no tensor-map encoder).
