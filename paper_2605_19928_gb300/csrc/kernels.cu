@@ -683,6 +683,8 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
     const TermTab tg(Gg.n_hands, Gg.hand_size, Gg.deck);
     unsigned char* buf = smt + kTab + tg.fold_len * 2 + (g & 1) * NV * bytes;
     const V* q = static_cast<const V*>(use_bar ? Gg.reach_bar : Gg.reach) + (size_t)(1 - i) * Gg.n_nodes * S;
+    // the block's own writes there (zeroed hands, another game's arrays) come before the copies
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     mbar_arrive_expect_tx(&bar[g & 1], NV * bytes);  // a short group repeats its last node
     for (int v = 0; v < NV; ++v) bulk_copy_g2s(buf + v * bytes, q + (size_t)term_src_node(d.src[v].row[1 - i]) * S, bytes, &bar[g & 1]);
   };
