@@ -140,9 +140,9 @@ __device__ __forceinline__ double f2d(float f) {
 }
 // double -> float, round to nearest even, on the integer pipe where the result is a normal float (or
 // overflows by rounding): 29 mantissa bits off with the carry, exponent - 896.  A conversion holds the
-// FP64 pipe as long as an addition: in the hand tiles' updates, of three more FP64 operations a row,
-// Leduc 5.44 -> 5.26 ms, resident river 4.12 -> 4.09, 256 rivers 69.4 -> 69.0.  The wide update, which
-// waits on memory, keeps the conversion (the exact turn got 0.3 % slower without).
+// FP64 pipe as long as an addition; without it a row of the hand tiles' updates needs that pipe three
+// times, not four: Leduc 5.44 -> 5.25 ms, resident river 4.12 -> 4.08, 256 rivers 69.4 -> 69.0.  The
+// wide update, which waits on memory, keeps the conversion (without it the exact turn is 0.3 % slower).
 __device__ __forceinline__ float d2f(double x) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), a = hi & 0x7fffffffu;
   if (a - 0x38100000u < 0x0fe00000u) {  // 2^-126 <= |x| < 2^128
@@ -1240,7 +1240,7 @@ __global__ void __launch_bounds__(kHandThreads, 1) k_hand(const GameDev* __restr
 //      reach of their children (Stage 1), in the array of A.
 // R and S are read and written once, straight from registers; L2 is asked for their lines at the
 // start, before the launch waits for its predecessor.  The arithmetic is k_hand's, in its order.
-// Bound: the FP64 pipe (four operations a row and hand: 88 us on the batch below) and issue slots.
+// Bound: the FP64 pipe (three operations a row and hand: 66 us on the batch below) and issue slots.
 // Measured, one player's update: 256 rivers, FP32 values 267 -> 180 us against the one-warp walk;
 // 64 rivers, pairs, Predictive CFR+ 321 -> 110 us.  Average pass 780 -> 167, best response 943 ->
 // 150 us (256 rivers, both players; k_hand before).
