@@ -392,7 +392,9 @@ int cfr_leaf_info(const cfr_tree* tree, int leaf, int* n_leaves, int* game, int*
 
 /* Read network rows of the last leaf evaluation into a host buffer (synchronises):
  * what 0 = inputs (n_rows x 2752 BF16 as uint16), 1 = outputs (n_rows x 2688 FP32), in
- * the slot layout cfr_set_leaf_net describes. */
+ * the slot layout cfr_set_leaf_net describes.  An alternating update evaluates its own player's
+ * outputs; the first read of outputs after it (or cfr_set_leaf_net, before it replaces the
+ * weights) runs the output layer once for both players. */
 int cfr_read_leaf_rows(cfr_tree* tree, int what, int row0, int n_rows, void* out);
 
 /* One dense layer of the depth-limit leaf network (Section 3, depth-limited solving; the

@@ -93,7 +93,9 @@ struct cfr_tree {
   std::vector<LeafDev> leaf_host;
   std::vector<int> leaf_col;    // network column of each card-pair slot (hand order, or the slot)
   bool leaf_net_set = false;
-  bool leaf_half = false;         // iterations have computed one player's network outputs at a time
+  // Players (mask) whose outputs of the last leaf evaluation are in leaf.Y: an alternating update's
+  // evaluation computes only its player's (complete_leaf_outputs adds the other's).
+  int leaf_have = 3;
   int64_t launches = 0;         // kernels launched (graph replays included)
   int64_t device_bytes = 0;
   int64_t h2d_bytes = 0;
@@ -1121,6 +1123,17 @@ int check_device_flag(cfr_tree* t) {
   return CFR_OK;
 }
 
+// The whole output layer of the last leaf evaluation, from its hidden rows, where its update took one
+// player's columns only.
+int complete_leaf_outputs(cfr_tree* t) {
+  if (t->leaf_have == 3) return CFR_OK;
+  if (launch_leaf_outputs(t->ctx, t->leaf, 3, t->stream) != 0) return fail(CFR_ECUDA, "leaf launch failed");
+  t->launches += 1;
+  const int rc = check_device_flag(t);
+  if (rc == CFR_OK) t->leaf_have = 3;
+  return rc;
+}
+
 int check_game(const cfr_tree* t, int game) {
   if (!t) return fail(CFR_EINVAL, "tree is NULL");
   if (game < 0 || game >= (int)t->host.size()) return fail(CFR_EINVAL, "game index out of range");
@@ -1168,7 +1181,7 @@ int cfr_iterate(cfr_tree* t, int n_iters) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
   }
   t->state_gen += 1;
-  if (t->leaf.n_leaves > 0 && t->opts.alternating) t->leaf_half = true;
+  if (t->leaf.n_leaves > 0) t->leaf_have = t->opts.alternating ? 2 : 3;  // the last update's players
   if (t->ctx.resident) {  // one cooperative launch per 2^20 iterations (its barrier count stays in 32 bits)
     for (int done = 0; done < n_iters; done += 1 << 20) {
       const int n = std::min(n_iters - done, 1 << 20);
@@ -1251,6 +1264,7 @@ int cfr_exploitability_async(cfr_tree* t) {
     CK(cudaGraphLaunch(t->expl_graph, t->stream));
   }
   t->avg_gen = -1;  // the pass rewrites sigbar with its own normalisation
+  t->leaf_have = 3;
   t->launches += terminal_launches(t) + pass_launches(t, kModeAvg, 3, 0) +
                  pass_launches(t, kModeBR, 3, 0) + leaf_launches(t, 3);
   return CFR_OK;
@@ -1469,6 +1483,7 @@ int cfr_stage_times(cfr_tree* t, int n_iters, double* ms, int64_t* launches) {
   if (err != cudaSuccess) return cuda_fail(err, "cudaEventRecord");
   if (serr != cudaSuccess) return cuda_fail(serr, "cudaStreamSynchronize");
   t->iters_done += n_iters;
+  t->leaf_have = 3;  // the closing exploitability pass evaluated both players
   for (int k = 0; k < CFR_N_STAGES; ++k) {
     ms[k] = cnt[k] ? tot[k] / (double)cnt[k] : 0.0;
     if (launches) launches[k] = cnt[k];
@@ -1495,6 +1510,9 @@ int cfr_set_leaf_net(cfr_tree* t, const uint16_t* const W[4], const float* const
   const size_t bn[4] = {(size_t)kLeafHidden, (size_t)kLeafHidden, (size_t)kLeafHidden, (size_t)kLeafOut};
   for (int k = 0; k < 4; ++k)
     if (!W[k] || !b[k]) return fail(CFR_EINVAL, "every layer needs weights and a bias");
+  // the outputs of the last evaluation stay readable: they are completed with the weights that made them
+  const int orc = complete_leaf_outputs(t);
+  if (orc) return orc;
   // the range inputs (columns of layer 1) and value outputs (rows of layer 4) move to the
   // handle's column order
   const std::vector<int>& col = t->leaf_col;
@@ -1537,6 +1555,7 @@ int cfr_eval_leaves(cfr_tree* t, int average) {
     t->avg_gen = -1;
   }
   if (enqueue_leaves(t, 3, average ? 1 : 0, t->stream) != 0) return fail(CFR_ECUDA, "leaf launch failed");
+  t->leaf_have = 3;
   t->launches += (average ? pass_launches(t, kModeAvg, 3, 0) : 0) + leaf_launches(t, 3);
   return cfr_sync(t);
 }
@@ -1562,10 +1581,8 @@ int cfr_read_leaf_rows(cfr_tree* t, int what, int row0, int n_rows, void* out) {
   std::vector<unsigned char> raw((size_t)n_rows * width * es);
   const unsigned char* src = what == 0 ? static_cast<const unsigned char*>(t->leaf.X)
                                        : reinterpret_cast<const unsigned char*>(t->leaf.Y);
-  if (what == 1 && t->leaf_half && n_rows) {  // both players' outputs, from the last evaluation's hidden rows
-    if (launch_leaf_outputs(t->ctx, t->leaf, 3, t->stream) != 0) return fail(CFR_ECUDA, "leaf launch failed");
-    t->launches += 1;
-  }
+  const int orc = what == 1 && n_rows ? complete_leaf_outputs(t) : CFR_OK;
+  if (orc) return orc;
   if (n_rows)
     CK(cudaMemcpyAsync(raw.data(), src + (size_t)row0 * width * es, raw.size(), cudaMemcpyDeviceToHost, t->stream));
   CK(cudaStreamSynchronize(t->stream));
@@ -1815,6 +1832,7 @@ extern "C" int cfr_exploitability_noalloc(cfr_tree* t, double* expl, double* br)
   t->avg_gen = -1;
   if (launch_avg_reach(c, s) || enqueue_leaves(t, 3, 1, s) || launch_terminals(t, 3, 1, s) || launch_br(c, s))
     return fail(CFR_ECUDA, "exploitability launch failed");
+  t->leaf_have = 3;
   k_br_root_static<<<2 * c.n_chunk_work, 32, 0, s>>>(c.games, c.chunk_work, c.n_chunk_work, c.precision, scratch);
   CK(cudaGetLastError());
   t->launches += terminal_launches(t) + pass_launches(t, kModeAvg, 3, 0) + pass_launches(t, kModeBR, 3, 0) +
