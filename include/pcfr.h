@@ -150,10 +150,10 @@ typedef struct cfr_game_spec {
  * CFR_ETIMEOUT and the handle's state is undefined.
  * CFR_SCHEDULE_AUTO (0) picks STREAM when the handle has at least 1216 such warps (8 per
  * SM) and every tree allows it, WIDE for one subgame too large to stage, else LEVEL.
- * term_nodes: fold and showdown nodes a block of the terminal launch evaluates together (nodes
- * of one board and kind; 0 = automatic: one while the nodes do not fill the GPU many times over,
- * four when they do -- two with pair values; otherwise 1 to 8, of which at most those many are
- * taken).  Results are the same bits for every value.
+ * term_nodes: fold and showdown nodes (of one board and kind) a block of the terminal launch
+ * evaluates: 1, one; 2 to 8, at most so many, one after the other or, with FP32 values on trees with
+ * many showdowns a board, two or four together; 0 = automatic: one while the nodes do not fill the
+ * GPU many times over, more when they do.  Results are the same bits for every value.
  * warp_hands: 64 asks the stream schedule for its one-warp walk with two hands per lane (needs
  * every subgame's hand rows padded to a multiple of 64, i.e. the hand count rounded up to 32 is a
  * multiple of 64, CFR_EINVAL otherwise); 0 (automatic) and 32: hand tiles, or the walk with one

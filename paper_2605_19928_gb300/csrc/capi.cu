@@ -24,8 +24,17 @@ using namespace pcfr;
 
 namespace {
 
-// Terminal nodes from which the launch evaluates them in groups (see create_impl).
+// Terminal nodes from which a block of the launch evaluates several (FP32 values), from which pairs take
+// the run form (with one node a block while they do not fill the GPU: more than one wave of the
+// one-node form's two blocks per SM; turn of 12 hands, 1,448 nodes: 22.5 -> 18.3 us), and showdown
+// nodes a board table from which FP32 values take groups of four (see create_impl).  Measured, one
+// player's launch with FP32 values, runs against groups: 7 showdowns a table (31,124-node flop, 513
+// hands) 158 against 197 us, 12 (the same flop's depth-limited form, 300 hands) 190 against 216, 30
+// (256 rivers of 406 hands) 100 against 79, 45 (turn of 1,128 hands) 49 against 44, 113 (exact turn)
+// 113 against 88.
 constexpr int kTermGroupMin = 152 * 16;
+constexpr int kTermRunMin = 152 * 2 + 1;
+constexpr int kTermGroupShows = 24;
 
 thread_local std::string g_last_error;
 cfr_alloc_fn g_alloc = nullptr;
@@ -57,6 +66,7 @@ struct cfr_tree {
   Work* d_term_work = nullptr;
   TermGroup* d_term_groups = nullptr;
   Work* d_term_segments = nullptr;
+  Work* d_term_runs = nullptr;
   Work* d_warp_work = nullptr;
   Work* d_tile_work = nullptr;
   WideNode* d_wide_inner = nullptr;                // wide schedule: inner nodes, level by level
@@ -705,19 +715,29 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     }
   }
 
-  // Terminal nodes a block evaluates together: one while they do not fill the GPU many times over
-  // (a block per node then has the lower latency), else groups of four (two with pair values:
-  // 16-byte entries either way).
-  int n_ends = 0;
-  std::vector<char> shows(n_games, es == 8);  // its records are read: at showdowns, and pairs' folds
-  for (int g = 0; g < n_games; ++g)
-    for (int n : t->host[g].terminals)
-      if (ro.inside.empty() || !ro.inside[(size_t)n]) {
-        ++n_ends;
-        if (t->host[g].nodes[(size_t)n].type == kShowdown) shows[g] = 1;
-      }
-  const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= kTermGroupMin ? 4 : 1;
-  const int term_nv = term_nodes == 1 ? 1 : term_nodes < 4 || es == 8 ? 2 : 4;
+  // Terminal nodes a block evaluates: one while they do not fill the GPU many times over (a block per
+  // node then has the lower latency); then runs of up to eight, or, with FP32 values and board tables
+  // of kTermGroupShows showdown nodes or more on average, groups of four (k_terminal_vec), whose
+  // blocks load a table's lists once for many full groups.
+  int n_ends = 0, n_shows = 0, n_tables = 0;
+  std::vector<char> shows(n_games, 0);  // its per-hand records are read
+  for (int g = 0; g < n_games; ++g) {
+    const HostGame& h = t->host[g];
+    std::vector<char> seen((size_t)h.n_boards, 0);
+    for (int n : h.terminals) {
+      if (!ro.inside.empty() && ro.inside[(size_t)n]) continue;
+      ++n_ends;
+      const NodeDev& nd = h.nodes[(size_t)n];
+      if (nd.type != kShowdown) continue;
+      ++n_shows;
+      n_tables += !seen[(size_t)nd.row];
+      seen[(size_t)nd.row] = 1;
+    }
+    shows[g] = es == 8 || n_shows > 0;
+  }
+  const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= (es == 8 ? kTermRunMin : kTermGroupMin) ? 8 : 1;
+  const bool term_run = term_nodes > 1 && (es == 8 || n_shows < kTermGroupShows * n_tables);
+  const int term_nv = term_run || term_nodes == 1 ? 1 : term_nodes < 4 ? 2 : 4;
 
   std::vector<Work> chunk_work, term_work, warp_work;
   // each game's device tables, prepared on the host in parallel, then packed in game order
@@ -889,14 +909,25 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     }
   // grouped terminal launch: groups of up to term_nv nodes of one game, board table and kind, and
   // each block's stretch of them -- two blocks per SM, equal shares of the work (a showdown group
-  // costs about twice a fold group with FP32 values, the same with pairs)
+  // costs about twice a fold group)
   std::vector<TermGroup> term_groups;
   std::vector<Work> term_segments;
+  std::vector<Work> term_runs;
+  auto key = [&](const Work& w) {
+    const NodeDev& nd = t->host[w.game].nodes[(size_t)w.unit];
+    return nd.type == kShowdown ? nd.row : -1;
+  };
+  if (term_run) {  // as long as the runs still fill the GPU eight times over
+    const int per = o.term_nodes ? o.term_nodes : std::max(1, std::min(8, (int)term_work.size() / (152 * 8)));
+    for (size_t a = 0; a < term_work.size(); ++a) {
+      const Work w = term_work[a];
+      if (!term_runs.empty() && term_runs.back().unit < per && term_work[a - 1].game == w.game && key(term_work[a - 1]) == key(w))
+        term_runs.back().unit += 1;
+      else
+        term_runs.push_back({(int)a, 1});
+    }
+  }
   if (term_nv > 1) {
-    auto key = [&](const Work& w) {
-      const NodeDev& nd = t->host[w.game].nodes[(size_t)w.unit];
-      return nd.type == kShowdown ? nd.row : -1;
-    };
     for (size_t a = 0; a < term_work.size();) {
       TermGroup q{};
       const Work w0 = term_work[a];
@@ -913,9 +944,8 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
         for (int p = 0; p < 2; ++p) q.below |= (term_src[a].row[p] < 0) << p;
         q.board[q.count] = nd.board;
         for (int i = 0; i < 2; ++i) {
-          const float* pay = &prep[w.game].pay32[2 * (size_t)w.unit];
-          const bool neg = nd.type == kFold && nd.player == i;
-          q.pay[i][q.count] = {neg ? -pay[0] : pay[0], neg ? -pay[1] : pay[1]};
+          const float pay = prep[w.game].pay32[2 * (size_t)w.unit];
+          q.pay[i][q.count] = nd.type == kFold && nd.player == i ? -pay : pay;
         }
       }
       for (int v = q.count; v < term_nv; ++v) {  // a short group repeats its last node, unwritten
@@ -926,22 +956,30 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       }
       term_groups.push_back(q);
     }
-    auto cost = [&](const TermGroup& q) { return es == 4 && q.kind == kFold ? 1 : 2; };
-    long total = 0, done = 0, cut = 0;
+    auto cost = [](const TermGroup& q) { return q.kind == kFold ? 1 : 2; };
+    long total = 0;
     for (const TermGroup& q : term_groups) total += cost(q);
-    const long share = (total + 2 * n_sms - 1) / (2 * n_sms);
-    for (size_t a = 0; a < term_groups.size(); ++a) {
-      if (term_segments.empty() || done >= cut || term_segments.back().unit == kTermSegment) {
-        term_segments.push_back({(int)a, 0});
-        cut = done + share;
+    // the shortest stretches that make whole waves of two blocks per SM: kTermSegment bounds a stretch, so
+    // stretches of one wave's share may be more than a wave (one player of 40 rivers of 771 nodes:
+    // 357 blocks, 218 us; in two even waves 152)
+    for (long waves = 1;; ++waves) {
+      const long blocks = 2 * n_sms * waves, share = (total + blocks - 1) / blocks;
+      term_segments.clear();
+      long done = 0, cut = 0;
+      for (size_t a = 0; a < term_groups.size(); ++a) {
+        if (term_segments.empty() || done >= cut || term_segments.back().unit == kTermSegment) {
+          term_segments.push_back({(int)a, 0});
+          cut = done + share;
+        }
+        term_segments.back().unit += 1;
+        done += cost(term_groups[a]);
       }
-      term_segments.back().unit += 1;
-      done += cost(term_groups[a]);
+      if ((long)term_segments.size() <= blocks || share <= 1) break;
     }
   }
   size_t smem_term = 0;
   for (const HostGame& h : t->host)
-    smem_term = std::max(smem_term, terminal_smem_size(h.n_hands, h.hand_size, h.deck, h.hstride, es, term_nv));
+    smem_term = std::max(smem_term, terminal_smem_size(h.n_hands, h.hand_size, h.deck, h.hstride, es, term_nv, term_run));
   // stream schedule: blocks of kStreamWarps warps of one game, largest trees first so that
   // their long walks start at once and the small trees fill in behind them
   std::vector<int> by_size(n_games);
@@ -957,7 +995,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   if ((rc = upload(t, t->dev, &t->d_games)) || (rc = upload(t, chunk_work, &t->d_chunk_work)) ||
       (rc = upload(t, term_work, &t->d_term_work)) || (rc = upload(t, warp_work, &t->d_warp_work)) ||
       (rc = upload(t, term_src, &t->d_term_src)) ||
-      (rc = upload(t, term_groups, &t->d_term_groups)) || (rc = upload(t, term_segments, &t->d_term_segments)) ||
+      (rc = upload(t, term_groups, &t->d_term_groups)) || (rc = upload(t, term_segments, &t->d_term_segments)) || (rc = upload(t, term_runs, &t->d_term_runs)) ||
       (rc = upload(t, tile_work, &t->d_tile_work)) ||
       (rc = zeros(t, 1, &t->d_iter)) ||
       (rc = zeros(t, 1, &t->d_done)) || (rc = zeros(t, 1, &t->d_err)) || (rc = zeros(t, 3, &t->d_res_sync)) ||
@@ -976,6 +1014,8 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.term_groups = t->d_term_groups;
   c.term_segments = t->d_term_segments;
   c.n_term_segments = (int)term_segments.size();
+  c.term_runs = t->d_term_runs;
+  c.n_term_runs = (int)term_runs.size();
   c.term_nv = term_nv;
   c.iter = t->d_iter;
   c.done = t->d_done;

@@ -335,21 +335,27 @@ __device__ __forceinline__ void acc_join(float& a, float b) { a = __fadd_rn(a, b
 __device__ __forceinline__ void acc_join(acc2& a, acc2 b) { acc_merge(a, b); }
 
 // Exclusive prefix sums of NV arrays of n values by GT consecutive threads, in two halves with a block
-// barrier between.  Each thread owns a run of ceil(n / GT) entries, whose values are in registers
-// (a[0 .. cnt)): first x receives the inclusive sum of its warp's runs up to its own, and the warp's
-// total goes to red[warp].  Sums are plain FP32 with FP32 values, compensated with pairs.
-template <typename P, int NV>
-__device__ __forceinline__ void scan_runs(const Vec<P, NV> (&a)[ScanPer<P>::n], int cnt, VecAcc<P, NV>* red, int gtid,
-                                          VecAcc<P, NV>& x) {
+// barrier between.  Each thread owns a run of ceil(n / GT) entries, entry e at at(e) -- in registers
+// (REGS: ScanPer of them at most), or in the output array itself: first x receives the inclusive sum
+// of its warp's runs up to its own, and the warp's total goes to red[warp].  Sums are plain FP32 with
+// FP32 values, compensated with pairs.
+template <typename P, int NV, bool REGS, typename F>
+__device__ __forceinline__ void scan_runs(F at, int cnt, VecAcc<P, NV>* red, int gtid, VecAcc<P, NV>& x) {
   const int lane = gtid & 31;
 #pragma unroll
   for (int v = 0; v < NV; ++v) x.v[v] = P::acc0();
+  auto add = [&](int e) {
+    const Vec<P, NV> y = at(e);
 #pragma unroll
-  for (int e = 0; e < ScanPer<P>::n; ++e)
-    if (e < cnt) {
+    for (int v = 0; v < NV; ++v) P::acc(x.v[v], y.v[v]);
+  };
+  if constexpr (REGS) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) P::acc(x.v[v], a[e].v[v]);
-    }
+    for (int e = 0; e < ScanPer<P>::n; ++e)
+      if (e < cnt) add(e);
+  } else {
+    for (int e = 0; e < cnt; ++e) add(e);
+  }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
@@ -362,10 +368,9 @@ __device__ __forceinline__ void scan_runs(const Vec<P, NV> (&a)[ScanPer<P>::n], 
 
 // After the barrier: the exclusive prefix sums of the thread's run into out (out[n] = totals).  Every
 // warp scans the GT / 32 warp totals itself.
-template <typename P, int NV, int GT>
-__device__ __forceinline__ void scan_write(const Vec<P, NV> (&a)[ScanPer<P>::n], int begin, int cnt, int n,
-                                           const VecAcc<P, NV>* red, int gtid, const VecAcc<P, NV>& x,
-                                           Vec<P, NV>* out) {
+template <typename P, int NV, int GT, bool REGS, typename F>
+__device__ __forceinline__ void scan_write(F at, int begin, int cnt, int n, const VecAcc<P, NV>* red, int gtid,
+                                           const VecAcc<P, NV>& x, Vec<P, NV>* out) {
   const int lane = gtid & 31, warp = gtid >> 5;
   VecAcc<P, NV> run;
   Vec<P, NV> total;
@@ -383,17 +388,23 @@ __device__ __forceinline__ void scan_write(const Vec<P, NV> (&a)[ScanPer<P>::n],
     if (warp > 0) acc_join(run.v[v], before);
     total.v[v] = P::value(acc_from(w, GT / 32 - 1));
   }
+  auto put = [&](int e) {
+    const Vec<P, NV> y = at(e);
+    Vec<P, NV> o;
 #pragma unroll
-  for (int e = 0; e < ScanPer<P>::n; ++e)
-    if (e < cnt) {
-      Vec<P, NV> o;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        o.v[v] = P::value(run.v[v]);
-        P::acc(run.v[v], a[e].v[v]);
-      }
-      out[begin + e] = o;
+    for (int v = 0; v < NV; ++v) {
+      o.v[v] = P::value(run.v[v]);
+      P::acc(run.v[v], y.v[v]);
     }
+    out[begin + e] = o;
+  };
+  if constexpr (REGS) {
+#pragma unroll
+    for (int e = 0; e < ScanPer<P>::n; ++e)
+      if (e < cnt) put(e);
+  } else {
+    for (int e = 0; e < cnt; ++e) put(e);
+  }
   if (gtid == 0) out[n] = total;
 }
 
@@ -431,9 +442,15 @@ struct TermLane {
 template <typename P>
 struct TermStaged {
   TermRun<P> run;
-  const uint16_t *list, *cards, *gs, *ge, *lo, *hi;  // list: the thread's run, or null (hand order)
+  const uint16_t *list, *perm, *cards, *gs, *ge, *lo, *hi;  // list: the thread's run, or null (hand order)
   __device__ __forceinline__ int hand(int e) const {
     return e >= run.cnt ? 0 : list ? list[run.begin + e] : run.begin + e;
+  }
+  __device__ __forceinline__ void set(const TermTab& tt, const uint16_t* tab, int H, int k, bool show) {
+    run = TermRun<P>(H, k);
+    perm = tab + tt.perm;
+    list = (int)threadIdx.x >= run.gp ? tab + tt.clh : show ? perm : nullptr;
+    cards = tab + tt.cards, gs = tab + tt.gs, ge = tab + tt.ge, lo = tab + tt.lo, hi = tab + tt.hi;
   }
   __device__ __forceinline__ uint4 record(int, int h) const {
     return make_uint4(cards[h] | (uint32_t)gs[h] << 16, ge[h] | (uint32_t)lo[2 * h] << 16,
@@ -461,7 +478,7 @@ __device__ __forceinline__ void term_lane_load(TermLane<P>& L, const GameDev& G,
 
 // Values at one node: q its reach row, ft the fold part of its board table (card lists, cards, list
 // offsets) and CP [k H + 1], Ps [H + 1] in shared memory; put(h, value) takes the results.
-template <typename P, typename LT, typename F>
+template <typename P, bool REGS = true, typename LT, typename F>
 __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int deck, bool show, uint64_t board, ff u,
                                               const typename P::V* q, const uint16_t* ft, typename P::V* CP,
                                               typename P::V* Ps, F put) {
@@ -511,17 +528,27 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
     }
   }
   {
-    V1 a[ScanPer<P>::n];
+    V1 a[REGS ? ScanPer<P>::n : 1];
     VecAcc<P, 1> x;
-#pragma unroll
-    for (int e = 0; e < ScanPer<P>::n; ++e) a[e].v[0] = q[L.hand(e)];
+    V1* ps = reinterpret_cast<V1*>(Ps);
+    V1* cp = reinterpret_cast<V1*>(CP);
     const int gtid = tid < gp ? tid : tid - gp;
-    scan_runs<P, 1>(a, L.run.cnt, red[tid >= gp], gtid, x);
+    if constexpr (REGS) {
+#pragma unroll
+      for (int e = 0; e < ScanPer<P>::n; ++e) a[e].v[0] = q[L.hand(e)];
+    } else {  // gathered into the arrays that the scan turns into prefix sums in place
+      for (int j = tid; j < H; j += kTermThreads) ps[j].v[0] = q[show ? L.perm[j] : j];
+      for (int j = tid; j < k * H; j += kTermThreads) cp[j].v[0] = q[clh[j]];
+      __syncthreads();
+    }
+    V1* mine = (tid < gp ? ps : cp) + L.run.begin;
+    auto at = [&](int e) { return REGS ? a[REGS ? e : 0] : mine[e]; };
+    scan_runs<P, 1, REGS>(at, L.run.cnt, red[tid >= gp], gtid, x);
     __syncthreads();
     if (tid < gp)
-      scan_write<P, 1, gp>(a, L.run.begin, L.run.cnt, H, red[0], gtid, x, reinterpret_cast<V1*>(Ps));
+      scan_write<P, 1, gp, REGS>(at, L.run.begin, L.run.cnt, H, red[0], gtid, x, ps);
     else
-      scan_write<P, 1, kTermThreads - gp>(a, L.run.begin, L.run.cnt, k * H, red[1], gtid, x, reinterpret_cast<V1*>(CP));
+      scan_write<P, 1, kTermThreads - gp, REGS>(at, L.run.begin, L.run.cnt, k * H, red[1], gtid, x, cp);
   }
   __syncthreads();
   const V T = Ps[H], us = P::scale(u);
@@ -618,9 +645,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __r
   if (tid == 0) bulk_copy_g2s(q, qsrc + (size_t)term_src_node(from) * stride, q_bytes, &bar);
   const ff u = terminal_payoff(G, nd, n, i);
   TermStaged<P> L;
-  L.run = TermRun<P>(H, k);
-  L.list = tid >= L.run.gp ? tab + tt.clh : show ? tab + tt.perm : nullptr;
-  L.cards = tab + tt.cards, L.gs = tab + tt.gs, L.ge = tab + tt.ge, L.lo = tab + tt.lo, L.hi = tab + tt.hi;
+  L.set(tt, tab, H, k, show);
   const bool ok = tid >= 32 || mbar_wait_bounded(&bar, 0, g_first_wait_polls);  // one warp polls
   if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
     if (tid == 0) {
@@ -638,10 +663,98 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __r
   terminal_node<P>(L, H, k, G.deck, show, nd.board, u, q, tab, CP, Ps, [&](int h, V v) { dst[h] = v; });
 }
 
-// ---- several nodes at once: the throughput form for handles whose terminals fill the GPU
+// ---- the run form, for handles whose terminals fill the GPU many times over
+//
+// A block takes up to eight nodes of one game, board table and kind one after the other: the table is
+// staged once, and each node's reach row lands (two buffers) while the node before is computed.  A
+// node is a chain of four block barriers with little between them, so what counts is how many chains
+// an SM holds: four blocks, which the scans' in-place form leaves room for (40 registers; 64 with the
+// entries in registers hold two).  Pairs always run so (groups of two nodes a thread spilled, and
+// took 419 us a player on 256 rivers of 1,081 hands where this form takes 309); FP32 values where a
+// board table has few showdown nodes (see create_impl).  Measured, one player: 256 rivers, pairs, 309
+// us (four blocks; 317 three, 342 two); exact turn, pairs, 214; the 31,124-node flop of 513 hands,
+// FP32 values 158, pairs 275.
+template <typename P>
+__global__ void __launch_bounds__(kTermThreads, 4) k_terminal_run(const GameDev* __restrict__ games,
+                                                            const Work* __restrict__ work,
+                                                            const TermSrc* __restrict__ src,
+                                                            const Work* __restrict__ runs, int n_runs,
+                                                            int player_mask, int use_bar, int* err) {
+  using V = typename P::V;
+  int i;
+  const Work r = runs[terminal_item(n_runs, player_mask, i)];  // (first entry of work, count)
+  const int first = r.game, count = r.unit, tid = threadIdx.x;
+  const GameDev& G = games[work[first].game];
+  const NodeDev nd0 = G.nodes[work[first].unit];
+  const int H = G.n_hands, k = G.hand_size;
+  const size_t stride = (size_t)G.hstride;
+  const TermTab tt(H, k, G.deck);
+  const bool show = nd0.type == kShowdown;
+  const unsigned tab_bytes = (unsigned)(show ? tt.len : tt.fold_len) * 2u, q_bytes = (unsigned)(stride * sizeof(V));
+  const V* qsrc = static_cast<const V*>(use_bar ? G.reach_bar : G.reach) + (size_t)(1 - i) * G.n_nodes * stride;
+  V* dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
+
+  extern __shared__ __align__(128) unsigned char smt[];
+  __shared__ __align__(8) uint64_t bar[2];
+  const uint16_t* tab = reinterpret_cast<const uint16_t*>(smt);  // [tt.len]
+  V* rows = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);       // [2][hstride]
+  V* CP = rows + 2 * stride;                                     // [k H + 1]
+  V* Ps = CP + (k * H + 1);                                      // [H + 1]
+  if (tid == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  auto copy_row = [&](int j) {
+    bulk_copy_g2s(rows + (j & 1) * stride, qsrc + (size_t)term_src_node(src[first + j].row[1 - i]) * stride, q_bytes, &bar[j & 1]);
+  };
+  if (tid == 0) {
+    mbar_arrive_expect_tx(&bar[0], tab_bytes + q_bytes);
+    bulk_copy_g2s(smt, G.term_tab + (size_t)(show ? nd0.row : 0) * tt.len, tab_bytes, &bar[0]);
+  }
+  pdl_wait();  // the reach rows come from the launch just before this one
+  pdl_trigger();
+  if (tid == 0) copy_row(0);
+  TermStaged<P> L;
+  L.set(tt, tab, H, k, show);
+  for (int j = 0; j < count; ++j) {
+    const int n = work[first + j].unit, from = src[first + j].row[1 - i];
+    const uint64_t board = G.nodes[n].board;
+    const ff u = terminal_payoff(G, G.nodes[n], n, i);
+    if (tid == 0 && j + 1 < count) {
+      // the other buffer's last readers are behind the barrier that closed node j - 1; the block's own
+      // writes there (zeroed hands) come before the copy
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive_expect_tx(&bar[(j + 1) & 1], q_bytes);
+      copy_row(j + 1);
+    }
+    const bool ok = tid >= 32 || mbar_wait_bounded(&bar[j & 1], (j >> 1) & 1, j == 0 ? g_first_wait_polls : kWaitLimit);
+    if (__syncthreads_or(!ok)) {  // a copy did not land: report, let the copies drain, leave
+      if (tid == 0) {
+        atomicExch(err, 1);
+        mbar_wait_bounded(&bar[j & 1], (j >> 1) & 1);
+        if (j + 1 < count) mbar_wait_bounded(&bar[(j + 1) & 1], ((j + 1) >> 1) & 1);
+      }
+      __syncthreads();
+      return;
+    }
+    V* q = rows + (j & 1) * stride;
+    if (from < 0) {  // below an all-in run-out: its reach, without the hands holding a card dealt since
+      for (int h = tid; h < H; h += kTermThreads)
+        if (holds_board_card(L.cards, h, k, board)) q[h] = P::zero();
+      __syncthreads();
+    }
+    V* out = dst + (size_t)n * stride;
+    terminal_node<P, false>(L, H, k, G.deck, show, board, u, q, tab, CP, Ps, [&](int h, V v) { out[h] = v; });
+    __syncthreads();  // the row and the scan arrays are free
+  }
+}
+
+// ---- several nodes at once: the throughput form of FP32 values
 //
 // A group is up to NV nodes of one game, one kind (folds or showdowns) and one board table.  The
-// scan arrays of terminal_values become arrays of NV values (16 bytes), so each table entry and
+// scan arrays of terminal_node become arrays of NV values (16 bytes), so each table entry and
 // each address is read and computed once for NV nodes and a gather is one 16-byte shared-memory
 // access.  Component v runs exactly the one-node form's operations in its order (the same runs
 // of entries per thread, the same combination of threads and warps), so the bits are the same.
@@ -655,16 +768,15 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __r
 // Measured against blocks that take their nodes one by one: exact turn 119 -> 88 us per player,
 // 256 rivers 132 -> 129, with one block per group and its descriptors read node by node 147.
 
-template <typename P, int NV>
+template <int NV>
 __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev* __restrict__ games,
                                                                 const TermGroup* __restrict__ groups,
                                                                 const Work* __restrict__ segments, int n_segments,
                                                                 int player_mask, int use_bar, int* err) {
-  using V = typename P::V;
+  using P = Single;
   using VV = Vec<P, NV>;
-  constexpr bool single = std::is_same<P, Single>::value;
   constexpr int kScanPer = ScanPer<P>::n;
-  constexpr int gp = single ? 5 * 32 : kTermThreads / 2;  // threads on the rank order; the rest on the card lists
+  constexpr int gp = TermRun<P>::gp;  // threads on the rank order; the rest on the card lists
   int i;
   const Work seg = segments[terminal_item(n_segments, player_mask, i)];  // (first group, count <= kTermSegment)
   const int tid = threadIdx.x, lane = tid & 31;
@@ -672,7 +784,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
   extern __shared__ __align__(128) unsigned char smt[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ VecAcc<P, NV> red[2][kTermThreads / 32];
-  __shared__ float Cs[NV][kMaxDeck], Ts[NV];  // fold groups, FP32 values
+  __shared__ float Cs[NV][kMaxDeck], Ts[NV];  // fold groups
   TermGroup* desc = reinterpret_cast<TermGroup*>(smt);
   const uint4* gsrc = reinterpret_cast<const uint4*>(groups + seg.game);
   for (int k = tid; k < seg.unit * (int)(sizeof(TermGroup) / 16); k += kTermThreads)
@@ -689,7 +801,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
   // Ps [H + 1]
   constexpr int kTab = kTermSegment * (int)sizeof(TermGroup);
   int game = -1, table = -1, kind = -1, H = 0, k = 0, stride = 0, begin = 0, cnt = 0, rows = 0;
-  V* dst = nullptr;
+  float* dst = nullptr;
   const uint4* rec = nullptr;
   uint32_t at[kScanPer / 2];  // hands of the thread's run (rank order or card lists), two in a word
 
@@ -697,10 +809,10 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
     const TermGroup& d = desc[g];
     const GameDev& Gg = games[d.game];
     const size_t S = (size_t)Gg.hstride;
-    const unsigned bytes = (unsigned)(S * sizeof(V));
+    const unsigned bytes = (unsigned)(S * sizeof(float));
     const TermTab tg(Gg.n_hands, Gg.hand_size, Gg.deck);
     unsigned char* buf = smt + kTab + tg.fold_len * 2 + (g & 1) * NV * bytes;
-    const V* q = static_cast<const V*>(use_bar ? Gg.reach_bar : Gg.reach) + (size_t)(1 - i) * Gg.n_nodes * S;
+    const float* q = static_cast<const float*>(use_bar ? Gg.reach_bar : Gg.reach) + (size_t)(1 - i) * Gg.n_nodes * S;
     // the block's own writes there (zeroed hands, another game's arrays) come before the copies
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     mbar_arrive_expect_tx(&bar[g & 1], NV * bytes);  // a short group repeats its last node
@@ -725,7 +837,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
       if (other) {
         stride = G.hstride;
         rows = kTab + tt.fold_len * 2;
-        dst = static_cast<V*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
+        dst = static_cast<float*>(use_bar ? G.cfv_br : G.cfv) + (size_t)i * G.n_nodes * stride;
       }
       const uint16_t* gt = G.term_tab + (size_t)d.table * tt.len;
       if (other || d.table != table) {
@@ -737,7 +849,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
       }
       game = d.game;
       kind = d.kind;
-      if (show || !single) {
+      if (show) {
         const int n = tid < gp ? H : k * H, gt_n = tid < gp ? gp : kTermThreads - gp, gtid = tid < gp ? tid : tid - gp;
         const int per = (n + gt_n - 1) / gt_n;
         begin = min(gtid * per, n);
@@ -745,7 +857,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
 #pragma unroll
         for (int e = 0; e < kScanPer; ++e) {
           const int j = begin + e;
-          const uint32_t h = e >= cnt ? 0 : tid >= gp ? gt[tt.clh + j] : show ? gt[tt.perm + j] : j;
+          const uint32_t h = e >= cnt ? 0 : gt[(tid >= gp ? tt.clh : tt.perm) + j];
           at[e / 2] = e & 1 ? at[e / 2] | h << 16 : h;
         }
       }
@@ -764,110 +876,94 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
     const uint16_t* clh = reinterpret_cast<const uint16_t*>(smt + kTab);
     const uint16_t* cards = clh + k * H;
     const uint16_t* cloff = cards + H;
-    V* q = reinterpret_cast<V*>(smt + rows) + (g & 1) * NV * stride;  // node v's row at q + v * stride
-    VV* CP = reinterpret_cast<VV*>(reinterpret_cast<V*>(smt + rows) + 2 * NV * stride);
+    float* q = reinterpret_cast<float*>(smt + rows) + (g & 1) * NV * stride;  // node v's row at q + v * stride
+    VV* CP = reinterpret_cast<VV*>(reinterpret_cast<float*>(smt + rows) + 2 * NV * stride);
     VV* Ps = CP + (k * H + 1);
     if (d.below >> (1 - i) & 1) {  // nodes below an all-in run-out: its reach, without the hands holding a card dealt since
       for (int v = 0; v < NV; ++v)
         if (d.src[v].row[1 - i] < 0)
           for (int h = tid; h < H; h += kTermThreads)
-            if (holds_board_card(cards, h, k, d.board[v])) q[v * stride + h] = P::zero();
+            if (holds_board_card(cards, h, k, d.board[v])) q[v * stride + h] = 0.f;
       __syncthreads();
     }
 
-    if constexpr (single) {
-      if (!show) {  // terminal_values' FP32 fold sums: T of node v by warp v, C[c] of (v, c) by one thread
-        const int deck = games[game].deck;
-        if (tid < 32 * NV) {
-          const float* qv = q + (tid >> 5) * stride;
-          float t = 0.f;
+    if (!show) {  // terminal_node's fold sums: T of node v by warp v, C[c] of (v, c) by one thread
+      const int deck = games[game].deck;
+      if (tid < 32 * NV) {
+        const float* qv = q + (tid >> 5) * stride;
+        float t = 0.f;
 #pragma unroll 8
-          for (int h = lane; h < H; h += 32) t = __fadd_rn(t, qv[h]);
-          for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
-          if (lane == 0) Ts[tid >> 5] = t;
-        } else if (tid - 32 * NV < NV * deck) {
-          const int x = tid - 32 * NV, v = x / deck, c = x - v * deck;
-          const float* qv = q + v * stride;
-          float s = 0.f;
+        for (int h = lane; h < H; h += 32) t = __fadd_rn(t, qv[h]);
+        for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+        if (lane == 0) Ts[tid >> 5] = t;
+      } else if (tid - 32 * NV < NV * deck) {
+        const int x = tid - 32 * NV, v = x / deck, c = x - v * deck;
+        const float* qv = q + v * stride;
+        float s = 0.f;
 #pragma unroll 8
-          for (int j = cloff[c]; j < cloff[c + 1]; ++j) s = __fadd_rn(s, qv[clh[j]]);
-          Cs[v][c] = s;
-        }
-        __syncthreads();
-        for (int h = tid; h < H; h += kTermThreads) {
-          const unsigned cw = cards[h];
-          const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
-          const uint64_t own = (1ull << c1) | (k == 2 ? 1ull << c2 : 0ull);
-#pragma unroll
-          for (int v = 0; v < NV; ++v)
-            if (v < d.count) {
-              float m = __fsub_rn(Ts[v], Cs[v][c1]);
-              if (k == 2) m = __fadd_rn(__fsub_rn(m, Cs[v][c2]), q[v * stride + h]);
-              dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? 0.f : __fmul_rn(d.pay[i][v].hi, m);
-            }
-        }
-        continue;
+        for (int j = cloff[c]; j < cloff[c + 1]; ++j) s = __fadd_rn(s, qv[clh[j]]);
+        Cs[v][c] = s;
       }
+      __syncthreads();
+      for (int h = tid; h < H; h += kTermThreads) {
+        const unsigned cw = cards[h];
+        const unsigned c1 = cw & 0xffu, c2 = cw >> 8;
+        const uint64_t own = (1ull << c1) | (k == 2 ? 1ull << c2 : 0ull);
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          if (v < d.count) {
+            float m = __fsub_rn(Ts[v], Cs[v][c1]);
+            if (k == 2) m = __fadd_rn(__fsub_rn(m, Cs[v][c2]), q[v * stride + h]);
+            dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? 0.f : __fmul_rn(d.pay[i][v], m);
+          }
+      }
+      continue;
     }
-    {  // the reach in rank order (pair values' folds: in hand order) and along the card lists
+    {  // the reach in rank order and along the card lists
       VV a[kScanPer];
       VecAcc<P, NV> x;
 #pragma unroll
       for (int e = 0; e < kScanPer; ++e)
         if (e < cnt) {
-          const V* qe = q + (at[e / 2] >> (e & 1 ? 16 : 0) & 0xffffu);
+          const float* qe = q + (at[e / 2] >> (e & 1 ? 16 : 0) & 0xffffu);
 #pragma unroll
           for (int v = 0; v < NV; ++v) a[e].v[v] = qe[v * stride];
         }
       const int gtid = tid < gp ? tid : tid - gp;
-      scan_runs<P, NV>(a, cnt, red[tid >= gp], gtid, x);
+      auto entry = [&](int e) { return a[e]; };
+      scan_runs<P, NV, true>(entry, cnt, red[tid >= gp], gtid, x);
       __syncthreads();
       if (tid < gp)
-        scan_write<P, NV, gp>(a, begin, cnt, H, red[0], gtid, x, Ps);
+        scan_write<P, NV, gp, true>(entry, begin, cnt, H, red[0], gtid, x, Ps);
       else
-        scan_write<P, NV, kTermThreads - gp>(a, begin, cnt, k * H, red[1], gtid, x, CP);
+        scan_write<P, NV, kTermThreads - gp, true>(entry, begin, cnt, k * H, red[1], gtid, x, CP);
     }
     __syncthreads();
     for (int h = tid; h < H; h += kTermThreads) {
       const uint4 hr = __ldg(rec + h);
       const unsigned c1 = hr.x & 0xffu, c2 = (hr.x >> 8) & 0xffu;
       uint64_t own = 1ull << c1;
-      VV d0;
-      if (show) {
-        const VV T = Ps[H];
-        VV Wn = Ps[hr.x >> 16], Ln = Ps[hr.y & 0xffffu];
+      const VV T = Ps[H];
+      VV Wn = Ps[hr.x >> 16], Ln = Ps[hr.y & 0xffffu];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) Ln.v[v] = P::sub(T.v[v], Ln.v[v]);
-        auto one = [&](unsigned c, unsigned lo, unsigned hi) {
-          const VV a = CP[lo], a0 = CP[cloff[c]], z0 = CP[cloff[c + 1]], z = CP[hi];
+      for (int v = 0; v < NV; ++v) Ln.v[v] = P::sub(T.v[v], Ln.v[v]);
+      auto one = [&](unsigned c, unsigned lo, unsigned hi) {
+        const VV a = CP[lo], a0 = CP[cloff[c]], z0 = CP[cloff[c + 1]], z = CP[hi];
 #pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            Wn.v[v] = P::sub(Wn.v[v], P::sub(a.v[v], a0.v[v]));
-            Ln.v[v] = P::sub(Ln.v[v], P::sub(z0.v[v], z.v[v]));
-          }
-        };
-        one(c1, hr.y >> 16, hr.z & 0xffffu);
-        if (k == 2) {
-          one(c2, hr.z >> 16, hr.w & 0xffffu);
-          own |= 1ull << c2;
+        for (int v = 0; v < NV; ++v) {
+          Wn.v[v] = P::sub(Wn.v[v], P::sub(a.v[v], a0.v[v]));
+          Ln.v[v] = P::sub(Ln.v[v], P::sub(z0.v[v], z.v[v]));
         }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) d0.v[v] = P::sub(Wn.v[v], Ln.v[v]);
-      } else {  // pair values' folds
-        const VV T = Ps[H], a = CP[cloff[c1 + 1]], a0 = CP[cloff[c1]];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) d0.v[v] = P::sub(T.v[v], P::sub(a.v[v], a0.v[v]));
-        if (k == 2) {
-          own |= 1ull << c2;
-          const VV b = CP[cloff[c2 + 1]], b0 = CP[cloff[c2]];
-#pragma unroll
-          for (int v = 0; v < NV; ++v) d0.v[v] = P::add(P::sub(d0.v[v], P::sub(b.v[v], b0.v[v])), q[v * stride + h]);
-        }
+      };
+      one(c1, hr.y >> 16, hr.z & 0xffffu);
+      if (k == 2) {
+        one(c2, hr.z >> 16, hr.w & 0xffffu);
+        own |= 1ull << c2;
       }
 #pragma unroll
       for (int v = 0; v < NV; ++v)
         if (v < d.count)
-          dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? P::zero() : P::mul(P::scale(d.pay[i][v]), d0.v[v]);
+          dst[(size_t)d.node[v] * stride + h] = (d.board[v] & own) ? 0.f : P::mul(d.pay[i][v], P::sub(Wn.v[v], Ln.v[v]));
     }
   }
 }
@@ -2998,10 +3094,10 @@ size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es)
   return hand_smem_bytes(n_nodes, n_levels, rows_max, W, es);
 }
 
-size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv) {
+size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv, bool runs) {
   const TermTab tt(n_hands, hand_size, deck);
   const size_t scan = (size_t)(hand_size * n_hands + 1 + n_hands + 1);
-  if (nv == 1) return (size_t)tt.len * 2 + (size_t)hstride * es + scan * es;
+  if (nv == 1) return (size_t)tt.len * 2 + (size_t)(runs ? 2 : 1) * hstride * es + scan * es;
   return kTermSegment * sizeof(TermGroup) + (size_t)tt.fold_len * 2 + 2 * (size_t)nv * hstride * es + scan * nv * es;
 }
 
@@ -3050,8 +3146,7 @@ static cudaError_t configure_precision() {
   cudaError_t e = configure_hand<P, true>();
   if (e == cudaSuccess) e = configure_hand<P, false>();
   if (e == cudaSuccess) e = configure_one(k_terminal<P>, 200 * 1024);
-  if (e == cudaSuccess) e = configure_one(k_terminal_vec<P, 2>, 200 * 1024);
-  if (e == cudaSuccess && sizeof(typename P::V) == 4) e = configure_one(k_terminal_vec<Single, 4>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal_run<P>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_average_rows<P>, 0);
   if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false, false>, kTileSmem);
   if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false, false>, kTileSmem);
@@ -3077,6 +3172,8 @@ int set_first_wait_polls(long polls) {
 int configure_kernels() {
   cudaError_t e = configure_precision<Pairs>();
   if (e == cudaSuccess) e = configure_precision<Single>();
+  if (e == cudaSuccess) e = configure_one(k_terminal_vec<2>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal_vec<4>, 200 * 1024);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: kernel attribute setup failed: %s\n", cudaGetErrorString(e));
     return -1;
@@ -3307,11 +3404,18 @@ int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stre
     return launch_kernel(kernel, c.n_term_segments * players, kTermThreads, c.smem_term, stream, pdl, c.games,
                          c.term_groups, c.term_segments, c.n_term_segments, player_mask, use_bar, c.err);
   };
+  auto run = [&](auto kernel) {
+    return launch_kernel(kernel, c.n_term_runs * players, kTermThreads, c.smem_term, stream, pdl, c.games, c.term_work,
+                         c.term_src, c.term_runs, c.n_term_runs, player_mask, use_bar, c.err);
+  };
+  const bool single = c.precision == kPrecisionSingle;
   cudaError_t e;
-  if (c.precision == kPrecisionSingle)
-    e = c.term_nv == 4 ? vec(k_terminal_vec<Single, 4>) : c.term_nv == 2 ? vec(k_terminal_vec<Single, 2>) : one(k_terminal<Single>);
+  if (c.n_term_runs > 0)
+    e = single ? run(k_terminal_run<Single>) : run(k_terminal_run<Pairs>);
+  else if (c.term_nv > 1)
+    e = c.term_nv == 4 ? vec(k_terminal_vec<4>) : vec(k_terminal_vec<2>);
   else
-    e = c.term_nv == 2 ? vec(k_terminal_vec<Pairs, 2>) : one(k_terminal<Pairs>);
+    e = single ? one(k_terminal<Single>) : one(k_terminal<Pairs>);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_terminal failed: %s\n", cudaGetErrorString(e));
     return -1;

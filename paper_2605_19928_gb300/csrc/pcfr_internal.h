@@ -203,7 +203,7 @@ struct TermSrc {
 };
 __host__ __device__ inline int term_src_node(int32_t row) { return row < 0 ? ~row : row; }
 
-// Up to four terminal nodes of one game, board table and kind, evaluated together.
+// Up to four terminal nodes of one game, board table and kind, evaluated together (FP32 values).
 struct alignas(16) TermGroup {
   int32_t game;
   int32_t table;      // board table (folds read table 0)
@@ -213,10 +213,10 @@ struct alignas(16) TermGroup {
   int32_t node[4];
   TermSrc src[4];
   uint64_t board[4];
-  PairF pay[2][4];    // per player: payoff * kappa, negative where the player folded
+  float pay[2][4];    // per player: payoff * kappa, negative where the player folded
 };
-static_assert(sizeof(TermGroup) == 160, "TermGroup is 160 bytes");
-constexpr int kTermSegment = 16;  // groups a block of the grouped terminal launch walks at most
+static_assert(sizeof(TermGroup) == 128, "TermGroup is 128 bytes");
+constexpr int kTermSegment = 32;  // groups a block of the grouped terminal launch walks at most
 
 // Wide schedule: an inner node, and a node that makes a new reach row of one player.
 struct alignas(16) WideNode {
@@ -254,8 +254,11 @@ struct LaunchCtx {
   const Work* term_work;       // device [n_term_work]: (game, terminal node), grouped by game,
                                // board table and kind (folds, then showdowns)
   int n_term_work;
-  int term_nv;                 // nodes a block evaluates together: 1, or term_groups of up to 2 or 4
+  int term_nv;                 // nodes a block evaluates together: 1 (in runs when n_term_runs > 0), or
+                               // term_groups of up to 2 or 4
   const TermGroup* term_groups;   // device (term_nv > 1)
+  const Work* term_runs;       // device [n_term_runs]: (first entry of term_work, count), one block's (run form)
+  int n_term_runs;
   const Work* term_segments;      // device [n_term_segments]: (first group, count), one block's
   int n_term_segments;
   const TermSrc* term_src;     // device [n_term_work]: reach rows of each terminal
@@ -317,8 +320,8 @@ int launch_average_rows(const LaunchCtx& c, void* stream);
 // kModeBR, as the per-hand kernel's modes).
 int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advance);
 int hand_kernel_smem_limit();
-// Shared memory of one block of the terminal launch for one game (nv: LaunchCtx::term_nv).
-size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv);
+// Shared memory of one block of the terminal launch for one game (nv: LaunchCtx::term_nv; runs: its run form).
+size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv, bool runs);
 // Shared memory the per-hand kernel needs to stage one game (es = bytes per value).
 size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es);
 int configure_kernels();  // once per process, before the first launch
