@@ -88,7 +88,7 @@ struct TileHead {
   // at it, HostGame::reach_row), level by level; first of each level; levels
   int32_t fwd[2], flevel[2], flevels[2];
   int32_t all[2];              // per player: [n_nodes] reach_row
-  int32_t pad;
+  int32_t deal;                // uint8 [n_nodes] card dealt to each node (none without chance nodes)
 };
 static_assert(sizeof(TileHead) % 16 == 0, "the table's TileNodes start 16-byte aligned");
 // One inner node of a tile table, 8 bytes.

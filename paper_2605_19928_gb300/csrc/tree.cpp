@@ -776,6 +776,12 @@ std::vector<uint16_t> tile_table(const HostGame& g) {
     head.flevels[p] = (int32_t)flevel[p].size() - 1;
     head.all[p] = put(all[p].data(), all[p].size());
   }
+  std::vector<uint16_t> deal;
+  if (std::any_of(inner.begin(), inner.end(), [](const TileNode& t) { return t.kids >> 6 == 2; })) {
+    deal.resize(((size_t)N + 1) / 2);
+    for (int n = 0; n < N; ++n) reinterpret_cast<uint8_t*>(deal.data())[n] = g.nodes[(size_t)n].deal;
+  }
+  head.deal = put(deal.data(), deal.size());
   memcpy(out.data(), &head, sizeof head);
   out.resize((out.size() + 7) / 8 * 8, 0);
   return out;
