@@ -624,17 +624,18 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   }
   if (staged || resident) {
     bool fit = staged;
+    // a wave of blocks takes each phase in one step with 512 threads; more blocks overlap instead
+    const int threads = resident || chunks_of(chunk[0]) <= n_sms ? 512 : 256;
     for (int g = 0; g < n_games; ++g) {
       while (1 << tile_wlog[g] < chunk[g]) ++tile_wlog[g];
       if (tile_tabs[g].empty()) {
         fit = false;
         continue;
       }
-      tile_group[g] = tile_walkers(t->host[g], chunk[g]);
+      tile_group[g] = tile_walkers(t->host[g], chunk[g], threads);
       smem_tile = std::max(smem_tile, tile_bytes(g, tile_wlog[g], 1));
     }
-    // a wave of blocks takes each phase in one step with 512 threads; more blocks overlap instead
-    if (fit && smem_tile <= (size_t)kTileSmemStaged) tile_threads = chunks_of(chunk[0]) <= n_sms ? 512 : 256;
+    if (fit && smem_tile <= (size_t)kTileSmemStaged) tile_threads = threads;
   }
   const bool tiles = tile_threads > 0;
   RunoutPlan ro;

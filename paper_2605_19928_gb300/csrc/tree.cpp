@@ -787,14 +787,14 @@ std::vector<uint16_t> tile_table(const HostGame& g) {
   return out;
 }
 
-int tile_walkers(const HostGame& g, int W) {
+int tile_walkers(const HostGame& g, int W, int most) {
   int widest = 1;
   for (size_t l = 0; l + 1 < g.level_start.size(); ++l) {
     int cnt = 0;
     for (int n = g.level_start[l]; n < g.level_start[l + 1]; ++n) cnt += !is_terminal(g.nodes[(size_t)n]);
     widest = std::max(widest, cnt);
   }
-  return std::min((widest * W + 31) / 32 * 32, 256);
+  return std::min((widest * W + 31) / 32 * 32, most);
 }
 
 void plan_runouts(const HostGame& h, RunoutPlan& r) {

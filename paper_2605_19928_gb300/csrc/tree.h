@@ -93,8 +93,8 @@ std::vector<int32_t> stream_tables(const HostGame& g, const std::vector<int32_t>
 std::vector<uint16_t> tile_table(const HostGame& g);
 
 // Threads that walk the levels of a tile of W hands in the latency form: enough for the widest level in
-// one step, a multiple of 32 from 32 to 256.
-int tile_walkers(const HostGame& g, int W);
+// one step, a multiple of 32 up to `most`, the block's.
+int tile_walkers(const HostGame& g, int W, int most);
 
 // All-in run-outs of one game evaluated by win-minus-loss tables (runout.h): a run-out's top
 // is a chance node below a decision whose subtree holds only chance and showdown nodes, all of
