@@ -1064,6 +1064,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const int pairs = (h.n_hands + 1) / 2;  // two hands a thread, blocks of even size
     c.wide_segments = (pairs + 255) / 256;
     c.wide_threads = ((pairs + c.wide_segments - 1) / c.wide_segments + 31) / 32 * 32;
+    c.wide_pairs = pairs;
     int dmax = 0;
     for (int p = 0; p < 2; ++p) {
       int cnt = 0;

@@ -2934,24 +2934,38 @@ __global__ void k_average_rows(const GameDev* __restrict__ games, int n_games) {
 // ------------------------------------------------------------------ wide schedule
 //
 // For one tree too large to stage in shared memory, each pass of the per-hand kernel becomes one
-// launch per level over all of that level's (node, hand) pairs.  A block takes one node (or, when
-// its hands are more than 512, an even share of them), two consecutive hands a thread: the node's
-// description is one 16-byte load, branches are the block's, and rows are read and written 16
-// bytes a thread (FP64) or 8 (FP32 values).  The arithmetic per (node, hand) -- the order of every
-// sum over children, regret matching, the Stage 7 update -- is the per-hand kernel's, so the
-// schedules agree bit for bit.  Bound by DRAM where a level holds many nodes and by the launches'
-// latency where it does not.  Measured, one player's update with FP32 values: exact turn 355 -> 225 us,
-// learned flop 204 -> 144 us against one thread per (node, hand) that found its node by division
-// and stored every node's reach; average pass of the turn 278 -> 143, best response 192 -> 110.
-// Three blocks of 85 registers per SM (nodes of six actions and more spill) beat two without
-// spills (253 us).
+// launch per level over all of that level's (node, hand) pairs.  In the bottom-up step a block takes
+// one node (or, when its hands are more than 512, an even share of them), two consecutive hands a
+// thread: the node's description is one 16-byte load, branches are the block's, and rows are read and
+// written 16 bytes a thread (FP64) or 8 (FP32 values); the row passes lay the nodes' hands end to end
+// (wide_at).  The arithmetic per (node, hand) -- the order of every sum over children, regret matching,
+// the Stage 7 update -- is the per-hand kernel's, so the schedules agree bit for bit.  Bound by DRAM
+// where a level holds many nodes and by the launches' latency where it does not.  Measured, one
+// player's update with FP32 values: exact turn 354 -> 211 us, learned flop 204 -> 135 us against one
+// thread per (node, hand) that found its node by division and stored every node's reach; average pass
+// of the turn (both players) 271 -> 142, best response 190 -> 98.  Three blocks of 80 registers per SM
+// beat two without spills.
 
-constexpr int kWideThreads = 256;  // at most; LaunchCtx::wide_threads
+constexpr int kWideThreads = 256;  // at most (k_wide_back: LaunchCtx::wide_threads)
+constexpr int kWideKids = 8;
 
 template <typename P>
 struct alignas(2 * sizeof(typename P::V)) V2 {  // two consecutive hands' values
   typename P::V v[2];
 };
+
+// The node of a list and the first of the two hands of this thread of the passes that only read and
+// write rows: the nodes' `pairs` of hands laid end to end over the blocks.  (k_wide_back keeps a block
+// to a node: its branches and action counts differ from node to node.)  Average pass of the 31,124-node
+// flop of 12 hands 53 -> 20 us, of a 43,509-node turn of 200 hands 123 -> 92, against a block a node.
+struct WideAt {
+  int node, h;
+};
+__device__ __forceinline__ WideAt wide_at(int pairs) {
+  // (below 2^32: a node and pair of hands takes more than 64 bytes of device memory)
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x, node = e / (unsigned)pairs;
+  return {(int)node, 2 * (int)(e - node * (unsigned)pairs)};
+}
 
 // Two hands of a row; `both`: the second exists (it is not stored otherwise).
 template <typename T2, typename T>
@@ -2974,6 +2988,62 @@ __device__ __forceinline__ V2<P> wide_decision(const typename P::V* __restrict__
                                                double* __restrict__ Sp, double* __restrict__ Mp, size_t S,
                                                const Discount& d, int variant, bool both) {
   using V = typename P::V;
+  if constexpr (NA > 3) {
+    // more actions: their rows would not fit the registers, so each is read when its turn comes (the
+    // children's values and the strategy twice, the second time from L1).  Update of a 1,581-node river
+    // of 1,081 hands and up to 7 actions, FP32 values 69 -> 50 us, pairs 101 -> 80; exact turn 238 ->
+    // 226 (every row loaded first, spilling, before)
+    const bool plus = variant == 1 || variant == 3;
+    typename P::Acc a0 = P::acc0(), a1 = P::acc0();
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      const V2<P> s = load2<V2<P>>(sgp + (size_t)a * S), x = load2<V2<P>>(c + (size_t)a * S);
+      P::acc_mul(a0, s.v[0], x.v[0]);
+      P::acc_mul(a1, s.v[1], x.v[1]);
+    }
+    V2<P> val;
+    val.v[0] = P::value(a0), val.v[1] = P::value(a1);
+    const V2<P> pi = load2<V2<P>>(pip);
+    V2<P> y[NA];
+    V tot[2] = {P::zero(), P::zero()};
+    int npos[2] = {0, 0};
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      const V2<P> s = load2<V2<P>>(sgp + (size_t)a * S), x = load2<V2<P>>(c + (size_t)a * S);
+      double2 R = load2<double2>(Rp + (size_t)a * S), Sv = load2<double2>(Sp + (size_t)a * S), rd;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const double r = P::to_double(P::sub(x.v[j], val.v[j]));
+        const double contrib = P::to_double(P::mul(pi.v[j], s.v[j]));
+        double z = (j ? R.y : R.x) + r;
+        if (variant == 2) z *= __double_as_longlong(z) > 0 ? d.dpos : d.dneg;
+        if (plus && __double_as_longlong(z) < 0) z = 0.0;
+        (j ? Sv.y : Sv.x) = fma(j ? Sv.y : Sv.x, d.dS, plus ? d.wS * contrib : contrib);
+        (j ? R.y : R.x) = z;
+        (j ? rd.y : rd.x) = r;
+        const double m = variant == 3 ? z + r : z;  // Predictive CFR+ matches R + M
+        const V p = __double_as_longlong(m) > 0 ? P::of_double(m) : P::zero();
+        y[a].v[j] = p;
+        npos[j] += P::positive(p);
+        tot[j] = P::add(tot[j], p);
+      }
+      store2(Rp + (size_t)a * S, R, both);
+      store2(Sp + (size_t)a * S, Sv, both);
+      if (variant == 3) store2(Mp + (size_t)a * S, rd, both);
+    }
+    const V inv[2] = {P::recip(tot[0]), P::recip(tot[1])}, uni = P::uniform(NA);
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      V2<P> o;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const V z = y[a].v[j], many = P::mul(z, inv[j]);
+        o.v[j] = npos[j] > 1 ? many : npos[j] == 1 ? (P::positive(z) ? P::one() : P::zero()) : uni;
+      }
+      store2<P>(sgp + (size_t)a * S, o, both);
+    }
+    return val;
+  }
   V2<P> cc[NA], sg[NA];
   double2 R[NA], Sv[NA];
 #pragma unroll
@@ -3049,11 +3119,22 @@ __global__ void __launch_bounds__(kWideThreads, 3) k_wide_back(const GameDev* __
     // children values already carry the card probabilities; cards in the hand are out
     const uint64_t m0 = G.hand_mask[h], m1 = both ? G.hand_mask[h + 1] : 0ull;
     typename P::Acc a0 = P::acc0(), a1 = P::acc0();
-    for (int a = 0; a < A; ++a) {
-      const int deal = G.nodes[w.first_kid + a].deal;
-      const V2<P> x = load2<V2<P>>(c + (size_t)a * S);
-      if (!((m0 >> deal) & 1ull)) P::acc(a0, x.v[0]);
-      if (!((m1 >> deal) & 1ull)) P::acc(a1, x.v[1]);
+    // up to 49 children in one thread's sum: eight children's loads go out together (best response of the
+    // 31,124-node flop of 33 hands with pairs 93 -> 67 us)
+    for (int a = 0; a < A; a += kWideKids) {
+      int deal[kWideKids];
+      V2<P> x[kWideKids];
+#pragma unroll
+      for (int e = 0; e < kWideKids; ++e) {
+        const int k = min(a + e, A - 1);
+        deal[e] = G.nodes[w.first_kid + k].deal;
+        x[e] = load2<V2<P>>(c + (size_t)k * S);
+      }
+#pragma unroll
+      for (int e = 0; e < kWideKids; ++e) {
+        if (a + e < A && !((m0 >> deal[e]) & 1ull)) P::acc(a0, x[e].v[0]);
+        if (a + e < A && !((m1 >> deal[e]) & 1ull)) P::acc(a1, x[e].v[1]);
+      }
     }
     val.v[0] = P::value(a0), val.v[1] = P::value(a1);
   } else if (kind != p) {
@@ -3096,14 +3177,14 @@ __global__ void __launch_bounds__(kWideThreads, 3) k_wide_back(const GameDev* __
 // average S / sum S into sigbar (avg = 1), as the per-hand kernel computes them: positive parts in
 // the value type, their sum in action order.
 template <typename P>
-__global__ void __launch_bounds__(kWideThreads) k_wide_rows(const GameDev* __restrict__ games, int segments, int avg) {
+__global__ void __launch_bounds__(kWideThreads) k_wide_rows(const GameDev* __restrict__ games, int pairs, int avg) {
   using V = typename P::V;
   pdl_wait();
   pdl_trigger();
   const GameDev& G = games[0];
-  const int p = blockIdx.y, k = (int)(blockIdx.x / (unsigned)segments);
+  const WideAt at0 = wide_at(pairs);
+  const int p = blockIdx.y, k = at0.node, h0 = at0.h;
   const int db = G.dec_begin[p], ndec = G.dec_begin[p + 1] - db;
-  const int h0 = 2 * ((int)(blockIdx.x % (unsigned)segments) * (int)blockDim.x + (int)threadIdx.x);
   if (k >= ndec || h0 >= G.n_hands) return;
   const size_t S = (size_t)G.hstride;
   const NodeDev nd = G.nodes[G.dec_nodes[db + k]];
@@ -3131,12 +3212,12 @@ __global__ void __launch_bounds__(kWideThreads) k_wide_rows(const GameDev* __res
 template <typename P>
 __global__ void __launch_bounds__(kWideThreads) k_wide_fwd(const GameDev* __restrict__ games,
                                                            const WideReach* __restrict__ list0, int cnt0,
-                                                           const WideReach* __restrict__ list1, int cnt1, int segments,
+                                                           const WideReach* __restrict__ list1, int cnt1, int pairs,
                                                            int player_mask, int avg) {
   using V = typename P::V;
   const int p = player_mask == 3 ? (int)blockIdx.y : (player_mask == 1 ? 0 : 1);
-  const int k = (int)(blockIdx.x / (unsigned)segments);
-  const int h = 2 * ((int)(blockIdx.x % (unsigned)segments) * (int)blockDim.x + (int)threadIdx.x);
+  const WideAt at0 = wide_at(pairs);
+  const int k = at0.node, h = at0.h;
   if (k >= (p ? cnt1 : cnt0)) return;  // (a launch's blocks may leave before its trigger)
   const WideReach w = (p ? list1 : list0)[k];
   pdl_wait();
@@ -3354,6 +3435,11 @@ static cudaError_t launch_wide(void (*kernel)(KArgs...), unsigned blocks, int pl
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Blocks of the row passes over cnt nodes (wide_at).
+static unsigned wide_blocks(const LaunchCtx& c, int cnt) {
+  return (unsigned)(((size_t)cnt * c.wide_pairs + kWideThreads - 1) / kWideThreads);
+}
+
 template <int MODE, typename P>
 static cudaError_t wide_backward(const LaunchCtx& c, int player_mask, void* stream) {
   const int players = player_mask == 3 ? 2 : 1;
@@ -3380,9 +3466,9 @@ static cudaError_t wide_forward(const LaunchCtx& c, int player_mask, int avg, in
     const int c0 = player_mask & 1 ? wide_fwd_count(c, 0, d) : 0, c1 = player_mask & 2 ? wide_fwd_count(c, 1, d) : 0;
     const int cnt = c0 > c1 ? c0 : c1;
     if (cnt == 0) continue;
-    const cudaError_t e = launch_wide(k_wide_fwd<P>, (unsigned)cnt * c.wide_segments, players, c.wide_threads, stream,
+    const cudaError_t e = launch_wide(k_wide_fwd<P>, wide_blocks(c, cnt), players, kWideThreads, stream,
                                       c.pdl != 0, c.games, c.wide_fwd[0] + (c0 ? c.wide_fwd_off[0][d] : 0), c0,
-                                      c.wide_fwd[1] + (c1 ? c.wide_fwd_off[1][d] : 0), c1, c.wide_segments, player_mask, avg);
+                                      c.wide_fwd[1] + (c1 ? c.wide_fwd_off[1][d] : 0), c1, c.wide_pairs, player_mask, avg);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -3391,8 +3477,8 @@ static cudaError_t wide_forward(const LaunchCtx& c, int player_mask, int avg, in
 template <typename P>
 static cudaError_t wide_rows(const LaunchCtx& c, int avg, void* stream) {
   // rows of both players: the larger player's decision-node count sizes the grid
-  return launch_wide(k_wide_rows<P>, (unsigned)c.wide_max_dec * c.wide_segments, 2, c.wide_threads, stream, c.pdl != 0,
-                     c.games, c.wide_segments, avg);
+  return launch_wide(k_wide_rows<P>, wide_blocks(c, c.wide_max_dec), 2, kWideThreads, stream, c.pdl != 0, c.games,
+                     c.wide_pairs, avg);
 }
 
 template <typename P>

@@ -297,8 +297,9 @@ struct LaunchCtx {
   int wide_fwd_levels[2];
   const int* wide_fwd_off[2];  // host [wide_fwd_levels + 1]
   const WideReach* wide_fwd[2];  // device
-  int wide_segments;           // blocks per node, and
-  int wide_threads;            // threads of each (two hands a thread)
+  int wide_pairs;              // pairs of hands: a thread takes one
+  int wide_segments;           // k_wide_back: blocks per node, and
+  int wide_threads;            // threads of each
   int wide_max_dec;            // decision nodes of the player who has more
   // resident schedule (cfr_iterate only; the other passes use the level schedule's kernels)
   int resident;                // cfr_iterate runs k_resident
