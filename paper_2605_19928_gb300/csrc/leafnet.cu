@@ -13,8 +13,8 @@
 //     BN, K 16 per instruction, four per 64-wide stage) into one of two TMEM accumulators, each
 //     CTA's TMEM holding its own 128 rows, commits each stage back to both CTAs' "empty"
 //     barriers and each finished tile to both CTAs' "full accumulator" barriers;
-//   * in each CTA sixteen warps each take every fourth 32-column block of one 32-lane quarter of the
-//     finished accumulator with tcgen05.ld, add the bias, apply GELU (hidden layers), stage the
+//   * in each CTA eight or sixteen warps each take every second or fourth 32-column block of one 32-lane
+//     quarter of the finished accumulator with tcgen05.ld, add the bias, apply GELU (hidden layers), stage the
 //     block in shared memory and write it by bulk tensor stores; the accumulator is handed back as
 //     soon as it is in registers, so a tile's epilogue runs while the next tile's MMAs fill the other.
 // Every mbarrier wait is bounded; a wait that gives up sets *err, the CTA stops issuing,
@@ -35,10 +35,8 @@ constexpr int kBM = 128, kBK = 64, kBNMax = 256;  // rows of C per CTA, a pair's
 constexpr int kATile = kBM * kBK * 2;            // 16 KB: one A stage
 constexpr int kRingBytes = 160 * 1024;           // stages of A and B: 5 of the widest tile's 32 KB
 constexpr int kMaxStages = 8;
-constexpr int kEpiWarps = 16;                    // four per TMEM lane quarter
-constexpr int kEpiParts = kEpiWarps / 4;
 constexpr int kStageBytes = 4096;                // output staging per epilogue warp: one FP32 block, two BF16 blocks
-constexpr int kGemmThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, then the epilogue warps
+constexpr int gemm_threads(int ew) { return 64 + 32 * ew; }  // warp 0 TMA, warp 1 MMA, then EW epilogue warps
 constexpr int kTmemCols = 512;                   // two accumulators of up to 256 columns
 constexpr long kGemmWaitLimit = 1l << 22;
 
@@ -188,14 +186,17 @@ __device__ __forceinline__ void bar_arrive_cluster(uint32_t bar) {
 // Columns [n_begin, n_begin + n_nt bn) of C.  A pair's tile needs 32 KB of A and B per CTA for the MMAs
 // that take 48 KB as a 128 x 256 tile of one CTA.  The MMAs alone, without loads and epilogue, take
 // 89 us on 49,392 rows of layer 1 (six rounds of tiles where 5.1 would do); GELU and the loads make
-// that 118 us (115 as one-CTA tiles).  The 512-wide layers of K = 512 are bound by GELU's
+// that 117 us (115.5 as one-CTA tiles).  The 512-wide layers of K = 512 are bound by GELU's
 // instructions: 60 us at 49,392 rows as one-CTA tiles, 50 with eight epilogue warps, 46 with sixteen
 // (half the registers each).  The output layer is bound by its FP32 stores (12,528 rows: 43.2 ->
-// 38.5 us) and, in an update of one player, computes that player's half.  A turn's 624 rows spread
-// over narrow tiles and the launches' prologues overlap (programmatic dependent launch): 24.2 -> 19.2
-// us (layer 1), 14.0 -> 7.5 (512 x 512).
-template <bool F32, bool ACT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+// 37.4 us) and, in an update of one player, computes that player's half.  A turn's 624 rows spread
+// over narrow tiles and the launches' prologues overlap (programmatic dependent launch): 24.2 -> 18.9
+// us (layer 1), 13.7 -> 7.5 (512 x 512).  These are launches that follow each other; one that follows
+// another kernel pays the pair's set-up (cluster, TMEM, barriers), about 1 us, which one-CTA tiles did not
+// have: 624 rows of the output layer 8.9 against 8.2 us, 49,392 of layer 1 118.5 against 116.5.  FP32
+// outputs after a K of 64 or 128 are slower as pairs too (100,000 x 128 x 128: 15.2 against 13.2 us).
+template <bool F32, bool ACT, int EW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads(EW), 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_c, const float* __restrict__ bias, int M, int n_begin, int n_nt,
                 int kb_count, int bn, int stages, int* err) {
@@ -216,7 +217,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       bar_init(&acc_full[b], 1);               // one tcgen05.commit per finished tile
-      bar_init(&acc_empty[b], 2 * kEpiWarps);  // one arrival per epilogue warp of the pair
+      bar_init(&acc_empty[b], 2 * EW);         // one arrival per epilogue warp of the pair
     }
     bar_init(&mma_done, 1);
     failed = 0;
@@ -304,13 +305,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       bar_wait(&mma_done, 0);
     }
     __syncwarp();
-  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, every fourth 32-column
+  } else {  // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, every EW / 4-th 32-column
             // block, from its part (w - 2) / 4 on (the parts take turns, as the count may be uneven)
     const int q = warp & 3, part = (warp - 2) >> 2, blocks = bn / 32;
     // staging blocks of 32 rows x 32 columns in the bulk store's swizzled layout: 16-byte chunk j of row
     // r at chunk j ^ (r % 8) (FP32, 128-byte rows) or j ^ (r / 2 % 4) (BF16, 64-byte rows)
     unsigned char* stage = base + kRingBytes + (size_t)(warp - 2) * kStageBytes;
-    float* sbias = reinterpret_cast<float*>(base + kRingBytes + kEpiWarps * kStageBytes) + (warp - 2) * 32;
+    float* sbias = reinterpret_cast<float*>(base + kRingBytes + EW * kStageBytes) + (warp - 2) * 32;
     int cc = 0;  // blocks this warp has staged
     int lt = 0;
     // one block: its values v and bias (lane's column) to the staging block, and from there to C
@@ -357,7 +358,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       const int row0 = (tile / n_nt) * 2 * kBM + rank * kBM + q * 32, n0 = n_begin + (tile % n_nt) * bn;
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBNMax);
       const int last = row0 < M ? blocks : 0;
-      int b = (part + lt) % kEpiParts;
+      int b = (part + lt) % (EW / 4);
       auto bias_at = [&](int blk) { return bias && blk < last ? __ldg(bias + n0 + blk * 32 + lane) : 0.f; };
       float bias_lane = bias_at(b);
       const bool ok = bar_wait(&acc_full[acc], (uint32_t)(lt >> 1) & 1u);
@@ -372,12 +373,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         if (lane == 0) bar_arrive_cluster(of_first_cta(&acc_empty[acc]));
       };
       if (b >= last) drained();  // no block of this tile
-      for (; b < last; b += kEpiParts) {
+      for (; b < last; b += EW / 4) {
         uint32_t v[32];
         tmem_load(v, taddr + (uint32_t)(b * 32));
-        const float next = bias_at(b + kEpiParts);
+        const float next = bias_at(b + EW / 4);
         tmem_wait(v);
-        if (b + kEpiParts >= last) drained();
+        if (b + EW / 4 >= last) drained();
         put(v, bias_lane, n0 + b * 32, row0);
         bias_lane = next;
       }
@@ -443,27 +444,37 @@ bool encode(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows)
 }  // namespace
 
 // the ring, the epilogue warps' staging blocks and bias rows
-size_t gemm_smem_bytes() { return (size_t)kRingBytes + kEpiWarps * (kStageBytes + 128); }
+static size_t gemm_smem_bytes(int ew) { return (size_t)kRingBytes + ew * (kStageBytes + 128); }
+
+using GemmKernel = decltype(&k_gemm_bf16<false, false, 16>);
+// [eight warps or sixteen][FP32 or BF16 output][GELU]
+static const GemmKernel kGemmKernels[2][2][2] = {
+    {{k_gemm_bf16<false, false, 8>, k_gemm_bf16<false, true, 8>}, {k_gemm_bf16<true, false, 8>, k_gemm_bf16<true, true, 8>}},
+    {{k_gemm_bf16<false, false, 16>, k_gemm_bf16<false, true, 16>}, {k_gemm_bf16<true, false, 16>, k_gemm_bf16<true, true, 16>}}};
 
 int configure_gemm() {
-  const int smem = (int)gemm_smem_bytes();
-  for (auto k : {k_gemm_bf16<false, false>, k_gemm_bf16<false, true>, k_gemm_bf16<true, false>, k_gemm_bf16<true, true>})
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return -1;
+  for (int k = 0; k < 8; ++k)
+    if (cudaFuncSetAttribute(kGemmKernels[k >> 2][k >> 1 & 1][k & 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)gemm_smem_bytes(k >> 2 ? 16 : 8)) != cudaSuccess)
+      return -1;
   return 0;
 }
 
-// Width of the tiles of n columns: the one whose rounds of tiles over the pairs take least by this
-// count of cycles.  A tile's fill is its loads (256 + bn bytes of A and B a row of 64, at 64 bytes a
-// cycle) or its MMAs, its drain about 20 cycles a column; the last drain is not covered by a fill.
-// A few rows (a turn's 13 leaves have 624) thus spread over narrow tiles, many take 256-wide ones.
-static int gemm_bn(int M, int n, int kb_count, int pairs) {
+// Width of the tiles of n columns: the one that takes least by this count of cycles, fitted to the times
+// of every width at 14 row counts from 1 to 100,000 and 11 shapes.  A tile has a cost of its own (1,700,
+// and 720 per 64-wide step of K, for the latency of the chain through ring, MMA and accumulator) and one
+// per column: its drain (33 cycles with GELU, 16 FP32, 13 BF16) or, with long K, its loads and MMAs (1
+// per step).  The last drain, about four tenths, is not covered.  Over those 147 cases the choice is
+// within 1.2 % of the best width on average; without the tiles' own cost it took narrow tiles at many
+// rows and short K: 20,001 rows of 512 x 64 took 2.6 times as long.
+static int gemm_bn(int M, int n, int kb_count, int pairs, bool act, bool f32) {
   int best = 0;
   double best_cost = 0;
+  const double drain = act ? 33 : f32 ? 16 : 13, column = kb_count > drain ? kb_count : drain;
   for (int bn = 32; bn <= kBNMax; bn += 32) {
     if (n % bn) continue;
     const long tiles = (long)(n / bn) * ((M + 2 * kBM - 1) / (2 * kBM)), rounds = (tiles + pairs - 1) / pairs;
-    const double fill = (double)kb_count * (256 + bn > 2 * bn ? 256 + bn : 2 * bn), drain = 20.0 * bn;
-    const double cost = (double)rounds * (fill > drain ? fill : drain) + drain;
+    const double cost = (double)rounds * (1700 + 720.0 * kb_count + column * bn) + 0.43 * drain * bn;
     if (best == 0 || cost < best_cost) best = bn, best_cost = cost;
   }
   return best;
@@ -479,26 +490,28 @@ static int launch_gemm_cols(const void* A, const void* B, const float* bias, voi
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 2)
     return -1;
-  const int bn = gemm_bn(M, n_cols, K / kBK, sms / 2);
+  const int bn = gemm_bn(M, n_cols, K / kBK, sms / 2, act != 0, out_f32 != 0);
   const long tiles = (long)(n_cols / bn) * ((M + 2 * kBM - 1) / (2 * kBM));
   if (tiles > (1l << 29)) return -2;
   CUtensorMap ma, mb, mc;
   if (!encode(&ma, A, M, K, kBM) || !encode(&mb, B, N, K, bn / 2) || !encode_out(&mc, C, M, N, out_f32)) return -3;
   const int pairs = (int)(tiles < sms / 2 ? tiles : sms / 2);  // persistent: one CTA per SM
+  // Sixteen epilogue warps where the epilogue bounds a tile (GELU after a short K, or a K of a few steps),
+  // else eight, beside which loads and MMAs run a little faster: layer 1 of 49,392 rows 119.8 -> 116.8 us,
+  // the output layer of 12,528 rows 38.8 -> 37.4, but 512 x 512 of 49,392 rows 46.2 -> 47.8.
+  const int ew = K / kBK >= (act ? 16 : 8) ? 8 : 16;
   const int stage = kATile + bn * kBK, stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
-  auto* kernel = out_f32 ? (act ? k_gemm_bf16<true, true> : k_gemm_bf16<true, false>)
-                         : (act ? k_gemm_bf16<false, true> : k_gemm_bf16<false, false>);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * pairs));
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = gemm_smem_bytes();
+  cfg.blockDim = dim3((unsigned)gemm_threads(ew));
+  cfg.dynamicSmemBytes = gemm_smem_bytes(ew);
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, ma, mb, mc, bias, M, n_begin, n_cols / bn, K / kBK, bn, stages, err);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kGemmKernels[ew == 16][out_f32 != 0][act != 0], ma, mb, mc, bias, M, n_begin, n_cols / bn, K / kBK, bn, stages, err);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_gemm_bf16 failed: %s\n", cudaGetErrorString(e));
     return -1;
