@@ -500,53 +500,46 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     if (all_fit) smem_hand = std::max(smem_hand, hand_smem(h, chunk[g], es));
   }
 
-  // Update schedule: one warp per 32 hands when the handle has enough of them to fill the
-  // GPU (8 warps per SM) and every tree fits the warp's registers and stack.
-  std::vector<std::vector<int32_t>> programs(n_games);
-  std::vector<std::array<int, 4>> prog_meta(n_games);  // depth, max actions, fits, max loads of a node
-  parallel_games(n_games, [&](int g) {
-    int depth = 0, amax = 0, loads = 0;
-    bool fits = false;
-    programs[g] = dfs_program(t->host[g], &depth, &amax, &fits);
-    for (int n : programs[g])
-      for (int p = 0; p < 2; ++p)
-        loads = std::max(loads, (int)node_loads(t->host[g], n, p, true, (uint32_t)t->host[g].hstride,
-                                                o.variant == CFR_VARIANT_PCFRPLUS).size());
-    prog_meta[g] = {depth, amax, fits ? 1 : 0, loads};
-  });
-  int stream_depth = 1, stream_warps = 0, actions_max = 0;
-  bool stream_ok = true;
+  // Update schedule: the stream schedule when the handle has enough hands to fill the GPU (8 warps of 32
+  // per SM) and every tree fits a warp's registers and stack.  Only a handle that may take it needs the
+  // trees' programs, and only one that walks them (below) their load tables.
+  int stream_warps = 0, actions_max = 0;
   for (int g = 0; g < n_games; ++g) {
-    stream_ok = stream_ok && prog_meta[g][2];
-    stream_depth = std::max(stream_depth, prog_meta[g][0]);
-    actions_max = std::max(actions_max, prog_meta[g][1]);
-    stream_ok = stream_ok && prog_meta[g][1] <= kStreamMaxActions;
     stream_warps += (t->host[g].n_hands + 31) / 32;
+    for (const NodeDev& nd : t->host[g].nodes)
+      if (nd.type == kDecision) actions_max = std::max(actions_max, (int)nd.n_kids);
   }
-  // the program of the largest tree is staged in shared memory when it takes at most 64 KB
-  int max_prog = 0, max_loads = 0;
+  const bool pred = o.variant == CFR_VARIANT_PCFRPLUS;
+  bool stream_ok = o.schedule == CFR_SCHEDULE_STREAM || (o.schedule == CFR_SCHEDULE_AUTO && stream_warps >= 8 * 152);
+  std::vector<std::vector<int32_t>> programs(n_games);
+  struct ProgramMeta {
+    int depth = 1, max_loads = 0, units[4] = {0, 0, 0, 0};
+    bool fits = true;
+  };
+  std::vector<ProgramMeta> prog_meta(n_games);
+  if (stream_ok)
+    parallel_games(n_games, [&](int g) {
+      ProgramMeta& m = prog_meta[g];
+      int amax = 0;
+      programs[g] = dfs_program(t->host[g], &m.depth, &amax, &m.fits);
+      stream_counts(t->host[g], programs[g], pred, m.units, &m.max_loads);
+    });
+  stream_ok = stream_ok && actions_max <= kStreamMaxActions;
+  // the program of the largest tree is staged in shared memory when it takes at most 64 KB, with its
+  // load tables (units per player: both passes)
+  int stream_depth = 1, max_prog = 0, max_loads = 0, stream_units_max = 0;
   for (int g = 0; g < n_games; ++g) {
+    const ProgramMeta& m = prog_meta[g];
+    stream_ok = stream_ok && m.fits;
+    stream_depth = std::max(stream_depth, m.depth);
     max_prog = std::max(max_prog, (int)programs[g].size());
-    max_loads = std::max(max_loads, prog_meta[g][3]);
-  }
-  const int stream_prog = max_prog * (int)sizeof(ProgOp) <= 64 * 1024 ? max_prog : 0;
-  const int stream_half = std::max(kStreamHalfMin, max_loads);
-  // load tables of every game (units per player: both passes), and their largest size
-  std::vector<std::vector<uint32_t>> unit_lists(n_games);
-  std::vector<std::vector<int32_t>> chunk_lists(n_games);
-  std::vector<std::array<int, 16>> table_meta(n_games);
-  int stream_units_max = 0;
-  parallel_games(n_games, [&](int g) {
-    std::array<int, 16>& m = table_meta[g];
-    chunk_lists[g] = stream_tables(t->host[g], programs[g], stream_half, o.variant == CFR_VARIANT_PCFRPLUS,
-                                   unit_lists[g], &m[0], &m[4], &m[8], &m[12]);
-  });
-  for (int g = 0; g < n_games; ++g) {
-    const std::array<int, 16>& m = table_meta[g];
-    for (int p = 0; p < 2; ++p) stream_units_max = std::max(stream_units_max, m[4 + p] + m[4 + 2 + p]);
+    max_loads = std::max(max_loads, m.max_loads);
+    for (int p = 0; p < 2; ++p) stream_units_max = std::max(stream_units_max, m.units[p] + m.units[2 + p]);
     const size_t span = std::max(t->host[g].nodes.size(), (size_t)t->host[g].n_rows) * (size_t)t->host[g].hstride;
     stream_ok = stream_ok && span < (1u << kArrShift);
   }
+  const int stream_prog = max_prog * (int)sizeof(ProgOp) <= 64 * 1024 ? max_prog : 0;
+  const int stream_half = std::max(kStreamHalfMin, max_loads);
   stream_units_max = (stream_units_max + 3) / 4 * 4;  // keeps the ring 16-byte aligned
   const int stream_units = stream_prog ? stream_units_max : 0;
   // hands per lane: one (32 per warp) unless the options ask for 64 per warp.  Two per lane
@@ -572,7 +565,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
                                   " actions per decision node and a stack that fits shared memory");
     }
     schedule = kScheduleStream;
-  } else if (o.schedule == CFR_SCHEDULE_AUTO && stream_ok && stream_warps >= 8 * 152) {
+  } else if (o.schedule == CFR_SCHEDULE_AUTO && stream_ok) {
     schedule = kScheduleStream;
   }
   // Wide schedule: one subgame whose tree a block cannot stage (the per-hand pass would walk
@@ -603,12 +596,19 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   std::vector<int> tile_wlog(n_games, 0), tile_group(n_games, 0);
   size_t smem_tile = 0;
   int tile_threads = 0;
-  if (stream_tiles || staged || resident) parallel_games(n_games, [&](int g) { tile_tabs[g] = tile_table(t->host[g]); });
   auto tile_bytes = [&](int g, int wl, int with_rs) {
     const HostGame& h = t->host[g];
     const int rows_max = std::max(h.row_begin[1] - h.row_begin[0], h.row_begin[2] - h.row_begin[1]);
     return tile_smem_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, 1 << wl, es, with_rs);
   };
+  // (no tables where a tree is too large for a tile even without one)
+  auto too_large = [&](int g) {
+    return stream_tiles ? tile_bytes(g, 3, 0) > (size_t)kTileSmem
+                        : !resident && tile_bytes(g, __builtin_ctz((unsigned)chunk[g]), 1) > (size_t)kTileSmemStaged;
+  };
+  bool tabled = stream_tiles || staged || resident;
+  for (int g = 0; g < n_games; ++g) tabled = tabled && !too_large(g);
+  if (tabled) parallel_games(n_games, [&](int g) { tile_tabs[g] = tile_table(t->host[g]); });
   for (int small = es == 4; stream_tiles && small >= 0 && !tile_threads; --small) {
     const size_t limit = small ? kTileSmemSmall : kTileSmem;
     bool fit = true;
@@ -637,7 +637,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     }
     if (fit && smem_tile <= (size_t)kTileSmemStaged) tile_threads = threads;
   }
-  const bool tiles = tile_threads > 0;
+  const bool tiles = tile_threads > 0, walk = schedule == kScheduleStream && !tiles;
   RunoutPlan ro;
   if (o.runout_tables) {
     if (schedule != kScheduleWide || t->host[0].hand_size != 2) {
@@ -653,7 +653,6 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // Resident schedule: one block per SM holds a chunk's state of both players beside a terminal
   // node's board table, and every chunk has a block.
   size_t res_term = 0, res_hand = 0;
-  bool tabled = true;
   if (resident) {
     for (int g = 0; g < n_games; ++g) {
       const HostGame& h = t->host[g];
@@ -747,8 +746,12 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     std::vector<float> rv, pay32;
     std::vector<uint16_t> tab, rec, tile;
     std::vector<int32_t> rown, decn;
-    std::vector<ProgOp> ops;
     int dec_begin[3];
+    // where the tree is walked: its program and load tables
+    std::vector<ProgOp> ops;
+    std::vector<uint32_t> units;
+    std::vector<int32_t> chunks;
+    int unit_off[4], unit_count[4], chunk_off[4], chunk_count[4];
   };
   std::vector<Prepared> prep(n_games);
   parallel_games(n_games, [&](int g) {
@@ -771,9 +774,22 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       q.pay32[2 * n] = (float)x;
       q.pay32[2 * n + 1] = (float)(x - (double)q.pay32[2 * n]);
     }
-    q.ops = program_ops(h, programs[g]);
+    if (walk) {
+      q.ops = program_ops(h, programs[g]);
+      q.chunks = stream_tables(h, programs[g], stream_half, pred, q.units, q.unit_off, q.unit_count, q.chunk_off, q.chunk_count);
+    }
   });
   Packer packer;
+  size_t table_bytes = 0;  // reserved at once: growing would copy the tables of hundreds of games again and again
+  for (int g = 0; g < n_games; ++g) {
+    const HostGame& h = t->host[g];
+    const Prepared& q = prep[g];
+    table_bytes += 14 * 256 + h.nodes.size() * (sizeof(NodeDev) + 8) + (h.level_start.size() + q.rown.size() + q.decn.size()) * 4 +
+                   (h.hand_mask.size() + q.r64.size()) * 8 + (q.rv.size() + q.pay32.size()) * 4 +
+                   (q.tab.size() + q.rec.size() + q.tile.size()) * 2 + q.ops.size() * sizeof(ProgOp) +
+                   (q.units.size() + q.chunks.size()) * 4;
+  }
+  packer.stage.reserve(table_bytes);
   packer.zeroed((size_t)2 * n_games * sizeof(double), &t->d_br_all);
   t->dev.resize(n_games);  // not resized again: the packer holds the addresses of its fields
   for (int g = 0; g < n_games; ++g) {
@@ -803,12 +819,11 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const std::vector<int32_t>& rown = q.rown;
     const std::vector<int32_t>& decn = q.decn;
     const std::vector<float>& pay32 = q.pay32;
-    const std::vector<ProgOp>& ops = q.ops;
-    for (int q = 0; q < 4; ++q) {
-      d.unit_off[q] = table_meta[g][q];
-      d.unit_count[q] = table_meta[g][4 + q];
-      d.chunk_off[q] = table_meta[g][8 + q];
-      d.chunk_count[q] = table_meta[g][12 + q];
+    for (int k = 0; walk && k < 4; ++k) {
+      d.unit_off[k] = q.unit_off[k];
+      d.unit_count[k] = q.unit_count[k];
+      d.chunk_off[k] = q.chunk_off[k];
+      d.chunk_count[k] = q.chunk_count[k];
     }
     packer.table(h.nodes, &d.nodes);
     packer.table(h.level_start, &d.level_start);
@@ -825,10 +840,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     d.tile_wlog = tile_wlog[g];
     d.tile_group = tile_group[g];
     packer.table(decn, &d.dec_nodes);
-    packer.table(ops, &d.prog);
-    packer.table(chunk_lists[g], &d.chunks);
-    packer.table(unit_lists[g], &d.units);
-    d.prog_len = (int)programs[g].size();
+    packer.table(q.ops, &d.prog);
+    packer.table(q.chunks, &d.chunks);
+    packer.table(q.units, &d.units);
+    d.prog_len = (int)q.ops.size();
     const size_t rows = (size_t)h.n_rows * S, cells = 2 * N * S;
     packer.zeroed(rows * 8, &d.R);
     packer.zeroed(rows * 8, &d.S);
@@ -992,7 +1007,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     for (int u = 0; tiles && u << tile_wlog[g] < t->host[g].n_hands; ++u) tile_work.push_back({g, u});
   const int warp_span = 32 * stream_hp;
   for (int g : by_size)
-    for (int u = 0; u < (t->host[g].n_hands + warp_span - 1) / warp_span; u += kStreamWarps) warp_work.push_back({g, u});
+    for (int u = 0; walk && u < (t->host[g].n_hands + warp_span - 1) / warp_span; u += kStreamWarps) warp_work.push_back({g, u});
   if ((rc = upload(t, t->dev, &t->d_games)) || (rc = upload(t, chunk_work, &t->d_chunk_work)) ||
       (rc = upload(t, term_work, &t->d_term_work)) || (rc = upload(t, warp_work, &t->d_warp_work)) ||
       (rc = upload(t, term_src, &t->d_term_src)) ||

@@ -679,6 +679,23 @@ std::vector<int32_t> stream_tables(const HostGame& g, const std::vector<int32_t>
   return chunks;
 }
 
+void stream_counts(const HostGame& g, const std::vector<int32_t>& pre, bool pred, int unit_count[4], int* max_loads) {
+  *max_loads = 0;
+  for (int q = 0; q < 4; ++q) unit_count[q] = 0;
+  for (int n : pre) {
+    const NodeDev& nd = g.nodes[(size_t)n];
+    int ends = 0;  // the bottom-up passes load the values of the terminal children
+    for (int a = 0; a < nd.n_kids; ++a) ends += is_terminal(g.nodes[(size_t)(nd.first_kid + a)]);
+    for (int p = 0; p < 2; ++p) {
+      const bool own = nd.type == kDecision && nd.player == p;
+      const int back = ends + (own ? (pred ? 3 : 2) * nd.n_kids + 1 : 0);
+      unit_count[p] += back;
+      unit_count[2 + p] += own ? (pred ? 2 : 1) * nd.n_kids : 0;
+      *max_loads = std::max(*max_loads, back);
+    }
+  }
+}
+
 std::vector<uint32_t> node_loads(const HostGame& g, int n, int p, bool backward, uint32_t S, bool pred) {
   std::vector<uint32_t> mine;
   const NodeDev& nd = g.nodes[(size_t)n];

@@ -86,6 +86,10 @@ std::vector<int32_t> stream_tables(const HostGame& g, const std::vector<int32_t>
                                    std::vector<uint32_t>& units, int unit_off[4], int unit_count[4],
                                    int chunk_off[4], int chunk_count[4]);
 
+// What stream_tables would list, counted: the units of each of its four passes, and the most loads one
+// node of the bottom-up passes has.
+void stream_counts(const HostGame& g, const std::vector<int32_t>& pre, bool pred, int unit_count[4], int* max_loads);
+
 // The hand-tile table of one subgame (TileHead and its lists, pcfr_internal.h), or empty when its
 // tree does not suit them (node or row ids beyond 16 bits).
 // Nodes of one level are ordered by kind and action count, so that the slots sharing a warp take the

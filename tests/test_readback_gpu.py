@@ -100,3 +100,15 @@ def test_a_read_that_launches_reports_a_wait_that_gave_up():
             capi.cfr_debug_first_wait_polls(-1)
     finally:
         capi.cfr_tree_destroy(tree)
+
+
+def test_only_walked_trees_upload_their_programs():
+    spec = synth.river_subgame(n_hands=64, seed=3, range_seed=4)
+    sent = {}
+    for schedule, warp_hands, chunk in (("level", 0, 2), ("stream", 0, 0), ("stream", 64, 0)):
+        opts = capi.make_opts("dcfr", precision="single", schedule=schedule, warp_hands=warp_hands, chunk_hands=chunk)
+        tree = capi.cfr_tree_create(spec, opts)
+        sent[schedule, warp_hands] = capi.cfr_counters(tree)["h2d_bytes"]
+        capi.cfr_tree_destroy(tree)
+    # the per-hand kernels' handle sends less than the one that walks its tree, although its chunks are more
+    assert sent["level", 0] < sent["stream", 64]
