@@ -1279,8 +1279,9 @@ int cfr_strategy(cfr_tree* t, int game, int node, int average, float* out, size_
     t->launches += 1;
     t->avg_gen = t->state_gen;
   }
-  if (!average && t->ctx.schedule == kScheduleStream && t->cur_gen != t->state_gen) {
-    // the stream schedule keeps no strategy rows: regret-match R for the read-back
+  if (!average && t->ctx.schedule == kScheduleStream && t->ctx.n_tile_work == 0 && t->cur_gen != t->state_gen) {
+    // the one-warp walk keeps no strategy rows: regret-match R for the read-back (hand tiles store them,
+    // and their next update reads them)
     if (launch_current_rows(t->ctx, t->stream) != 0) return fail(CFR_ECUDA, "strategy launch failed");
     t->launches += 1;
     t->cur_gen = t->state_gen;

@@ -1,5 +1,5 @@
-"""What a handle reads back between calls: the rows of the last leaf evaluation, whatever ran or was
-set since."""
+"""What a handle keeps, sends and reads back between calls: the rows of the last leaf evaluation, whatever
+ran or was set since; the current strategy; the tables its kernels read."""
 import numpy as np
 import pytest
 
@@ -100,6 +100,23 @@ def test_a_read_that_launches_reports_a_wait_that_gave_up():
             capi.cfr_debug_first_wait_polls(-1)
     finally:
         capi.cfr_tree_destroy(tree)
+
+
+@pytest.mark.parametrize("variant", ["dcfr", "pcfr+"])
+def test_current_strategy_of_hand_tiles_is_read_where_it_is_kept(variant):
+    specs = [synth.river_subgame(n_hands=60 + 7 * k, seed=3 * k, range_seed=3 * k + 1) for k in range(3)]
+    rows = {}
+    for schedule in ("level", "stream"):
+        tree = capi.cfr_batch_create(specs, capi.make_opts(variant, precision="single", schedule=schedule))
+        try:
+            capi.cfr_iterate(tree, 4)
+            l0 = _launches(tree)
+            rows[schedule] = [capi.cfr_strategy(tree, 0, game=g) for g in range(3)]
+            assert _launches(tree) == l0
+        finally:
+            capi.cfr_tree_destroy(tree)
+    for x, y in zip(rows["level"], rows["stream"]):
+        assert np.array_equal(x, y)
 
 
 def test_only_walked_trees_upload_their_programs():
