@@ -134,10 +134,13 @@ typedef struct cfr_game_spec {
  * batches (highest throughput; needs at most 8 actions per decision node): one block per tile
  * of 8 to 32 hands keeps its subgame's values, strategy and reach in shared memory and streams R
  * and S; where a tree is too large for a tile, or warp_hands is 64, or chunk_hands is above 8, one
- * warp per 32 (or 64) hands walks a depth-first program of its tree instead.  CFR_SCHEDULE_WIDE: every pass (update, initial strategy, average, best
- * response) is one launch per tree level over all of that level's (node, hand) pairs, one
- * thread each (for one tree too large for a block to stage in shared memory: exact turns
- * and flops; one subgame per handle, at most 8 actions per decision node).
+ * warp per 32 (or 64) hands walks a depth-first program of its tree instead (one such subgame takes
+ * its whole handle there).  CFR_SCHEDULE_WIDE: every pass (update, initial strategy, average, best
+ * response) is one launch per tree level over all of that level's (node, hand) pairs, two hands a
+ * thread (for one tree too large for a block to stage in shared memory: exact turns and flops; one
+ * subgame per handle, at most 8 actions per decision node).  The level and wide schedules of trees
+ * that do fit a block's shared memory with 4 hands or more take one launch a pass, a block per
+ * chunk_hands hands.
  * CFR_SCHEDULE_RESIDENT: cfr_iterate runs all its iterations in one cooperative launch;
  * each block keeps one chunk of hands of both players (regrets, strategy sums, strategy,
  * reach) in shared memory for the whole launch, and an iteration's phases (the terminal values

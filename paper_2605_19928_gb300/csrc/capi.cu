@@ -589,7 +589,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // chunk_hands beyond 8 for best-response sums a tile cannot form.
   // The level and wide schedules (one subgame, or few) run their passes as the latency form of the
   // same kernel when every tree fits it with chunk_hands hands a tile (4 or more: 16-byte pieces),
-  // and the resident schedule walks the same tables.
+  // and the resident schedule walks the same tables.  It is the faster one up to the limit of shared
+  // memory: an iteration of a river of 1,081 hands as tiles or a launch a level, FP32 values, 525 nodes 48
+  // or 86 us, 1,353 nodes 65 or 106; pairs, 525 nodes 61 or 125, 1,137 nodes 95 or 172; of 27 hands, 1,353
+  // nodes, 57 or 76.  One subgame that does not fit keeps the whole handle from tiles.
   const bool stream_tiles = schedule == kScheduleStream && o.warp_hands != 64 && chunk[0] <= 8;
   const bool staged = schedule != kScheduleStream && chunk[0] >= 4 && !o.runout_tables;
   std::vector<std::vector<uint16_t>> tile_tabs(n_games);
