@@ -298,8 +298,8 @@ __device__ __forceinline__ bool holds_board_card(const uint16_t* cards, int h, i
 // Sums and differences are double-float with FP32-pair values (whose folds take T and C[c] from
 // the same prefix sums, in hand order), plain FP32 with FP32 values.
 
-// Entries of a thread's run at most, for the 1176 hands a flop leaves: 1176 over 160 threads (8) and
-// 2352 over 352 (7) with FP32 values, 2352 over 256 (10) with pairs.
+// Entries of a thread's run at most: kMaxHands over 160 threads (8) and twice as many over 352 (7) with
+// FP32 values, over 256 (10) with pairs.
 template <typename P>
 struct ScanPer {
   static constexpr int n = std::is_same<P, Single>::value ? 8 : 10;
@@ -398,12 +398,15 @@ __device__ __forceinline__ void scan_write(F at, int begin, int cnt, int n, cons
 
 // ---- one node, all of a block of kTermThreads threads: the latency form
 
-constexpr int kTermHands = 3;  // hands per thread: at most 1176 of them
+constexpr int kTermHands = 3;  // hands per thread
+static_assert(kTermHands * kTermThreads >= kMaxHands, "every hand has a thread");
 
 // The threads on the rank order (the others take the card lists), and a thread's run of them.
 template <typename P>
 struct TermRun {
   static constexpr int gp = std::is_same<P, Single>::value ? 5 * 32 : kTermThreads / 2;
+  static_assert(ScanPer<P>::n * gp >= kMaxHands && ScanPer<P>::n * (kTermThreads - gp) >= 2 * kMaxHands,
+                "a thread's run holds its share of the hands and of the card lists");
   int begin, cnt;
   __device__ __forceinline__ TermRun() : begin(0), cnt(0) {}
   __device__ __forceinline__ TermRun(int H, int k) {

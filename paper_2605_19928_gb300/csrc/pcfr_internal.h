@@ -12,7 +12,7 @@
 // A decision node with A actions owns rows [row, row + A); player 0's rows come first.
 //
 // Terminal tables, one block of uint16 per showdown board (TermTab gives the offsets), all
-// indices below 2^15 because a player has at most 1326 hands:
+// indices below 2^15 because a player has at most kMaxHands hands:
 //   clh    [k * H]   per-card lists of hands, each list in rank-sorted order, concatenated
 //   cards  [H]       card ids of each hand, c1 | c2 << 8 (c2 = 255 for one-card hands)
 //   cloff  [deck+1]  start of each card's list in clh
@@ -41,6 +41,7 @@ enum NodeType : uint8_t { kDecision = 0, kFold = 1, kShowdown = 2, kChance = 3, 
 __host__ __device__ inline bool is_end(int type) { return type == kFold || type == kShowdown || type == kLeaf; }
 
 constexpr int kMaxActions = 16;
+constexpr int kMaxHands = 1176;  // of a player: two of the 49 cards that a flop leaves
 constexpr int kMaxDeck = 52;
 constexpr uint8_t kNoCard = 255;
 constexpr int kPrecisionPairs = 0;   // values as double-float FP32 pairs

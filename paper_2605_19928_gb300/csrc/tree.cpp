@@ -256,6 +256,10 @@ int build_game(const cfr_game_spec& spec, HostGame& g, std::string& err) {
   R.deck = g.deck;
   R.n_streets = g.n_streets;
   const int H = g.n_hands;
+  if (H > kMaxHands) {  // (three board cards and distinct hands leave no more)
+    err = "more than " + std::to_string(kMaxHands) + " hands";
+    return CFR_EINVAL;
+  }
   g.hstride = (H + 31) / 32 * 32;
 
   // ranges: non-negative, finite, normalised to sum 1
