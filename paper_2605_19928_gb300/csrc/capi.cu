@@ -1685,7 +1685,12 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
-  // time one candidate; +inf when the layout does not apply (e.g. a tree the stream form refuses)
+  // Layouts of the terminal launch timed with the fastest schedule: several term_nodes can give one.
+  using TermLayout = std::array<int, 3>;
+  std::vector<TermLayout> term_timed;
+  TermLayout term_last{}, term_top{};
+  // time one candidate; +inf when the layout does not apply (e.g. a tree the stream form refuses) or its
+  // terminal layout has been timed
   auto trial = [&](const cfr_solver_opts& o, double* ms) -> int {
     *ms = INFINITY;
     cfr_tree* t = nullptr;
@@ -1693,6 +1698,11 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
     // the level schedule takes every valid handle: its refusal is the caller's error
     if (rc == CFR_EINVAL && o.schedule != CFR_SCHEDULE_LEVEL) return CFR_OK;
     if (rc) return rc;
+    term_last = {t->ctx.term_nv, t->ctx.n_term_runs, t->ctx.n_term_segments};
+    if (std::find(term_timed.begin(), term_timed.end(), term_last) != term_timed.end()) {
+      delete t;
+      return CFR_OK;
+    }
     t->leaf_net_set = true;  // leaves, if any, run with the all-zero network the handle starts with
     rc = cfr_iterate(t, 2);
     cudaError_t e = cudaSuccess;
@@ -1719,7 +1729,7 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
     cand.schedule = CFR_SCHEDULE_LEVEL;
     cand.chunk_hands = chunks[k];
     rc = trial(cand, &ms);
-    if (!rc && ms < top_ms) top_ms = ms, top = cand;
+    if (!rc && ms < top_ms) top_ms = ms, top = cand, term_top = term_last;
   }
   for (int sch : {CFR_SCHEDULE_STREAM, CFR_SCHEDULE_WIDE}) {
     if (rc || (sch == CFR_SCHEDULE_WIDE && n_games != 1)) continue;
@@ -1730,7 +1740,7 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
       if (rc || (sch == CFR_SCHEDULE_WIDE && wh == 64)) continue;
       cand.warp_hands = sch == CFR_SCHEDULE_STREAM ? wh : 0;
       rc = trial(cand, &ms);
-      if (!rc && ms < top_ms) top_ms = ms, top = cand;
+      if (!rc && ms < top_ms) top_ms = ms, top = cand, term_top = term_last;
     }
     cand.warp_hands = 0;
   }
@@ -1740,15 +1750,17 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
     cand.warp_hands = 0;
     cand.runout_tables = 0;
     rc = trial(cand, &ms);
-    if (!rc && ms < top_ms) top_ms = ms, top = cand;
+    if (!rc && ms < top_ms) top_ms = ms, top = cand, term_top = term_last;
   }
   cand = top;
+  term_timed.push_back(term_top);
   for (int tn : {1, 2, 4, 8}) {  // terminal nodes per block, for the fastest layout
     if (cand.schedule == CFR_SCHEDULE_RESIDENT) break;  // one node per block item: no runs
     if (rc) break;
     cand.term_nodes = tn;
     rc = trial(cand, &ms);
-    if (!rc && ms < top_ms) top_ms = ms, top = cand;
+    if (!rc) term_timed.push_back(term_last);
+    if (!rc && ms < top_ms) top_ms = ms, top = cand, term_top = term_last;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
