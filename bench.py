@@ -503,8 +503,8 @@ def run_ours(args):
         # the roofline model counts 4-byte values whatever the storage precision
         alg = sum(algorithmic_bytes(sh, dom, 4) for sh in shapes)
         achieved = alg / (stages[dom][0] * 1e-3) / 1e9
-        upd_kernel = "k_tile<update>"
-        roofline = {"bound": "hbm", "kernel": upd_kernel if dom == "update" else "k_terminal",
+        term_kernel, upd_kernel = capi.cfr_kernel_names(tree)
+        roofline = {"bound": "hbm", "kernel": upd_kernel if dom == "update" else term_kernel,
                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": f"{peak_kind} hbm_gbs",
                     "traffic": profiled_traffic(dom, "batch256" if batch else "river1081"),

@@ -280,6 +280,10 @@ int cfr_autotune(const cfr_game_spec* specs, int n_games, const cfr_solver_opts*
  * CFR_SCHEDULE_WIDE or CFR_SCHEDULE_RESIDENT), or a negative status. */
 int cfr_schedule(const cfr_tree* tree);
 
+/* The names of the kernels that the handle's terminal launches and updates run (static strings, either
+ * may be NULL): within one schedule they depend on the trees' sizes. */
+int cfr_kernel_names(const cfr_tree* tree, const char** terminal, const char** update);
+
 /* Sizes of one subgame and the number of iterations done.  Any out pointer may be NULL. */
 int cfr_tree_info(const cfr_tree* tree, int game, int* n_nodes, int* n_hands, int* iters_done);
 

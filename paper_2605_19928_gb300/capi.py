@@ -35,7 +35,7 @@ CFR_STAGES = ("terminal", "update", "avg_reach", "br_terminal", "br", "leaf")
 EXPORTS = ("cfr_set_allocator", "cfr_tree_create", "cfr_batch_create", "cfr_iterate", "cfr_strategy",
            "cfr_exploitability", "cfr_tree_info", "cfr_node_info", "cfr_read_values", "cfr_sync",
            "cfr_stage_times", "cfr_counters", "cfr_exploitability_async", "cfr_exploitability_result",
-           "cfr_reset", "cfr_tree_destroy", "cfr_last_error", "cfr_exploitability_noalloc", "cfr_schedule",
+           "cfr_reset", "cfr_tree_destroy", "cfr_last_error", "cfr_exploitability_noalloc", "cfr_schedule", "cfr_kernel_names",
            "cfr_gemm_bf16", "cfr_set_leaf_net", "cfr_leaf_info", "cfr_read_leaf_rows",
            "cfr_eval_leaves", "cfr_write_values", "cfr_autotune", "cfr_debug_first_wait_polls")
 
@@ -100,6 +100,7 @@ def load(path: str = LIB_PATH):
         lib.cfr_reset.argtypes = [P]
         lib.cfr_exploitability_noalloc.argtypes = [P, pd, pd]
         lib.cfr_schedule.argtypes = [P]
+        lib.cfr_kernel_names.argtypes = [P, C.POINTER(C.c_char_p), C.POINTER(C.c_char_p)]
         lib.cfr_gemm_bf16.argtypes = [P, P, P, P, I, I, I, I, I, P, P]
         lib.cfr_debug_first_wait_polls.argtypes = [C.c_long]
         lib.cfr_set_leaf_net.argtypes = [P, C.POINTER(P), C.POINTER(P)]
@@ -323,6 +324,13 @@ def cfr_schedule(tree) -> int:
     if rc < 0:
         _check(rc)
     return rc
+
+
+def cfr_kernel_names(tree) -> tuple[str, str]:
+    """Names of the handle's terminal and update kernels."""
+    a, b = C.c_char_p(), C.c_char_p()
+    _check(load().cfr_kernel_names(tree, C.byref(a), C.byref(b)))
+    return a.value.decode(), b.value.decode()
 
 
 def cfr_tree_info(tree, game: int = 0):

@@ -1381,6 +1381,18 @@ int cfr_schedule(const cfr_tree* t) {
                                             : CFR_SCHEDULE_LEVEL;
 }
 
+int cfr_kernel_names(const cfr_tree* t, const char** terminal, const char** update) {
+  if (!t) return fail(CFR_EINVAL, "tree is NULL");
+  const LaunchCtx& c = t->ctx;
+  if (terminal)
+    *terminal = c.resident ? "k_resident" : c.n_term_work == 0 ? "" : c.n_term_runs > 0 ? "k_terminal_run"
+                : c.term_nv > 1 ? "k_terminal_vec" : "k_terminal";
+  if (update)
+    *update = c.resident ? "k_resident" : c.n_tile_work > 0 ? "k_tile" : c.schedule == kScheduleStream ? "k_stream_update"
+              : c.schedule == kScheduleWide ? "k_wide_back" : "k_hand";
+  return CFR_OK;
+}
+
 int cfr_tree_info(const cfr_tree* t, int game, int* n_nodes, int* n_hands, int* iters_done) {
   int rc = check_game(t, game);
   if (rc) return rc;

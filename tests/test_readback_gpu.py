@@ -129,3 +129,24 @@ def test_only_walked_trees_upload_their_programs():
         capi.cfr_tree_destroy(tree)
     # the per-hand kernels' handle sends less than the one that walks its tree, although its chunks are more
     assert sent["level", 0] < sent["stream", 64]
+
+
+def test_kernel_names_follow_what_the_handle_runs():
+    A = synth.ALL_IN
+    small = synth.river_subgame(n_hands=64, seed=3, range_seed=4)
+    large = synth.river_subgame(n_hands=64, seed=3, range_seed=4, bet_sizes=(0.33, 0.5, 0.75, 1.0, 2.0, A), max_raises=4,
+                                stack=3000.0)
+    batch = synth.batch_rivers(256, n_hands=40)
+    cases = [([small], dict(schedule="level"), ("k_terminal", "k_tile")),
+             ([small], dict(schedule="level", chunk_hands=2), ("k_terminal", "k_hand")),
+             ([large], dict(schedule="wide"), ("k_terminal_vec", "k_wide_back")),
+             ([small], dict(schedule="stream", warp_hands=64), ("k_terminal", "k_stream_update")),
+             ([small], dict(schedule="resident"), ("k_resident", "k_resident")),
+             (batch, dict(schedule="stream"), ("k_terminal_vec", "k_tile")),
+             (batch, dict(schedule="stream", precision="pairs"), ("k_terminal_run", "k_tile"))]
+    for specs, kw, want in cases:
+        tree = capi.cfr_batch_create(specs, capi.make_opts("dcfr", **{"precision": "single", **kw}))
+        try:
+            assert capi.cfr_kernel_names(tree) == want
+        finally:
+            capi.cfr_tree_destroy(tree)
