@@ -1600,6 +1600,14 @@ __device__ __forceinline__ void tile_reach(const TileLane& T, typename P::V* rch
   }
 }
 
+// Whether the walk's regret matching runs ahead of it: with pairs, but not on trees of one or two such
+// levels, where the barrier costs as much as it saves (river of 275 hands with pairs, resident, 18.8 us an
+// iteration inside the walk, 20.6 ahead).
+template <typename P>
+__device__ __forceinline__ bool match_ahead(const TileLane& T) {
+  return std::is_same<P, Pairs>::value && T.head->flevels[T.p] > 2;
+}
+
 // Regret matching of all the player's nodes ahead of the walk, by nslots slots of W lanes (slot, from
 // them, this lane's): the strategy replaces the positive parts in sg.  The latency forms take it with
 // pairs: a node's reciprocal and products are a long chain in double-float arithmetic, paid once here
@@ -1908,7 +1916,7 @@ __global__ void __launch_bounds__(LAT ? 2 * kTileThreads : kTileThreads, LAT ? 2
   auto put_reach = [&](int n, V y) {
     if (MODE == kModeUpdate && valid) grch[(size_t)n * stride + h] = y;
   };
-  if constexpr (LAT && sizeof(V) == 8) {
+  if (LAT && match_ahead<P>(T)) {
     tile_match_all<P>(T, sg, slot, nslots, put_sigma);
     __syncthreads();
     if (tid < T.group) tile_reach_matched<P>(T, val, sg, put_reach);
@@ -2313,7 +2321,7 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
           };
           if (tid < W) put_reach(0, srch[p][0]);
           auto put_sigma = [&](int r, V y) { ssg[p][r << wlog] = y; };
-          if constexpr (es == 8) {
+          if (match_ahead<P>(T)) {
             tile_match_all<P>(T, ssg[p], slot, nslots, [](int, V) {});
             __syncthreads();
             if (tid < T.group) tile_reach_matched<P>(T, srch[p], ssg[p], put_reach);
