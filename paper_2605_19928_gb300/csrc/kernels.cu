@@ -2216,6 +2216,13 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
   const int it0 = *iter;             // written only by the last block to finish
   const uint32_t stamp0 = sync[2];  // too
   const int steps = alternating ? 2 : 1;
+  // A step's terminal items, of the one or both players.  Each block takes neighbours of the list, which
+  // is sorted by board table and kind, so that what it keeps of the table stays (taking every
+  // gridDim.x-th, Leduc's blocks met a fold and a showdown in turn: 38.4 against 34.6 us an iteration,
+  // with pairs 56.0 against 50.2).
+  const int items = (alternating ? 1 : 2) * n_term_work, share = items / (int)gridDim.x, over = items % (int)gridDim.x;
+  const int item0 = (int)blockIdx.x * share + min((int)blockIdx.x, over),
+            item1 = item0 + share + ((int)blockIdx.x < over);
   unsigned nbar = 0;
   bool ok = true;
   ResidentTerm<P> term;
@@ -2229,14 +2236,8 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
       const int p0 = pm == 2 ? 1 : 0, np = pm == 3 ? 2 : 1;
       const long limit = it == 0 ? g_first_wait_polls : kWaitLimit;
       // ---- terminal values of the player(s) of this step (Stages 2-4)
-      // Each block takes neighbours of the list, which is sorted by board table and kind, so that what it
-      // keeps of the table stays (taking every gridDim.x-th, Leduc's blocks met a fold and a showdown in
-      // turn: 38.4 against 34.6 us an iteration, with pairs 56.0 against 50.2).
-      const int items = np * n_term_work, share = items / (int)gridDim.x, over = items % (int)gridDim.x,
-                item0 = (int)blockIdx.x * share + min((int)blockIdx.x, over),
-                item1 = item0 + share + ((int)blockIdx.x < over);
       for (int item = item0; item < item1 && ok; ++item) {
-        const int e = item % n_term_work, i = p0 + item / n_term_work;
+        const int e = item < n_term_work ? item : item - n_term_work, i = p0 + (item >= n_term_work);
         // player 0's first terminals read what the launch before left
         ok = resident_terminal<P>(games, term_work, term_src, e, i, smr, term, alternating && (it > 0 || step > 0),
                                   step == 0 ? stamp - 1u : stamp, alternating != 0, stamp, !alternating || last, limit, err);
