@@ -1363,16 +1363,39 @@ struct TileLane {
 
 // Value of a chance node for one lane: the sum over its A children c[a * W] but those whose card is in
 // the hand (children values carry the card probabilities).  One thread adds up to 49 children, so the
-// cards are in the tile's table and the loads of eight children go out together: with the cards in
-// global memory an update of a 537-node turn took 27.1 us, now 18.5.
-template <typename P>
+// cards are in the tile's table and several children are loaded ahead of the sum: with the cards in
+// global memory an update of a 537-node turn with FP32 values took 27.1 us, now 18.5.  FP32 values take
+// eight a step.  Pairs take four, added to a copy of the sum that the card's test then keeps or drops
+// (turn to a leaf network, 997 hands: 24.0 us an update with eight and a branch at each, 19.1 so), and
+// so does FP32 in the resident kernel, where the longer code costs rivers that have no such node
+// (187 hands: 13.7 and 13.5 us an iteration).
+template <typename P, bool LEAN>
 __device__ __forceinline__ typename P::V tile_chance(const TileLane& T, const TileNode& nd, const typename P::V* c, int W) {
   const uint8_t* deal = reinterpret_cast<const uint8_t*>(T.tab + T.head->deal) + nd.first_kid;
   const int A = nd.kids & 63;
   typename P::Acc acc = P::acc0();
+  if constexpr (LEAN || std::is_same<P, Pairs>::value) {
+    constexpr int kAhead = 4;
+    for (int a0 = 0; a0 < A; a0 += kAhead) {
+      typename P::V y[kAhead];
+      int card[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const int a = min(a0 + u, A - 1);
+        y[u] = c[a * W], card[u] = deal[a];
+      }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        typename P::Acc with = acc;
+        P::acc(with, y[u]);
+        if (a0 + u < A && !((T.hmask >> card[u]) & 1ull)) acc = with;
+      }
+    }
+  } else {
 #pragma unroll 8
-  for (int a = 0; a < A; ++a)
-    if (!((T.hmask >> deal[a]) & 1ull)) P::acc(acc, c[a * W]);
+    for (int a = 0; a < A; ++a)
+      if (!((T.hmask >> deal[a]) & 1ull)) P::acc(acc, c[a * W]);
+  }
   return P::value(acc);
 }
 
@@ -1387,7 +1410,7 @@ __device__ __forceinline__ void group_barrier(int group) {
 // Phase A: the inner nodes' values from the deepest level up (Stage 6, Eq. backward; kModeBR: the
 // best response's), by the first `group` threads.  gv: the player's value rows; the values are
 // stored there when `store` is set, the root's always.
-template <int MODE, typename P>
+template <int MODE, typename P, bool LEAN = false>
 __device__ __forceinline__ void tile_values(const TileLane& T, typename P::V* val, const typename P::V* sg,
                                             typename P::V* gv, bool store) {
   using V = typename P::V;
@@ -1402,7 +1425,7 @@ __device__ __forceinline__ void tile_values(const TileLane& T, typename P::V* va
       const V* c = val + (nd.first_kid << wlog);
       V x;
       if (kind == 2) {
-        x = tile_chance<P>(T, nd, c, 1 << wlog);
+        x = tile_chance<P, LEAN>(T, nd, c, 1 << wlog);
       } else if (MODE == kModeBR && kind == T.p) {
         x = c[0];
         for (int a = 1; a < A; ++a) x = P::vmax(x, c[a << wlog]);
@@ -1432,7 +1455,7 @@ __device__ __forceinline__ void tile_values(const TileLane& T, typename P::V* va
 // river of 1,081 hands and 75 nodes 16.6 -> 16.2 us, with pairs 31.7 -> 27.1, of 27 nodes 14.0 -> 13.0;
 // 165-node river of 300 hands with pairs, level schedule, 32.8 -> 30.7.
 constexpr int kTileSlack = 4;  // rows of slack behind a tile's strategy
-template <int MODE, typename P>
+template <int MODE, typename P, bool LEAN = false>
 __device__ __forceinline__ void tile_values8(const TileLane& T, typename P::V* val, const typename P::V* sg,
                                              typename P::V* gv, bool store) {
   using V = typename P::V;
@@ -1447,7 +1470,7 @@ __device__ __forceinline__ void tile_values8(const TileLane& T, typename P::V* v
       const V* c = val + nd.first_kid * 8;
       V x;
       if (kind == 2) {
-        x = tile_chance<P>(T, nd, c, 8);
+        x = tile_chance<P, LEAN>(T, nd, c, 8);
       } else {
         V cc[4];
 #pragma unroll
@@ -2295,8 +2318,8 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
           if (!ok) break;
           // A: later iterations of the launch overwrite the inner values, so only the last stores them
           if (tid < T.group) {
-            if (wlog == 3) tile_values8<kModeUpdate, P>(T, val, ssg[p], gv, last);
-            else tile_values<kModeUpdate, P>(T, val, ssg[p], gv, last);
+            if (wlog == 3) tile_values8<kModeUpdate, P, true>(T, val, ssg[p], gv, last);
+            else tile_values<kModeUpdate, P, true>(T, val, ssg[p], gv, last);
           }
           __syncthreads();
           // B
