@@ -354,11 +354,11 @@ __device__ __forceinline__ void scan_runs(F at, int cnt, VecAcc<P, NV>* red, int
   if (lane == 31) red[gtid >> 5] = x;
 }
 
-// After the barrier: the exclusive prefix sums of the thread's run into out (out[n] = totals).  Every
-// warp scans the GT / 32 warp totals itself.
-template <typename P, int NV, int GT, bool REGS, typename F>
+// After the barrier: the exclusive prefix sums of the thread's run into out (out[place(n)] = totals).
+// Every warp scans the GT / 32 warp totals itself.
+template <typename P, int NV, int GT, bool REGS, typename F, typename M>
 __device__ __forceinline__ void scan_write(F at, int begin, int cnt, int n, const VecAcc<P, NV>* red, int gtid,
-                                           const VecAcc<P, NV>& x, Vec<P, NV>* out) {
+                                           const VecAcc<P, NV>& x, Vec<P, NV>* out, M place) {
   const int lane = gtid & 31, warp = gtid >> 5;
   VecAcc<P, NV> run;
   Vec<P, NV> total;
@@ -384,7 +384,7 @@ __device__ __forceinline__ void scan_write(F at, int begin, int cnt, int n, cons
       o.v[v] = P::value(run.v[v]);
       P::acc(run.v[v], y.v[v]);
     }
-    out[begin + e] = o;
+    out[place(begin + e)] = o;
   };
   if constexpr (REGS) {
 #pragma unroll
@@ -393,7 +393,7 @@ __device__ __forceinline__ void scan_write(F at, int begin, int cnt, int n, cons
   } else {
     for (int e = 0; e < cnt; ++e) put(e);
   }
-  if (gtid == 0) out[n] = total;
+  if (gtid == 0) out[place(n)] = total;
 }
 
 // ---- one node, all of a block of kTermThreads threads: the latency form
@@ -518,6 +518,13 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
       return;
     }
   }
+  // In place, threads walk the arrays a run apart: runs of a multiple of eight entries would meet in a few
+  // banks, so the entries of such an array swap places within each eight of them (by the number of the
+  // eight).  106 rivers of 900 hands with pairs (runs of 8 along the card lists): 173 -> 137 us a player.
+  constexpr int gc = kTermThreads - gp;
+  const int pmask = !REGS && (H + gp - 1) / gp % 8 == 0 ? 7 : 0, cmask = !REGS && (k * H + gc - 1) / gc % 8 == 0 ? 7 : 0;
+  auto pat = [&](int j) { return REGS ? j : j ^ (j >> 3 & pmask); };
+  auto cat = [&](int j) { return REGS ? j : j ^ (j >> 3 & cmask); };
   {
     V1 a[REGS ? ScanPer<P>::n : 1];
     VecAcc<P, 1> x;
@@ -528,21 +535,22 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
 #pragma unroll
       for (int e = 0; e < ScanPer<P>::n; ++e) a[e].v[0] = q[L.hand(e)];
     } else {  // gathered into the arrays that the scan turns into prefix sums in place
-      for (int j = tid; j < H; j += kTermThreads) ps[j].v[0] = q[show ? L.perm[j] : j];
-      for (int j = tid; j < k * H; j += kTermThreads) cp[j].v[0] = q[clh[j]];
+      for (int j = tid; j < H; j += kTermThreads) ps[pat(j)].v[0] = q[show ? L.perm[j] : j];
+      for (int j = tid; j < k * H; j += kTermThreads) cp[cat(j)].v[0] = q[clh[j]];
       __syncthreads();
     }
-    V1* mine = (tid < gp ? ps : cp) + L.run.begin;
-    auto at = [&](int e) { return REGS ? a[REGS ? e : 0] : mine[e]; };
+    V1* mine = tid < gp ? ps : cp;
+    const int mask = tid < gp ? pmask : cmask, begin = L.run.begin;
+    auto at = [&](int e) { return REGS ? a[REGS ? e : 0] : mine[(begin + e) ^ ((begin + e) >> 3 & mask)]; };
     scan_runs<P, 1, REGS>(at, L.run.cnt, red[tid >= gp], gtid, x);
     __syncthreads();
     if (tid < gp)
-      scan_write<P, 1, gp, REGS>(at, L.run.begin, L.run.cnt, H, red[0], gtid, x, ps);
+      scan_write<P, 1, gp, REGS>(at, L.run.begin, L.run.cnt, H, red[0], gtid, x, ps, pat);
     else
-      scan_write<P, 1, kTermThreads - gp, REGS>(at, L.run.begin, L.run.cnt, k * H, red[1], gtid, x, cp);
+      scan_write<P, 1, gc, REGS>(at, L.run.begin, L.run.cnt, k * H, red[1], gtid, x, cp, cat);
   }
   __syncthreads();
-  const V T = Ps[H], us = P::scale(u);
+  const V T = Ps[pat(H)], us = P::scale(u);
 #pragma unroll
   for (int s = 0; s < kTermHands; ++s) {
     const int h = tid + s * kTermThreads;
@@ -550,23 +558,23 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
       const uint4 r = L.record(s, h);
       const unsigned c1 = r.x & 0xffu, c2 = (r.x >> 8) & 0xffu;
       bool blocked = (board >> c1) & 1ull;
-      const V a0 = CP[cloff[c1]], z0 = CP[cloff[c1 + 1]];
+      const V a0 = CP[cat(cloff[c1])], z0 = CP[cat(cloff[c1 + 1])];
       V d;
       if (show) {
-        V Wn = Ps[r.x >> 16], Ln = P::sub(T, Ps[r.y & 0xffffu]);
-        Wn = P::sub(Wn, P::sub(CP[r.y >> 16], a0));
-        Ln = P::sub(Ln, P::sub(z0, CP[r.z & 0xffffu]));
+        V Wn = Ps[pat(r.x >> 16)], Ln = P::sub(T, Ps[pat(r.y & 0xffffu)]);
+        Wn = P::sub(Wn, P::sub(CP[cat(r.y >> 16)], a0));
+        Ln = P::sub(Ln, P::sub(z0, CP[cat(r.z & 0xffffu)]));
         if (k == 2) {
           blocked = blocked || ((board >> c2) & 1ull);
-          Wn = P::sub(Wn, P::sub(CP[r.z >> 16], CP[cloff[c2]]));
-          Ln = P::sub(Ln, P::sub(CP[cloff[c2 + 1]], CP[r.w & 0xffffu]));
+          Wn = P::sub(Wn, P::sub(CP[cat(r.z >> 16)], CP[cat(cloff[c2])]));
+          Ln = P::sub(Ln, P::sub(CP[cat(cloff[c2 + 1])], CP[cat(r.w & 0xffffu)]));
         }
         d = P::sub(Wn, Ln);
       } else {
         d = P::sub(T, P::sub(z0, a0));
         if (k == 2) {
           blocked = blocked || ((board >> c2) & 1ull);
-          d = P::add(P::sub(d, P::sub(CP[cloff[c2 + 1]], CP[cloff[c2]])), q[h]);
+          d = P::add(P::sub(d, P::sub(CP[cat(cloff[c2 + 1])], CP[cat(cloff[c2])])), q[h]);
         }
       }
       put(h, blocked ? P::zero() : P::mul(us, d));
@@ -659,7 +667,7 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __r
 // A block takes up to eight nodes of one game, board table and kind one after the other: the table is
 // staged once, and each node's reach row lands (two buffers) while the node before is computed.  A
 // node is a chain of four block barriers with little between them, so what counts is how many chains
-// an SM holds: four blocks, which the scans' in-place form leaves room for (40 registers; 64 with the
+// an SM holds: four blocks, which the scans' in-place form leaves room for (32 registers; 64 with the
 // entries in registers hold two).  Pairs always run so (groups of two nodes a thread spilled, and
 // took 419 us a player on 256 rivers of 1,081 hands where this form takes 309); FP32 values where a
 // board table has few showdown nodes (see create_impl).  Measured, one player: 256 rivers, pairs, 309
@@ -689,8 +697,8 @@ __global__ void __launch_bounds__(kTermThreads, 4) k_terminal_run(const GameDev*
   __shared__ __align__(8) uint64_t bar[2];
   const uint16_t* tab = reinterpret_cast<const uint16_t*>(smt);  // [tt.len]
   V* rows = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);       // [2][hstride]
-  V* CP = rows + 2 * stride;                                     // [k H + 1]
-  V* Ps = CP + (k * H + 1);                                      // [H + 1]
+  V* CP = rows + 2 * stride;                                     // [k H + 1], in eights
+  V* Ps = CP + TermTab::round8(k * H + 1);                       // [H + 1], in eights
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -922,12 +930,13 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal_vec(const GameDev*
         }
       const int gtid = tid < gp ? tid : tid - gp;
       auto entry = [&](int e) { return a[e]; };
+      auto same = [](int j) { return j; };
       scan_runs<P, NV, true>(entry, cnt, red[tid >= gp], gtid, x);
       __syncthreads();
       if (tid < gp)
-        scan_write<P, NV, gp, true>(entry, begin, cnt, H, red[0], gtid, x, Ps);
+        scan_write<P, NV, gp, true>(entry, begin, cnt, H, red[0], gtid, x, Ps, same);
       else
-        scan_write<P, NV, kTermThreads - gp, true>(entry, begin, cnt, k * H, red[1], gtid, x, CP);
+        scan_write<P, NV, kTermThreads - gp, true>(entry, begin, cnt, k * H, red[1], gtid, x, CP, same);
     }
     __syncthreads();
     for (int h = tid; h < H; h += kTermThreads) {
@@ -3317,7 +3326,10 @@ size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es)
 size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv, bool runs) {
   const TermTab tt(n_hands, hand_size, deck);
   const size_t scan = (size_t)(hand_size * n_hands + 1 + n_hands + 1);
-  if (nv == 1) return (size_t)tt.len * 2 + (size_t)(runs ? 2 : 1) * hstride * es + scan * es;
+  if (runs)
+    return (size_t)tt.len * 2 + 2 * (size_t)hstride * es +
+           (size_t)(TermTab::round8(hand_size * n_hands + 1) + TermTab::round8(n_hands + 1)) * es;
+  if (nv == 1) return (size_t)tt.len * 2 + (size_t)hstride * es + scan * es;
   return kTermSegment * sizeof(TermGroup) + (size_t)tt.fold_len * 2 + 2 * (size_t)nv * hstride * es + scan * nv * es;
 }
 

@@ -33,6 +33,9 @@ CASES = {
     # games of different hand counts and kinds side by side
     "mixed": lambda: [synth.leduc(), _river(33, 7), synth.kuhn(),
                       synth.turn_subgame(n_hands=301, seed=9, range_seed=10, bet_sizes=(ALL_IN,), max_raises=1)],
+    # hand counts at which a thread's run of the prefix sums is 7, 8 and 9 entries, and few showdowns a board
+    "eights": lambda: [_river(h, h, bet_sizes=(ALL_IN,), max_raises=1) for h in (559, 561, 640, 896, 897, 900, 1024, 1025, 1081)]
+    + [synth.turn_subgame(n_hands=h, seed=9, range_seed=10, bet_sizes=(ALL_IN,), max_raises=1) for h in (1120, 1121, 1128)],
 }
 
 
