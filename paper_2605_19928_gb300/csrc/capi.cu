@@ -25,15 +25,16 @@ using namespace pcfr;
 namespace {
 
 // Terminal nodes from which a block of the launch evaluates several (FP32 values), from which pairs take
-// the run form (with one node a block while they do not fill the GPU: more than one wave of the
-// one-node form's two blocks per SM; turn of 12 hands, 1,448 nodes: 22.5 -> 18.3 us), and showdown
-// nodes a board table from which FP32 values take groups of four (see create_impl).  Measured, one
+// the run form (with one node a block while they do not fill the GPU) with many hands and with up to
+// 128, and showdown nodes a board table from which FP32 values take groups of four (see create_impl).
+// Pairs, one node a block or runs: 430 nodes of 12 hands 14.0 and 11.9 us, of 1,128 hands 20.5 and 22.2
+// (8 rivers of 452 hands, an iteration, 39.0 and 42.2); 1,448 nodes of 12 hands 22.5 and 18.3.  One
 // player's launch with FP32 values, runs against groups: 7 showdowns a table (31,124-node flop, 513
 // hands) 158 against 197 us, 12 (the same flop's depth-limited form, 300 hands) 190 against 216, 30
 // (256 rivers of 406 hands) 100 against 79, 45 (turn of 1,128 hands) 49 against 44, 113 (exact turn)
 // 113 against 88.
 constexpr int kTermGroupMin = 152 * 16;
-constexpr int kTermRunMin = 152 * 2 + 1;
+constexpr int kTermRunMin = 152 * 4, kTermRunMinFew = 152 * 2 + 1;
 constexpr int kTermGroupShows = 24;
 
 thread_local std::string g_last_error;
@@ -738,7 +739,10 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     }
     shows[g] = es == 8 || n_shows > 0;
   }
-  const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= (es == 8 ? kTermRunMin : kTermGroupMin) ? 8 : 1;
+  int most_hands = 0;
+  for (const HostGame& h : t->host) most_hands = std::max(most_hands, h.n_hands);
+  const int several = es == 4 ? kTermGroupMin : most_hands <= 128 ? kTermRunMinFew : kTermRunMin;
+  const int term_nodes = o.term_nodes ? o.term_nodes : n_ends >= several ? 8 : 1;
   const bool term_run = term_nodes > 1 && (es == 8 || n_shows < kTermGroupShows * n_tables);
   const int term_nv = term_run || term_nodes == 1 ? 1 : term_nodes < 4 ? 2 : 4;
 
@@ -936,8 +940,9 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const NodeDev& nd = t->host[w.game].nodes[(size_t)w.unit];
     return nd.type == kShowdown ? nd.row : -1;
   };
-  if (term_run) {  // as long as the runs still fill the GPU eight times over
-    const int per = o.term_nodes ? o.term_nodes : std::max(1, std::min(8, (int)term_work.size() / (152 * 8)));
+  if (term_run) {  // as long as the runs still fill the GPU (two waves of four blocks per SM), also where
+                   // term_nodes asks for more: 8 rivers of 684 hands in runs of four 17 us, in the shorter ones 11
+    const int per = std::max(1, std::min(o.term_nodes ? o.term_nodes : 8, (int)term_work.size() / (152 * 8)));
     for (size_t a = 0; a < term_work.size(); ++a) {
       const Work w = term_work[a];
       if (!term_runs.empty() && term_runs.back().unit < per && term_work[a - 1].game == w.game && key(term_work[a - 1]) == key(w))
