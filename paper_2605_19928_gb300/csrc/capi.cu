@@ -940,8 +940,14 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
     const NodeDev& nd = t->host[w.game].nodes[(size_t)w.unit];
     return nd.type == kShowdown ? nd.row : -1;
   };
+  bool term_swap = false;
   if (term_run) {  // as long as the runs still fill the GPU (two waves of four blocks per SM), also where
                    // term_nodes asks for more: 8 rivers of 684 hands in runs of four 17 us, in the shorter ones 11
+    // Where more than a quarter of the terminals' scans would meet in a few banks, the entries are swapped:
+    // 106 rivers of 900 hands with pairs 173 -> 137 us a player; 256 of 1,081, which do not, 310 -> 336.
+    int n_eights = 0;
+    for (const Work& w : term_work) n_eights += scans_in_eights(t->host[w.game].n_hands, t->host[w.game].hand_size, es);
+    term_swap = 4 * n_eights > (int)term_work.size();
     const int per = std::max(1, std::min(o.term_nodes ? o.term_nodes : 8, (int)term_work.size() / (152 * 8)));
     for (size_t a = 0; a < term_work.size(); ++a) {
       const Work w = term_work[a];
@@ -1040,6 +1046,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.n_term_segments = (int)term_segments.size();
   c.term_runs = t->d_term_runs;
   c.n_term_runs = (int)term_runs.size();
+  c.term_swap = term_swap;
   c.term_nv = term_nv;
   c.iter = t->d_iter;
   c.done = t->d_done;

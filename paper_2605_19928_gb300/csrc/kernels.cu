@@ -469,7 +469,7 @@ __device__ __forceinline__ void term_lane_load(TermLane<P>& L, const GameDev& G,
 
 // Values at one node: q its reach row, ft the fold part of its board table (card lists, cards, list
 // offsets) and CP [k H + 1], Ps [H + 1] in shared memory; put(h, value) takes the results.
-template <typename P, bool REGS = true, typename LT, typename F>
+template <typename P, bool REGS = true, bool SWAP = false, typename LT, typename F>
 __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int deck, bool show, uint64_t board, ff u,
                                               const typename P::V* q, const uint16_t* ft, typename P::V* CP,
                                               typename P::V* Ps, F put) {
@@ -519,12 +519,12 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
     }
   }
   // In place, threads walk the arrays a run apart: runs of a multiple of eight entries would meet in a few
-  // banks, so the entries of such an array swap places within each eight of them (by the number of the
-  // eight).  106 rivers of 900 hands with pairs (runs of 8 along the card lists): 173 -> 137 us a player.
+  // banks, so with SWAP the entries of such an array swap places within each eight of them (by the number
+  // of the eight; see scans_in_eights).
   constexpr int gc = kTermThreads - gp;
-  const int pmask = !REGS && (H + gp - 1) / gp % 8 == 0 ? 7 : 0, cmask = !REGS && (k * H + gc - 1) / gc % 8 == 0 ? 7 : 0;
-  auto pat = [&](int j) { return REGS ? j : j ^ (j >> 3 & pmask); };
-  auto cat = [&](int j) { return REGS ? j : j ^ (j >> 3 & cmask); };
+  const int pmask = SWAP && (H + gp - 1) / gp % 8 == 0 ? 7 : 0, cmask = SWAP && (k * H + gc - 1) / gc % 8 == 0 ? 7 : 0;
+  auto pat = [&](int j) { return !SWAP ? j : j ^ (j >> 3 & pmask); };
+  auto cat = [&](int j) { return !SWAP ? j : j ^ (j >> 3 & cmask); };
   {
     V1 a[REGS ? ScanPer<P>::n : 1];
     VecAcc<P, 1> x;
@@ -541,7 +541,7 @@ __device__ __forceinline__ void terminal_node(const LT& L, int H, int k, int dec
     }
     V1* mine = tid < gp ? ps : cp;
     const int mask = tid < gp ? pmask : cmask, begin = L.run.begin;
-    auto at = [&](int e) { return REGS ? a[REGS ? e : 0] : mine[(begin + e) ^ ((begin + e) >> 3 & mask)]; };
+    auto at = [&](int e) { return REGS ? a[REGS ? e : 0] : mine[!SWAP ? begin + e : (begin + e) ^ ((begin + e) >> 3 & mask)]; };
     scan_runs<P, 1, REGS>(at, L.run.cnt, red[tid >= gp], gtid, x);
     __syncthreads();
     if (tid < gp)
@@ -667,13 +667,14 @@ __global__ void __launch_bounds__(kTermThreads, 2) k_terminal(const GameDev* __r
 // A block takes up to eight nodes of one game, board table and kind one after the other: the table is
 // staged once, and each node's reach row lands (two buffers) while the node before is computed.  A
 // node is a chain of four block barriers with little between them, so what counts is how many chains
-// an SM holds: four blocks, which the scans' in-place form leaves room for (32 registers; 64 with the
+// an SM holds: four blocks (with pairs up to about 950 hands, three above, whose arrays fill its shared
+// memory), which the scans' in-place form leaves room for (32 registers; 64 with the
 // entries in registers hold two).  Pairs always run so (groups of two nodes a thread spilled, and
 // took 419 us a player on 256 rivers of 1,081 hands where this form takes 309); FP32 values where a
 // board table has few showdown nodes (see create_impl).  Measured, one player: 256 rivers, pairs, 309
-// us (four blocks; 317 three, 342 two); exact turn, pairs, 214; the 31,124-node flop of 513 hands,
-// FP32 values 158, pairs 275.
-template <typename P>
+// us (317 held to three blocks' registers, 342 with the entries in registers); exact turn, pairs, 214;
+// the 31,124-node flop of 513 hands, FP32 values 158, pairs 275.
+template <typename P, bool SWAP>
 __global__ void __launch_bounds__(kTermThreads, 4) k_terminal_run(const GameDev* __restrict__ games,
                                                             const Work* __restrict__ work,
                                                             const TermSrc* __restrict__ src,
@@ -697,8 +698,8 @@ __global__ void __launch_bounds__(kTermThreads, 4) k_terminal_run(const GameDev*
   __shared__ __align__(8) uint64_t bar[2];
   const uint16_t* tab = reinterpret_cast<const uint16_t*>(smt);  // [tt.len]
   V* rows = reinterpret_cast<V*>(smt + (size_t)tt.len * 2);       // [2][hstride]
-  V* CP = rows + 2 * stride;                                     // [k H + 1], in eights
-  V* Ps = CP + TermTab::round8(k * H + 1);                       // [H + 1], in eights
+  V* CP = rows + 2 * stride;                                     // [k H + 1], with SWAP in eights
+  V* Ps = CP + (SWAP ? TermTab::round8(k * H + 1) : k * H + 1);  // [H + 1]
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -745,7 +746,7 @@ __global__ void __launch_bounds__(kTermThreads, 4) k_terminal_run(const GameDev*
       __syncthreads();
     }
     V* out = dst + (size_t)n * stride;
-    terminal_node<P, false>(L, H, k, G.deck, show, board, u, q, tab, CP, Ps, [&](int h, V v) { out[h] = v; });
+    terminal_node<P, false, SWAP>(L, H, k, G.deck, show, board, u, q, tab, CP, Ps, [&](int h, V v) { out[h] = v; });
     __syncthreads();  // the row and the scan arrays are free
   }
 }
@@ -3323,6 +3324,11 @@ size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es)
   return hand_smem_bytes(n_nodes, n_levels, rows_max, W, es);
 }
 
+bool scans_in_eights(int n_hands, int hand_size, size_t es) {
+  const int gp = es == 4 ? TermRun<Single>::gp : TermRun<Pairs>::gp, gc = kTermThreads - gp;
+  return (n_hands + gp - 1) / gp % 8 == 0 || (hand_size * n_hands + gc - 1) / gc % 8 == 0;
+}
+
 size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv, bool runs) {
   const TermTab tt(n_hands, hand_size, deck);
   const size_t scan = (size_t)(hand_size * n_hands + 1 + n_hands + 1);
@@ -3378,7 +3384,8 @@ static cudaError_t configure_precision() {
   cudaError_t e = configure_hand<P, true>();
   if (e == cudaSuccess) e = configure_hand<P, false>();
   if (e == cudaSuccess) e = configure_one(k_terminal<P>, 200 * 1024);
-  if (e == cudaSuccess) e = configure_one(k_terminal_run<P>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal_run<P, false>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_terminal_run<P, true>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_average_rows<P>, 0);
   if (e == cudaSuccess) e = configure_one(k_tile<kModeInit, P, false, false>, kTileSmem);
   if (e == cudaSuccess) e = configure_one(k_tile<kModeUpdate, P, false, false>, kTileSmem);
@@ -3648,7 +3655,8 @@ int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stre
   const bool single = c.precision == kPrecisionSingle;
   cudaError_t e;
   if (c.n_term_runs > 0)
-    e = single ? run(k_terminal_run<Single>) : run(k_terminal_run<Pairs>);
+    e = c.term_swap ? (single ? run(k_terminal_run<Single, true>) : run(k_terminal_run<Pairs, true>))
+                    : (single ? run(k_terminal_run<Single, false>) : run(k_terminal_run<Pairs, false>));
   else if (c.term_nv > 1)
     e = c.term_nv == 4 ? vec(k_terminal_vec<4>) : vec(k_terminal_vec<2>);
   else

@@ -260,6 +260,7 @@ struct LaunchCtx {
   const TermGroup* term_groups;   // device (term_nv > 1)
   const Work* term_runs;       // device [n_term_runs]: (first entry of term_work, count), one block's (run form)
   int n_term_runs;
+  bool term_swap;              // run form: scan arrays with entries swapped within eights
   const Work* term_segments;      // device [n_term_segments]: (first group, count), one block's
   int n_term_segments;
   const TermSrc* term_src;     // device [n_term_work]: reach rows of each terminal
@@ -323,6 +324,8 @@ int launch_average_rows(const LaunchCtx& c, void* stream);
 int wide_launch_count(const LaunchCtx& c, int which, int player_mask, int advance);
 int hand_kernel_smem_limit();
 // Shared memory of one block of the terminal launch for one game (nv: LaunchCtx::term_nv; runs: its run form).
+// Whether a thread's run of either scan of the run form is a multiple of eight entries.
+bool scans_in_eights(int n_hands, int hand_size, size_t es);
 size_t terminal_smem_size(int n_hands, int hand_size, int deck, int hstride, size_t es, int nv, bool runs);
 // Shared memory the per-hand kernel needs to stage one game (es = bytes per value).
 size_t hand_smem_size(int n_nodes, int n_levels, int rows_max, int W, size_t es);
