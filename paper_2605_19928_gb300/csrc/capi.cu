@@ -657,6 +657,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   // Resident schedule: one block per SM holds a chunk's state of both players beside a terminal
   // node's board table, and every chunk has a block.
   size_t res_term = 0, res_hand = 0;
+  bool res_ahead = false;  // match_ahead for a player of some tree
   if (resident) {
     for (int g = 0; g < n_games; ++g) {
       const HostGame& h = t->host[g];
@@ -664,6 +665,9 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
       res_term = std::max(res_term, resident_term_size(h.n_hands, h.hand_size, h.deck, h.hstride, es));
       res_hand = std::max(res_hand, resident_hand_size((int)tile_tabs[g].size() / 8, (int)h.nodes.size(), rows_max, chunk[g], es));
       tabled = tabled && !tile_tabs[g].empty();
+      if (tile_tabs[g].empty()) continue;
+      const TileHead* head = reinterpret_cast<const TileHead*>(tile_tabs[g].data());
+      res_ahead = res_ahead || (es == 8 && std::max(head->flevels[0], head->flevels[1]) > 2);
     }
     const int per_sm = tabled && res_term + res_hand <= 200 * 1024 ? resident_blocks_per_sm(o.precision, res_term + res_hand) : 0;
     const long chunks = chunks_of(chunk[0]);  // reads the handle's games
@@ -1076,6 +1080,7 @@ int create_impl(const cfr_game_spec* specs, int n_games, const cfr_solver_opts* 
   c.resident_sync = t->d_res_sync;
   if (resident) {
     c.resident_term = (unsigned)res_term;
+    c.resident_ahead = res_ahead;
     c.smem_resident = res_term + res_hand;
     const long items = (long)term_work.size() * (o.alternating ? 1 : 2);
     c.resident_grid = (int)std::max<long>(chunk_work.size(), std::min<long>(items, n_sms));

@@ -2190,7 +2190,10 @@ __device__ __forceinline__ bool resident_terminal(const GameDev* __restrict__ ga
 // finished; the last block to finish resets both and advances *iter and sync[2] by n_iters.  The
 // stamps are counted on the device, over the handle's life, so that a launch replayed from a
 // captured graph takes new ones too; every word is rewritten every iteration, so they may wrap.
-template <typename P>
+// AHEAD: some tree of the handle has its regrets matched ahead of the walk (match_ahead).  Handles without
+// such trees are faster without that code (river of 789 hands and two levels with pairs 23.7 -> 22.1 us an
+// iteration).
+template <typename P, bool AHEAD>
 __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
     const GameDev* __restrict__ games, const Work* __restrict__ chunk_work, int n_chunk_work,
     const Work* __restrict__ term_work, const TermSrc* __restrict__ term_src, int n_term_work, int alternating,
@@ -2355,7 +2358,7 @@ __global__ void __launch_bounds__(kTermThreads, 1) k_resident(
           };
           if (tid < W) put_reach(0, srch[p][0]);
           auto put_sigma = [&](int r, V y) { ssg[p][r << wlog] = y; };
-          if (match_ahead<P>(T)) {
+          if (AHEAD && match_ahead<P>(T)) {
             tile_match_all<P>(T, ssg[p], slot, nslots, [](int, V) {});
             __syncthreads();
             if (tid < T.group) tile_reach_matched<P>(T, srch[p], ssg[p], put_reach);
@@ -3351,11 +3354,15 @@ size_t resident_hand_size(int tab16, int n_nodes, int rows_max, int W, size_t es
   return resident_hand_bytes(tab16, n_nodes, rows_max, W, es);
 }
 int resident_blocks_per_sm(int precision, size_t smem) {
-  int n = 0;
-  const cudaError_t e =
-      precision == kPrecisionSingle
-          ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_resident<Single>, kTermThreads, smem)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_resident<Pairs>, kTermThreads, smem);
+  int n = 0, m = 0;
+  cudaError_t e;
+  if (precision == kPrecisionSingle) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_resident<Single, false>, kTermThreads, smem);
+  } else {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_resident<Pairs, false>, kTermThreads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_resident<Pairs, true>, kTermThreads, smem);
+    n = n < m ? n : m;
+  }
   return e == cudaSuccess ? n : 0;
 }
 
@@ -3399,7 +3406,8 @@ static cudaError_t configure_precision() {
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 1>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_stream_update<P, 2>, 200 * 1024);
   if (e == cudaSuccess) e = configure_one(k_current_rows<P>, 0);
-  if (e == cudaSuccess) e = configure_one(k_resident<P>, 200 * 1024);
+  if (e == cudaSuccess) e = configure_one(k_resident<P, false>, 200 * 1024);
+  if (e == cudaSuccess && std::is_same<P, Pairs>::value) e = configure_one(k_resident<Pairs, true>, 200 * 1024);
   return e;
 }
 
@@ -3670,7 +3678,7 @@ int launch_terminal(const LaunchCtx& c, int player_mask, int use_bar, void* stre
 
 // One cooperative launch: every block is resident at once, which the grid barriers need
 // (the launch fails rather than run a grid that does not fit).
-template <typename P>
+template <typename P, bool AHEAD>
 static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c.resident_grid);
@@ -3682,14 +3690,15 @@ static cudaError_t launch_resident_p(const LaunchCtx& c, int n_iters, void* stre
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_resident<P>, c.games, c.chunk_work, c.n_chunk_work, c.term_work,
+  return cudaLaunchKernelEx(&cfg, k_resident<P, AHEAD>, c.games, c.chunk_work, c.n_chunk_work, c.term_work,
                             c.term_src, c.n_term_work, c.alternating, n_iters, c.iter,
                             c.disc, c.variant, c.resident_sync, c.err, c.resident_term);
 }
 
 int launch_resident(const LaunchCtx& c, int n_iters, void* stream) {
-  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single>(c, n_iters, stream)
-                                                        : launch_resident_p<Pairs>(c, n_iters, stream);
+  const cudaError_t e = c.precision == kPrecisionSingle ? launch_resident_p<Single, false>(c, n_iters, stream)
+                        : c.resident_ahead              ? launch_resident_p<Pairs, true>(c, n_iters, stream)
+                                                        : launch_resident_p<Pairs, false>(c, n_iters, stream);
   if (e != cudaSuccess) {
     fprintf(stderr, "pcfr: launch of k_resident failed: %s\n", cudaGetErrorString(e));
     return -1;

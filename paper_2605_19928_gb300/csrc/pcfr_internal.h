@@ -308,6 +308,7 @@ struct LaunchCtx {
   int resident_grid;           // blocks of the cooperative launch (>= n_chunk_work)
   size_t smem_resident;        // its dynamic shared memory: terminal region, then hand region
   unsigned resident_term;      // bytes of the terminal region
+  bool resident_ahead;         // some tree's regrets are matched ahead of the walk (with pairs)
   unsigned* resident_sync;     // device [3]: barrier arrivals, blocks finished (zero between launches), the last stamp used
   int alternating;
 };
